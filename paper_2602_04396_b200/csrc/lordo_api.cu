@@ -1,4 +1,5 @@
 // Host layer of the LoRDO hot path: context, workspace carving, launch plans, the C ABI.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -14,8 +15,9 @@ using namespace lordo;
 namespace {
 
 constexpr int kMaxK = 64;
+constexpr long long kPairs = 74;  // CTA pairs that the work of a refresh is planned for (148 SMs)
 
-enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_NORM = 6, ST_EIG = 7 };
+enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_NORM = 6, ST_EIG = 7, ST_GRAM = 8 };
 enum Phase { PH_SUBSPACE = 0, PH_ROTATE = 1, PH_COMMIT = 2 };
 
 // One launch of the refresh / init / inner-step plans. The entries it works on are a contiguous
@@ -42,6 +44,7 @@ struct SlotBuilder {
     std::vector<ConvProblem> cv;
     std::vector<NormProblem> nm;
     std::vector<EigProblem> eg;
+    std::vector<GramProblem> gr;
   };
   std::vector<Slot> slots;
   size_t cur = 0;
@@ -93,6 +96,7 @@ struct lordo_ctx {
   ConvProblem* d_convs = nullptr;
   NormProblem* d_norms = nullptr;
   EigProblem* d_eigs = nullptr;
+  GramProblem* d_grams = nullptr;
   float* d_scratch = nullptr;
   long long total_chunks = 0, total_mom_tiles = 0, total_wblks = 0, total_sblks = 0;
 
@@ -132,6 +136,7 @@ struct lordo_ctx {
   std::vector<ConvProblem> h_convs;
   std::vector<NormProblem> h_norms;
   std::vector<EigProblem> h_eigs;
+  std::vector<GramProblem> h_grams;
   struct SketchBufs {
     __nv_bfloat16 *om16 = nullptr, *pn16 = nullptr, *zq16 = nullptr;
     // hi|lo planes of the tensor-core QR and rotation (null when those run in fp32)
@@ -287,6 +292,24 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   // every step of the refresh is one launch over a whole group.
   constexpr size_t kRefreshScratchFloats = size_t(1) << 33;  // 32 GiB: fewer, fuller launches (a launch of the factorisation kernel takes as long for 64 matrices as for 148)
   std::vector<size_t> mat_scratch(n_mats);
+  // Ranges of k that the two sums of a tensor-core Gram matrix are dealt out in (`gram_sum_kernel` adds them).
+  // A Gram matrix has only ceil(r / 256) output tiles, so without ranges a launch over few matrices leaves most
+  // of the CTA pairs idle (7 matrices of r = 256: 265 us in 7 pairs, 30 us in 70): the count with the shortest
+  // last wave is taken, a range costing about four steps of 64 k on top of its own (start of the pipeline,
+  // epilogue). A range is also kept below 64 steps, because the tensor cores' fp32 accumulation truncates and
+  // the ranges meet in fp64.
+  long long gram_tiles = 0;
+  for (int i = 0; i < n_mats; ++i) gram_tiles += 2ll * (local ? K : 1) * ((cfg.mats[i].r + 255) / 256);
+  auto gram_ranges = [&](long long rows) {
+    const long long steps = 2 * ((rows + 63) / 64);
+    int best = 1;
+    long long best_cost = -1;
+    for (int ns = (int)((steps + 63) / 64); ns <= 32 && (ns == 1 || steps / ns >= 4); ++ns) {
+      const long long cost = ((gram_tiles * ns + kPairs - 1) / kPairs) * ((steps + ns - 1) / ns + 4);
+      if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = ns; }
+    }
+    return best;
+  };
   std::vector<int> group_of(n_mats);
   size_t scratch_floats = 0;
   {
@@ -308,6 +331,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         // (per batch entry) and the two moment operands of every worker in two
         per += 3 * (size_t)maxd * a.r / 2 + pm * a.r + 7 * (size_t)a.r * a.r / 2 + 128;
         states16 = 2 * (size_t)K * a.r * ln + 64;
+        per += 2 * (size_t)std::max(gram_ranges(pm), gram_ranges(ln)) * a.r * a.r;
       }
       mat_scratch[i] = nb * per + states16;
       if (acc > 0 && acc + mat_scratch[i] > kRefreshScratchFloats) { ++grp; acc = 0; }
@@ -428,7 +452,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
 
   // ---------------- launch plans ----------------
   std::vector<GemmProblem>& P = c->h_probs;
-  P.clear(); c->h_chols.clear(); c->h_rands.clear(); c->h_copies.clear(); c->h_sks.clear(); c->h_convs.clear(); c->h_norms.clear(); c->h_eigs.clear(); c->h_diag.clear();
+  P.clear(); c->h_chols.clear(); c->h_rands.clear(); c->h_copies.clear(); c->h_sks.clear(); c->h_convs.clear(); c->h_norms.clear(); c->h_eigs.clear(); c->h_grams.clear(); c->h_diag.clear();
   c->h_skbufs.assign(n_mats, lordo_ctx::SketchBufs());
   const bool tc_sketch = c->tc && c->tma && cfg.oversample == 0;  // products of the refresh on tensor cores
   auto gemm_prob = [&](int M, int N, int Kd, const Operand& A, const Operand& B, const Operand* B2, const Epilogue& ep) {
@@ -474,6 +498,9 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       } else if (st.type == ST_EIG) {
         st.first = (long long)c->h_eigs.size(); st.count = (int)sl.eg.size(); st.r_max = 0;
         for (const EigProblem& x : sl.eg) { if (x.w > st.r_max) st.r_max = x.w; c->h_eigs.push_back(x); }
+      } else if (st.type == ST_GRAM) {
+        st.first = (long long)c->h_grams.size(); st.count = (int)sl.gr.size(); st.tiles = 0;
+        for (GramProblem& x : sl.gr) { const long long b = (x.r + 31) / 32; x.blk_start = st.tiles; st.tiles += b * (b + 1) / 2; c->h_grams.push_back(x); }
       } else if (st.type == ST_NORM) {
         st.first = (long long)c->h_norms.size(); st.count = (int)sl.nm.size(); st.tiles = 0;
         for (NormProblem& x : sl.nm) { x.blk_start = st.tiles; st.tiles += (x.r + 31) / 32; c->h_norms.push_back(x); }
@@ -607,6 +634,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       c->h_skbufs[i].om16 = om16; c->h_skbufs[i].pn16 = pn16; c->h_skbufs[i].zq16 = zq16;
       // tensor-core QR and rotation: bf16 planes, plane p of batch entry b at index p * nb + b
       __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr, *uh16 = nullptr, *wr16 = nullptr;
+      float* gpart = nullptr;  // partial sums of the Gram matrices
       if (tc_sketch) {
         auto take16 = [&](size_t floats) { __nv_bfloat16* p16 = reinterpret_cast<__nv_bfloat16*>(s); s += floats + 16; return p16; };
         x16 = take16(3 * (size_t)nb * maxd * r / 2);
@@ -616,6 +644,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         sq16 = take16((size_t)nb * r * r);
         uh16 = take16((size_t)K * r * n);
         wr16 = take16((size_t)K * r * n);
+        gpart = s; s += (size_t)nb * 2 * std::max(gram_ranges(m), gram_ranges(n)) * r * r;
         lordo_ctx::SketchBufs& kb = c->h_skbufs[i];
         kb.x16 = x16; kb.rinv16 = rinv16; kb.phl = phl; kb.rt16 = rt16; kb.sq16 = sq16; kb.uh16 = uh16; kb.wr16 = wr16;
       }
@@ -638,7 +667,9 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         std::memset(&sp, 0, sizeof(sp));
         sp.M = (int)Mo; sp.Kd = (int)Kd; sp.r = r; sp.r_n = (r + 15) / 16 * 16;
         sp.a_mn = a_mn; sp.a_c2 = a_b; sp.a_pl = a_nb; sp.b_c2 = b_b; sp.b_pl = b_nb;
-        sp.split = np; sp.c_trans = c_trans;
+        sp.c_trans = c_trans;
+        // 3 planes: (0,0) (0,1) (1,0) (1,1) (0,2) (2,0); 2 planes: the first three
+        sp.pa = 0x201100u; sp.pb = 0x021010u; sp.j0 = 0; sp.j1 = (np == 3 ? 6 : 3) * (int)((Kd + 63) / 64);
         sp.map_a = map_a; sp.map_b = map_b; sp.C = C; sp.ldc = ldc;
         sl.sk.push_back(sp);
       };
@@ -661,8 +692,21 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           float* dst = pass == 0 ? T : O;
           const long long sd = pass == 0 ? st : so;
           conv_split(sb, phase, src, ss, x16, rows * r, 3);
+          const int ns = gram_ranges(rows), steps = 2 * (int)((rows + 63) / 64);
           SlotBuilder::Slot& g = sb.next(ST_SKETCH, phase);
-          for (int b = 0; b < nb; ++b) sk_split(g, 1, x_sw, b, nb, x_sw, b, nb, r, rows, gram + (long long)b * r * r, r, 0, 3);
+          for (int b = 0; b < nb; ++b)
+            for (int x = 0; x < 2 * ns; ++x) {  // the smaller pair of each sum first: less is truncated
+              sk_split(g, 1, x_sw, b, nb, x_sw, b, nb, r, rows, gpart + (size_t)(b * 2 * ns + x) * r * r, r, 0, 3);
+              SkProblem& sp = g.sk.back();
+              sp.pa = x < ns ? 0x01u : 0x00u; sp.pb = x < ns ? 0x01u : 0x12u;
+              sp.j0 = (int)((long long)steps * (x % ns) / ns); sp.j1 = (int)((long long)steps * (x % ns + 1) / ns);
+            }
+          SlotBuilder::Slot& gs = sb.next(ST_GRAM, phase);
+          for (int b = 0; b < nb; ++b) {
+            GramProblem gp;
+            gp.part = gpart + (size_t)b * 2 * ns * r * r; gp.gram = gram + (long long)b * r * r; gp.blk_start = 0; gp.r = r; gp.ns = ns;
+            gs.gr.push_back(gp);
+          }
           SlotBuilder::Slot& ch = sb.next(ST_CHOL, phase);
           for (int b = 0; b < nb; ++b) {
             CholProblem cp;
@@ -693,7 +737,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         for (int b = 0; b < nb; ++b) {
           SkProblem sp;
           std::memset(&sp, 0, sizeof(sp));
-          sp.M = (int)Mo; sp.Kd = (int)Kd; sp.r = r; sp.r_n = (r + 15) / 16 * 16;
+          sp.M = (int)Mo; sp.Kd = (int)Kd; sp.r = r; sp.r_n = (r + 15) / 16 * 16; sp.j1 = (int)((Kd + 63) / 64);
           const int st_mn = a_mn ^ sd;  // how the stored signal lies with respect to this product
           sp.a_mn = st_mn; sp.a_c2 = local ? b : 0; sp.b_c2 = b;
           TmaMatMaps* mm = c->d_maps + i;
@@ -898,6 +942,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   c->d_convs = cv.take<ConvProblem>(c->h_convs.size() + 1);
   c->d_norms = cv.take<NormProblem>(c->h_norms.size() + 1);
   c->d_eigs = cv.take<EigProblem>(c->h_eigs.size() + 1);
+  c->d_grams = cv.take<GramProblem>(c->h_grams.size() + 1);
   c->d_diag = cv.take<DiagProblem>(c->h_diag.size() + 1);
 
   c->last_G.assign(n_mats, nullptr);
@@ -977,6 +1022,10 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       launch_colnorm_grouped(c->d_norms + s.first, s.count, s.tiles, st);
       c->launches += 1;
       return check_launch(c, "colnorm");
+    case ST_GRAM:
+      launch_gram_sum(c->d_grams + s.first, s.count, s.tiles, st);
+      c->launches += 1;
+      return check_launch(c, "gram_sum");
     case ST_COPY:
       launch_copy_grouped(c->d_copies + s.first, s.count, s.tiles, st);
       c->launches += 1;
@@ -1119,6 +1168,7 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
   if (!c->h_convs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_convs, c->h_convs.data(), sizeof(ConvProblem) * c->h_convs.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_norms.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_norms, c->h_norms.data(), sizeof(NormProblem) * c->h_norms.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_eigs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_eigs, c->h_eigs.data(), sizeof(EigProblem) * c->h_eigs.size(), cudaMemcpyHostToDevice, st));
+  if (!c->h_grams.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_grams, c->h_grams.data(), sizeof(GramProblem) * c->h_grams.size(), cudaMemcpyHostToDevice, st));
   INIT_CUDA(cudaMemsetAsync(c->d_status, 0, 256, st));
   if (c->tc) {
     if (!c->tma) INIT_CUDA(tc_configure(c->tc_rn_max, c->tc_rk_max));  // register-staged kernels (fp32 storage)

@@ -223,6 +223,17 @@ struct ConvProblem {
 };
 void launch_convert_grouped(const ConvProblem* probs, int nprobs, long long total_blocks, const GemmScalars& sc, cudaStream_t st);
 
+// Gram matrix of a tensor-core QR from its partial products: gram = sum_s S_s + sum_s (T_s + T_s^T), the S
+// and T of `ns` ranges of k each, all r x r, S first. With X ~ p0 + p1 + p2, S = p1^T p1 + p0^T p0 and
+// T = p0^T p2 + p0^T p1, so that four of the six pairs of planes are multiplied.
+struct GramProblem {
+  const float* part;
+  float* gram;
+  long long blk_start;
+  int r, ns;
+};
+void launch_gram_sum(const GramProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
+
 // Columns of X [rows][r] scaled to unit length (sums of squares in fp64), one block per 32 columns.
 // The tensor-core Gram matrix underestimates its diagonal (an fp32 accumulator that truncates, over
 // thousands of positive addends), which leaves every column of Q a few 1e-5 too long; the
@@ -241,7 +252,10 @@ struct SkProblem {
   long long tile_start;      // first 256-row tile (128 rows per CTA of a pair) of this problem within the launch
   int M, Kd, r, r_n;
   int a_mn, a_c2, b_c2;      // third TMA coordinate (worker / batch index) of A and of B
-  int split;                 // 0: one product; 2 or 3: operands split in that many bf16 planes, 3 or 6 passes over k
+  // operands split in bf16 planes: the k loop runs over pairs of planes, pair s being nibble s of pa (plane of A)
+  // and of pb (plane of B); a problem covers the steps [j0, j1) of 64 k of the pairs laid end to end
+  unsigned pa, pb;
+  int j0, j1;
   int a_pl, b_pl;            // third-coordinate distance between the planes of A and of B
   int c_trans, pad;          // 1: C is stored transposed, C[col * ldc + row]
   const void* map_a;         // 64 x 64 swizzled boxes (a_mn) or 64 x 128 swizzled boxes

@@ -338,6 +338,55 @@ __global__ void __launch_bounds__(256) convert_grouped_kernel(const ConvProblem*
   }
 }
 
+// One block per 32 x 32 block on or below the diagonal, which it also mirrors; the partial products meet in
+// fp64, so that what is left of the tensor cores' truncating accumulation is that of one range of k.
+// Bound by the reads of the partial products: r = 512, 16 matrices, 2 x 8 ranges in 21 us.
+__global__ void __launch_bounds__(256) gram_sum_kernel(const GramProblem* __restrict__ probs, int nprobs) {
+  __shared__ float tt[32][33];
+  const long long blk = blockIdx.x;
+  int lo = 0, hi = nprobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (probs[mid].blk_start <= blk) lo = mid; else hi = mid - 1;
+  }
+  const GramProblem pb = probs[lo];
+  const int r = pb.r;
+  const size_t rr = (size_t)r * r;
+  int bi = 0, rest = (int)(blk - pb.blk_start);
+  while (rest > bi) rest -= ++bi;  // block row bi has bi + 1 blocks
+  const int bj = rest;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int s = 0; s < pb.ns; ++s) {
+    const float* S = pb.part + s * rr;
+    const float* T = pb.part + (pb.ns + s) * rr;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = bj * 32 + y + 8 * q, j = bi * 32 + x;  // the mirrored block of T
+      tt[y + 8 * q][x] = (i < r && j < r) ? T[(size_t)i * r + j] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = bi * 32 + y + 8 * q, j = bj * 32 + x;
+      if (i < r && j < r) acc[q] += (double)S[(size_t)i * r + j] + ((double)T[(size_t)i * r + j] + (double)tt[x][y + 8 * q]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = bi * 32 + y + 8 * q, j = bj * 32 + x;
+    tt[y + 8 * q][x] = (float)acc[q];
+    if (i < r && j < r && (bi != bj || j <= i)) pb.gram[(size_t)i * r + j] = (float)acc[q];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = bj * 32 + y + 8 * q, j = bi * 32 + x;
+    if (i < r && j < r && (bi != bj || j > i)) pb.gram[(size_t)i * r + j] = tt[x][y + 8 * q];
+  }
+}
+
 __global__ void __launch_bounds__(256) colnorm_grouped_kernel(const NormProblem* __restrict__ probs, int nprobs) {
   __shared__ double part[8][32];
   const long long blk = blockIdx.x;
@@ -440,6 +489,9 @@ void launch_fill_random_grouped(const RandProblem* probs, int nprobs, long long 
 }
 void launch_convert_grouped(const ConvProblem* probs, int nprobs, long long total_blocks, const GemmScalars& sc, cudaStream_t st) {
   convert_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs, sc.inv_bc1, sc.inv_bc2, sc.bc1, sc.bc2);
+}
+void launch_gram_sum(const GramProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
+  gram_sum_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
 }
 void launch_colnorm_grouped(const NormProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
   colnorm_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);

@@ -723,7 +723,6 @@ constexpr int kSMaxStages = 4;
 constexpr uint32_t kSSmemBytes = 196608 + 1024;  // 4 stages of A 16 KB | E 16 KB | B 16 KB, or 3 with 32 KB of B
 constexpr int kSThreads = (2 + 4 + 4) * 32;  // TMA, MMA, 4 transform warps, 4 epilogue warps
 constexpr uint32_t kIdescBMajorMN = 1u << 16;
-__device__ __forceinline__ int sk_passes(int split) { return split == 3 ? 6 : (split == 2 ? 3 : 1); }
 
 __device__ __forceinline__ int find_sk(const SkProblem* __restrict__ probs, int nprobs, long long tile) {
   int lo = 0, hi = nprobs - 1;
@@ -774,12 +773,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
         const int n_lo = pr->r_n < 256 ? pr->r_n : 256, n_hi = pr->r_n - n_lo;
         const int c_lo = (int)rank * (n_lo / 2), c_hi = 256 + (int)rank * (n_hi / 2);
         const int nbox_lo = (n_lo / 2 + 63) / 64, nbox_hi = (n_hi / 2 + 63) / 64;
-        const int nkb = nkb1 * sk_passes(pr->split);
         const bool has_e = pr->map_e != nullptr;
         const uint32_t tx = 16384u + (has_e ? 16384u : 0u) + (uint32_t)(nbox_lo + nbox_hi) * 8192u;
-        for (int j = 0; j < nkb; ++j, ++it) {
-          const int seg = j / nkb1, kb = j - seg * nkb1;  // plane pairs (0,0) (0,1) (1,0) (1,1) (0,2) (2,0)
-          const int a_c2 = pr->a_c2 + ((0x201100 >> (4 * seg)) & 3) * pr->a_pl, b_c2 = pr->b_c2 + ((0x021010 >> (4 * seg)) & 3) * pr->b_pl;
+        const int j1 = pr->j1;
+        int seg = pr->j0 / nkb1, kb = pr->j0 - seg * nkb1;
+        for (int j = pr->j0; j < j1; ++j, ++it, ++kb) {
+          if (kb == nkb1) { kb = 0; ++seg; }
+          const int a_c2 = pr->a_c2 + (int)((pr->pa >> (4 * seg)) & 15u) * pr->a_pl, b_c2 = pr->b_c2 + (int)((pr->pb >> (4 * seg)) & 15u) * pr->b_pl;
           const int s = it % ST;
           ok = mbar_wait(&empty_bar[s], ((it / ST) & 1u) ^ 1u, status);
           if (!ok) break;
@@ -810,7 +810,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
       const uint32_t af0 = cluster_addr(&acc_full[0], 0), af1 = cluster_addr(&acc_full[0], 1);
       for (long long tile = tile_first; tile < total_tiles && ok; tile += tile_step, ++si) {
         const SkProblem* __restrict__ pr = probs + find_sk(probs, nprobs, tile);
-        const int nkb = ((pr->Kd + 63) / 64) * sk_passes(pr->split);
+        const int nkb = pr->j1 - pr->j0;
         const bool a_mn = pr->a_mn != 0;
         const uint32_t n_lo = pr->r_n < 256 ? (uint32_t)pr->r_n : 256u, n_hi = (uint32_t)pr->r_n - n_lo;
         const uint32_t majors = kIdescBMajorMN | (a_mn ? kIdescAMajorMN : 0u);
@@ -842,7 +842,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
     const uint32_t xf = cluster_addr(&xform_bar[0], 0);
     for (long long tile = tile_first; tile < total_tiles && ok; tile += tile_step) {
       const SkProblem* __restrict__ pr = probs + find_sk(probs, nprobs, tile);
-      const int nkb = ((pr->Kd + 63) / 64) * sk_passes(pr->split);
+      const int nkb = pr->j1 - pr->j0;
       const bool has_e = pr->map_e != nullptr;
       const float c = pr->cptr ? *pr->cptr : 1.f;
       for (int kb = 0; kb < nkb; ++kb, ++it) {

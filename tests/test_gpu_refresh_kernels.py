@@ -1,0 +1,28 @@
+"""Edges of the kernels of the tensor-core refresh, against the oracle on the CUDA path's own state."""
+import pytest
+
+from paper_2602_04396_b200 import synth
+from tests import harness as hz
+from tests.harness import RunSpec
+
+pytestmark = pytest.mark.gpu
+
+ANGLE_TOL, ORTH_TOL, ROT_TOL = 1e-3, 1e-5, 16 * 2.0 ** -16  # as for the other refresh tests
+
+
+def _refresh(m, n, r, K=1, variant=1, grad="gauss", q=0, **kw):
+    wl = synth.Workload(f"t{m}x{n}r{r}", ((m, n, r),), K=K, H=1, rounds=2, grad=grad, clip_rho=30.0, power_iters=q,
+                        w_dtype="bf16", g_dtype="bf16", e_dtype="bf16", **kw)
+    opt, _, worst = hz.run_lockstep_refresh(RunSpec(wl, variant=variant, form=1, lr=0.01, check_mode=0, eps=0.05), rounded_signal=True)
+    assert opt.poll_status() == 0
+    opt.close()
+    return worst
+
+
+@pytest.mark.parametrize("shape", [(64, 72, 8), (1096, 264, 8), (2056, 520, 264), (600, 4104, 40), (1544, 768, 512)])
+def test_gram_in_ranges_of_k(shape):
+    """Gram matrices in one range of k, in many, with a ragged last step and at both tile counts (r up to 256
+    and above). Gaussian noise as the signal: the sketch has exact operands, only the QR is left to differ."""
+    w = _refresh(*shape)
+    assert w["P_angle"] < ANGLE_TOL and w["P_orth"] < ORTH_TOL, w
+    assert w["rot_u"] < ROT_TOL and w["rot_v"] < 2 * ROT_TOL, w
