@@ -999,7 +999,7 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       c->launches += 1;
       return check_launch(c, "gemm");
     case ST_CHOL:
-      launch_chol_inverse(c->d_chols + s.first, s.count, s.r_max, c->d_status, st);
+      launch_chol_inverse(c->d_chols + s.first, s.count, s.r_max, c->sm_count, c->d_status, st);
       c->launches += 1;
       return check_launch(c, "chol_inverse");
     case ST_RANDOM:
@@ -1170,6 +1170,12 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
   if (!c->h_eigs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_eigs, c->h_eigs.data(), sizeof(EigProblem) * c->h_eigs.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_grams.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_grams, c->h_grams.data(), sizeof(GramProblem) * c->h_grams.size(), cudaMemcpyHostToDevice, st));
   INIT_CUDA(cudaMemsetAsync(c->d_status, 0, 256, st));
+  {
+    int dev = 0;
+    INIT_CUDA(cudaGetDevice(&dev));
+    INIT_CUDA(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev));
+    INIT_CUDA(chol_configure());
+  }
   if (c->tc) {
     if (!c->tma) INIT_CUDA(tc_configure(c->tc_rn_max, c->tc_rk_max));  // register-staged kernels (fp32 storage)
     INIT_CUDA(cudaMemsetAsync(c->d_tc_bf16, 0, c->tc_bf16_bytes, st));
@@ -1178,9 +1184,6 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
     INIT_CUDA(cudaMemcpyAsync(c->d_tc_prep, c->h_prep.data(), sizeof(TcPrep) * c->h_prep.size(), cudaMemcpyHostToDevice, st));
     INIT_CUDA(cudaMemcpyAsync(c->d_prep_start, c->h_prep_start.data(), 8 * c->h_prep_start.size(), cudaMemcpyHostToDevice, st));
     if (c->tma) {
-      int dev = 0;
-      INIT_CUDA(cudaGetDevice(&dev));
-      INIT_CUDA(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev));
       if (c->sm_count < 2) return bail(LORDO_ERR_UNSUPPORTED);  // the projection and the refresh products run as CTA pairs
       std::vector<TmaMatMaps> hm(nm);
       bool good = tmap_encoder() != nullptr;

@@ -170,7 +170,8 @@ struct CholProblem {
   float* rinv;
   int r, pad;
 };
-void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, unsigned* status, cudaStream_t st);
+void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, int sm_count, unsigned* status, cudaStream_t st);
+cudaError_t chol_configure();
 
 // Rayleigh-Ritz truncation of an oversampled basis: C = (Q^T S)(Q^T S)^T is w x w symmetric (w = r + p
 // <= 600). The kernel diagonalises C with a parallel cyclic Jacobi method (one CTA per problem) and

@@ -1,7 +1,8 @@
 """Edges of the kernels of the tensor-core refresh, against the oracle on the CUDA path's own state."""
 import pytest
+import torch
 
-from paper_2602_04396_b200 import synth
+from paper_2602_04396_b200 import lordo, synth
 from tests import harness as hz
 from tests.harness import RunSpec
 
@@ -26,3 +27,19 @@ def test_gram_in_ranges_of_k(shape):
     w = _refresh(*shape)
     assert w["P_angle"] < ANGLE_TOL and w["P_orth"] < ORTH_TOL, w
     assert w["rot_u"] < ROT_TOL and w["rot_v"] < 2 * ROT_TOL, w
+
+
+@pytest.mark.parametrize("r,count", [(8, 1), (32, 1), (40, 3), (256, 2), (264, 40), (504, 1), (296, 80), (512, 75)])
+def test_cholesky_panels_and_clusters(r, count):
+    """The factorisation behind P_0 = Q of a 2r x r integer matrix, against a QR in fp64: one panel, whole and
+    ragged panels, clusters of eight CTAs (few matrices) down to one (many), more blocks per CTA than it sums at
+    once (r = 296, 512 in one CTA). The condition of such a matrix is about 6 (the ratio of the edges of its
+    singular values): CholeskyQR2 in fp32 is off by a small multiple of 6^2 2^-24 = 2e-6."""
+    mats = [(2 * r, r, r)] * count
+    opt = lordo.Lordo(mats, 1, 1, [torch.zeros(2 * r, r)] * count, check_mode=0, seed=5)
+    assert opt.poll_status() == 0
+    for i in {0, count // 2, count - 1}:
+        q, t = torch.linalg.qr(lordo.fill_random(5, 1, i, 0, 0, 2 * r, r).double())
+        q = q * torch.sign(torch.diagonal(t))
+        assert ((opt.P[i].double() - q).norm() / q.norm()).item() < 1e-5
+    opt.close()
