@@ -577,7 +577,8 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       SlotBuilder::Slot& ch = sb.next(ST_CHOL, phase);
       for (int b = 0; b < nb; ++b) {
         CholProblem cp;
-        cp.gram = gram + (long long)b * r * r; cp.lwork = lw + (long long)b * r * r; cp.rinv = rinv + (long long)b * r * r; cp.r = r; cp.pad = 0;
+        std::memset(&cp, 0, sizeof(cp));
+        cp.gram = gram + (long long)b * r * r; cp.lwork = lw + (long long)b * r * r; cp.rinv = rinv + (long long)b * r * r; cp.r = r;
         ch.ch.push_back(cp);
       }
       SlotBuilder::Slot& ap = sb.next(ST_GEMM, phase, 0, 0, 0);
@@ -673,25 +674,20 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         sp.map_a = map_a; sp.map_b = map_b; sp.C = C; sp.ldc = ldc;
         sl.sk.push_back(sp);
       };
-      // CholeskyQR2 with the Gram matrices and the products with R^-1 on tensor cores, operands in three
-      // planes: the Gram matrix then carries fp32's rounding noise, which the breakdown threshold of the
+      // CholeskyQR2 of the matrix in x16 (three planes, left there by the epilogue of the product before it) with
+      // the Gram matrices and the products with R^-1 on tensor cores, operands in three planes: the Gram matrix then carries fp32's rounding noise, which the breakdown threshold of the
       // Cholesky step assumes
       // `last` = false: the result only serves as the right-hand side of the next product of the subspace
-      // iteration. Such a basis has to span the same subspace and be well conditioned, no more: one pass
+      // iteration, O16 in bf16. Such a basis has to span the same subspace and be well conditioned, no more: one pass
       // instead of two, which leaves it orthonormal to cond(X)^2 * 1e-7. Both products keep their three
       // planes: with fewer, the rounding of X (relative 2^-9 or 2^-17) times cond(X) would enter the
       // weak directions of the span (measured: angles of 0.03..0.1 rad with one plane on a sketch of
       // condition 1e3).
-      auto cholqr2_tc = [&](SlotBuilder& sb, int phase, float* X, long long sx, float* T, long long st, float* O, long long so, long long rows,
-                            bool last) {
+      auto cholqr2_tc = [&](SlotBuilder& sb, int phase, float* O, long long so, __nv_bfloat16* O16, long long rows, bool last) {
         const bool by_m = rows == m;
         const unsigned char* x_sw = by_m ? mmi->xm_sw : mmi->xn_sw;
         const unsigned char* x_kb = by_m ? mmi->xm_kb : mmi->xn_kb;
-        float* src = X; long long ss = sx;
         for (int pass = last ? 0 : 1; pass < 2; ++pass) {
-          float* dst = pass == 0 ? T : O;
-          const long long sd = pass == 0 ? st : so;
-          conv_split(sb, phase, src, ss, x16, rows * r, 3);
           const int ns = gram_ranges(rows), steps = 2 * (int)((rows + 63) / 64);
           SlotBuilder::Slot& g = sb.next(ST_SKETCH, phase);
           for (int b = 0; b < nb; ++b)
@@ -711,12 +707,18 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           for (int b = 0; b < nb; ++b) {
             CholProblem cp;
             cp.gram = gram + (long long)b * r * r; cp.lwork = lw + (long long)b * r * r; cp.rinv = rinv + (long long)b * r * r; cp.r = r; cp.pad = 0;
+            cp.rinv16 = rinv16 + (size_t)b * r * r; cp.plane = (long long)nb * r * r;
             ch.ch.push_back(cp);
           }
-          conv_split(sb, phase, rinv, (long long)r * r, rinv16, (long long)r * r, 3);
           SlotBuilder::Slot& ap = sb.next(ST_SKETCH, phase);
-          for (int b = 0; b < nb; ++b) sk_split(ap, 0, x_kb, b, nb, mmi->rinv_sw, b, nb, rows, r, dst + b * sd, r, 0, 3);
-          src = dst; ss = sd;
+          for (int b = 0; b < nb; ++b) {
+            // the first pass hands its result on as planes (in place), the last one as O
+            const bool to_planes = pass == 0, to_rhs = pass == 1 && !last;
+            sk_split(ap, 0, x_kb, b, nb, mmi->rinv_sw, b, nb, rows, r, to_planes || to_rhs ? nullptr : O + b * so, r, 0, 3);
+            SkProblem& sp = ap.sk.back();
+            if (to_planes) { sp.C16 = x16 + (size_t)b * rows * r; sp.plane = (long long)nb * rows * r; sp.planes = 3; }
+            if (to_rhs) { sp.C16 = O16 + (size_t)b * rows * r; sp.planes = 1; }
+          }
         }
         if (!last) return;
         SlotBuilder::Slot& nr = sb.next(ST_NORM, phase);  // the columns of Q back to unit length
@@ -727,12 +729,12 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         }
       };
       auto qr2 = [&](SlotBuilder& sb, int phase, float* X, long long sx, float* T, long long st, float* O, long long so, long long rows, int w,
-                     bool last = true) {
-        if (tc_sketch) cholqr2_tc(sb, phase, X, sx, T, st, O, so, rows, last);
+                     __nv_bfloat16* O16 = nullptr, bool last = true) {
+        if (tc_sketch) cholqr2_tc(sb, phase, O, so, O16, rows, last);
         else cholqr2(sb, phase, X, sx, T, st, O, so, rows, w, nb, gram, lw, rinv);
       };
-      // S * B on tensor cores: a_mn = 0 -> S rows are the output rows (Y = S B), 1 -> S^T B
-      auto sketch = [&](SlotBuilder& sb, int a_mn, unsigned char* map_b, float* C, long long cstride, long long Mo, long long Kd) {
+      // S * B on tensor cores, into the three planes of x16: a_mn = 0 -> S rows are the output rows (Y = S B), 1 -> S^T B
+      auto sketch = [&](SlotBuilder& sb, int a_mn, unsigned char* map_b, long long Mo, long long Kd) {
         SlotBuilder::Slot& sl = sb.next(ST_SKETCH, PH_SUBSPACE);
         for (int b = 0; b < nb; ++b) {
           SkProblem sp;
@@ -749,7 +751,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
             sp.map_a = st_mn ? mm->d_sw : mm->d_kb;
           }
           sp.map_b = map_b;
-          sp.C = C + (long long)b * cstride; sp.ldc = r;
+          sp.C16 = x16 + (size_t)b * Mo * r; sp.plane = (long long)nb * Mo * r; sp.planes = 3;
           sl.sk.push_back(sp);
         }
       };
@@ -774,7 +776,8 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       };
       if (warm) {  // block power iteration warm-started from the current basis
         if (tc_sketch && !local) convert(R, md.Delta, md.Delta16, (size_t)m * n);
-        add_copy(R, PH_SUBSPACE, Pn, md.P, (size_t)nb * m * r * sizeof(float));
+        if (tc_sketch) convert(R, md.P, pn16, (size_t)nb * m * r);
+        else add_copy(R, PH_SUBSPACE, Pn, md.P, (size_t)nb * m * r * sizeof(float));
       } else {
         {
           SlotBuilder::Slot& f = R.next(ST_RANDOM, PH_SUBSPACE);
@@ -788,30 +791,28 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         }
         if (tc_sketch) {  // Y = S Omega
           if (!local) convert(R, md.Delta, md.Delta16, (size_t)m * n);  // bf16 copy of the Global signal
-          sketch(R, 0, (c->d_maps + i)->om16, Ya, m * r, m, n);
+          sketch(R, 0, (c->d_maps + i)->om16, m, n);
         } else {
           SlotBuilder::Slot& g = R.next(ST_GEMM, PH_SUBSPACE, sd, 0, 0);
           for (int b = 0; b < nb; ++b) g.g.push_back(gemm_prob((int)m, rs, (int)n, signal(b), plain(Om + (long long)b * n * rs, rs), nullptr, store_epi(Ya + (long long)b * m * rs, rs)));
         }
-        qr2(R, PH_SUBSPACE, Ya, m * rs, Yb, maxd * rs, Pn, m * rs, m, rs, q == 0 || rr);
+        qr2(R, PH_SUBSPACE, Ya, m * rs, Yb, maxd * rs, Pn, m * rs, m, rs, pn16, q == 0 || rr);
       }
       for (int it = 0; it < q; ++it) {
         if (tc_sketch) {  // Z = S^T P'
-          convert(R, Pn, pn16, (size_t)nb * m * r);
-          sketch(R, 1, (c->d_maps + i)->pn16, Za, n * r, n, m);
+          sketch(R, 1, (c->d_maps + i)->pn16, n, m);
         } else {
           SlotBuilder::Slot& g = R.next(ST_GEMM, PH_SUBSPACE, 1 - sd, 0, 0);
           for (int b = 0; b < nb; ++b) g.g.push_back(gemm_prob((int)n, rs, (int)m, signal(b), plain(Pn + (long long)b * m * rs, rs), nullptr, store_epi(Za + (long long)b * n * rs, rs)));
         }
-        qr2(R, PH_SUBSPACE, Za, n * rs, Yb, maxd * rs, Zq, n * rs, n, rs, rr);
+        qr2(R, PH_SUBSPACE, Za, n * rs, Yb, maxd * rs, Zq, n * rs, n, rs, zq16, rr);
         if (tc_sketch) {  // Y = S Z
-          convert(R, Zq, zq16, (size_t)nb * n * r);
-          sketch(R, 0, (c->d_maps + i)->zq16, Ya, m * r, m, n);
+          sketch(R, 0, (c->d_maps + i)->zq16, m, n);
         } else {
           SlotBuilder::Slot& g = R.next(ST_GEMM, PH_SUBSPACE, sd, 0, 0);
           for (int b = 0; b < nb; ++b) g.g.push_back(gemm_prob((int)m, rs, (int)n, signal(b), plain(Zq + (long long)b * n * rs, rs), nullptr, store_epi(Ya + (long long)b * m * rs, rs)));
         }
-        qr2(R, PH_SUBSPACE, Ya, m * rs, Yb, maxd * rs, Pn, m * rs, m, rs, it == q - 1 || rr);
+        qr2(R, PH_SUBSPACE, Ya, m * rs, Yb, maxd * rs, Pn, m * rs, m, rs, pn16, it == q - 1 || rr);
       }
       if (rr) {
         // Rayleigh-Ritz truncation of the (r + p)-column basis Q (in Pn): Z = S^T Q, C = Z^T Z, the

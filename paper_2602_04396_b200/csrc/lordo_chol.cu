@@ -109,7 +109,10 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
     const int rows = r - b * kB < kB ? r - b * kB : kB;
     for (int e = tid; e < rows * b * (kB / 4); e += nt) {
       const int rr = e / (b * (kB / 4)), cc = e - rr * (b * (kB / 4));
-      *reinterpret_cast<float4*>(Z + (size_t)(b * kB + rr) * r + cc * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+      const size_t at = (size_t)(b * kB + rr) * r + cc * 4;
+      if (!pb.rinv16) *reinterpret_cast<float4*>(Z + at) = make_float4(0.f, 0.f, 0.f, 0.f);
+      else
+        for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(pb.rinv16 + p * pb.plane + at) = make_uint2(0u, 0u);
     }
   }
   float md = 0.f;
@@ -260,7 +263,19 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
 #pragma unroll
           for (int n = 0; n < 4; ++n) {
             const int col = 8 * n + 2 * (lane & 3);
-            if (col < kw) *reinterpret_cast<float2*>(out + col) = make_float2((float)c[n][0], (float)c[n][1]);
+            if (col >= kw) continue;
+            float x = (float)c[n][0], y = (float)c[n][1];
+            *reinterpret_cast<float2*>(out + col) = make_float2(x, y);
+            if (b <= k && pb.rinv16) {
+              __nv_bfloat16* o16 = pb.rinv16 + (size_t)row * r + k0 + col;
+#pragma unroll
+              for (int p = 0; p < 3; ++p, o16 += pb.plane) {
+                const uint32_t w = pack_bf16x2(x, y);
+                *reinterpret_cast<uint32_t*>(o16) = w;
+                x -= __uint_as_float(w << 16);
+                y -= __uint_as_float(w & 0xFFFF0000u);
+              }
+            }
           }
         }
       }

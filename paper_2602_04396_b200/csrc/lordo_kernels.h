@@ -163,11 +163,13 @@ void launch_error_norms(const MatDev* mats, int n_mats, int K, int e_dt, float* 
 
 // Cholesky factor of a batch of r x r Gram matrices and the inverse of its transpose:
 // gram = R^T R (R upper triangular, positive diagonal); rinv = R^-1, row-major, zeros below the
-// diagonal. lwork: r*r floats per problem. Strides in floats between batch entries.
+// diagonal. lwork: r*r floats per problem.
 struct CholProblem {
   const float* gram;
   float* lwork;
   float* rinv;
+  __nv_bfloat16* rinv16;  // R^-1 as three bf16 planes, `plane` elements apart, zeros below the diagonal; or null: then the zeros
+  long long plane;        // are written to rinv instead
   int r, pad;
 };
 void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, int sm_count, unsigned* status, cudaStream_t st);
@@ -249,6 +251,8 @@ void launch_colnorm_grouped(const NormProblem* probs, int nprobs, long long tota
 // Tensor-core sketch products of the refresh (lordo_tma.cu): C[M x r] (fp32) = S * B with the big
 // signal matrix S streamed by TMA as bf16 (optionally formed as c*G + E in shared memory) and
 // B [Kd][r] in bf16. a_mn = 1: S is stored [Kd][M] (the product S^T P'); 0: stored [M][Kd].
+// Where the result is only an operand of a later product it leaves the kernel as its bf16 planes: an fp32 store, a
+// pass to split it and a launch less per product (4096 x 11008, r = 512, K = 16: refresh 14.8 -> 13.6 ms).
 struct SkProblem {
   long long tile_start;      // first 256-row tile (128 rows per CTA of a pair) of this problem within the launch
   int M, Kd, r, r_n;
@@ -263,8 +267,11 @@ struct SkProblem {
   const void* map_e;         // same shape over E, or null
   const void* map_b;         // 64 x 64 swizzled boxes over B [batch][Kd][r]
   const float* cptr;         // scale of A when map_e is set (clip coefficient), else null
-  float* C;
-  long long ldc;
+  float* C;                  // fp32 output, or null: then `planes` bf16 planes (1 or 3), C16 [M][r] and `plane` elements on.
+  long long ldc;             // C16 may be A's own storage: a tile reads no rows of A but those it writes, and has read them all
+  __nv_bfloat16* C16;
+  long long plane;
+  int planes, pad2;
 };
 void launch_sketch_tma(const SkProblem* probs, int nprobs, long long total_tiles, int grid, int big, unsigned* status, cudaStream_t st);
 

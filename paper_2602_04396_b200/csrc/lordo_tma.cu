@@ -721,7 +721,7 @@ using namespace umma;
 namespace {
 constexpr int kSMaxStages = 4;
 constexpr uint32_t kSSmemBytes = 196608 + 1024;  // 4 stages of A 16 KB | E 16 KB | B 16 KB, or 3 with 32 KB of B
-constexpr int kSThreads = (2 + 4 + 4) * 32;  // TMA, MMA, 4 transform warps, 4 epilogue warps
+constexpr int kSThreads = (2 + 4 + 8) * 32;  // TMA, MMA, 4 transform warps, 8 epilogue warps
 constexpr uint32_t kIdescBMajorMN = 1u << 16;
 
 __device__ __forceinline__ int find_sk(const SkProblem* __restrict__ probs, int nprobs, long long tile) {
@@ -752,7 +752,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
 
   if (tid == 0) {
     for (int s = 0; s < ST; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&xform_bar[s], 8); mbar_init(&empty_bar[s], 1); }
-    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 8); }
+    for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], 16); }
     mbar_init_fence();
   }
   if (warp == 1) tmem_alloc_pair(&tmem_slot, 512);
@@ -870,8 +870,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
       }
     }
   } else {
-    // epilogue: lane = row of the tile, r_n fp32 columns out of tensor memory
-    const int q = warp & 3;
+    // epilogue: lane = row of the tile, r_n fp32 columns out of tensor memory, every other 16 of them per warp
+    const int q = warp & 3, half = (warp - 6) >> 2;
     uint32_t si = 0;
     bool ok = true;
     const uint32_t ae = cluster_addr(&acc_empty[0], 0);
@@ -880,15 +880,31 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
       const long long row = (2 * (tile - pr->tile_start) + rank) * 128 + q * 32 + lane;
       const bool row_ok = row < pr->M;
       float* __restrict__ crow = pr->C + (row_ok ? row : 0) * pr->ldc;
-      const int r = pr->r, r_n = pr->r_n;
+      const int r = pr->r, r_n = pr->r_n, planes = pr->planes;
       const uint32_t buf = BIG ? 0u : (si & 1u);
       ok = mbar_wait<64>(&acc_full[buf], (BIG ? si : (si >> 1)) & 1u, status);
       if (!ok) break;
       tc_fence_after_sync();
-      for (int ch = 0; ch < r_n / 16; ++ch) {
+      for (int ch = half; ch < r_n / 16; ch += 2) {
         float v[16];
         tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + buf * 256 + (uint32_t)(ch * 16), v);
-        if (row_ok && !pr->c_trans) {
+        if (planes) {
+          // rounded to bf16, the residual being the next plane's value
+          __nv_bfloat16* d = pr->C16 + (row_ok ? row : 0) * r + ch * 16;
+          for (int p = 0; p < planes; ++p, d += pr->plane) {
+            uint32_t w[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              w[j] = pack2_bf16(v[2 * j], v[2 * j + 1]);
+              v[2 * j] -= bf_lo(w[j]);
+              v[2 * j + 1] -= bf_hi(w[j]);
+            }
+            if (row_ok) {
+              *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+              if (ch * 16 + 8 < r) *reinterpret_cast<uint4*>(d + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+            }
+          }
+        } else if (row_ok && !pr->c_trans) {
 #pragma unroll
           for (int j = 0; j < 16; j += 4)
             if (ch * 16 + j < r) *reinterpret_cast<float4*>(crow + ch * 16 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
