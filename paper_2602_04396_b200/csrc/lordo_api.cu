@@ -17,7 +17,7 @@ namespace {
 constexpr int kMaxK = 64;
 constexpr long long kPairs = 74;  // CTA pairs that the work of a refresh is planned for (148 SMs)
 
-enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_NORM = 6, ST_EIG = 7, ST_GRAM = 8 };
+enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_COLSQ = 6, ST_EIG = 7, ST_GRAM = 8, ST_BASIS = 9, ST_ROT = 10 };
 enum Phase { PH_SUBSPACE = 0, PH_ROTATE = 1, PH_COMMIT = 2 };
 
 // One launch of the refresh / init / inner-step plans. The entries it works on are a contiguous
@@ -42,7 +42,8 @@ struct SlotBuilder {
     std::vector<CopyProblem> cp;
     std::vector<SkProblem> sk;
     std::vector<ConvProblem> cv;
-    std::vector<NormProblem> nm;
+    std::vector<BasisProblem> bs;
+    std::vector<RotProblem> rt;
     std::vector<EigProblem> eg;
     std::vector<GramProblem> gr;
   };
@@ -94,7 +95,8 @@ struct lordo_ctx {
   CopyProblem* d_copies = nullptr;
   SkProblem* d_sks = nullptr;
   ConvProblem* d_convs = nullptr;
-  NormProblem* d_norms = nullptr;
+  BasisProblem* d_bases = nullptr;
+  RotProblem* d_rots = nullptr;
   EigProblem* d_eigs = nullptr;
   GramProblem* d_grams = nullptr;
   float* d_scratch = nullptr;
@@ -134,7 +136,8 @@ struct lordo_ctx {
   std::vector<DiagProblem> h_diag;  // one per rotation matrix, ordered by matrix then batch entry
   DiagProblem* d_diag = nullptr;
   std::vector<ConvProblem> h_convs;
-  std::vector<NormProblem> h_norms;
+  std::vector<BasisProblem> h_bases;
+  std::vector<RotProblem> h_rots;
   std::vector<EigProblem> h_eigs;
   std::vector<GramProblem> h_grams;
   struct SketchBufs {
@@ -160,6 +163,7 @@ struct lordo_ctx {
   int steps_in_round = 0;
   bool after_outer = false;
   bool rot_valid = false;       // the rotation matrices in the workspace were written by a refresh of this context
+  bool refresh_makes_copies = false;  // the refresh plan itself writes the bf16 operand copies of P
   bool p_copies_stale = false;  // the caller may have restored P: the bf16 operand copies are remade before the next use
   std::string err;
 
@@ -300,16 +304,19 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   // the ranges meet in fp64.
   long long gram_tiles = 0;
   for (int i = 0; i < n_mats; ++i) gram_tiles += 2ll * (local ? K : 1) * ((cfg.mats[i].r + 255) / 256);
-  auto gram_ranges = [&](long long rows) {
-    const long long steps = 2 * ((rows + 63) / 64);
+  auto ranges = [&](long long tiles, long long steps, long long most) {
     int best = 1;
     long long best_cost = -1;
-    for (int ns = (int)((steps + 63) / 64); ns <= 32 && (ns == 1 || steps / ns >= 4); ++ns) {
-      const long long cost = ((gram_tiles * ns + kPairs - 1) / kPairs) * ((steps + ns - 1) / ns + 4);
+    for (int ns = (int)((steps + 63) / 64); ns <= most && (ns == 1 || steps / ns >= 4); ++ns) {
+      const long long cost = ((tiles * ns + kPairs - 1) / kPairs) * ((steps + ns - 1) / ns + 4);
       if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = ns; }
     }
     return best;
   };
+  auto gram_ranges = [&](long long rows) { return ranges(gram_tiles, 2 * ((rows + 63) / 64), 32); };
+  // Rot has half the tiles and three pairs of planes; its partial products share the Gram matrices' buffer
+  auto rot_ranges = [&](long long rows) { return ranges(gram_tiles / 2, 3 * ((rows + 63) / 64), 64); };
+  auto part_matrices = [&](long long pm, long long ln) { return std::max(2 * std::max(gram_ranges(pm), gram_ranges(ln)), rot_ranges(pm)); };
   std::vector<int> group_of(n_mats);
   size_t scratch_floats = 0;
   {
@@ -331,7 +338,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         // (per batch entry) and the two moment operands of every worker in two
         per += 3 * (size_t)maxd * a.r / 2 + pm * a.r + 7 * (size_t)a.r * a.r / 2 + 128;
         states16 = 2 * (size_t)K * a.r * ln + 64;
-        per += 2 * (size_t)std::max(gram_ranges(pm), gram_ranges(ln)) * a.r * a.r;
+        per += (size_t)part_matrices(pm, ln) * a.r * a.r + 2 * (size_t)((pm + kNormRows - 1) / kNormRows) * a.r + 16;
       }
       mat_scratch[i] = nb * per + states16;
       if (acc > 0 && acc + mat_scratch[i] > kRefreshScratchFloats) { ++grp; acc = 0; }
@@ -370,6 +377,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
     if (cfg.mats[i].r > (cfg.w_dtype == LORDO_BF16 ? 512 : 256) || (cfg.mats[i].side && cfg.w_dtype != LORDO_BF16)) c->tc = false;
   c->h_tc.clear(); c->h_prep.clear(); c->h_prep_start.assign(1, 0);
   c->tc_strips = 0; c->tc_strips_p = 0; c->tc_rn_max = 0; c->tc_rk_max = 0;
+  std::vector<size_t> h_prep_first(n_mats, 0);  // first entry of a matrix in h_prep
   if (c->tc) {
     auto up = [](long long x, long long q) { return (x + q - 1) / q * q; };
     (void)cv.take<char>(0);
@@ -387,6 +395,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       float* dcol2 = nsplit == 2 ? cv.take<float>((size_t)K * md.ln) : nullptr;
       if (r_n > c->tc_rn_max) c->tc_rn_max = r_n;
       if (r_k > c->tc_rk_max) c->tc_rk_max = r_k;
+      h_prep_first[i] = c->h_prep.size();
       for (int k = 0; k < copies; ++k) {
         TcPrep pp;
         std::memset(&pp, 0, sizeof(pp));
@@ -452,9 +461,10 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
 
   // ---------------- launch plans ----------------
   std::vector<GemmProblem>& P = c->h_probs;
-  P.clear(); c->h_chols.clear(); c->h_rands.clear(); c->h_copies.clear(); c->h_sks.clear(); c->h_convs.clear(); c->h_norms.clear(); c->h_eigs.clear(); c->h_grams.clear(); c->h_diag.clear();
+  P.clear(); c->h_chols.clear(); c->h_rands.clear(); c->h_copies.clear(); c->h_sks.clear(); c->h_convs.clear(); c->h_bases.clear(); c->h_rots.clear(); c->h_eigs.clear(); c->h_grams.clear(); c->h_diag.clear();
   c->h_skbufs.assign(n_mats, lordo_ctx::SketchBufs());
   const bool tc_sketch = c->tc && c->tma && cfg.oversample == 0;  // products of the refresh on tensor cores
+  c->refresh_makes_copies = tc_sketch;
   auto gemm_prob = [&](int M, int N, int Kd, const Operand& A, const Operand& B, const Operand* B2, const Epilogue& ep) {
     GemmProblem g;
     std::memset(&g, 0, sizeof(g));
@@ -501,9 +511,21 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       } else if (st.type == ST_GRAM) {
         st.first = (long long)c->h_grams.size(); st.count = (int)sl.gr.size(); st.tiles = 0;
         for (GramProblem& x : sl.gr) { const long long b = (x.r + 31) / 32; x.blk_start = st.tiles; st.tiles += b * (b + 1) / 2; c->h_grams.push_back(x); }
-      } else if (st.type == ST_NORM) {
-        st.first = (long long)c->h_norms.size(); st.count = (int)sl.nm.size(); st.tiles = 0;
-        for (NormProblem& x : sl.nm) { x.blk_start = st.tiles; st.tiles += (x.r + 31) / 32; c->h_norms.push_back(x); }
+      } else if (st.type == ST_COLSQ) {
+        // the table of the commit that follows: its entries carry the first block in either launch
+        st.first = (long long)c->h_bases.size(); st.count = (int)sl.bs.size(); st.tiles = 0;
+        for (const BasisProblem& x : sl.bs) st.tiles += (x.m + kNormRows - 1) / kNormRows * ((x.r + 127) / 128);
+      } else if (st.type == ST_BASIS) {
+        st.first = (long long)c->h_bases.size(); st.count = (int)sl.bs.size(); st.tiles = 0;
+        long long sq = 0;
+        for (BasisProblem& x : sl.bs) {
+          x.sq_start = sq; sq += (x.m + kNormRows - 1) / kNormRows * ((x.r + 127) / 128);
+          x.tile_start = st.tiles; st.tiles += (x.m + 63) / 64 * ((x.r + 63) / 64);
+          c->h_bases.push_back(x);
+        }
+      } else if (st.type == ST_ROT) {
+        st.first = (long long)c->h_rots.size(); st.count = (int)sl.rt.size(); st.tiles = 0;
+        for (RotProblem& x : sl.rt) { const long long b = (x.r + 31) / 32; x.blk_start = st.tiles; st.tiles += b * b; c->h_rots.push_back(x); }
       } else {
         st.first = (long long)c->h_copies.size(); st.count = (int)sl.cp.size(); st.tiles = 0;
         for (CopyProblem& x : sl.cp) { x.blk_start = st.tiles; st.tiles += (x.chunks + 1023) / 1024; c->h_copies.push_back(x); }
@@ -635,7 +657,8 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       c->h_skbufs[i].om16 = om16; c->h_skbufs[i].pn16 = pn16; c->h_skbufs[i].zq16 = zq16;
       // tensor-core QR and rotation: bf16 planes, plane p of batch entry b at index p * nb + b
       __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr, *uh16 = nullptr, *wr16 = nullptr;
-      float* gpart = nullptr;  // partial sums of the Gram matrices
+      float* gpart = nullptr;   // partial sums of the Gram matrices and of Rot
+      double* colsq = nullptr;  // partial sums of squares of the new basis' columns
       if (tc_sketch) {
         auto take16 = [&](size_t floats) { __nv_bfloat16* p16 = reinterpret_cast<__nv_bfloat16*>(s); s += floats + 16; return p16; };
         x16 = take16(3 * (size_t)nb * maxd * r / 2);
@@ -645,22 +668,14 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         sq16 = take16((size_t)nb * r * r);
         uh16 = take16((size_t)K * r * n);
         wr16 = take16((size_t)K * r * n);
-        gpart = s; s += (size_t)nb * 2 * std::max(gram_ranges(m), gram_ranges(n)) * r * r;
+        gpart = s; s += (size_t)nb * part_matrices(m, n) * r * r;
+        s = c->d_scratch + ((s - c->d_scratch + 3) & ~(ptrdiff_t)3);
+        colsq = reinterpret_cast<double*>(s); s += 2 * (size_t)nb * ((m + kNormRows - 1) / kNormRows) * r;
         lordo_ctx::SketchBufs& kb = c->h_skbufs[i];
         kb.x16 = x16; kb.rinv16 = rinv16; kb.phl = phl; kb.rt16 = rt16; kb.sq16 = sq16; kb.uh16 = uh16; kb.wr16 = wr16;
       }
       TmaMatMaps* mmi = c->d_maps + i;
       auto conv = [&](SlotBuilder& sb, int phase, const ConvProblem& cp) { sb.next(ST_CONVERT, phase).cv.push_back(cp); };
-      auto conv_split = [&](SlotBuilder& sb, int phase, const float* src, long long sstride, __nv_bfloat16* planes, long long elems, int np) {
-        SlotBuilder::Slot& sl = sb.next(ST_CONVERT, phase);
-        for (int b = 0; b < nb; ++b) {
-          ConvProblem cp;
-          std::memset(&cp, 0, sizeof(cp));
-          cp.mode = CONV_SPLIT; cp.src = src ? src + b * sstride : nullptr; cp.count = elems;
-          cp.dst = planes + (long long)b * elems; cp.plane = (long long)nb * elems; cp.planes = np;
-          sl.cv.push_back(cp);
-        }
-      };
       // C = A B as the sum of the products of np-plane split operands; planes as above. a_mn: A stored [Kd][M].
       auto sk_split = [&](SlotBuilder::Slot& sl, int a_mn, const unsigned char* map_a, int a_b, int a_nb, const unsigned char* map_b, int b_b, int b_nb,
                           long long Mo, long long Kd, float* C, long long ldc, int c_trans, int np) {
@@ -719,13 +734,6 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
             if (to_planes) { sp.C16 = x16 + (size_t)b * rows * r; sp.plane = (long long)nb * rows * r; sp.planes = 3; }
             if (to_rhs) { sp.C16 = O16 + (size_t)b * rows * r; sp.planes = 1; }
           }
-        }
-        if (!last) return;
-        SlotBuilder::Slot& nr = sb.next(ST_NORM, phase);  // the columns of Q back to unit length
-        for (int b = 0; b < nb; ++b) {
-          NormProblem np;
-          np.X = O + b * so; np.blk_start = 0; np.rows = (int)rows; np.r = r;
-          nr.nm.push_back(np);
         }
       };
       auto qr2 = [&](SlotBuilder& sb, int phase, float* X, long long sx, float* T, long long st, float* O, long long so, long long rows, int w,
@@ -845,21 +853,37 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         c->h_diag.push_back(dp);
       }
       if (tc_sketch) {
-        // Rot = P'^T P and the rotated moments on tensor cores, operands in two planes (16 bits each)
-        conv_split(R, PH_SUBSPACE, Pn, m * r, x16, m * r, 2);
-        conv_split(R, PH_SUBSPACE, md.P, md.p_stride, phl, m * r, 2);
-        {
-          SlotBuilder::Slot& g = R.next(ST_SKETCH, PH_SUBSPACE);
-          for (int b = 0; b < nb; ++b) sk_split(g, 1, mmi->xm_sw, b, nb, mmi->phl_sw, b, nb, r, m, rot + (long long)b * r * r, r, 0, 2);
+        // the new basis takes the old one's place; Rot = P'^T P and the rotated moments on tensor cores, operands in
+        // two planes (16 bits each)
+        std::vector<BasisProblem> bases(nb);
+        for (int b = 0; b < nb; ++b) {
+          BasisProblem& bp = bases[b];
+          const TcPrep& pp = c->h_prep[h_prep_first[i] + b];
+          std::memset(&bp, 0, sizeof(bp));
+          bp.Q = Pn + (size_t)b * m * r; bp.sq = colsq + (size_t)b * ((m + kNormRows - 1) / kNormRows) * r;
+          bp.P = md.P ? md.P + b * md.p_stride : nullptr;
+          bp.q16 = x16 + (size_t)b * m * r; bp.p16 = phl + (size_t)b * m * r; bp.q_plane = bp.p_plane = (long long)nb * m * r;
+          bp.P16 = pp.P16; bp.PT16 = pp.PT16; bp.m = m; bp.r = r; bp.r_k = pp.r_k; bp.m_k = pp.m_k;
         }
-        {  // Rot^T and its element-wise square as right-hand sides
-          SlotBuilder::Slot& sl = R.next(ST_CONVERT, PH_ROTATE);
+        for (int type : {ST_COLSQ, ST_BASIS}) {
+          SlotBuilder::Slot& sl = R.next(type, PH_SUBSPACE);
+          sl.bs.insert(sl.bs.end(), bases.begin(), bases.end());
+        }
+        {
+          const int ns = rot_ranges(m), steps = 3 * (int)((m + 63) / 64);
+          SlotBuilder::Slot& g = R.next(ST_SKETCH, PH_SUBSPACE);
+          for (int b = 0; b < nb; ++b)
+            for (int x = 0; x < ns; ++x) {  // the smaller pairs first: less is truncated
+              sk_split(g, 1, mmi->xm_sw, b, nb, mmi->phl_sw, b, nb, r, m, gpart + (size_t)(b * ns + x) * r * r, r, 0, 2);
+              SkProblem& sp = g.sk.back();
+              sp.pa = 0x010u; sp.pb = 0x001u; sp.j0 = (int)((long long)steps * x / ns); sp.j1 = (int)((long long)steps * (x + 1) / ns);
+            }
+          SlotBuilder::Slot& rs_ = R.next(ST_ROT, PH_SUBSPACE);
           for (int b = 0; b < nb; ++b) {
-            ConvProblem cp;
-            std::memset(&cp, 0, sizeof(cp));
-            cp.mode = CONV_ROT_T; cp.src = rot + (long long)b * r * r; cp.count = (long long)r * r; cp.ld = r;
-            cp.dst = rt16 + (long long)b * r * r; cp.dst2 = sq16 + (long long)b * r * r; cp.plane = (long long)nb * r * r; cp.planes = 2;
-            sl.cv.push_back(cp);
+            RotProblem rp;
+            rp.part = gpart + (size_t)b * ns * r * r; rp.rot = rot + (size_t)b * r * r; rp.rt16 = rt16 + (size_t)b * r * r; rp.sq16 = sq16 + (size_t)b * r * r;
+            rp.plane = (long long)nb * r * r; rp.blk_start = 0; rp.r = r; rp.ns = ns;
+            rs_.rt.push_back(rp);
           }
         }
         {  // u^ and v^ - u^ u^ of all workers as hi|lo planes [2K][r][n]
@@ -870,12 +894,11 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           conv(R, PH_ROTATE, cp);
         }
         {  // (Rot u^)^T = u^^T Rot^T, stored back as [r][n] into the transient g^ area; same for the second moment
-          SlotBuilder::Slot& g1 = R.next(ST_SKETCH, PH_ROTATE);
-          for (int k = 0; k < K; ++k)
-            sk_split(g1, 1, mmi->uh_sw, k, K, mmi->rt_sw, local ? k : 0, nb, n, r, md.ghat + (long long)k * r * n, n, 1, 2);
-          SlotBuilder::Slot& g2 = R.next(ST_SKETCH, PH_ROTATE);
-          for (int k = 0; k < K; ++k)
-            sk_split(g2, 1, mmi->wr_sw, k, K, mmi->sq_sw, local ? k : 0, nb, n, r, md.util + (long long)k * r * n, n, 1, 2);
+          SlotBuilder::Slot& g = R.next(ST_SKETCH, PH_ROTATE);
+          for (int k = 0; k < K; ++k) {
+            sk_split(g, 1, mmi->uh_sw, k, K, mmi->rt_sw, local ? k : 0, nb, n, r, md.ghat + (long long)k * r * n, n, 1, 2);
+            sk_split(g, 1, mmi->wr_sw, k, K, mmi->sq_sw, local ? k : 0, nb, n, r, md.util + (long long)k * r * n, n, 1, 2);
+          }
         }
         {  // u = bc1 (Rot u^), v = bc2 |Rot^2 (v^ - u^ u^) + (Rot u^)^2|
           ConvProblem cp;
@@ -904,7 +927,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           add_copy(R, PH_ROTATE, md.v, md.util, (size_t)K * r * n * sizeof(float));
         }
       }
-      add_copy(R, PH_COMMIT, md.P, Pn, (size_t)nb * m * r * sizeof(float));
+      if (!tc_sketch) add_copy(R, PH_COMMIT, md.P, Pn, (size_t)nb * m * r * sizeof(float));
       if (!local) {  // P_0 = orthonormalised random m x r matrix
         RandProblem rp;
         rp.out = Ya; rp.out16 = nullptr; rp.count = m * r; rp.blk_start = 0; rp.purpose = 1; rp.mat = i; rp.replica = 0; rp.pad = 0;
@@ -941,7 +964,8 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   c->d_copies = cv.take<CopyProblem>(c->h_copies.size() + 1);
   c->d_sks = cv.take<SkProblem>(c->h_sks.size() + 1);
   c->d_convs = cv.take<ConvProblem>(c->h_convs.size() + 1);
-  c->d_norms = cv.take<NormProblem>(c->h_norms.size() + 1);
+  c->d_bases = cv.take<BasisProblem>(c->h_bases.size() + 1);
+  c->d_rots = cv.take<RotProblem>(c->h_rots.size() + 1);
   c->d_eigs = cv.take<EigProblem>(c->h_eigs.size() + 1);
   c->d_grams = cv.take<GramProblem>(c->h_grams.size() + 1);
   c->d_diag = cv.take<DiagProblem>(c->h_diag.size() + 1);
@@ -1019,10 +1043,18 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       launch_jacobi_projector(c->d_eigs + s.first, s.count, s.r_max, st);
       c->launches += 1;
       return check_launch(c, "jacobi_projector");
-    case ST_NORM:
-      launch_colnorm_grouped(c->d_norms + s.first, s.count, s.tiles, st);
+    case ST_COLSQ:
+      launch_colsq(c->d_bases + s.first, s.count, s.tiles, st);
       c->launches += 1;
-      return check_launch(c, "colnorm");
+      return check_launch(c, "colsq");
+    case ST_BASIS:
+      launch_commit_basis(c->d_bases + s.first, s.count, s.tiles, st);
+      c->launches += 1;
+      return check_launch(c, "commit_basis");
+    case ST_ROT:
+      launch_rot_sum(c->d_rots + s.first, s.count, s.tiles, st);
+      c->launches += 1;
+      return check_launch(c, "rot_sum");
     case ST_GRAM:
       launch_gram_sum(c->d_grams + s.first, s.count, s.tiles, st);
       c->launches += 1;
@@ -1167,7 +1199,8 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
   if (!c->h_sks.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_sks, c->h_sks.data(), sizeof(SkProblem) * c->h_sks.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_diag.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_diag, c->h_diag.data(), sizeof(DiagProblem) * c->h_diag.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_convs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_convs, c->h_convs.data(), sizeof(ConvProblem) * c->h_convs.size(), cudaMemcpyHostToDevice, st));
-  if (!c->h_norms.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_norms, c->h_norms.data(), sizeof(NormProblem) * c->h_norms.size(), cudaMemcpyHostToDevice, st));
+  if (!c->h_bases.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_bases, c->h_bases.data(), sizeof(BasisProblem) * c->h_bases.size(), cudaMemcpyHostToDevice, st));
+  if (!c->h_rots.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_rots, c->h_rots.data(), sizeof(RotProblem) * c->h_rots.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_eigs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_eigs, c->h_eigs.data(), sizeof(EigProblem) * c->h_eigs.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_grams.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_grams, c->h_grams.data(), sizeof(GramProblem) * c->h_grams.size(), cudaMemcpyHostToDevice, st));
   INIT_CUDA(cudaMemsetAsync(c->d_status, 0, 256, st));
@@ -1484,7 +1517,7 @@ int lordo_refresh_subspace(lordo_ctx* c, const void* const* G, float beta1, void
       rc = run_plan_step(c, s, gs, st);
       if (rc != LORDO_OK) return rc;
     }
-    if (c->tc) {  // bf16 operand copies of the new P
+    if (c->tc && !c->refresh_makes_copies) {  // bf16 operand copies of the new P
       launch_prep_projection(c->d_tc_prep, c->d_prep_start, (int)c->h_prep.size(), c->prep_blocks, st);
       c->launches += 1;
       rc = check_launch(c, "prep_projection");

@@ -210,10 +210,8 @@ void launch_copy_grouped(const CopyProblem* probs, int nprobs, long long total_b
 // [three planes: 24 bits, the accuracy of an fp32 product].
 enum ConvMode {
   CONV_BF16 = 0,     // dst = bf16(src)
-  CONV_SPLIT = 1,    // dst = split(src)
-  CONV_STATES = 2,   // dst = split(u^ = inv_bc1 src), dst2 = split(inv_bc2 src2 - u^ u^)
-  CONV_ROT_T = 3,    // src is Rot [ld][ld]: dst = split(Rot^T), dst2 = split(Rot^T o Rot^T)
-  CONV_COMBINE = 4   // outf = bc1 src, outf2 = bc2 |src2 + src src|   (rotated moments from the two products)
+  CONV_STATES = 1,   // dst = split(u^ = inv_bc1 src), dst2 = split(inv_bc2 src2 - u^ u^)
+  CONV_COMBINE = 2   // outf = bc1 src, outf2 = bc2 |src2 + src src|   (rotated moments from the two products)
 };
 struct ConvProblem {
   const float* src;
@@ -222,7 +220,7 @@ struct ConvProblem {
   float *outf, *outf2;
   long long count, blk_start;  // count is a multiple of 8
   long long plane;             // elements between the planes of dst and of dst2
-  int mode, ld, planes, pad;
+  int mode, planes;
 };
 void launch_convert_grouped(const ConvProblem* probs, int nprobs, long long total_blocks, const GemmScalars& sc, cudaStream_t st);
 
@@ -237,16 +235,35 @@ struct GramProblem {
 };
 void launch_gram_sum(const GramProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
 
-// Columns of X [rows][r] scaled to unit length (sums of squares in fp64), one block per 32 columns.
-// The tensor-core Gram matrix underestimates its diagonal (an fp32 accumulator that truncates, over
-// thousands of positive addends), which leaves every column of Q a few 1e-5 too long; the
-// off-diagonal part is already at fp32 level.
-struct NormProblem {
-  float* X;
-  long long blk_start;
-  int rows, r;
+// Rot = P'^T P from its products over `ns` ranges of k, with the two right-hand sides of the moments' rotation:
+// Rot^T and Rot^T o Rot^T as two bf16 planes each, `plane` elements apart.
+struct RotProblem {
+  const float* part;  // [ns][r][r]
+  float* rot;         // [r][r]
+  __nv_bfloat16 *rt16, *sq16;
+  long long plane, blk_start;
+  int r, ns;
 };
-void launch_colnorm_grouped(const NormProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
+void launch_rot_sum(const RotProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
+
+// A new basis in place of the old one, one block per 64 x 64 tile: the columns of Q scaled to unit length (the
+// tensor cores' fp32 accumulation truncates and leaves them a few 1e-6 off; the off-diagonal part is at
+// fp32 level) become P, its operand copies P16 and PT16 and two planes for Rot; the old P becomes two planes too.
+// sq: sums of squares of Q's columns over chunks of kNormRows rows, [chunks][r], from launch_colsq.
+constexpr int kNormRows = 256;
+struct BasisProblem {
+  const float* Q;                    // [m][r]
+  double* sq;
+  float* P;                          // [m][r]
+  __nv_bfloat16 *q16, *p16;          // planes of the new and of the old basis, q_plane and p_plane elements apart
+  __nv_bfloat16 *P16, *PT16;         // [m_k][r_k], [r_n][m_k]
+  long long q_plane, p_plane;
+  long long sq_start, tile_start;    // first block of this problem in the two launches
+  long long m;
+  int r, r_k, m_k, pad;
+};
+void launch_colsq(const BasisProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
+void launch_commit_basis(const BasisProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
 
 // Tensor-core sketch products of the refresh (lordo_tma.cu): C[M x r] (fp32) = S * B with the big
 // signal matrix S streamed by TMA as bf16 (optionally formed as c*G + E in shared memory) and

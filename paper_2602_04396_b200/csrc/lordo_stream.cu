@@ -309,21 +309,9 @@ __global__ void __launch_bounds__(256) convert_grouped_kernel(const ConvProblem*
   const ConvProblem pb = probs[lo];
   const long long e = ((blk - pb.blk_start) * 256 + threadIdx.x) * 4;  // count is a multiple of 8
   if (e >= pb.count) return;
-  if (pb.mode == CONV_ROT_T) {  // element e of the transposed matrix: (k, j) <- Rot[j][k]
-    float t[4];
-    for (int x = 0; x < 4; ++x) {
-      const long long k = (e + x) / pb.ld, j = (e + x) - k * pb.ld;
-      t[x] = pb.src[j * pb.ld + k];
-    }
-    split_store4(pb.dst, pb.plane, pb.planes, e, make_float4(t[0], t[1], t[2], t[3]));
-    split_store4(pb.dst2, pb.plane, pb.planes, e, make_float4(t[0] * t[0], t[1] * t[1], t[2] * t[2], t[3] * t[3]));
-    return;
-  }
   const float4 v = *reinterpret_cast<const float4*>(pb.src + e);
   if (pb.mode == CONV_BF16) {
     store4(pb.dst, LORDO_BF16, e, v);
-  } else if (pb.mode == CONV_SPLIT) {
-    split_store4(pb.dst, pb.plane, pb.planes, e, v);
   } else if (pb.mode == CONV_STATES) {
     const float4 w = *reinterpret_cast<const float4*>(pb.src2 + e);
     const float4 uh = make_float4(inv_bc1 * v.x, inv_bc1 * v.y, inv_bc1 * v.z, inv_bc1 * v.w);
@@ -387,35 +375,137 @@ __global__ void __launch_bounds__(256) gram_sum_kernel(const GramProblem* __rest
   }
 }
 
-__global__ void __launch_bounds__(256) colnorm_grouped_kernel(const NormProblem* __restrict__ probs, int nprobs) {
-  __shared__ double part[8][32];
+// One block per 32 x 32 block of Rot, whose transpose it writes.
+__global__ void __launch_bounds__(256) rot_sum_kernel(const RotProblem* __restrict__ probs, int nprobs) {
+  __shared__ float tt[32][33];
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (probs[mid].blk_start <= blk) lo = mid; else hi = mid - 1;
   }
-  const NormProblem pb = probs[lo];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int col = (int)(blk - pb.blk_start) * 32 + lane;
-  const bool live = col < pb.r;
-  double s = 0.0;
-  if (live)
-    for (int row = w; row < pb.rows; row += 8) {
-      const float x = pb.X[(long long)row * pb.r + col];
-      s += (double)x * (double)x;
+  const RotProblem pb = probs[lo];
+  const int r = pb.r, nb = (r + 31) / 32;
+  const int bi = (int)(blk - pb.blk_start) / nb, bj = (int)(blk - pb.blk_start) - bi * nb;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = bi * 32 + y + 8 * q, j = bj * 32 + x;
+    if (i < r && j < r) {
+      double a = 0.0;
+      for (int s = 0; s < pb.ns; ++s) a += (double)pb.part[(size_t)s * r * r + (size_t)i * r + j];
+      pb.rot[(size_t)i * r + j] = (float)a;
+      tt[y + 8 * q][x] = (float)a;
     }
-  part[w][lane] = s;
-  __syncthreads();
-  if (w == 0) {
-    double t = 0.0;
-    for (int k = 0; k < 8; ++k) t += part[k][lane];
-    part[0][lane] = t > 0.0 ? 1.0 / sqrt(t) : 1.0;
   }
   __syncthreads();
-  const float sc = (float)part[0][lane];
-  if (live)
-    for (int row = w; row < pb.rows; row += 8) pb.X[(long long)row * pb.r + col] *= sc;
+  for (int e = threadIdx.x; e < 256; e += 256) {  // four neighbouring elements of a row of Rot^T per thread
+    const int i = bj * 32 + (e >> 3), j = bi * 32 + (e & 7) * 4;
+    if (i < r && j < r) {  // r is a multiple of 8
+      const int c = e >> 3, k = (e & 7) * 4;
+      const float4 t = make_float4(tt[k][c], tt[k + 1][c], tt[k + 2][c], tt[k + 3][c]);
+      const long long at = (long long)i * r + j;
+      split_store4(pb.rt16, pb.plane, 2, at, t);
+      split_store4(pb.sq16, pb.plane, 2, at, make_float4(t.x * t.x, t.y * t.y, t.z * t.z, t.w * t.w));
+    }
+  }
+}
+
+// Sums of squares of 128 columns over kNormRows rows, in fp64. One block per 32 columns over all rows took 346 us
+// for 7 matrices of up to 5632 x 256 (and 400 us for 16 of 4096 x 512).
+__global__ void __launch_bounds__(256) colsq_kernel(const BasisProblem* __restrict__ probs, int nprobs) {
+  __shared__ double red[8][128];
+  const long long blk = blockIdx.x;
+  int lo = 0, hi = nprobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (probs[mid].sq_start <= blk) lo = mid; else hi = mid - 1;
+  }
+  const BasisProblem pb = probs[lo];
+  const int nc = (pb.r + 127) / 128;
+  const long long chunk = (blk - pb.sq_start) / nc;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c0 = (int)(blk - pb.sq_start - chunk * nc) * 128;
+  const int col = c0 + 4 * lane;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  if (col < pb.r) {
+    const long long end = min((long long)pb.m, (chunk + 1) * kNormRows);
+#pragma unroll 4
+    for (long long row = chunk * kNormRows + w; row < end; row += 8) {
+      const float4 v = *reinterpret_cast<const float4*>(pb.Q + row * pb.r + col);
+      s[0] += (double)v.x * (double)v.x; s[1] += (double)v.y * (double)v.y;
+      s[2] += (double)v.z * (double)v.z; s[3] += (double)v.w * (double)v.w;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) red[w][4 * lane + i] = s[i];
+  __syncthreads();
+  if (threadIdx.x < 128 && c0 + threadIdx.x < pb.r) {
+    double t = 0.0;
+    for (int k = 0; k < 8; ++k) t += red[k][threadIdx.x];
+    pb.sq[chunk * pb.r + c0 + threadIdx.x] = t;
+  }
+}
+
+__global__ void __launch_bounds__(256) commit_basis_kernel(const BasisProblem* __restrict__ probs, int nprobs) {
+  __shared__ __nv_bfloat16 tile[64][66];
+  __shared__ float scale[64];
+  __shared__ double part[4][64];
+  const long long blk = blockIdx.x;
+  int lo = 0, hi = nprobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (probs[mid].tile_start <= blk) lo = mid; else hi = mid - 1;
+  }
+  const BasisProblem pb = probs[lo];
+  const int r = pb.r, nc = (r + 63) / 64;
+  const long long row0 = (blk - pb.tile_start) / nc * 64;
+  const int col0 = (int)((blk - pb.tile_start) % nc) * 64;
+  const int t = threadIdx.x;
+  float4 q[4], p[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int rr = (t >> 4) + 16 * i, cc = (t & 15) * 4;
+    q[i] = p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row0 + rr < pb.m && col0 + cc < r) {
+      const long long at = (row0 + rr) * r + col0 + cc;
+      q[i] = *reinterpret_cast<const float4*>(pb.Q + at);
+      p[i] = *reinterpret_cast<const float4*>(pb.P + at);
+    }
+  }
+  {
+    const int c = t & 63, w = t >> 6;
+    double s = 0.0;
+    if (col0 + c < r) {
+      const int chunks = (int)((pb.m + kNormRows - 1) / kNormRows);
+      for (int k = w; k < chunks; k += 4) s += pb.sq[(long long)k * r + col0 + c];
+    }
+    part[w][c] = s;
+  }
+  __syncthreads();
+  if (t < 64) {
+    const double s = (part[0][t] + part[1][t]) + (part[2][t] + part[3][t]);
+    scale[t] = (float)(s > 0.0 ? 1.0 / sqrt(s) : 1.0);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int rr = (t >> 4) + 16 * i, cc = (t & 15) * 4;
+    if (row0 + rr < pb.m && col0 + cc < r) {
+      const long long at = (row0 + rr) * r + col0 + cc;
+      const float4 n = make_float4(q[i].x * scale[cc], q[i].y * scale[cc + 1], q[i].z * scale[cc + 2], q[i].w * scale[cc + 3]);
+      *reinterpret_cast<float4*>(pb.P + at) = n;
+      split_store4(pb.q16, pb.q_plane, 2, at, n);
+      split_store4(pb.p16, pb.p_plane, 2, at, p[i]);
+      store4(pb.P16, LORDO_BF16, (row0 + rr) * pb.r_k + col0 + cc, n);
+      tile[rr][cc] = __float2bfloat16_rn(n.x); tile[rr][cc + 1] = __float2bfloat16_rn(n.y);
+      tile[rr][cc + 2] = __float2bfloat16_rn(n.z); tile[rr][cc + 3] = __float2bfloat16_rn(n.w);
+    }
+  }
+  __syncthreads();
+  for (int e = t; e < 64 * 64; e += 256) {
+    const int cc = e >> 6, rr = e & 63;
+    if (row0 + rr < pb.m && col0 + cc < r) pb.PT16[(long long)(col0 + cc) * pb.m_k + row0 + rr] = tile[rr][cc];
+  }
 }
 
 // Device-to-device copies of many buffers in one launch (16-byte chunks).
@@ -493,8 +583,14 @@ void launch_convert_grouped(const ConvProblem* probs, int nprobs, long long tota
 void launch_gram_sum(const GramProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
   gram_sum_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
 }
-void launch_colnorm_grouped(const NormProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
-  colnorm_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+void launch_rot_sum(const RotProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
+  rot_sum_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+}
+void launch_colsq(const BasisProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
+  colsq_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+}
+void launch_commit_basis(const BasisProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
+  commit_basis_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
 }
 void launch_copy_grouped(const CopyProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
   copy_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
