@@ -1024,7 +1024,7 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       c->launches += 1;
       return check_launch(c, "gemm");
     case ST_CHOL:
-      launch_chol_inverse(c->d_chols + s.first, s.count, s.r_max, c->sm_count, c->d_status, st);
+      launch_chol_inverse(c->d_chols + s.first, s.count, s.r_max, c->d_status, st);
       c->launches += 1;
       return check_launch(c, "chol_inverse");
     case ST_RANDOM:

@@ -10,58 +10,94 @@
 // sums run in fp64 on the tensor cores (mma.sync m8n8k4, measured at 64 FMA a clock and SM, the rate of the
 // fp64 pipe), L and rinv are kept in fp32. A row block belongs to CTA (block mod cluster size); the block of
 // the diagonal is summed, factored and inverted by every CTA for itself, which leaves one barrier a panel.
+// While one warp factors the diagonal block of panel k, the others already sum panel k + 1 over the panels
+// before k, so that a panel waits for the newest 32 columns only.
 //
-// What bounds it: the chain of r columns (a reciprocal square root and two multiply-adds each) and one pass
-// over the stored factors out of L2 per panel. Against one CTA per matrix with a thread per row: r = 512, 16
-// matrices 2200 -> 669 us; r = 256, 7 matrices 580 -> 136 us; r = 128, 56 matrices 197 -> 67 us.
+// What bounds it: the chain of r columns, 200 to 350 clocks each (shuffle, reciprocal square root, multiply-adds),
+// and per panel one trip to L2 for the newest columns, the small products and the barrier; for few CTAs per matrix
+// the fp64 products. One CTA per matrix with a thread per row took 2200 us for r = 512 and 16 matrices, 580 us
+// for r = 256 and 7, 197 us for r = 128 and 56; clusters that summed a whole panel at its turn 654, 131 and 62 us;
+// this one 392, 117 and 60 us.
 #include "lordo_kernels.h"
 
 namespace lordo {
 namespace {
 
 constexpr int kB = 32;                       // panel width
-constexpr int kCholWarps = 12;               // 4 on the diagonal block, 8 on the other blocks of the panel
-constexpr int kUnits = 8;                    // partial sums of 32 x 32 blocks in flight, one per warp
-constexpr int kLd = 40;                      // row stride of a partial sum: 16-byte stores of two rows meet no bank twice
+constexpr int kCholWarps = 8;                // 255 registers a thread: with 168 the column chain takes twice as long
+constexpr int kUnits = 4;                    // partial sums of 32 x 32 blocks in flight, one per warp
+constexpr int kLd = 36;                      // row stride of the partial sums and of the inverse: 8 rows x 4 columns meet no bank twice
 constexpr int kPartDoubles = kB * kLd;
-constexpr size_t kCholSmem = sizeof(double) * (size_t)((4 + kUnits) * kPartDoubles + kB * (2 * kB + 1) + kB);
+constexpr size_t kCholSmem = sizeof(double) * (size_t)((4 + kUnits) * kPartDoubles + kB * kB + kB + kB * kLd);
 
 __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b) {
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1},{%2},{%3},{%0,%1};" : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
 }
 
-// c (+)= X_j L_j^T over the 32-column blocks j = j0, j0 + dj, ... < j1 of two row blocks (32 rows from xr, lr on).
-// Lane l holds rows l/4 + 8a and, of every 8 columns, columns 2(l%4) and +1: the same permutation of the
-// summation index on both sides. Rows from r on read as zeros.
-__device__ __forceinline__ void block_sum(double (&c)[4][4][2], const float* X, int xr, const float* L, int lr, int r, int j0, int j1, int dj) {
-  const int lane = threadIdx.x & 31, row = lane >> 2, kc = (lane & 3) * 2;
+// Sums of products of rows: lane l of a warp holds rows l/4 + 8i of both 32-row blocks (rows from r on read as
+// zeros). The columns may be dealt to the lanes in any order as long as it is the same on both sides.
+// c += X_cols L_cols^T over 8 columns from `col` on.
+__device__ __forceinline__ void block_cols(double (&c)[4][4][2], const float* X, int xr, const float* L, int lr, int r, int col) {
+  const int lane = threadIdx.x & 31, row = lane >> 2, kc = col + (lane & 3) * 2;
   float2 a[4], b[4];
-  auto fetch = [&](int col) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int ra = xr + row + 8 * i, rb = lr + row + 8 * i;
+    a[i] = b[i] = make_float2(0.f, 0.f);
+    if (ra < r) a[i] = *reinterpret_cast<const float2*>(X + (size_t)ra * r + kc);
+    if (rb < r) b[i] = *reinterpret_cast<const float2*>(L + (size_t)rb * r + kc);
+  }
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int n = 0; n < 4; ++n) dmma(c[i][n][0], c[i][n][1], (double)(t ? a[i].y : a[i].x), (double)(t ? b[n].y : b[n].x));
+}
+
+__device__ __forceinline__ void fetch16(float4 (&a)[4], float4 (&b)[4], const float* X, int xr, const float* L, int lr, int r, int col) {
+  const int lane = threadIdx.x & 31, row = lane >> 2, kc = col + (lane & 3) * 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int ra = xr + row + 8 * i, rb = lr + row + 8 * i;
+    a[i] = b[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ra < r) a[i] = *reinterpret_cast<const float4*>(X + (size_t)ra * r + kc);
+    if (rb < r) b[i] = *reinterpret_cast<const float4*>(L + (size_t)rb * r + kc);
+  }
+}
+__device__ __forceinline__ void mma16(double (&c)[4][4][2], const float4 (&a)[4], const float4 (&b)[4]) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    double bv[4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) bv[n] = (double)(t == 0 ? b[n].x : t == 1 ? b[n].y : t == 2 ? b[n].z : b[n].w);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int ra = xr + row + 8 * i, rb = lr + row + 8 * i;
-      a[i] = b[i] = make_float2(0.f, 0.f);
-      if (ra < r) a[i] = *reinterpret_cast<const float2*>(X + (size_t)ra * r + col);
-      if (rb < r) b[i] = *reinterpret_cast<const float2*>(L + (size_t)rb * r + col);
-    }
-  };
-  if (j0 < j1) fetch(j0 * kB + kc);
-  for (int j = j0; j < j1; j += dj) {
-#pragma unroll 1
-    for (int h = 0; h < 4; ++h) {
-      double av[4][2], bv[4][2];
+      const double av = (double)(t == 0 ? a[i].x : t == 1 ? a[i].y : t == 2 ? a[i].z : a[i].w);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { av[i][0] = a[i].x; av[i][1] = a[i].y; bv[i][0] = b[i].x; bv[i][1] = b[i].y; }
-      if (h < 3) fetch(j * kB + (h + 1) * 8 + kc);  // the next 8 columns are on their way while these are multiplied
-      else if (j + dj < j1) fetch((j + dj) * kB + kc);
-#pragma unroll
-      for (int t = 0; t < 2; ++t)
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int n = 0; n < 4; ++n) dmma(c[i][n][0], c[i][n][1], av[i][t], bv[n][t]);
+      for (int n = 0; n < 4; ++n) dmma(c[i][n][0], c[i][n][1], av, bv[n]);
     }
   }
+}
+// c += X_j L_j^T over the 32-column blocks j = j0, j0 + dj, ... < j1, 16 columns on their way while 16 are multiplied.
+__device__ __forceinline__ void block_sum(double (&c)[4][4][2], const float* X, int xr, const float* L, int lr, int r, int j0, int j1, int dj) {
+  if (j0 >= j1) return;
+  float4 a0[4], b0[4], a1[4], b1[4];
+  fetch16(a0, b0, X, xr, L, lr, r, j0 * kB);
+#pragma unroll 1
+  for (int j = j0; j < j1; j += dj) {
+    fetch16(a1, b1, X, xr, L, lr, r, j * kB + 16);
+    mma16(c, a0, b0);
+    if (j + dj < j1) fetch16(a0, b0, X, xr, L, lr, r, (j + dj) * kB);
+    mma16(c, a1, b1);
+  }
+}
+
+__device__ __forceinline__ void clear(double (&c)[4][4][2]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int n = 0; n < 4; ++n) c[i][n][0] = c[i][n][1] = 0.0;
 }
 
 __device__ __forceinline__ void store_part(double* p, const double (&c)[4][4][2]) {
@@ -88,12 +124,13 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
 
 __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const CholProblem* __restrict__ probs, unsigned* __restrict__ status) {
   extern __shared__ __align__(16) double csm[];
-  double* dpart = csm;                               // [4] quarters of the diagonal block's sum
+  double* dpart = csm;                               // [4] parts of the diagonal block's sum
   double* part = dpart + 4 * kPartDoubles;           // [kUnits] partial sums of the other blocks
-  double* Li = part + kUnits * kPartDoubles;         // [kB][kB + 1] inverse of the diagonal block of L
-  double* Lc = Li + kB * (kB + 1);                   // [kB][kB] columns of the diagonal block of L
+  double* Lc = part + kUnits * kPartDoubles;         // [kB][kB] columns of the diagonal block of L
   double* dinv = Lc + kB * kB;                       // [kB] 1 / its diagonal
+  double* Li = dinv + kB;                            // [kB][kLd] inverse of the diagonal block
   __shared__ float wmax[kCholWarps];
+  __shared__ float ga[kB * kB];                      // the Gram matrix' diagonal block of the coming panel, for warp 0
 
   const uint32_t rank = cluster_ctarank(), csize = cluster_nctarank();
   const CholProblem pb = probs[blockIdx.x / csize];
@@ -129,142 +166,183 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
   constexpr float kBreakdown = 3e-5f;
   const float abs_floor = md > 0.f ? md * 1e-12f : 1.f;
 
+  // Warps 0 and 4 (one scheduler's fp64 pipe, kept free of the products) factor and invert the diagonal block,
+  // warps 1 and 2 sum the diagonal block, the other four the row blocks.
+  const int u = warp == 3 ? 0 : warp > 4 ? warp - 4 : kUnits;
+  const int own = (int)rank < nb ? (nb - 1 - (int)rank) / (int)csize + 1 : 0;  // this CTA's row blocks: rank, rank + csize, ...
+  const bool ahead = own <= kUnits;  // every block of a panel has a warp of its own, so its sum may begin early
+  auto has = [&](int k) { return k % (int)csize == (int)rank; };
+  auto tiles = [&](int k) { return own - (has(k) ? 1 : 0); };                  // ... without the block of the diagonal
+  auto tile_block = [&](int k, int t) { return (int)rank + (int)csize * ((has(k) && t >= k / (int)csize) ? t + 1 : t); };
+  // slices of the summation index per block, so that a batch of `cnt` blocks has work for every warp
+  auto slices = [&](int cnt) { return cnt > 0 && cnt <= kUnits ? kUnits / cnt : 1; };
+  auto a_diag = [&](int k, int j) {  // element (lane, j) of the Gram matrix' diagonal block; A is symmetric
+    const int k0 = k * kB, kw = r - k0 < kB ? r - k0 : kB;
+    return lane < kw && j < kw ? A[(size_t)(k0 + j) * r + k0 + lane] : (lane == j ? 1.f : 0.f);
+  };
+
+  double c[4][4][2];  // a product warp's sum, begun one panel ahead
+  clear(c);
+  if (warp == 0)
+#pragma unroll
+    for (int j = 0; j < kB; ++j) ga[j * kB + lane] = a_diag(0, j);
+
+#pragma unroll 1
   for (int k = 0; k < nb; ++k) {
     const int k0 = k * kB, kw = r - k0 < kB ? r - k0 : kB;  // this panel's columns
-    // this CTA's other row blocks: b = rank, rank + csize, ... without k
-    const int own = ((int)rank < nb ? (nb - 1 - (int)rank) / (int)csize + 1 : 0);
-    const bool has_k = k % (int)csize == (int)rank;
-    const int ntiles = own - (has_k ? 1 : 0);
-    const int kpos = k / (int)csize;  // position of k in this CTA's list when has_k
-    auto tile_block = [&](int t) { return (int)rank + (int)csize * ((has_k && t >= kpos) ? t + 1 : t); };
-    // slices of the summation index per block, so that a batch of `cnt` blocks has work for every warp
-    auto slices = [&](int cnt) {
-      const int s = cnt > 0 ? kUnits / cnt : 1;
-      return s < 1 ? 1 : s > k && k > 0 ? k : k > 0 ? s : 1;
-    };
-    auto unit = [&](int base, int cnt, int s) {  // a warp's share of a batch of `cnt` blocks in `s` slices each
-      const int u = warp - 4;
-      if (u >= cnt * s) return;
-      const int b = tile_block(base + u / s), sl = u % s;
-      double c[4][4][2];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int n = 0; n < 4; ++n) c[i][n][0] = c[i][n][1] = 0.0;
-      block_sum(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + sl, k, s);
-      store_part(part + u * kPartDoubles, c);
-    };
-    const int first = ntiles < kUnits ? ntiles : kUnits;  // blocks of the first batch
+    const bool has_k = has(k);
+    const int ntiles = tiles(k), first = ntiles < kUnits ? ntiles : kUnits;
 
-    if (warp < 4) {
-      double c[4][4][2];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int n = 0; n < 4; ++n) c[i][n][0] = c[i][n][1] = 0.0;
-      block_sum(c, L, k0, L, k0, r, warp, k, 4);
-      store_part(dpart + warp * kPartDoubles, c);
+    // ---- the newest 32 columns (or, without a head start, all of them) and the sums to shared memory
+    if (u == kUnits) {
+      const int w = warp == 4 ? 3 : warp;
+      if (k > 0) block_cols(c, L, k0, L, k0, r, k0 - kB + w * 8);
+      store_part(dpart + w * kPartDoubles, c);
+      clear(c);
+    } else if (u < first * slices(first)) {
+      const int s = slices(first), b = tile_block(k, u / s), sl = u % s;
+      const float* X = b > k ? L : Z;
+      if (!ahead) block_sum(c, X, b * kB, L, k0, r, (b > k ? 0 : b) + sl, k, s);
+      else if (k > 0)
+        for (int h = sl; h < 4; h += s) block_cols(c, X, b * kB, L, k0, r, k0 - kB + h * 8);
+      store_part(part + u * kPartDoubles, c);
+      clear(c);
+    }
+
+    if (warp == 0) {
+      // Factor of the diagonal block: lane i holds row i of what is left of the block. The next pivot is kept up to
+      // date by its own lane (dg), so that the chain from column to column is a shuffle, a reciprocal square root
+      // (one Newton step in fp64 on rsqrtf's 22 bits: 44 bits) and two multiply-adds; the update of the columns
+      // behind the next one fills its gaps.
       asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (warp == 0) {
-        // Factor of the diagonal block: lane i holds row i of what is left of the block. The next pivot is kept
-        // up to date by its own lane (dg), so that the chain from column to column is a reciprocal square root
-        // (one Newton step in fp64 on rsqrtf's 22 bits: 44 bits) and two multiply-adds; the update of the
-        // columns behind the next one runs beside it.
-        double a[kB], dg = 1.0;
-        float own_floor = 0.f;
+      double a[kB], dg = 1.0, fl = 0.0;
 #pragma unroll
-        for (int j = 0; j < kB; ++j) {
-          const bool in = lane < kw && j < kw;
-          double s = in ? (double)A[(size_t)(k0 + j) * r + k0 + lane] : (lane == j ? 1.0 : 0.0);  // A is symmetric
-          if (in && lane == j) own_floor = fmaxf(kBreakdown * (float)s, abs_floor);
-          const double* q = dpart + lane * kLd + j;
-          s -= ((q[0] + q[kPartDoubles]) + (q[2 * kPartDoubles] + q[3 * kPartDoubles]));
-          a[j] = s;
-          if (lane == j) dg = s;
-        }
-        bool broke = false;
-#pragma unroll
-        for (int j = 0; j < kB; ++j) {
-          double d = __shfl_sync(0xffffffffu, dg, j);
-          float df = (float)d;
-          const float fl = __shfl_sync(0xffffffffu, own_floor, j);
-          if (!(df > fl)) {  // also catches NaN
-            broke = true;
-            df = fl;
-            d = (double)fl;
-          }
-          const double y0 = (double)rsqrtf(df);
-          const double y = fma(y0 * fma(-d * y0, y0, 1.0), 0.5, y0);  // 1 / L_jj
-          const double l = lane == j ? d * y : (lane > j ? a[j] * y : 0.0);
-          dg -= l * l;
-          Lc[j * kB + lane] = l;
-          if (lane == 0) dinv[j] = y;
-          __syncwarp();
-          if (j % 8 == 7) asm volatile("bar.arrive %0, 64;" ::"r"(2 + j / 8) : "memory");  // eight more columns for the inverse
-#pragma unroll
-          for (int j2 = j + 1; j2 < kB; ++j2) a[j2] -= l * Lc[j * kB + j2];
-        }
-        if (broke && lane == 0 && rank == 0) atomicOr(status, LORDO_FLAG_QR_BREAKDOWN);
-      } else if (warp == 1) {
-        // inverse of the diagonal block, column `lane`, eight columns of the factor behind warp 0
-        double x[kB];
-#pragma unroll
-        for (int i = 0; i < kB; ++i) x[i] = lane == i ? 1.0 : 0.0;
-#pragma unroll
-        for (int p = 0; p < kB; ++p) {
-          if (p % 8 == 0) asm volatile("bar.sync %0, 64;" ::"r"(2 + p / 8) : "memory");
-          x[p] *= dinv[p];
-          Li[p * (kB + 1) + lane] = x[p];
-#pragma unroll
-          for (int i = p + 1; i < kB; ++i) x[i] -= Lc[p * kB + i] * x[p];
+      for (int j = 0; j < kB; ++j) {
+        const double* q = dpart + j * kLd + lane;  // symmetric too
+        const float ga_j = ga[j * kB + lane];
+        a[j] = (double)ga_j - ((q[0] + q[kPartDoubles]) + (q[2 * kPartDoubles] + q[3 * kPartDoubles]));
+        if (lane == j) {
+          dg = a[j];
+          if (j < kw) fl = (double)fmaxf(kBreakdown * ga_j, abs_floor);
         }
       }
-    } else {
-      unit(0, first, slices(first));
+      bool broke = false;
+      double d, y;
+      auto pivot = [&](int j) {  // every lane offers its own; !(x > y) also catches NaN
+        const bool low = !(dg > fl);
+        if (lane == j) broke |= low;
+        d = __shfl_sync(0xffffffffu, low ? fl : dg, j);
+        const double y0 = (double)rsqrtf((float)d);
+        y = fma(0.5 * y0, fma(-d * y0, y0, 1.0), y0);  // 1 / L_jj
+      };
+      pivot(0);
+#pragma unroll
+      for (int j = 0; j < kB; ++j) {
+        const double l = lane == j ? d * y : (lane > j ? a[j] * y : 0.0);
+        dg -= l * l;
+        Lc[j * kB + lane] = l;
+        if (lane == 0) dinv[j] = y;
+        __syncwarp();
+        if (j % 8 == 7) asm volatile("bar.arrive %0, 64;" ::"r"(2 + j / 8) : "memory");  // eight more columns for the inverse
+        if (j + 1 < kB) {
+          a[j + 1] -= l * Lc[j * kB + j + 1];
+          pivot(j + 1);
+        }
+#pragma unroll
+        for (int j2 = (j + 2) & ~1; j2 < kB; j2 += 2) {
+          const double2 v = *reinterpret_cast<const double2*>(Lc + j * kB + j2);
+          if (j2 > j + 1) a[j2] -= l * v.x;
+          a[j2 + 1] -= l * v.y;
+        }
+      }
+      if (broke && rank == 0) atomicOr(status, LORDO_FLAG_QR_BREAKDOWN);
+      clear(c);  // not held in registers meanwhile
+    } else if (warp < 3) {
+      asm volatile("bar.arrive 1, 128;" ::: "memory");
+      if (k + 1 < nb) block_sum(c, L, k0 + kB, L, k0 + kB, r, warp - 1, k, 2);
+    } else if (warp == 4) {
+      asm volatile("bar.arrive 1, 128;" ::: "memory");
+      // inverse of the diagonal block, column `lane`, eight columns of the factor behind warp 0
+      double x[kB];
+#pragma unroll
+      for (int i = 0; i < kB; ++i) x[i] = lane == i ? 1.0 : 0.0;
+#pragma unroll
+      for (int p = 0; p < kB; ++p) {
+        if (p % 8 == 0) asm volatile("bar.sync %0, 64;" ::"r"(2 + p / 8) : "memory");
+        x[p] *= dinv[p];
+        Li[p * kLd + lane] = x[p];
+#pragma unroll
+        for (int i = (p + 1) & ~1; i < kB; i += 2) {
+          const double2 v = *reinterpret_cast<const double2*>(Lc + p * kB + i);
+          if (i > p) x[i] -= v.x * x[p];
+          x[i + 1] -= v.y * x[p];
+        }
+      }
+      clear(c);
+    } else if (ahead && k + 1 < nb) {
+      const int n1 = tiles(k + 1), s = slices(n1);
+      if (u < n1 * s) {
+        const int b = tile_block(k + 1, u / s), sl = u % s;
+        block_sum(c, b > k + 1 ? L : Z, b * kB, L, k0 + kB, r, (b > k + 1 ? 0 : b) + sl, k, s);
+      }
     }
-    __syncthreads();  // the inverse of the diagonal block and the partial sums of the first batch are there
 
+    // ---- Z_k = M Lkk^-T, eight rows of a block per warp and turn; the panel's own rows of rinv with the first batch
+    const int lr = lane >> 2, lc = lane & 3;
+    auto gram_init = [&](int b, int row, float (&g)[8]) {  // below the diagonal k0 + 32 <= row, so the columns exist
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) g[kk] = b > k && row < r ? A[(size_t)row * r + k0 + kk * 4 + lc] : 0.f;
+    };
+    float g[8];
+    if (warp < first * 4) gram_init(tile_block(k, warp >> 2), tile_block(k, warp >> 2) * kB + (warp & 3) * 8 + lr, g);
+    __syncthreads();  // the inverse of the diagonal block and the sums of the first batch are there
     for (int base = 0; base < ntiles || base == 0; base += kUnits) {
       const int cnt = ntiles - base < kUnits ? ntiles - base : kUnits;
       const int s = slices(cnt);
       if (base > 0) {
-        __syncthreads();  // the batch before is done with its partial sums
-        if (warp >= 4) unit(base, cnt, s);
+        __syncthreads();  // the batch before is done with its sums
+        if (u < cnt * s) {
+          const int b = tile_block(k, base + u / s);
+          block_sum(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + u % s, k, s);
+          store_part(part + u * kPartDoubles, c);
+          clear(c);
+        }
         __syncthreads();
       }
-      // Z_k = M Lkk^-T, eight rows of a block per warp and turn; the panel's own rows of rinv with the first batch
       const int strips = cnt * 4 + (base == 0 && has_k ? 4 : 0);
       for (int q = warp; q < strips; q += kCholWarps) {
         const int t = q >> 2, r8 = (q & 3) * 8;
         const bool diag = t == cnt;
-        const int b = diag ? k : tile_block(base + t);
-        const int row = b * kB + r8 + (lane >> 2);
-        double c[4][2];
+        const int b = diag ? k : tile_block(k, base + t);
+        const int row = b * kB + r8 + lr;
+        if (!diag && (q != warp || base > 0)) gram_init(b, row, g);
+        double z[4][2];
 #pragma unroll
-        for (int n = 0; n < 4; ++n) c[n][0] = c[n][1] = 0.0;
+        for (int n = 0; n < 4; ++n) z[n][0] = z[n][1] = 0.0;
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
-          const int col = kk * 4 + (lane & 3);
+          const int col = kk * 4 + lc;
           double m;
           if (diag) {
-            m = (r8 + (lane >> 2)) == col ? 1.0 : 0.0;
+            m = r8 + lr == col ? 1.0 : 0.0;
           } else {
-            m = (b > k && row < r) ? (double)A[(size_t)row * r + k0 + col] : 0.0;  // below the diagonal k0 + 32 <= row, so the columns exist
-            const double* q0 = part + (size_t)t * s * kPartDoubles + (r8 + (lane >> 2)) * kLd + col;
+            const double* q0 = part + (size_t)t * s * kPartDoubles + (r8 + lr) * kLd + col;
             double sum = 0.0;
-            for (int sl = 0; sl < s; ++sl) sum += q0[(size_t)sl * kPartDoubles];
-            m -= sum;
+#pragma unroll
+            for (int sl = 0; sl < kUnits; ++sl)
+              if (sl < s) sum += q0[(size_t)sl * kPartDoubles];
+            m = (double)g[kk] - sum;
           }
 #pragma unroll
-          for (int n = 0; n < 4; ++n) dmma(c[n][0], c[n][1], m, Li[(8 * n + (lane >> 2)) * (kB + 1) + col]);
+          for (int n = 0; n < 4; ++n) dmma(z[n][0], z[n][1], m, Li[(8 * n + lr) * kLd + col]);
         }
         if (row < r) {
           float* out = (b > k ? L : Z) + (size_t)row * r + k0;
 #pragma unroll
           for (int n = 0; n < 4; ++n) {
-            const int col = 8 * n + 2 * (lane & 3);
+            const int col = 8 * n + 2 * lc;
             if (col >= kw) continue;
-            float x = (float)c[n][0], y = (float)c[n][1];
+            float x = (float)z[n][0], y = (float)z[n][1];
             *reinterpret_cast<float2*>(out + col) = make_float2(x, y);
             if (b <= k && pb.rinv16) {
               __nv_bfloat16* o16 = pb.rinv16 + (size_t)row * r + k0 + col;
@@ -281,25 +359,45 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
       }
     }
     // the panel is in memory for every CTA of the cluster
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (warp == 0 && k + 1 < nb)
+#pragma unroll
+      for (int j = 0; j < kB; ++j) ga[j * kB + lane] = a_diag(k + 1, j);
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
 }
 
-// CTAs per problem: as many as the device has room for, up to the portable cluster size. More than half the
-// problem's panels would idle.
-void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, int sm_count, unsigned* status, cudaStream_t st) {
+static int g_clusters[9] = {};  // clusters of c CTAs that the device holds at once, set by chol_configure (one device model per process)
+
+static cudaLaunchConfig_t chol_launch(cudaLaunchAttribute* at, int nprobs, int c, cudaStream_t st) {
+  cudaLaunchConfig_t lc = {};
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = (unsigned)c; at->val.clusterDim.y = 1; at->val.clusterDim.z = 1;
+  lc.gridDim = dim3((unsigned)(nprobs * c), 1, 1); lc.blockDim = dim3(kCholWarps * 32, 1, 1); lc.dynamicSmemBytes = kCholSmem; lc.stream = st;
+  lc.attrs = at; lc.numAttrs = 1;
+  return lc;
+}
+
+// CTAs per problem: as many, up to the portable cluster size, as leave every problem a place on the device at
+// once (sixteen clusters of eight do not fit 148 SMs and would take two turns) and
+// every CTA at least two row blocks.
+void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, unsigned* status, cudaStream_t st) {
   const int panels = (r_max + kB - 1) / kB;
   int c = 1;
-  while (c < 8 && 2 * c <= panels && 2 * c * nprobs <= sm_count) c *= 2;
-  cudaLaunchConfig_t lc = {};
+  while (c < 8 && 2 * c <= panels && nprobs <= g_clusters[2 * c]) c *= 2;
   cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-  lc.gridDim = dim3((unsigned)(nprobs * c), 1, 1); lc.blockDim = dim3(kCholWarps * 32, 1, 1); lc.dynamicSmemBytes = kCholSmem; lc.stream = st;
-  lc.attrs = &at; lc.numAttrs = 1;
+  const cudaLaunchConfig_t lc = chol_launch(&at, nprobs, c, st);
   cudaLaunchKernelEx(&lc, chol_inverse_kernel, probs, status);
 }
 
-cudaError_t chol_configure() { return cudaFuncSetAttribute(chol_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmem); }
+cudaError_t chol_configure() {
+  cudaError_t e = cudaFuncSetAttribute(chol_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmem);
+  for (int c = 2; c <= 8 && e == cudaSuccess; c *= 2) {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t lc = chol_launch(&at, 256, c, nullptr);
+    e = cudaOccupancyMaxActiveClusters(&g_clusters[c], chol_inverse_kernel, &lc);
+  }
+  return e;
+}
 
 }  // namespace lordo

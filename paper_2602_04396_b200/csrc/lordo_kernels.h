@@ -172,7 +172,7 @@ struct CholProblem {
   long long plane;        // are written to rinv instead
   int r, pad;
 };
-void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, int sm_count, unsigned* status, cudaStream_t st);
+void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, unsigned* status, cudaStream_t st);
 cudaError_t chol_configure();
 
 // Rayleigh-Ritz truncation of an oversampled basis: C = (Q^T S)(Q^T S)^T is w x w symmetric (w = r + p
