@@ -25,7 +25,7 @@ enum Phase { PH_SUBSPACE = 0, PH_ROTATE = 1, PH_COMMIT = 2 };
 struct PlanStep {
   int type = ST_GEMM, phase = PH_SUBSPACE;
   int atrans = 0, dual = 0, a_square = 0;  // gemm
-  int r_max = 0;                           // chol
+  int r_max = 0;                           // chol, eig: largest size; gemm: longest contraction
   int p0 = 0;                              // random: 1 = initial projection (draw index 0), 0 = sketch (index = refresh count)
   long long first = 0, tiles = 0;          // tiles: gemm tiles or 256-thread blocks
   int count = 0;
@@ -487,7 +487,9 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       PlanStep st = sl.st;
       if (st.type == ST_GEMM) {
         st.first = (long long)P.size(); st.count = (int)sl.g.size(); st.tiles = 0;
+        st.r_max = 0;
         for (GemmProblem& g : sl.g) {
+          if (g.Kd > st.r_max) st.r_max = g.Kd;
           g.tile_start = st.tiles;
           st.tiles += (long long)((g.M + 63) / 64) * g.tiles_n;
           P.push_back(g);
@@ -1020,7 +1022,7 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
   switch (s.type) {
     case ST_GEMM:
       sc.a_square = s.a_square;
-      launch_gemm(c->d_probs + s.first, s.count, s.tiles, s.atrans, s.dual, c->cfg.check_mode != 0, sc, st);
+      launch_gemm(c->d_probs + s.first, s.count, s.tiles, s.r_max, s.atrans, s.dual, c->cfg.check_mode != 0, c->sm_count, sc, st);
       c->launches += 1;
       return check_launch(c, "gemm");
     case ST_CHOL:
@@ -1208,6 +1210,7 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
     int dev = 0;
     INIT_CUDA(cudaGetDevice(&dev));
     INIT_CUDA(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev));
+    INIT_CUDA(gemm_configure());
     INIT_CUDA(chol_configure());
   }
   if (c->tc) {

@@ -10,59 +10,152 @@ namespace lordo {
 
 constexpr int BM = 64, BN = 64, BK = 16, PADS = 4;
 
-__device__ __forceinline__ const void* operand_base(const Operand& op) {
-  return op.p0_ind ? *op.p0_ind : op.p0;
+// An operand as the main loop reads it, resolved once per tile.
+struct Source {
+  const void *p0, *p1;
+  long long ld;
+  float s0;
+  int dt0, dt1, kind;
+};
+__device__ __forceinline__ Source resolve(const Operand& op) {
+  Source s;
+  const void* base = op.p0_ind ? *op.p0_ind : op.p0;
+  s.p0 = reinterpret_cast<const char*>(base) + op.p0_off * (op.dt0 == LORDO_F32 ? 4 : 2);
+  s.p1 = op.p1; s.ld = op.ld; s.s0 = op.s0_ptr ? *op.s0_ptr : 1.f; s.dt0 = op.dt0; s.dt1 = op.dt1; s.kind = op.kind;
+  return s;
 }
 
-// Four consecutive stored elements (row, col..col+3) of an operand, zero outside (rows, cols).
-__device__ __forceinline__ float4 operand_load4(const Operand& op, const void* base, float s0, const GemmScalars& sc, long long row,
-                                                long long col, long long rows, long long cols) {
-  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+// Four consecutive stored elements (row, col..col+3) of an operand as loaded, zero outside (rows, cols); their
+// value is formed when they are put into shared memory, so that nothing waits for a load before that.
+struct Raw {
+  float4 a, b;
+};
+__device__ __forceinline__ Raw source_load(const Source& op, long long row, long long col, long long rows, long long cols) {
+  Raw o;
+  o.a = o.b = make_float4(0.f, 0.f, 0.f, 0.f);
   if (row >= rows || col >= cols) return o;
   const long long idx = row * op.ld + col;
   if (col + 3 < cols) {
-    const float4 a = load4(base, op.dt0, op.p0_off + idx);
-    if (op.kind == OP_PLAIN) {
-      o = make_float4(s0 * a.x, s0 * a.y, s0 * a.z, s0 * a.w);
-      if (op.p1) {
-        const float4 b = load4(op.p1, op.dt1, idx);
-        o.x += b.x; o.y += b.y; o.z += b.z; o.w += b.w;
-      }
-    } else if (op.kind == OP_UHAT) {
-      o = make_float4(sc.inv_bc1 * a.x, sc.inv_bc1 * a.y, sc.inv_bc1 * a.z, sc.inv_bc1 * a.w);
-    } else {
-      const float4 b = load4(op.p1, op.dt1, idx);
-      const float ux = sc.inv_bc1 * a.x, uy = sc.inv_bc1 * a.y, uz = sc.inv_bc1 * a.z, uw = sc.inv_bc1 * a.w;
-      o = make_float4(sc.inv_bc2 * b.x - ux * ux, sc.inv_bc2 * b.y - uy * uy, sc.inv_bc2 * b.z - uz * uz,
-                      sc.inv_bc2 * b.w - uw * uw);
+    o.a = load4(op.p0, op.dt0, idx);
+    if (op.p1) o.b = load4(op.p1, op.dt1, idx);
+  } else {
+    float t[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int e = 0; e < 4 && col + e < cols; ++e) {
+      t[e] = load1(op.p0, op.dt0, idx + e);
+      if (op.p1) u[e] = load1(op.p1, op.dt1, idx + e);
     }
-    return o;
+    o.a = make_float4(t[0], t[1], t[2], t[3]);
+    o.b = make_float4(u[0], u[1], u[2], u[3]);
   }
-  float t[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int e = 0; e < 4 && col + e < cols; ++e) {
-    const float a = load1(base, op.dt0, op.p0_off + idx + e);
-    if (op.kind == OP_PLAIN) {
-      t[e] = s0 * a + (op.p1 ? load1(op.p1, op.dt1, idx + e) : 0.f);
-    } else if (op.kind == OP_UHAT) {
-      t[e] = sc.inv_bc1 * a;
-    } else {
-      const float uh = sc.inv_bc1 * a;
-      t[e] = sc.inv_bc2 * load1(op.p1, op.dt1, idx + e) - uh * uh;
-    }
-  }
-  return make_float4(t[0], t[1], t[2], t[3]);
+  return o;
+}
+__device__ __forceinline__ float4 source_value(const Source& op, const Raw& x, const GemmScalars& sc) {
+  if (op.kind == OP_PLAIN) return make_float4(op.s0 * x.a.x + x.b.x, op.s0 * x.a.y + x.b.y, op.s0 * x.a.z + x.b.z, op.s0 * x.a.w + x.b.w);
+  const float4 u = make_float4(sc.inv_bc1 * x.a.x, sc.inv_bc1 * x.a.y, sc.inv_bc1 * x.a.z, sc.inv_bc1 * x.a.w);
+  if (op.kind == OP_UHAT) return u;
+  return make_float4(sc.inv_bc2 * x.b.x - u.x * u.x, sc.inv_bc2 * x.b.y - u.y * u.y, sc.inv_bc2 * x.b.z - u.z * u.z, sc.inv_bc2 * x.b.w - u.w * u.w);
 }
 
+// One output row, columns col .. col+3 (N is a multiple of 4).
+template <int DUAL>
+__device__ __forceinline__ void gemm_epilogue(const Epilogue& ep, const GemmScalars& sc, int N, long long row, long long col, const float (&a)[4],
+                                              const float (&a2)[4]) {
+  if (ep.kind == EPI_STORE && ep.trans) {  // C[col][row]
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float* cp = ep.C + (col + j) * ep.ldc + row;
+      *cp = ep.pad ? *cp + a[j] : a[j];
+    }
+  } else if (ep.kind == EPI_STORE) {
+    float4* cp = reinterpret_cast<float4*>(ep.C + row * ep.ldc + col);
+    float4 o = make_float4(a[0], a[1], a[2], a[3]);
+    if (ep.pad) {  // accumulate into C
+      const float4 old = *cp;
+      o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w;
+    }
+    *cp = o;
+  } else if (ep.kind == EPI_APPLY && ep.trans) {
+    // the product was formed for the transposed problem: output (row, col) is weight element (col, row),
+    // and the full-rank QHM scale belongs to the output column = the weight's row
+    if constexpr (DUAL) {
+      const float c = *ep.cptr;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const long long idx = (col + j) * ep.ldt + row;
+        const float g = load1(*ep.G_ind, sc.g_dt, ep.G_off + idx);
+        const float w = load1(ep.W, sc.w_dt, idx);
+        float upd = a2[j];
+        if (sc.form == LORDO_QHM_FULL) upd = (1.f - sc.omega) * (c * g) / ep.dcol[col + j] + sc.omega * upd;
+        if (sc.ef) store1(ep.E, sc.e_dt, idx, (c * g + load1(ep.E, sc.e_dt, idx)) - a[j]);
+        store1(ep.W, sc.w_dt, idx, w - sc.lr * upd);
+      }
+    }
+  } else if (ep.kind == EPI_APPLY) {
+    if constexpr (DUAL) {
+      const long long idx = row * (long long)N + col;
+      const float c = *ep.cptr;
+      const float4 g = load4(*ep.G_ind, sc.g_dt, ep.G_off + idx);
+      const float4 w = load4(ep.W, sc.w_dt, idx);
+      float4 upd = make_float4(a2[0], a2[1], a2[2], a2[3]);
+      if (sc.form == LORDO_QHM_FULL) {
+        const float4 d = *reinterpret_cast<const float4*>(ep.dcol + col);
+        const float w1 = 1.f - sc.omega;
+        upd.x = w1 * (c * g.x) / d.x + sc.omega * upd.x;
+        upd.y = w1 * (c * g.y) / d.y + sc.omega * upd.y;
+        upd.z = w1 * (c * g.z) / d.z + sc.omega * upd.z;
+        upd.w = w1 * (c * g.w) / d.w + sc.omega * upd.w;
+      }
+      if (sc.ef) {
+        const float4 e = load4(ep.E, sc.e_dt, idx);
+        float4 en;
+        en.x = (c * g.x + e.x) - a[0];
+        en.y = (c * g.y + e.y) - a[1];
+        en.z = (c * g.z + e.z) - a[2];
+        en.w = (c * g.w + e.w) - a[3];
+        store4(ep.E, sc.e_dt, idx, en);
+      }
+      store4(ep.W, sc.w_dt, idx, make_float4(w.x - sc.lr * upd.x, w.y - sc.lr * upd.y, w.z - sc.lr * upd.z, w.w - sc.lr * upd.w));
+    }
+  } else {  // EPI_ROTATE: a = Rot u^, a2 = (Rot o Rot)(v^ - u^ o u^)
+    if constexpr (DUAL) {
+      const long long idx = row * (long long)N + col;
+      float4 un, vn;
+      un.x = sc.bc1 * a[0]; un.y = sc.bc1 * a[1]; un.z = sc.bc1 * a[2]; un.w = sc.bc1 * a[3];
+      vn.x = sc.bc2 * fabsf(a2[0] + a[0] * a[0]);
+      vn.y = sc.bc2 * fabsf(a2[1] + a[1] * a[1]);
+      vn.z = sc.bc2 * fabsf(a2[2] + a[2] * a[2]);
+      vn.w = sc.bc2 * fabsf(a2[3] + a[3] * a[3]);
+      *reinterpret_cast<float4*>(ep.u_out + idx) = un;
+      *reinterpret_cast<float4*>(ep.v_out + idx) = vn;
+    }
+  }
+}
+
+// Four partial sums of the CTA of rank `rank` of the cluster.
+__device__ __forceinline__ void partials_of(const double* p, unsigned rank, double (&v)[4]) {
+  const unsigned here = (unsigned)__cvta_generic_to_shared(p);
+  unsigned there;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(here), "r"(rank));
+  asm volatile("ld.shared::cluster.v2.f64 {%0,%1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(there) : "memory");
+  asm volatile("ld.shared::cluster.v2.f64 {%0,%1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "r"(there + 16u) : "memory");
+}
+
+// A cluster of CTAs works on one output tile, each on a range of k; the partial sums meet in fp64 through
+// distributed shared memory, every CTA finishing its share of the tile's rows (see launch_gemm for the size).
 // CARRY = 1: slice sums carried across k-slices in fp64 (parity mode). CARRY = 0: plain fp32
 // accumulation, half the registers (the fp32 work of the fast mode: QR and moment rotation).
 template <int ATRANS, int DUAL, int CARRY>
-__global__ void __launch_bounds__(256) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
-  __shared__ __align__(16) float sA[BK][BM + PADS];
-  __shared__ __align__(16) float sB[BK][BN + PADS];
-  __shared__ __align__(16) float sB2[DUAL ? BK : 1][BN + PADS];
+__global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
+  __shared__ __align__(16) float sA[2][BK][BM + PADS];
+  __shared__ __align__(16) float sB[2][BK][BN + PADS];
+  __shared__ __align__(16) float sB2[2][DUAL ? BK : 1][BN + PADS];
+  extern __shared__ __align__(16) double part[];  // [1 or 2 products][BM][BN] partial sums of this CTA, clusters only
+  unsigned rank, csize;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
 
   // locate the problem of this block
-  const long long blk = blockIdx.x;
+  const long long blk = blockIdx.x / csize;
   int lo = 0, hi = nprobs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -74,13 +167,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(const GemmProblem* __res
   const int M = pr.M, N = pr.N, Kd = pr.Kd;
   const long long m0 = (long long)tile_m * BM, n0 = (long long)tile_n * BN;
 
-  const void* baseA = operand_base(pr.A);
-  const void* baseB = operand_base(pr.B);
-  const void* baseB2 = DUAL ? operand_base(pr.B2) : nullptr;
-  const float sA0 = pr.A.s0_ptr ? *pr.A.s0_ptr : 1.f;
-  const float sB0 = pr.B.s0_ptr ? *pr.B.s0_ptr : 1.f;
-  float sB20 = 1.f;
-  if constexpr (DUAL) sB20 = pr.B2.s0_ptr ? *pr.B2.s0_ptr : 1.f;
+  const Source A = resolve(pr.A), B = resolve(pr.B), B2 = resolve(DUAL ? pr.B2 : pr.B);
 
   const int t = threadIdx.x;
   const int tx = t & 15, ty = t >> 4;
@@ -103,32 +190,41 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(const GemmProblem* __res
       }
     }
 
-  float4 ra, rb, rb2 = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto fetch = [&](int k0) {
-    if (ATRANS) ra = operand_load4(pr.A, baseA, sA0, sc, k0 + ar, m0 + ac, Kd, M);
-    else ra = operand_load4(pr.A, baseA, sA0, sc, m0 + ar, k0 + ac, M, Kd);
-    rb = operand_load4(pr.B, baseB, sB0, sc, k0 + bk, n0 + bc, Kd, N);
-    if constexpr (DUAL) rb2 = operand_load4(pr.B2, baseB2, sB20, sc, k0 + bk, n0 + bc, Kd, N);
+  // Two slices of k are on their way in registers while a third, in one of two buffers, is multiplied.
+  struct Slice {
+    Raw a, b, b2;
   };
-  auto stash = [&]() {
+  auto fetch = [&](Slice& x, int k0) {
+    if (ATRANS) x.a = source_load(A, k0 + ar, m0 + ac, Kd, M);
+    else x.a = source_load(A, m0 + ar, k0 + ac, M, Kd);
+    x.b = source_load(B, k0 + bk, n0 + bc, Kd, N);
+    if constexpr (DUAL) x.b2 = source_load(B2, k0 + bk, n0 + bc, Kd, N);
+  };
+  auto stash = [&](const Slice& x, int buf) {
+    const float4 v = source_value(A, x.a, sc);
     if (ATRANS) {
-      *reinterpret_cast<float4*>(&sA[ar][ac]) = ra;
+      *reinterpret_cast<float4*>(&sA[buf][ar][ac]) = v;
     } else {
-      sA[ac + 0][ar] = ra.x; sA[ac + 1][ar] = ra.y; sA[ac + 2][ar] = ra.z; sA[ac + 3][ar] = ra.w;
+      sA[buf][ac + 0][ar] = v.x; sA[buf][ac + 1][ar] = v.y; sA[buf][ac + 2][ar] = v.z; sA[buf][ac + 3][ar] = v.w;
     }
-    *reinterpret_cast<float4*>(&sB[bk][bc]) = rb;
-    if constexpr (DUAL) *reinterpret_cast<float4*>(&sB2[bk][bc]) = rb2;
+    *reinterpret_cast<float4*>(&sB[buf][bk][bc]) = source_value(B, x.b, sc);
+    if constexpr (DUAL) *reinterpret_cast<float4*>(&sB2[buf][bk][bc]) = source_value(B2, x.b2, sc);
   };
 
-  fetch(0);
-  for (int k0 = 0; k0 < Kd; k0 += BK) {
-    stash();
-    __syncthreads();
-    if (k0 + BK < Kd) fetch(k0 + BK);
+  // this CTA's range of k
+  const int per = ((Kd + BK - 1) / BK + (int)csize - 1) / (int)csize * BK;
+  const int kbeg = min((int)rank * per, Kd), kend = min(kbeg + per, Kd);
+  Slice x0, x1;
+  if (kbeg < kend) fetch(x0, kbeg);
+  if (kbeg + BK < kend) fetch(x1, kbeg + BK);
+  if (kbeg < kend) stash(x0, 0);
+  __syncthreads();
+  int buf = 0;
+  auto multiply = [&]() {
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&sA[kk][ty * 4]);
-      const float4 b4 = *reinterpret_cast<const float4*>(&sB[kk][tx * 4]);
+      const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][kk][ty * 4]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&sB[buf][kk][tx * 4]);
       const float a[4] = {a4.x, a4.y, a4.z, a4.w};
       const float b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
@@ -136,7 +232,7 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(const GemmProblem* __res
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
       if constexpr (DUAL) {
-        const float4 c4 = *reinterpret_cast<const float4*>(&sB2[kk][tx * 4]);
+        const float4 c4 = *reinterpret_cast<const float4*>(&sB2[buf][kk][tx * 4]);
         const float c[4] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -156,7 +252,62 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(const GemmProblem* __res
           if constexpr (DUAL) { tot2[i][j] += (double)acc2[i][j]; acc2[i][j] = 0.f; }
         }
     }
-    __syncthreads();
+  };
+  // on entry to a turn `far` is free, `near` holds the slice after the one in `buf`
+  auto turn = [&](int k0, Slice& far, const Slice& near) {
+    if (k0 + 2 * BK < kend) fetch(far, k0 + 2 * BK);
+    multiply();
+    if (k0 + BK < kend) {
+      stash(near, buf ^ 1);
+      __syncthreads();
+    }
+    buf ^= 1;
+  };
+  for (int k0 = kbeg; k0 < kend; k0 += 2 * BK) {
+    turn(k0, x0, x1);
+    if (k0 + BK < kend) turn(k0 + BK, x1, x0);
+  }
+  const Epilogue& ep = pr.epi;
+  if (csize > 1) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      double v[4], v2[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if constexpr (CARRY) v[j] = tot[i][j]; else v[j] = (double)acc[i][j];
+        if constexpr (CARRY && DUAL) v2[j] = tot2[i][j]; else v2[j] = (double)acc2[DUAL ? i : 0][j];
+      }
+      double2* o = reinterpret_cast<double2*>(part + (ty * 4 + i) * BN + tx * 4);
+      o[0] = make_double2(v[0], v[1]); o[1] = make_double2(v[2], v[3]);
+      if constexpr (DUAL) {
+        double2* o2 = o + BM * BN / 2;
+        o2[0] = make_double2(v2[0], v2[1]); o2[1] = make_double2(v2[2], v2[3]);
+      }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int rows = BM / (int)csize;
+    for (int e = t; e < rows * (BN / 4); e += 256) {
+      const int lr = (int)rank * rows + e / (BN / 4), lc = (e % (BN / 4)) * 4;
+      const long long row = m0 + lr, col = n0 + lc;
+      if (row >= M || col >= N) continue;
+      double s1[4] = {0.0, 0.0, 0.0, 0.0}, s2[4] = {0.0, 0.0, 0.0, 0.0};
+      for (unsigned q = 0; q < csize; ++q) {
+        double v[4];
+        partials_of(part + lr * BN + lc, q, v);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s1[j] += v[j];
+        if constexpr (DUAL) {
+          partials_of(part + BM * BN + lr * BN + lc, q, v);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) s2[j] += v[j];
+        }
+      }
+      const float a1[4] = {(float)s1[0], (float)s1[1], (float)s1[2], (float)s1[3]}, a2[4] = {(float)s2[0], (float)s2[1], (float)s2[2], (float)s2[3]};
+      gemm_epilogue<DUAL>(ep, sc, N, row, col, a1, a2);
+    }
+    // nobody leaves while its partial sums may still be read
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return;
   }
   if constexpr (CARRY) {
 #pragma unroll
@@ -167,102 +318,61 @@ __global__ void __launch_bounds__(256) gemm_ffma_kernel(const GemmProblem* __res
         if constexpr (DUAL) acc2[i][j] = (float)tot2[i][j];
       }
   }
-
-  // ---- epilogue: each thread owns rows m0+ty*4.., columns n0+tx*4..+3 (N is a multiple of 4)
-  const Epilogue& ep = pr.epi;
+  // each thread owns rows m0+ty*4.., columns n0+tx*4..+3
   const long long col = n0 + tx * 4;
   if (col >= N) return;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const long long row = m0 + ty * 4 + i;
     if (row >= M) break;
-    if (ep.kind == EPI_STORE && ep.trans) {  // C[col][row]
-      const float o[4] = {acc[i][0], acc[i][1], acc[i][2], acc[i][3]};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float* cp = ep.C + (col + j) * ep.ldc + row;
-        *cp = ep.pad ? *cp + o[j] : o[j];
-      }
-    } else if (ep.kind == EPI_STORE) {
-      float4* cp = reinterpret_cast<float4*>(ep.C + row * ep.ldc + col);
-      float4 o = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-      if (ep.pad) {  // accumulate into C
-        const float4 old = *cp;
-        o.x += old.x; o.y += old.y; o.z += old.z; o.w += old.w;
-      }
-      *cp = o;
-    } else if (ep.kind == EPI_APPLY && ep.trans) {
-      // the product was formed for the transposed problem: output (row, col) is weight element (col, row),
-      // and the full-rank QHM scale belongs to the output column = the weight's row
-      if constexpr (DUAL) {
-        const float c = *ep.cptr;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const long long idx = (col + j) * ep.ldt + row;
-          const float g = load1(*ep.G_ind, sc.g_dt, ep.G_off + idx);
-          const float w = load1(ep.W, sc.w_dt, idx);
-          float upd = acc2[i][j];
-          if (sc.form == LORDO_QHM_FULL) upd = (1.f - sc.omega) * (c * g) / ep.dcol[col + j] + sc.omega * upd;
-          if (sc.ef) store1(ep.E, sc.e_dt, idx, (c * g + load1(ep.E, sc.e_dt, idx)) - acc[i][j]);
-          store1(ep.W, sc.w_dt, idx, w - sc.lr * upd);
-        }
-      }
-    } else if (ep.kind == EPI_APPLY) {
-      if constexpr (DUAL) {
-        const long long idx = row * (long long)N + col;
-        const float c = *ep.cptr;
-        const float4 g = load4(*ep.G_ind, sc.g_dt, ep.G_off + idx);
-        const float4 w = load4(ep.W, sc.w_dt, idx);
-        float4 upd = make_float4(acc2[i][0], acc2[i][1], acc2[i][2], acc2[i][3]);
-        if (sc.form == LORDO_QHM_FULL) {
-          const float4 d = *reinterpret_cast<const float4*>(ep.dcol + col);
-          const float w1 = 1.f - sc.omega;
-          upd.x = w1 * (c * g.x) / d.x + sc.omega * upd.x;
-          upd.y = w1 * (c * g.y) / d.y + sc.omega * upd.y;
-          upd.z = w1 * (c * g.z) / d.z + sc.omega * upd.z;
-          upd.w = w1 * (c * g.w) / d.w + sc.omega * upd.w;
-        }
-        if (sc.ef) {
-          const float4 e = load4(ep.E, sc.e_dt, idx);
-          float4 en;
-          en.x = (c * g.x + e.x) - acc[i][0];
-          en.y = (c * g.y + e.y) - acc[i][1];
-          en.z = (c * g.z + e.z) - acc[i][2];
-          en.w = (c * g.w + e.w) - acc[i][3];
-          store4(ep.E, sc.e_dt, idx, en);
-        }
-        store4(ep.W, sc.w_dt, idx, make_float4(w.x - sc.lr * upd.x, w.y - sc.lr * upd.y, w.z - sc.lr * upd.z, w.w - sc.lr * upd.w));
-      }
-    } else {  // EPI_ROTATE: acc = Rot u^, acc2 = (Rot o Rot)(v^ - u^ o u^)
-      if constexpr (DUAL) {
-        const long long idx = row * (long long)N + col;
-        float4 un, vn;
-        un.x = sc.bc1 * acc[i][0]; un.y = sc.bc1 * acc[i][1]; un.z = sc.bc1 * acc[i][2]; un.w = sc.bc1 * acc[i][3];
-        vn.x = sc.bc2 * fabsf(acc2[i][0] + acc[i][0] * acc[i][0]);
-        vn.y = sc.bc2 * fabsf(acc2[i][1] + acc[i][1] * acc[i][1]);
-        vn.z = sc.bc2 * fabsf(acc2[i][2] + acc[i][2] * acc[i][2]);
-        vn.w = sc.bc2 * fabsf(acc2[i][3] + acc[i][3] * acc[i][3]);
-        *reinterpret_cast<float4*>(ep.u_out + idx) = un;
-        *reinterpret_cast<float4*>(ep.v_out + idx) = vn;
-      }
-    }
+    gemm_epilogue<DUAL>(ep, sc, N, row, col, acc[i], acc2[DUAL ? i : 0]);
   }
 }
 
-void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int atrans, int dual, int carry, const GemmScalars& sc,
-                 cudaStream_t st) {
-  const unsigned grid = (unsigned)total_tiles;
+// CTAs per output tile: doubled, up to the portable cluster size, while all of them have a place on the device at
+// once and each is left two slices of k. A product with few tiles is a chain of slices, each about a trip to
+// memory long: 256 x 256, r = 16, two replicas, P^T (c G + E) in 8 CTAs 44 us, in 64 10.5; Gram matrices of 1000 rows
+// and r up to 136 in 14 CTAs 105 us, in 112 17.
+void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
+                 const GemmScalars& sc, cudaStream_t st) {
+  const long long room = (long long)sm_count * (dual && carry ? 1 : 2);  // by registers
+  const int slices = (kd_max + BK - 1) / BK;
+  int c = 1;
+  while (c < 8 && total_tiles * 2 * c <= room && slices >= 4 * c) c *= 2;
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(256, 1, 1); lc.stream = st;
+  lc.dynamicSmemBytes = c > 1 ? sizeof(double) * BM * BN * (dual ? 2 : 1) : 0;
+  lc.attrs = &at; lc.numAttrs = 1;
+#define LORDO_GEMM(A, B, C) cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, C>, probs, nprobs, sc)
   if (carry) {
-    if (atrans && !dual) gemm_ffma_kernel<1, 0, 1><<<grid, 256, 0, st>>>(probs, nprobs, sc);
-    else if (!atrans && !dual) gemm_ffma_kernel<0, 0, 1><<<grid, 256, 0, st>>>(probs, nprobs, sc);
-    else if (!atrans && dual) gemm_ffma_kernel<0, 1, 1><<<grid, 256, 0, st>>>(probs, nprobs, sc);
-    else gemm_ffma_kernel<1, 1, 1><<<grid, 256, 0, st>>>(probs, nprobs, sc);
+    if (atrans && !dual) LORDO_GEMM(1, 0, 1);
+    else if (!atrans && !dual) LORDO_GEMM(0, 0, 1);
+    else if (!atrans && dual) LORDO_GEMM(0, 1, 1);
+    else LORDO_GEMM(1, 1, 1);
   } else {
-    if (atrans && !dual) gemm_ffma_kernel<1, 0, 0><<<grid, 256, 0, st>>>(probs, nprobs, sc);
-    else if (!atrans && !dual) gemm_ffma_kernel<0, 0, 0><<<grid, 256, 0, st>>>(probs, nprobs, sc);
-    else if (!atrans && dual) gemm_ffma_kernel<0, 1, 0><<<grid, 256, 0, st>>>(probs, nprobs, sc);
-    else gemm_ffma_kernel<1, 1, 0><<<grid, 256, 0, st>>>(probs, nprobs, sc);
+    if (atrans && !dual) LORDO_GEMM(1, 0, 0);
+    else if (!atrans && !dual) LORDO_GEMM(0, 0, 0);
+    else if (!atrans && dual) LORDO_GEMM(0, 1, 0);
+    else LORDO_GEMM(1, 1, 0);
   }
+#undef LORDO_GEMM
+}
+
+// With its partial sums a CTA exceeds the 48 KB of shared memory that a launch may ask for unannounced.
+cudaError_t gemm_configure() {
+  const int one = (int)(sizeof(double) * BM * BN), two = 2 * one;
+  cudaError_t e = cudaSuccess;
+  auto set = [&](const void* kernel, int smem) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  };
+  set((const void*)gemm_ffma_kernel<0, 0, 0>, one); set((const void*)gemm_ffma_kernel<0, 0, 1>, one);
+  set((const void*)gemm_ffma_kernel<1, 0, 0>, one); set((const void*)gemm_ffma_kernel<1, 0, 1>, one);
+  set((const void*)gemm_ffma_kernel<0, 1, 0>, two); set((const void*)gemm_ffma_kernel<0, 1, 1>, two);
+  set((const void*)gemm_ffma_kernel<1, 1, 0>, two); set((const void*)gemm_ffma_kernel<1, 1, 1>, two);
+  return e;
 }
 
 // ---------------------------------------------------------------------------------------------

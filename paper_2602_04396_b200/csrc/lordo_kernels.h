@@ -65,8 +65,9 @@ struct GemmScalars {
   int form, ef, w_dt, e_dt, g_dt, a_square;
 };
 
-void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int atrans, int dual, int carry, const GemmScalars& sc,
-                 cudaStream_t st);
+void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
+                 const GemmScalars& sc, cudaStream_t st);
+cudaError_t gemm_configure();
 
 // ---------------------------------------------------------------------------------------------
 // Tensor-core path of the inner step (bf16 operands, fp32 accumulation), see lordo_tc.cu.

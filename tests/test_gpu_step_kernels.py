@@ -1,0 +1,26 @@
+"""Edges of the kernels of the inner step, against the oracle."""
+import pytest
+
+from paper_2602_04396_b200 import synth
+from tests import harness as hz
+from tests.harness import RunSpec
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape", [(8, 8, 8), (72, 64, 8), (136, 72, 64), (1000, 64, 16), (520, 600, 72)])
+@pytest.mark.parametrize("side", [0, 1])
+def test_fp32_products_in_ranges_of_k(shape, side):
+    """The fp32 products with their contraction in one CTA or dealt out over a cluster (few tiles, long
+    contraction), ranges without a slice and a ragged last slice among them. The ranges meet in fp64, so the
+    bound of the other check-mode tests (1e-3, a few fp32 ulps per step in fact) is held to 2e-5."""
+    m, n, r = shape
+    if side:
+        m, n = n, m
+    wl = synth.Workload("t", ((m, n, r),), K=2, H=2, rounds=1, grad="gauss", clip_rho=30.0, sides=(side,))
+    spec = RunSpec(wl, variant=1, form=2, lr=0.01, omega=0.9, eps=0.05, refresh=False)
+    opt, orc = hz.run_gpu(spec), hz.run_oracle(spec)
+    st = hz.compare_states(opt, orc)
+    assert opt.poll_status() == 0
+    assert max(st["W"], st["E"], st["u"], st["v"]) < 2e-5, st
+    opt.close()
