@@ -15,6 +15,7 @@ using namespace lordo;
 namespace {
 
 constexpr int kMaxK = 64;
+constexpr int kMaxWorkers = 256;  // CTAs (or CTA pairs) that walk a list of work
 constexpr long long kPairs = 74;  // CTA pairs that the work of a refresh is planned for (148 SMs)
 
 enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_COLSQ = 6, ST_EIG = 7, ST_GRAM = 8, ST_BASIS = 9, ST_ROT = 10 };
@@ -105,17 +106,16 @@ struct lordo_ctx {
   // tensor-core path of the inner step (check_mode == 0 and every r <= 256)
   bool tc = false;
   TcProblem* d_tc_probs = nullptr;
-  // the update kernel runs once per side present: its table lists the problems stored as they are
-  // projected first, then the ones stored transposed (matrices projected from the right)
-  TcProblem* d_tc_apply = nullptr;
-  std::vector<TcProblem> h_tc_apply;
-  int tc_n_left = 0;
-  long long tc_strips_left = 0;
+  // TMA-fed kernels: who does what, [0] projection, [1] update of the problems stored as they are projected,
+  // [2] of the ones stored transposed (matrices projected from the right)
+  TcSeg* d_segs[3] = {nullptr, nullptr, nullptr};
+  int* d_seg_start[3] = {nullptr, nullptr, nullptr};
+  int seg_workers[3] = {0, 0, 0};
   TcPrep* d_tc_prep = nullptr;
   long long* d_prep_start = nullptr;
   char* d_tc_bf16 = nullptr;  // all bf16 operand copies, zeroed once by lordo_init
   size_t tc_bf16_bytes = 0;
-  long long tc_strips = 0, tc_strips_p = 0, prep_blocks = 0;
+  long long tc_strips = 0, tc_pairs = 0, prep_blocks = 0;
   int tc_rn_max = 0, tc_rk_max = 0;
   // TMA-fed kernels (bf16 storage): tensor maps per matrix, gradient maps re-encoded per pointer change
   bool tma = false;
@@ -270,6 +270,52 @@ void prefix_arrays(const lordo_config& cfg, std::vector<long long>& chunk_start,
   }
 }
 
+// Deals the work of the TMA-fed kernels out, longest pieces first, each to the worker with the least so far.
+// An item is a strip (or a pair of strips) of `len` steps that costs `cost`; `lists` comes back with every worker's
+// pieces, `start` with their offsets. With `split` a strip that would take its worker past the even share is cut
+// there and the rest dealt on, so that all workers end together; a piece costs `head` on top of its steps (its
+// operands are fetched anew; about four steps) and has at least kMinPiece. Strips dealt round the grid ended apart
+// wherever they were few or of different lengths: 7 layers of 768 (r = 128, K = 8) update 183 us, dealt out 137 us.
+constexpr int kMinPiece = 8;
+struct WorkItem {
+  int prob, strip, len;
+  double cost;
+};
+void deal_out(std::vector<WorkItem> items, int workers, bool split, double head, std::vector<TcSeg>& list, std::vector<int>& start) {
+  std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.cost > b.cost; });
+  double total = 0.0;
+  for (const WorkItem& it : items) total += it.cost + head;
+  const double share = std::max(total / workers + (split ? head / 2 : 0.0), split ? kMinPiece + head : 0.0);
+  std::vector<std::vector<TcSeg>> lists(workers);
+  typedef std::pair<double, int> Load;  // what a worker has, the worker
+  std::vector<Load> heap;
+  for (int w = 0; w < workers; ++w) heap.push_back(Load(0.0, w));
+  const auto later = [](const Load& a, const Load& b) { return a > b; };
+  for (const WorkItem& it : items) {
+    int t0 = 0;
+    while (t0 < it.len) {
+      std::pop_heap(heap.begin(), heap.end(), later);
+      Load& ld = heap.back();
+      int n = it.len - t0;
+      if (split) {
+        const int room = (int)(share - ld.first - head + 0.5);
+        if (n > room) n = std::min(n, std::max(room, kMinPiece));
+        if (it.len - t0 - n < kMinPiece) n = it.len - t0;
+      }
+      lists[ld.second].push_back({it.prob, it.strip, t0, t0 + n});
+      ld.first += it.cost * n / it.len + head;
+      t0 += n;
+      std::push_heap(heap.begin(), heap.end(), later);
+    }
+  }
+  list.clear();
+  start.assign(1, 0);
+  for (const std::vector<TcSeg>& l : lists) {
+    list.insert(list.end(), l.begin(), l.end());
+    start.push_back((int)list.size());
+  }
+}
+
 // Builds everything that lives in the workspace. With ws == nullptr only the size is computed.
 size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   const lordo_config& cfg = c->cfg;
@@ -376,7 +422,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   for (int i = 0; i < n_mats; ++i)  // ranks above 512 (above 256 with fp32 storage) run on the fp32 path
     if (cfg.mats[i].r > (cfg.w_dtype == LORDO_BF16 ? 512 : 256) || (cfg.mats[i].side && cfg.w_dtype != LORDO_BF16)) c->tc = false;
   c->h_tc.clear(); c->h_prep.clear(); c->h_prep_start.assign(1, 0);
-  c->tc_strips = 0; c->tc_strips_p = 0; c->tc_rn_max = 0; c->tc_rk_max = 0;
+  c->tc_strips = 0; c->tc_pairs = 0; c->tc_rn_max = 0; c->tc_rk_max = 0;
   std::vector<size_t> h_prep_first(n_mats, 0);  // first entry of a matrix in h_prep
   if (c->tc) {
     auto up = [](long long x, long long q) { return (x + q - 1) / q * q; };
@@ -424,35 +470,24 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         tp.G_ind = c->d_Gtab + i; tp.G_off = wo;
         tp.cptr = c->d_coef + (size_t)i * K + k;
         tp.mat = i; tp.replica = k; tp.pcopy = pk;
-        tp.strip_start_p = c->tc_strips_p; tp.nsplit = nsplit; tp.dcol2 = dcol2 ? dcol2 + (long long)k * md.ln : nullptr;
+        tp.nsplit = nsplit; tp.dcol2 = dcol2 ? dcol2 + (long long)k * md.ln : nullptr;
         c->h_tc.push_back(tp);
         c->tc_strips += (md.ln + 127) / 128;
-        c->tc_strips_p += (long long)nsplit * ((md.ln + 255) / 256);  // the projection runs as CTA pairs: two strips each
+        c->tc_pairs += (long long)nsplit * ((md.ln + 255) / 256);  // the projection runs as CTA pairs: two strips each
       }
     }
     c->d_tc_bf16 = ws ? reinterpret_cast<char*>(ws) + bf16_begin : nullptr;
     c->tc_bf16_bytes = cv.off - bf16_begin;
     c->prep_blocks = c->h_prep_start.back();
     c->d_tc_probs = cv.take<TcProblem>(c->h_tc.size());
-    c->d_tc_apply = cv.take<TcProblem>(c->h_tc.size());
-    c->h_tc_apply.clear();
-    c->tc_n_left = 0; c->tc_strips_left = 0;
-    {
-      long long strips = 0;
-      for (int side = 0; side < 2; ++side) {
-        for (const TcProblem& tp : c->h_tc) {
-          if (tp.tr != side) continue;
-          TcProblem q2 = tp;
-          q2.strip_start = strips;
-          strips += (tp.n + 127) / 128;
-          c->h_tc_apply.push_back(q2);
-        }
-        if (side == 0) { c->tc_n_left = (int)c->h_tc_apply.size(); c->tc_strips_left = strips; }
+    c->tma = cfg.w_dtype == LORDO_BF16;
+    if (c->tma)
+      for (int l = 0; l < 3; ++l) {
+        c->d_segs[l] = cv.take<TcSeg>((size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers));
+        c->d_seg_start[l] = cv.take<int>(kMaxWorkers + 1);
       }
-    }
     c->d_tc_prep = cv.take<TcPrep>(c->h_prep.size());
     c->d_prep_start = cv.take<long long>(c->h_prep_start.size());
-    c->tma = cfg.w_dtype == LORDO_BF16;
     c->d_maps = cv.take<TmaMatMaps>(n_mats);
     c->d_gmaps = cv.take<TmaGradMaps>(n_mats);
     if (c->tma && !local)
@@ -1217,7 +1252,6 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
     if (!c->tma) INIT_CUDA(tc_configure(c->tc_rn_max, c->tc_rk_max));  // register-staged kernels (fp32 storage)
     INIT_CUDA(cudaMemsetAsync(c->d_tc_bf16, 0, c->tc_bf16_bytes, st));
     INIT_CUDA(cudaMemcpyAsync(c->d_tc_probs, c->h_tc.data(), sizeof(TcProblem) * c->h_tc.size(), cudaMemcpyHostToDevice, st));
-    INIT_CUDA(cudaMemcpyAsync(c->d_tc_apply, c->h_tc_apply.data(), sizeof(TcProblem) * c->h_tc_apply.size(), cudaMemcpyHostToDevice, st));
     INIT_CUDA(cudaMemcpyAsync(c->d_tc_prep, c->h_prep.data(), sizeof(TcPrep) * c->h_prep.size(), cudaMemcpyHostToDevice, st));
     INIT_CUDA(cudaMemcpyAsync(c->d_prep_start, c->h_prep_start.data(), 8 * c->h_prep_start.size(), cudaMemcpyHostToDevice, st));
     if (c->tma) {
@@ -1271,6 +1305,35 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
         INIT_CUDA(cudaMemcpyAsync(c->d_maps, hm.data(), sizeof(TmaMatMaps) * nm, cudaMemcpyHostToDevice, st));
         INIT_CUDA(cudaStreamSynchronize(st));
         INIT_CUDA(tma_configure());
+        for (int l = 0; l < 3; ++l) {
+          std::vector<WorkItem> items;
+          for (int x = 0; x < (int)c->h_tc.size(); ++x) {
+            const TcProblem& tp = c->h_tc[x];
+            if (l > 0 && tp.tr != l - 1) continue;
+            const int steps = tp.m_k / 64, strips = (tp.n + 127) / 128;
+            if (l == 0) {  // the longer of the two chains, k steps and moment update (16 ranks about as long as half a step)
+              const int half = tp.r_n < 256 ? tp.r_n : 256;
+              for (int s2 = 0; s2 < tp.nsplit * ((strips + 1) / 2); ++s2) items.push_back({x, s2, 1, std::max((double)steps, half / 32.0) + 1.0});
+            } else {
+              for (int s2 = 0; s2 < strips; ++s2) items.push_back({x, s2, steps, (double)steps});
+            }
+          }
+          if (items.empty()) continue;
+          std::vector<TcSeg> list;
+          std::vector<int> start;
+          long long steps = 0;
+          for (const WorkItem& it : items) steps += it.len;
+          // no more workers than there are pieces
+          const int most = l == 0 ? std::min(project_pairs(c->sm_count), (int)items.size())
+                                  : (int)std::min<long long>(c->sm_count, std::max<long long>((long long)items.size(), steps / kMinPiece));
+          deal_out(std::move(items), std::min(most, kMaxWorkers), l > 0, l > 0 ? 4.0 : 0.0, list, start);
+          while (start.size() > 1 && start[start.size() - 2] == (int)list.size()) start.pop_back();  // workers without work
+          c->seg_workers[l] = (int)start.size() - 1;
+          if (list.size() > (size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers)) return bail(LORDO_ERR_NOMEM);
+          INIT_CUDA(cudaMemcpyAsync(c->d_segs[l], list.data(), sizeof(TcSeg) * list.size(), cudaMemcpyHostToDevice, st));
+          INIT_CUDA(cudaMemcpyAsync(c->d_seg_start[l], start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, st));
+          INIT_CUDA(cudaStreamSynchronize(st));
+        }
         if (cudaHostAlloc((void**)&c->h_gmaps, 2 * sizeof(TmaGradMaps) * nm, cudaHostAllocDefault) != cudaSuccess) return bail(LORDO_ERR_NOMEM);
       } else {
         return bail(LORDO_ERR_CUDA);  // tensor maps could not be encoded (driver without cuTensorMapEncodeTiled?)
@@ -1351,25 +1414,16 @@ int lordo_inner_step(lordo_ctx* c, const void* const* G, float lr, float beta1, 
       const int big = c->tc_rn_max > 256;
       {
         ProfScope ps(c, st, PC_PROJECT);  // includes the moment update (fused epilogue)
-        launch_project_tma(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips_p, c->d_maps, c->d_gmaps, ss, c->sm_count, c->d_status, st);
+        launch_project_tma(c->d_tc_probs, c->d_segs[0], c->d_seg_start[0], c->seg_workers[0], c->d_maps, c->d_gmaps, ss, c->d_status, st);
       }
       {
         ProfScope ps(c, st, PC_APPLY);
-        const int n_all = (int)c->h_tc_apply.size();
         for (int side = 0; side < 2; ++side) {  // problems stored as projected, then the ones stored transposed
-          const TcProblem* pb = c->d_tc_apply + (side ? c->tc_n_left : 0);
-          const int np = side ? n_all - c->tc_n_left : c->tc_n_left;
-          const long long s0 = side ? c->tc_strips_left : 0, s1 = side ? c->tc_strips : c->tc_strips_left;
-          if (np == 0) continue;
-          if (!big) {
-            launch_apply_tma(pb, np, s0, s1, c->d_maps, c->d_gmaps, ss, c->sm_count, 0, side, c->d_status, st);
-            c->launches += 1;
-          } else {  // 256 < r <= 512: the error-feedback sweep, then the model-update sweep
-            if (c->cfg.error_feedback) {
-              launch_apply_tma(pb, np, s0, s1, c->d_maps, c->d_gmaps, ss, c->sm_count, 1, side, c->d_status, st);
-              c->launches += 1;
-            }
-            launch_apply_tma(pb, np, s0, s1, c->d_maps, c->d_gmaps, ss, c->sm_count, 2, side, c->d_status, st);
+          if (c->seg_workers[1 + side] == 0) continue;
+          // 256 < r <= 512: the error-feedback sweep, then the model-update sweep; else one sweep does both
+          for (int mode = big ? (c->cfg.error_feedback ? 1 : 2) : 0; mode <= (big ? 2 : 0); ++mode) {
+            launch_apply_tma(c->d_tc_probs, c->d_segs[1 + side], c->d_seg_start[1 + side], c->seg_workers[1 + side], c->d_maps, c->d_gmaps, ss,
+                             mode, side, c->d_status, st);
             c->launches += 1;
           }
         }

@@ -99,9 +99,8 @@ struct TcProblem {
   int tr;                      // 1: W, G, E are stored transposed with respect to this problem (a matrix projected from the
                                // right): m counts their columns, n their rows
   float* tb;                   // [r][n] time buffer of this worker (+= lr * U~ every step), or null
-  // the projection's own numbering, in CTA pairs: nsplit pairs per 256 columns (2 when 256 < r <= 512: one
-  // per half of the rank), and the second half's share of the column scale of the full-rank QHM term
-  long long strip_start_p;
+  // TMA-fed projection: nsplit CTA pairs per 256 columns (2 when 256 < r <= 512: one per half of the rank), and
+  // the second half's share of the column scale of the full-rank QHM term
   float* dcol2;                // [n], or null when nsplit == 1
   int nsplit, pad2;
 };
@@ -143,13 +142,20 @@ void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips,
                      unsigned* status, cudaStream_t st);
 
 // TMA-fed persistent kernels for bf16 storage (lordo_tma.cu).
+// A piece of work of one CTA (update) or CTA pair (projection): steps [t0, t1) of 64 rows of one strip, or one
+// pair of strips. Workers walk their own part of a list, [start[w], start[w + 1]), dealt out by lordo_init so
+// that all of them end together.
+struct TcSeg {
+  int prob, strip, t0, t1;
+};
 cudaError_t tma_configure();
-void launch_project_tma(const TcProblem* probs, int nprobs, long long total_strips_p, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
-                        const StepScalars& sc, int grid, unsigned* status, cudaStream_t st);
-// mode 0: r <= 256, one sweep; modes 1 and 2: the two sweeps for 256 < r <= 512. The launch covers the strips
-// [strip_begin, strip_end) of `probs` (problems of one side only: tr = 0 stored as the problem, tr = 1 transposed).
-void launch_apply_tma(const TcProblem* probs, int nprobs, long long strip_begin, long long strip_end, const TmaMatMaps* maps,
-                      const TmaGradMaps* gmaps, const StepScalars& sc, int grid, int mode, int tr, unsigned* status, cudaStream_t st);
+int project_pairs(int sm_count);  // CTA pairs of the projection that the device holds at once
+void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int pairs, const TmaMatMaps* maps,
+                        const TmaGradMaps* gmaps, const StepScalars& sc, unsigned* status, cudaStream_t st);
+// mode 0: r <= 256, one sweep; modes 1 and 2: the two sweeps for 256 < r <= 512. A launch covers problems of one
+// side only: tr = 0 stored as the problem, tr = 1 transposed.
+void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int ctas, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
+                      const StepScalars& sc, int mode, int tr, unsigned* status, cudaStream_t st);
 
 void launch_selftest_wait(unsigned* status, cudaStream_t st);
 

@@ -14,9 +14,11 @@
 //                       works on the swizzled tiles in shared memory (four neighbouring columns per
 //                       thread, 8-byte accesses) and the updated E and W tiles leave by TMA stores.
 //
-// One CTA per SM; a CTA (the update kernel) or a CTA pair (the projection) walks the list of 128-column
-// strips, or of pairs of strips, with the stride of the grid. Every role walks the same list, so stage
+// One CTA per SM; a CTA (the update kernel) or a CTA pair (the projection) walks its own list of
+// 128-column strips or parts of strips, or of pairs of strips. Every role walks the same list, so stage
 // and phase counters stay in step without further communication.
+#include <algorithm>
+
 #include "lordo_kernels.h"
 #include "lordo_umma.cuh"
 
@@ -28,33 +30,14 @@ namespace {
 
 constexpr int kStrip = 128;
 
-__device__ __forceinline__ int find_problem(const TcProblem* __restrict__ probs, int nprobs, long long strip) {
-  int lo = 0, hi = nprobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (probs[mid].strip_start <= strip) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-// the projection numbers its strips on its own: a problem with 256 < r <= 512 has two per 128 columns
-__device__ __forceinline__ int find_problem_p(const TcProblem* __restrict__ probs, int nprobs, long long strip) {
-  int lo = 0, hi = nprobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (probs[mid].strip_start_p <= strip) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 __device__ __forceinline__ float bf_lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t x) { return __uint_as_float(x & 0xFFFF0000u); }
 
 // ---- projection ---------------------------------------------------------------------------------
 constexpr int kPStages = 4;
 constexpr uint32_t kPStageBytes = 49152;  // G 16 KB | E 16 KB | this CTA's rows of the P^T tile, up to 16 KB
-constexpr int kPXformWarps = 4, kPEpiWarps = 8;
-constexpr int kPThreads = (2 + kPXformWarps + kPEpiWarps) * 32;  // 448
+constexpr int kPXformWarps = 4, kPEpiWarps = 16;
+constexpr int kPThreads = (2 + kPXformWarps + kPEpiWarps) * 32;  // 704
 
 // ---- update -------------------------------------------------------------------------------------
 constexpr int kARows = 64;                // rows of W per step = MMA N
@@ -79,11 +62,14 @@ constexpr int kAThreads = (3 + kAEpiWarps) * 32;  // 608: TMA inputs, MMA, 16 ep
 // strips of a problem (and the same half of the rank), one per CTA, and every MMA spans both (M = 256),
 // so each CTA fetches and keeps only half of the rows of the P^T tile. Each CTA's loads complete on
 // its own barrier; its transform warps pass the stage on to the MMA thread of the pair's first CTA.
-// strip_start_p and total_pairs count such pairs; a problem with an odd number of strips ends in a
-// pair whose second CTA reads zeros and stores nothing.
+// A problem with an odd number of strips ends in a pair whose second CTA reads zeros and stores nothing.
+//
+// Sixteen epilogue warps: the moment update (two loads, two stores, a square root and a division per low-rank
+// element) is as long as the k loop at r = m / 8 with eight. 14 layers of 2048 (r = 256, K = 8) 882 -> 790 us, 7 layers of
+// 768 (r = 128) 118 -> 91 us, the second with the strips dealt out by length as well.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
-    project_tma_kernel(const TcProblem* __restrict__ probs, int nprobs, long long total_pairs, const TmaMatMaps* __restrict__ maps,
-                       const TmaGradMaps* __restrict__ gmaps, StepScalars sc, unsigned* __restrict__ status) {
+    project_tma_kernel(const TcProblem* __restrict__ probs, const TcSeg* __restrict__ segs, const int* __restrict__ start,
+                       const TmaMatMaps* __restrict__ maps, const TmaGradMaps* __restrict__ gmaps, StepScalars sc, unsigned* __restrict__ status) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   constexpr int ST = kPStages;
@@ -92,12 +78,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   // warps of both CTAs; empty_bar and acc_full are signalled in both CTAs by that thread's commits
   __shared__ uint64_t full_bar[kPStages], xform_bar[kPStages], empty_bar[kPStages], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_slot;
-  __shared__ float dsum_s[kStrip];
+  __shared__ float dsum_s[3][kStrip];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool ef = sc.ef != 0;
   const uint32_t rank = cluster_rank();
-  const long long pair_first = blockIdx.x >> 1, pair_step = gridDim.x >> 1;
+  const int seg_begin = start[blockIdx.x >> 1], seg_end = start[(blockIdx.x >> 1) + 1];
 
   if (tid == 0) {
     for (int s = 0; s < ST; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&xform_bar[s], 2 * kPXformWarps); mbar_init(&empty_bar[s], 1); }
@@ -111,8 +97,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   const uint32_t tmem = tmem_slot;
   // pair lp of a problem -> this CTA's 128 columns and its half of the rank (split problems: the two
   // halves of a column pair are neighbouring pairs)
-#define LORDO_PAIR_COORDS(pr, pp)                                                              \
-  const int lp = (int)((pp) - (pr)->strip_start_p);                                            \
+#define LORDO_PAIR_COORDS(pr, lp)                                                              \
   const int cs = 2 * ((pr)->nsplit == 2 ? lp >> 1 : lp) + (int)rank;                          \
   const int r_lo = (pr)->nsplit == 2 ? (lp & 1) * 256 : 0;
 
@@ -121,9 +106,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (long long strip = pair_first; strip < total_pairs && ok; strip += pair_step) {
-        const TcProblem* __restrict__ pr = probs + find_problem_p(probs, nprobs, strip);
-        LORDO_PAIR_COORDS(pr, strip)
+      for (int e = seg_begin; e < seg_end && ok; ++e) {
+        const TcProblem* __restrict__ pr = probs + segs[e].prob;
+        LORDO_PAIR_COORDS(pr, segs[e].strip)
         const int n0 = cs * kStrip;
         const TmaMatMaps* mm = maps + pr->mat;
         const TmaGradMaps* gm = gmaps + pr->mat;
@@ -161,9 +146,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       // the barriers the commits arrive on, in this CTA and in the other (8 bytes apart within an array)
       const uint32_t eb0 = cluster_addr(&empty_bar[0], 0), eb1 = cluster_addr(&empty_bar[0], 1);
       const uint32_t af0 = cluster_addr(&acc_full[0], 0), af1 = cluster_addr(&acc_full[0], 1);
-      for (long long strip = pair_first; strip < total_pairs && ok; strip += pair_step, ++si) {
-        const TcProblem* __restrict__ pr = probs + find_problem_p(probs, nprobs, strip);
-        const int r_lo = pr->nsplit == 2 ? ((int)(strip - pr->strip_start_p) & 1) * 256 : 0;
+      for (int e = seg_begin; e < seg_end && ok; ++e, ++si) {
+        const TcProblem* __restrict__ pr = probs + segs[e].prob;
+        const int r_lo = pr->nsplit == 2 ? (segs[e].strip & 1) * 256 : 0;
         const int nkb = pr->m_k / 64;
         const uint32_t n_h = (uint32_t)(pr->r_n - r_lo < 256 ? pr->r_n - r_lo : 256);
         const bool tr = pr->tr != 0;  // the tile then lies as [128 strip elements][64 k]: a K-major operand
@@ -192,8 +177,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     uint32_t it = 0;
     bool ok = true;
     const uint32_t xf = cluster_addr(&xform_bar[0], 0);
-    for (long long strip = pair_first; strip < total_pairs && ok; strip += pair_step) {
-      const TcProblem* __restrict__ pr = probs + find_problem_p(probs, nprobs, strip);
+    for (int e = seg_begin; e < seg_end && ok; ++e) {
+      const TcProblem* __restrict__ pr = probs + segs[e].prob;
       const int nkb = pr->m_k / 64;
       const float c = *pr->cptr;
       for (int kb = 0; kb < nkb; ++kb, ++it) {
@@ -222,15 +207,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     }
   } else {
     // ---------------- epilogue: moments on this thread's column, out of tensor memory -----------
-    const int q = warp & 3, half = (warp - (2 + kPXformWarps)) >> 2;
+    const int q = warp & 3, part = (warp - (2 + kPXformWarps)) >> 2;
     const float b1 = sc.beta1, b2 = sc.beta2, w = sc.omega;
     const bool low = sc.form == LORDO_QHM_LOW;
     uint32_t si = 0;
     bool ok = true;
     const uint32_t ae = cluster_addr(&acc_empty[0], 0);
-    for (long long strip = pair_first; strip < total_pairs && ok; strip += pair_step, ++si) {
-      const TcProblem* __restrict__ pr = probs + find_problem_p(probs, nprobs, strip);
-      LORDO_PAIR_COORDS(pr, strip)
+    for (int e = seg_begin; e < seg_end && ok; ++e, ++si) {
+      const TcProblem* __restrict__ pr = probs + segs[e].prob;
+      LORDO_PAIR_COORDS(pr, segs[e].strip)
       const int n = pr->n, r = pr->r, r_k = pr->r_k;
       const int rn_h = pr->r_n - r_lo < 256 ? pr->r_n - r_lo : 256;  // rank rows of this strip, padded to 16
       const long long n0 = (long long)cs * kStrip;
@@ -249,7 +234,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       if (!ok) break;
       tc_fence_after_sync();
       float dsum = 0.f;
-      for (int ch = half; ch < rn_h / 16; ch += 2) {
+      for (int ch = part; ch < rn_h / 16; ch += kPEpiWarps / 4) {
         float u[16], v[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -296,10 +281,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(ae + 8u * buf);
       if (sc.form == LORDO_QHM_FULL) {  // mu(D): mean over the rank axis, one value per column (a split problem: this half's share)
-        if (half == 1) dsum_s[q * 32 + lane] = dsum;
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (half == 0 && e_ok) (r_lo ? pr->dcol2 : pr->dcol)[ecol] = (dsum + dsum_s[q * 32 + lane]) / (float)r;
-        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (part > 0) dsum_s[part - 1][q * 32 + lane] = dsum;
+        asm volatile("bar.sync 1, %0;" ::"n"(kPEpiWarps * 32) : "memory");
+        if (part == 0 && e_ok)
+          (r_lo ? pr->dcol2 : pr->dcol)[ecol] = ((dsum + dsum_s[0][q * 32 + lane]) + (dsum_s[1][q * 32 + lane] + dsum_s[2][q * 32 + lane])) / (float)r;
+        asm volatile("bar.sync 1, %0;" ::"n"(kPEpiWarps * 32) : "memory");
       }
     }
   }
@@ -319,8 +305,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
 // accumulator tile (lane = strip element, column = step element) already lies the way the tiles are
 // stored, so a thread works on 16 neighbouring stored columns of its own row.
 template <int MODE, bool TR>
-__global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem* __restrict__ probs, int nprobs, long long strip_begin,
-                                                                 long long strip_end, const TmaMatMaps* __restrict__ maps,
+__global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem* __restrict__ probs, const TcSeg* __restrict__ segs,
+                                                                 const int* __restrict__ start, const TmaMatMaps* __restrict__ maps,
                                                                  const TmaGradMaps* __restrict__ gmaps, StepScalars sc,
                                                                  unsigned* __restrict__ status) {
   extern __shared__ unsigned char smem_raw[];
@@ -339,6 +325,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool ef = sc.ef != 0;
+  const int seg_begin = start[blockIdx.x], seg_end = start[blockIdx.x + 1];
 
   if (tid == 0) {
     for (int s = 0; s < kAPStages; ++s) { mbar_init(&p_full[s], 1); mbar_init(&p_empty[s], 1); }
@@ -360,14 +347,14 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
     if (lane == 0) {
       uint32_t jt = 0;
       bool ok = true;
-      for (long long strip = strip_begin + blockIdx.x; strip < strip_end && ok; strip += gridDim.x) {
-        const TcProblem* __restrict__ pr = probs + find_problem(probs, nprobs, strip);
-        const int n0 = (int)(strip - pr->strip_start) * kStrip;
+      for (int e = seg_begin; e < seg_end && ok; ++e) {
+        const TcSeg sg = segs[e];
+        const TcProblem* __restrict__ pr = probs + sg.prob;
+        const int n0 = sg.strip * kStrip;
         const TmaMatMaps* mm = maps + pr->mat;
         const TmaGradMaps* gm = gmaps + pr->mat;
         const int rep = pr->replica;
-        const int nsteps = (pr->m + kARows - 1) / kARows;
-        for (int t = 0; t < nsteps; ++t, ++jt) {
+        for (int t = sg.t0; t < sg.t1; ++t, ++jt) {
           const int is = jt % INST;
           ok = mbar_wait(&in_free[is], ((jt / INST) & 1u) ^ 1u, status);
           if (!ok) break;
@@ -393,12 +380,12 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
     if (lane == 0) {
       uint32_t jt = 0;
       bool ok = true;
-      for (long long strip = strip_begin + blockIdx.x; strip < strip_end && ok; strip += gridDim.x) {
-        const TcProblem* __restrict__ pr = probs + find_problem(probs, nprobs, strip);
+      for (int e = seg_begin; e < seg_end && ok; ++e) {
+        const TcSeg sg = segs[e];
+        const TcProblem* __restrict__ pr = probs + sg.prob;
         const TmaMatMaps* mm = maps + pr->mat;
         const int nkb = pr->r_k / 64, pc = pr->pcopy;
-        const int nsteps = (pr->m + kARows - 1) / kARows;
-        for (int t = 0; t < nsteps; ++t, ++jt) {
+        for (int t = sg.t0; t < sg.t1; ++t, ++jt) {
           const int ps = jt % kAPStages;
           ok = mbar_wait(&p_empty[ps], ((jt / kAPStages) & 1u) ^ 1u, status);
           if (!ok) break;
@@ -413,13 +400,13 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
       const uint32_t idesc = idesc_bf16_f32(128, kARows);
       uint32_t jt = 0, si = 0;
       bool ok = true;
-      for (long long strip = strip_begin + blockIdx.x; strip < strip_end && ok; strip += gridDim.x, ++si) {
-        const TcProblem* __restrict__ pr = probs + find_problem(probs, nprobs, strip);
+      for (int e = seg_begin; e < seg_end && ok; ++e, ++si) {
+        const TcSeg sg = segs[e];
+        const TcProblem* __restrict__ pr = probs + sg.prob;
         const int nkb = pr->r_k / 64;
-        const int nsteps = (pr->m + kARows - 1) / kARows;
         ok = mbar_wait(&x_ready, si & 1u, status);
         if (!ok) break;
-        for (int t = 0; t < nsteps; ++t, ++jt) {
+        for (int t = sg.t0; t < sg.t1; ++t, ++jt) {
           const int ps = jt % kAPStages;
           const uint32_t b = jt & 1u;
           ok = mbar_wait(&p_full[ps], (jt / kAPStages) & 1u, status);
@@ -467,13 +454,13 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
     const float a2w = full ? om : 1.f;
     uint32_t jt = 0, si = 0;
     bool ok = true;
-    for (long long strip = strip_begin + blockIdx.x; strip < strip_end && ok; strip += gridDim.x, ++si) {
-      const TcProblem* __restrict__ pr = probs + find_problem(probs, nprobs, strip);
+    for (int e = seg_begin; e < seg_end && ok; ++e, ++si) {
+      const TcSeg sg = segs[e];
+      const TcProblem* __restrict__ pr = probs + sg.prob;
       const int n = pr->n, r_k = pr->r_k;
-      const int n0 = (int)(strip - pr->strip_start) * kStrip;
+      const int n0 = sg.strip * kStrip;
       const TmaMatMaps* mm = maps + pr->mat;
       const int rep = pr->replica;
-      const int nsteps = (pr->m + kARows - 1) / kARows;
       const long long col = (long long)n0 + colq;
       const float c = *pr->cptr;
       float cd[4];
@@ -489,7 +476,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
         const int per = r_k / 8;  // 32-bit columns of one operand handled by this row group
         // strip block [r_k/8][128][8]: this row group's k-chunks, this lane's column; a warp reads 512
         // contiguous bytes per instruction
-        const size_t lr_off = (size_t)(strip - pr->strip_start) * (size_t)r_k * 128 + (size_t)grp * (r_k / 32) * 1024 + (size_t)colq * 8;
+        const size_t lr_off = (size_t)sg.strip * (size_t)r_k * 128 + (size_t)grp * (r_k / 32) * 1024 + (size_t)colq * 8;
         const uint4* __restrict__ g16 = reinterpret_cast<const uint4*>(pr->gT16 + lr_off);
         const uint4* __restrict__ u16 = reinterpret_cast<const uint4*>(pr->uT16 + lr_off);
         const bool live = col < n;
@@ -509,7 +496,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
         tc_fence_before_sync();
         mbar_arrive(&x_ready);
       }
-      for (int t = 0; t < nsteps; ++t, ++jt) {
+      for (int t = sg.t0; t < sg.t1; ++t, ++jt) {
         const int is = jt % INST;
         const uint32_t b = jt & 1u;
         unsigned char* base = sIn + is * ISB;
@@ -673,21 +660,18 @@ cudaError_t tma_configure() {
   return cudaFuncSetAttribute(apply_tma_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
-void launch_project_tma(const TcProblem* probs, int nprobs, long long total_pairs, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
-                        const StepScalars& sc, int grid, unsigned* status, cudaStream_t st) {
-  if (total_pairs <= 0 || grid < 2) return;
-  long long pairs = grid / 2;
-  if (g_project_pairs > 0 && pairs > g_project_pairs) pairs = g_project_pairs;
-  const unsigned g = 2u * (unsigned)(total_pairs < pairs ? total_pairs : pairs);
-  project_tma_kernel<<<g, kPThreads, kPStages * kPStageBytes + 1024, st>>>(probs, nprobs, total_pairs, maps, gmaps, sc, status);
+int project_pairs(int sm_count) { return g_project_pairs > 0 ? std::min(sm_count / 2, g_project_pairs) : sm_count / 2; }
+
+void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int pairs, const TmaMatMaps* maps,
+                        const TmaGradMaps* gmaps, const StepScalars& sc, unsigned* status, cudaStream_t st) {
+  if (pairs <= 0) return;
+  project_tma_kernel<<<2u * (unsigned)pairs, kPThreads, kPStages * kPStageBytes + 1024, st>>>(probs, segs, start, maps, gmaps, sc, status);
 }
-void launch_apply_tma(const TcProblem* probs, int nprobs, long long strip_begin, long long strip_end, const TmaMatMaps* maps,
-                      const TmaGradMaps* gmaps, const StepScalars& sc, int grid, int mode, int tr, unsigned* status, cudaStream_t st) {
-  const long long total = strip_end - strip_begin;
-  if (total <= 0) return;
-  const unsigned g = (unsigned)(total < grid ? total : grid);
+void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int ctas, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
+                      const StepScalars& sc, int mode, int tr, unsigned* status, cudaStream_t st) {
+  if (ctas <= 0) return;
   const size_t small = kAPStages * kAPStageBytes + kAInStages * kAInStageBytes + 1024, large = kAPStages * 65536 + kAInStages * 32768 + 1024;
-#define LORDO_APPLY(M, T, SM) apply_tma_kernel<M, T><<<g, kAThreads, SM, st>>>(probs, nprobs, strip_begin, strip_end, maps, gmaps, sc, status)
+#define LORDO_APPLY(M, T, SM) apply_tma_kernel<M, T><<<(unsigned)ctas, kAThreads, SM, st>>>(probs, segs, start, maps, gmaps, sc, status)
   if (!tr) {
     if (mode == 0) LORDO_APPLY(0, false, small);
     else if (mode == 1) LORDO_APPLY(1, false, large);

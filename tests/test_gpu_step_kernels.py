@@ -24,3 +24,23 @@ def test_fp32_products_in_ranges_of_k(shape, side):
     assert opt.poll_status() == 0
     assert max(st["W"], st["E"], st["u"], st["v"]) < 2e-5, st
     opt.close()
+
+
+@pytest.mark.parametrize("mats", [((72, 64, 8),), ((2056, 136, 24), (136, 2088, 64)), ((4104, 136, 24),), ((1544, 264, 72), (520, 1032, 264))])
+@pytest.mark.parametrize("side", [0, 1])
+def test_strips_in_pieces(mats, side):
+    """The update's strips whole, in two pieces and in many (one matrix with few columns and many rows), shorter
+    than the shortest piece, of very different lengths in one list, with one sweep and with two (r > 256)."""
+    mats = tuple((n, m, r) if side else (m, n, r) for m, n, r in mats)
+    wl = synth.Workload("t", mats, K=2, H=2, rounds=1, grad="gauss", clip_rho=30.0, w_dtype="bf16", g_dtype="bf16", e_dtype="bf16",
+                        sides=(side,) * len(mats))
+    spec = RunSpec(wl, variant=0, form=2, lr=0.01, omega=0.9, check_mode=0, eps=0.05, refresh=False)
+    opt, orc = hz.run_gpu(spec), hz.run_oracle(spec)
+    st = hz.compare_states(opt, orc)
+    assert opt.poll_status() == 0
+    tol = 8 * 2.0 ** -9  # bf16 operands, as for the other fast-mode tests
+    assert st["u"] < tol and st["v"] < 2 * tol and st["E"] < 2 * tol, st
+    for i in range(len(mats)):
+        d = hz.bf16_ulp_distance(hz._np_state(opt.W[i]), orc.W[i])
+        assert (d <= 1).mean() > 0.99 and d.max() <= 8, ((d <= 1).mean(), d.max())
+    opt.close()
