@@ -89,6 +89,7 @@ struct lordo_ctx {
   const void** d_Gtab = nullptr;
   double *d_partial = nullptr, *d_sumsq = nullptr;
   float* d_coef = nullptr;
+  unsigned* d_tickets = nullptr;  // of the clip kernel
   unsigned* d_status = nullptr;
   GemmProblem* d_probs = nullptr;
   CholProblem* d_chols = nullptr;
@@ -255,14 +256,21 @@ Operand plain(const void* p0, long long ld, int dt0 = LORDO_F32) {
   return o;
 }
 
+long long clip_chunk(const lordo_config& cfg) {
+  long long elements = 0;
+  for (int i = 0; i < cfg.n_mats; ++i) elements += cfg.mats[i].m * cfg.mats[i].n * cfg.K;
+  return sq_chunk(elements);
+}
+
 void prefix_arrays(const lordo_config& cfg, std::vector<long long>& chunk_start, std::vector<long long>& mom_start,
                    std::vector<long long>& wblk, std::vector<long long>& sblk) {
   const int n_mats = cfg.n_mats, K = cfg.K;
   chunk_start.assign(n_mats + 1, 0); mom_start.assign(n_mats + 1, 0); wblk.assign(n_mats + 1, 0); sblk.assign(n_mats + 1, 0);
+  const long long chunk = clip_chunk(cfg);
   for (int i = 0; i < n_mats; ++i) {
     const lordo_mat& a = cfg.mats[i];
     const long long elems = a.m * a.n;
-    chunk_start[i + 1] = chunk_start[i] + (long long)K * ((elems + kSqChunk - 1) / kSqChunk);
+    chunk_start[i + 1] = chunk_start[i] + (long long)K * ((elems + chunk - 1) / chunk);
     const long long ln = a.side ? a.m : a.n;  // columns of the low-rank arrays
     mom_start[i + 1] = mom_start[i] + (long long)K * ((ln + 127) / 128);
     wblk[i + 1] = wblk[i] + (elems + 1023) / 1024;
@@ -335,6 +343,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   c->d_status = cv.take<unsigned>(64);
   c->d_sumsq = cv.take<double>((size_t)n_mats * K);
   c->d_coef = cv.take<float>((size_t)n_mats * K);
+  c->d_tickets = cv.take<unsigned>((size_t)n_mats * K + K);
 
   std::vector<long long> chunk_start, mom_start, wblk, sblk;
   prefix_arrays(cfg, chunk_start, mom_start, wblk, sblk);
@@ -1145,10 +1154,9 @@ int set_gradients(lordo_ctx* c, const void* const* G, cudaStream_t st) {
 
 int run_clip(lordo_ctx* c, cudaStream_t st) {
   if (!(c->cfg.clip_rho > 0.f)) return LORDO_OK;  // coefficients stay at 1
-  launch_sumsq_partial(c->d_mats, c->d_Gtab, c->d_chunk_start, c->n_mats, c->K, c->cfg.g_dtype, c->d_partial, c->total_chunks, st);
-  launch_clip_finalize(c->d_mats, c->d_chunk_start, c->n_mats, c->K, c->d_partial, c->cfg.clip_rho, c->cfg.clip_scope, c->d_coef,
-                       c->d_sumsq, c->d_status, st);
-  c->launches += 3;
+  launch_clip(c->d_mats, c->d_Gtab, c->d_chunk_start, c->n_mats, c->K, c->cfg.g_dtype, clip_chunk(c->cfg), c->d_partial, c->total_chunks,
+              c->cfg.clip_rho, c->cfg.clip_scope, c->d_coef, c->d_sumsq, c->d_tickets, c->d_status, st);
+  c->launches += 1;
   return check_launch(c, "clip");
 }
 
@@ -1241,6 +1249,7 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
   if (!c->h_eigs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_eigs, c->h_eigs.data(), sizeof(EigProblem) * c->h_eigs.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_grams.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_grams, c->h_grams.data(), sizeof(GramProblem) * c->h_grams.size(), cudaMemcpyHostToDevice, st));
   INIT_CUDA(cudaMemsetAsync(c->d_status, 0, 256, st));
+  INIT_CUDA(cudaMemsetAsync(c->d_tickets, 0, sizeof(unsigned) * ((size_t)nm * c->K + c->K), st));
   {
     int dev = 0;
     INIT_CUDA(cudaGetDevice(&dev));

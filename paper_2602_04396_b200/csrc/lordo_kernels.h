@@ -4,7 +4,13 @@
 
 namespace lordo {
 
-constexpr long long kSqChunk = 32768;  // elements per partial sum of squares
+// Elements per partial sum of squares: small enough that a step with few gradients still has a few thousand
+// threads in flight on every SM, and no smaller. Never below 2048 (256 threads of 8).
+inline long long sq_chunk(long long elements) {
+  long long c = 32768;
+  while (c > 2048 && elements / c < 4 * 148) c /= 2;
+  return c;
+}
 
 struct RandomKeys {
   unsigned long long key[64];
@@ -300,10 +306,10 @@ struct SkProblem {
 void launch_sketch_tma(const SkProblem* probs, int nprobs, long long total_tiles, int grid, int big, unsigned* status, cudaStream_t st);
 
 // streaming kernels
-void launch_sumsq_partial(const MatDev* mats, const void* const* G, const long long* chunk_start, int n_mats, int K, int g_dt,
-                          double* partial, long long total_chunks, cudaStream_t st);
-void launch_clip_finalize(const MatDev* mats, const long long* chunk_start, int n_mats, int K, const double* partial, float rho,
-                          int scope, float* coef, double* sumsq, unsigned* status, cudaStream_t st);
+// tickets: n_mats * K + K counters, zero before the first launch (every launch leaves them at zero)
+void launch_clip(const MatDev* mats, const void* const* G, const long long* chunk_start, int n_mats, int K, int g_dt, long long chunk,
+                 double* partial, long long total_chunks, float rho, int scope, float* coef, double* sumsq, unsigned* tickets, unsigned* status,
+                 cudaStream_t st);
 void launch_fill_float(float* p, long long count, float value, cudaStream_t st);
 void launch_moments(const MatDev* mats, const long long* tile_start, int n_mats, long long total_tiles, const StepScalars& sc,
                     cudaStream_t st);

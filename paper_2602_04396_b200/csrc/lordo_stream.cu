@@ -6,79 +6,103 @@ namespace lordo {
 
 // ---------------------------------------------------------------------------------------------
 // Clip coefficient (Algorithm 1, line "clip"): c = min(1, rho / (||G_k||_2 + 1e-6))
-// Pass 1: one partial sum of squares per block of kSqChunk elements. Pass 2: fixed-order sum.
+// One block per `chunk` elements writes a partial sum of squares; the last block of a (matrix, worker) to
+// finish adds that pair's partial sums, the last pair of a worker the matrices' sums, both in a fixed order
+// whichever block it is. Bound by HBM (7 TB/s on 14 layers of 2048); with the two sums as kernels of their own a small
+// step spent 8 us more on launches, and 256 x 256 with chunks of 32768 had four blocks (step 40.0 -> 34.6 us).
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) sumsq_partial_kernel(const MatDev* __restrict__ mats, const void* const* __restrict__ G,
-                                                            const long long* __restrict__ chunk_start, int n_mats, int K,
-                                                            int g_dt, double* __restrict__ partial) {
+__device__ __forceinline__ double block_sum_256(double x, double* red) {  // all threads return the sum
+  const int t = threadIdx.x;
+  red[t] = x;
+  __syncthreads();
+  for (int s = 128; s > 0; s >>= 1) {
+    if (t < s) red[t] += red[t + s];
+    __syncthreads();
+  }
+  const double r = red[0];
+  __syncthreads();
+  return r;
+}
+
+template <bool BF16>
+__global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ mats, const void* const* __restrict__ G,
+                                                   const long long* __restrict__ chunk_start, int n_mats, int K, long long chunk, double* partial,
+                                                   float rho, int scope, float* __restrict__ coef, double* sumsq, unsigned* __restrict__ tickets,
+                                                   unsigned* __restrict__ status) {
+  __shared__ double red[256];
+  __shared__ bool last_s;
+  const int t = threadIdx.x;
   const long long blk = blockIdx.x;
   const int i = find_segment(chunk_start, n_mats, blk);
   const long long elems = mats[i].m * mats[i].n;
-  const long long chunks = (elems + kSqChunk - 1) / kSqChunk;
-  const long long local = blk - chunk_start[i];
+  const unsigned chunks = (unsigned)((elems + chunk - 1) / chunk);
+  const unsigned local = (unsigned)(blk - chunk_start[i]);
   const int k = (int)(local / chunks);
-  const long long c = local - (long long)k * chunks;
-  const long long begin = c * kSqChunk;
-  long long end = begin + kSqChunk;
-  if (end > elems) end = elems;
-  const void* g = G[i];
-  const long long base = (long long)k * elems;
+  const long long begin = (long long)(local - (unsigned)k * chunks) * chunk;
+  const long long end = begin + chunk < elems ? begin + chunk : elems;
+  constexpr int kBytes = BF16 ? 2 : 4;
+  const char* g = reinterpret_cast<const char*>(G[i]) + (long long)k * elems * kBytes;
   float acc = 0.f;
-  for (long long e = begin + 4ll * threadIdx.x; e < end; e += 4ll * 256) {  // elems is a multiple of 8
-    float4 x = load4(g, g_dt, base + e);
-    acc += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+  for (long long e = begin + 8ll * t; e < end; e += 4 * 8 * 256) {  // elems is a multiple of 8
+    uint4 x[4][BF16 ? 1 : 2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const long long at = e + u * 8 * 256;
+#pragma unroll
+      for (int h = 0; h < (BF16 ? 1 : 2); ++h)
+        x[u][h] = at < end ? reinterpret_cast<const uint4*>(g + at * kBytes)[h] : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int h = 0; h < (BF16 ? 1 : 2); ++h) {
+        const uint32_t w[4] = {x[u][h].x, x[u][h].y, x[u][h].z, x[u][h].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (BF16) {
+            const float lo = __uint_as_float(w[j] << 16), hi = __uint_as_float(w[j] & 0xFFFF0000u);
+            acc += lo * lo + hi * hi;
+          } else {
+            const float v = __uint_as_float(w[j]);
+            acc += v * v;
+          }
+        }
+      }
   }
   double d = (double)acc;
   for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-  __shared__ double warp_sum[8];
-  if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = d;
+  if ((t & 31) == 0) red[t >> 5] = d;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (t == 0) {
     double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += warp_sum[w];
+    for (int w = 0; w < 8; ++w) s += red[w];
     partial[blk] = s;
+    __threadfence();
+    last_s = atomicInc(tickets + (long long)i * K + k, chunks - 1) == chunks - 1;  // back to zero with the last block
   }
-}
-
-// Step 1: one block per (matrix, replica) sums that pair's partials in a fixed order.
-__global__ void __launch_bounds__(256) clip_matrix_sums_kernel(const MatDev* __restrict__ mats, const long long* __restrict__ chunk_start,
-                                                               int K, const double* __restrict__ partial, float rho, int scope,
-                                                               float* __restrict__ coef, double* __restrict__ sumsq) {
-  const int i = blockIdx.x, k = blockIdx.y;
-  __shared__ double red[256];
-  const long long elems = mats[i].m * mats[i].n;
-  const long long chunks = (elems + kSqChunk - 1) / kSqChunk;
+  __syncthreads();
+  if (!last_s) return;
+  __threadfence();
   const double* p = partial + chunk_start[i] + (long long)k * chunks;
   double a = 0.0;
-  for (long long c = threadIdx.x; c < chunks; c += 256) a += p[c];
-  red[threadIdx.x] = a;
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double s_i = red[0];
+  for (unsigned c = t; c < chunks; c += 256) a += __ldcg(p + c);  // written by other SMs meanwhile: not from this one's L1
+  const double s_i = block_sum_256(a, red);
+  if (t == 0) {
     sumsq[(long long)i * K + k] = s_i;
     if (scope == 1) coef[(long long)i * K + k] = fminf(1.f, rho / ((float)sqrt(s_i) + 1e-6f));
-  }
-}
-
-// Step 2: one block per replica adds the matrices' sums in matrix order (thread 0, so the order
-// is fixed) and writes the coefficient of the per-worker norm.
-__global__ void __launch_bounds__(256) clip_finalize_kernel(int n_mats, int K, float rho, int scope, float* __restrict__ coef,
-                                                            const double* __restrict__ sumsq, unsigned* __restrict__ status) {
-  const int k = blockIdx.x;
-  __shared__ float c_s;
-  if (threadIdx.x == 0) {
-    double total = 0.0;
-    for (int i = 0; i < n_mats; ++i) total += sumsq[(long long)i * K + k];
-    if (!isfinite(total)) atomicOr(status, LORDO_FLAG_NONFINITE_GRAD);
-    c_s = fminf(1.f, rho / ((float)sqrt(total) + 1e-6f));
+    __threadfence();
+    last_s = atomicInc(tickets + (long long)n_mats * K + k, (unsigned)n_mats - 1) == (unsigned)n_mats - 1;
   }
   __syncthreads();
+  if (!last_s) return;
+  __threadfence();
+  a = 0.0;
+  for (int m = t; m < n_mats; m += 256) a += __ldcg(sumsq + (long long)m * K + k);
+  const double total = block_sum_256(a, red);
+  if (t == 0 && !isfinite(total)) atomicOr(status, LORDO_FLAG_NONFINITE_GRAD);
+  const float c = fminf(1.f, rho / ((float)sqrt(total) + 1e-6f));
   if (scope == 0)
-    for (int i = threadIdx.x; i < n_mats; i += 256) coef[(long long)i * K + k] = c_s;
+    for (int m = t; m < n_mats; m += 256) coef[(long long)m * K + k] = c;
 }
 
 __global__ void fill_float_kernel(float* __restrict__ p, long long count, float value) {
@@ -595,14 +619,13 @@ void launch_commit_basis(const BasisProblem* probs, int nprobs, long long total_
 void launch_copy_grouped(const CopyProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
   copy_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
 }
-void launch_sumsq_partial(const MatDev* mats, const void* const* G, const long long* chunk_start, int n_mats, int K, int g_dt,
-                          double* partial, long long total_chunks, cudaStream_t st) {
-  sumsq_partial_kernel<<<(unsigned)total_chunks, 256, 0, st>>>(mats, G, chunk_start, n_mats, K, g_dt, partial);
-}
-void launch_clip_finalize(const MatDev* mats, const long long* chunk_start, int n_mats, int K, const double* partial, float rho,
-                          int scope, float* coef, double* sumsq, unsigned* status, cudaStream_t st) {
-  clip_matrix_sums_kernel<<<dim3(n_mats, K), 256, 0, st>>>(mats, chunk_start, K, partial, rho, scope, coef, sumsq);
-  clip_finalize_kernel<<<K, 256, 0, st>>>(n_mats, K, rho, scope, coef, sumsq, status);
+void launch_clip(const MatDev* mats, const void* const* G, const long long* chunk_start, int n_mats, int K, int g_dt, long long chunk,
+                 double* partial, long long total_chunks, float rho, int scope, float* coef, double* sumsq, unsigned* tickets, unsigned* status,
+                 cudaStream_t st) {
+  if (g_dt == LORDO_BF16)
+    clip_kernel<true><<<(unsigned)total_chunks, 256, 0, st>>>(mats, G, chunk_start, n_mats, K, chunk, partial, rho, scope, coef, sumsq, tickets, status);
+  else
+    clip_kernel<false><<<(unsigned)total_chunks, 256, 0, st>>>(mats, G, chunk_start, n_mats, K, chunk, partial, rho, scope, coef, sumsq, tickets, status);
 }
 void launch_fill_float(float* p, long long count, float value, cudaStream_t st) {
   fill_float_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(p, count, value);

@@ -1,7 +1,8 @@
 """Edges of the kernels of the inner step, against the oracle."""
 import pytest
+import torch
 
-from paper_2602_04396_b200 import synth
+from paper_2602_04396_b200 import lordo, synth
 from tests import harness as hz
 from tests.harness import RunSpec
 
@@ -43,4 +44,27 @@ def test_strips_in_pieces(mats, side):
     for i in range(len(mats)):
         d = hz.bf16_ulp_distance(hz._np_state(opt.W[i]), orc.W[i])
         assert (d <= 1).mean() > 0.99 and d.max() <= 8, ((d <= 1).mean(), d.max())
+    opt.close()
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("mats,K", [(((8, 8, 8),), 1), (((256, 256, 16),), 2), (((200, 136, 24), (8, 2056, 8), (264, 520, 40)), 5),
+                                    (((24, 24, 8),) * 300, 3), (((2048, 2056, 8),), 3)])
+@pytest.mark.parametrize("scope", [0, 1])
+def test_clip_coefficients_in_one_launch(dt, mats, K, scope):
+    """One chunk and many per (matrix, worker), a ragged last chunk, more matrices than threads; three launches in
+    a row (the counters return to zero). Sums of squares: fp32 over at most 128 values, then fp64: 1e-5 relative."""
+    gdt = synth.torch_dtype(dt)
+    opt = lordo.Lordo(mats, K, 8, [torch.zeros(m, n, dtype=gdt) for m, n, _ in mats], g_dtype=gdt, e_dtype=gdt, clip_rho=2.0, clip_scope=scope)
+    gen = torch.Generator(device="cuda")
+    for step in range(3):
+        G = []
+        for i, (m, n, _) in enumerate(mats):
+            gen.manual_seed(100 * step + i)
+            G.append(torch.empty(K, m, n, device="cuda").normal_(generator=gen).to(gdt))
+        opt.inner_step(G, 0.01, 0.9, 0.9, 2)
+        sq = torch.stack([g.double().square().sum((1, 2)) for g in G])
+        ref = (2.0 / ((sq if scope else sq.sum(0, keepdim=True).expand_as(sq)).sqrt() + 1e-6)).clamp(max=1.0)
+        assert ((opt.clip_coefficients().double() - ref).abs() / ref).max().item() < 1e-5
+    assert opt.poll_status() == 0
     opt.close()
