@@ -123,6 +123,7 @@ __device__ __forceinline__ uint32_t cluster_nctarank() {
 }  // namespace
 
 __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const CholProblem* __restrict__ probs, unsigned* __restrict__ status) {
+  dep_begin();
   extern __shared__ __align__(16) double csm[];
   double* dpart = csm;                               // [4] parts of the diagonal block's sum
   double* part = dpart + 4 * kPartDoubles;           // [kUnits] partial sums of the other blocks
@@ -374,7 +375,9 @@ static cudaLaunchConfig_t chol_launch(cudaLaunchAttribute* at, int nprobs, int c
   at->id = cudaLaunchAttributeClusterDimension;
   at->val.clusterDim.x = (unsigned)c; at->val.clusterDim.y = 1; at->val.clusterDim.z = 1;
   lc.gridDim = dim3((unsigned)(nprobs * c), 1, 1); lc.blockDim = dim3(kCholWarps * 32, 1, 1); lc.dynamicSmemBytes = kCholSmem; lc.stream = st;
-  lc.attrs = at; lc.numAttrs = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at; lc.numAttrs = 2;
   return lc;
 }
 
@@ -385,16 +388,17 @@ void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, unsign
   const int panels = (r_max + kB - 1) / kB;
   int c = 1;
   while (c < 8 && 2 * c <= panels && nprobs <= g_clusters[2 * c]) c *= 2;
-  cudaLaunchAttribute at;
-  const cudaLaunchConfig_t lc = chol_launch(&at, nprobs, c, st);
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t lc = chol_launch(at, nprobs, c, st);
   cudaLaunchKernelEx(&lc, chol_inverse_kernel, probs, status);
 }
 
 cudaError_t chol_configure() {
   cudaError_t e = cudaFuncSetAttribute(chol_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmem);
   for (int c = 2; c <= 8 && e == cudaSuccess; c *= 2) {
-    cudaLaunchAttribute at;
-    const cudaLaunchConfig_t lc = chol_launch(&at, 256, c, nullptr);
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t lc = chol_launch(at, 256, c, nullptr);
+    lc.numAttrs = 1;  // the cluster size alone
     e = cudaOccupancyMaxActiveClusters(&g_clusters[c], chol_inverse_kernel, &lc);
   }
   return e;

@@ -89,6 +89,14 @@ __device__ __forceinline__ void store1(void* base, int dt, long long idx, float 
   }
 }
 
+// Launches by launch_dep (lordo_kernels.h) may begin before the kernel before them in the stream has ended: a kernel
+// sets itself up, then waits here for everything before it, and only then lets the kernel after it begin
+// (so that at most two are in flight, and one that holds tensor memory never starts behind one that still needs some).
+__device__ __forceinline__ void dep_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Largest index i in [0, count) with start[i] <= x (start is ascending, start[0] == 0).
 __device__ __forceinline__ int find_segment(const long long* __restrict__ start, int count, long long x) {
   int lo = 0, hi = count - 1;

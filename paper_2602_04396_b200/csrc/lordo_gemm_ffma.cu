@@ -146,6 +146,7 @@ __device__ __forceinline__ void partials_of(const double* p, unsigned rank, doub
 // accumulation, half the registers (the fp32 work of the fast mode: QR and moment rotation).
 template <int ATRANS, int DUAL, int CARRY>
 __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
+  dep_begin();
   __shared__ __align__(16) float sA[2][BK][BM + PADS];
   __shared__ __align__(16) float sB[2][BK][BN + PADS];
   __shared__ __align__(16) float sB2[2][DUAL ? BK : 1][BN + PADS];
@@ -340,12 +341,14 @@ void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, in
   int c = 1;
   while (c < 8 && total_tiles * 2 * c <= room && slices >= 4 * c) c *= 2;
   cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(256, 1, 1); lc.stream = st;
   lc.dynamicSmemBytes = c > 1 ? sizeof(double) * BM * BN * (dual ? 2 : 1) : 0;
-  lc.attrs = &at; lc.numAttrs = 1;
+  lc.attrs = at; lc.numAttrs = 2;
 #define LORDO_GEMM(A, B, C) cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, C>, probs, nprobs, sc)
   if (carry) {
     if (atrans && !dual) LORDO_GEMM(1, 0, 1);

@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
                                                    const long long* __restrict__ chunk_start, int n_mats, int K, long long chunk, double* partial,
                                                    float rho, int scope, float* __restrict__ coef, double* sumsq, unsigned* __restrict__ tickets,
                                                    unsigned* __restrict__ status) {
+  dep_begin();
   __shared__ double red[256];
   __shared__ bool last_s;
   const int t = threadIdx.x;
@@ -115,10 +116,12 @@ __global__ void fill_float_kernel(float* __restrict__ p, long long count, float 
 //   u <- b1 u + (1-b1) g ; v <- b2 v + (1-b2) g*g ; u^ = u/(1-b1^s) ; v^ = v/(1-b2^s)
 //   D = sqrt(v^) + eps ; U~ = u^/D (no / full-rank QHM) or (w u^ + (1-w) g)/D (low-rank QHM)
 //   full-rank QHM also needs mu(D) = mean over the rank axis, one value per column.
-// One block = 128 columns of one (matrix, replica); threadIdx.y strides over the r rows.
+// One block = 128 columns of one (matrix, replica); its warps stride over the r rows.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) moments_kernel(const MatDev* __restrict__ mats, const long long* __restrict__ tile_start,
                                                       int n_mats, StepScalars sc) {
+  dep_begin();
+  const int lane = threadIdx.x & 31, wrow = threadIdx.x >> 5;
   const long long blk = blockIdx.x;
   const int i = find_segment(tile_start, n_mats, blk);
   const MatDev md = mats[i];
@@ -127,14 +130,14 @@ __global__ void __launch_bounds__(256) moments_kernel(const MatDev* __restrict__
   const long long ctiles = (n + 127) / 128;
   const long long local = blk - tile_start[i];
   const int k = (int)(local / ctiles);
-  const long long col = (local - (long long)k * ctiles) * 128 + 4ll * threadIdx.x;
+  const long long col = (local - (long long)k * ctiles) * 128 + 4ll * lane;
   const bool active = col < n;
   const long long base = (long long)k * r * n + col;
   const float b1 = sc.beta1, b2 = sc.beta2, w = sc.omega;
   float dsum0 = 0.f, dsum1 = 0.f, dsum2 = 0.f, dsum3 = 0.f;
   if (active) {
 #pragma unroll 2
-    for (int a = threadIdx.y; a < r; a += 8) {
+    for (int a = wrow; a < r; a += 8) {
       const long long idx = base + (long long)a * n;
       const float4 g = *reinterpret_cast<const float4*>(md.ghat + idx);
       float4 u = *reinterpret_cast<const float4*>(md.u + idx);
@@ -165,12 +168,12 @@ __global__ void __launch_bounds__(256) moments_kernel(const MatDev* __restrict__
   }
   if (sc.form == LORDO_QHM_FULL) {  // uniform over the grid
     __shared__ float4 red[8][32];
-    red[threadIdx.y][threadIdx.x] = make_float4(dsum0, dsum1, dsum2, dsum3);
+    red[wrow][lane] = make_float4(dsum0, dsum1, dsum2, dsum3);
     __syncthreads();
-    if (threadIdx.y == 0 && active) {
-      float4 s = red[0][threadIdx.x];
+    if (wrow == 0 && active) {
+      float4 s = red[0][lane];
       for (int y = 1; y < 8; ++y) {
-        const float4 t = red[y][threadIdx.x];
+        const float4 t = red[y][lane];
         s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
       }
       const float inv_r = 1.f / (float)r;
@@ -188,6 +191,7 @@ __global__ void __launch_bounds__(256) moments_kernel(const MatDev* __restrict__
 __global__ void __launch_bounds__(256) outer_weights_kernel(const MatDev* __restrict__ mats, const long long* __restrict__ blk_start,
                                                             int n_mats, int K, int w_dt, int outer, float eta_s, float mu_s,
                                                             float delta_scale) {
+  dep_begin();
   const long long blk = blockIdx.x;
   const int i = find_segment(blk_start, n_mats, blk);
   const MatDev md = mats[i];
@@ -228,6 +232,7 @@ __global__ void __launch_bounds__(256) outer_weights_kernel(const MatDev* __rest
 // bit 2 = the time buffers (Global rule: one basis, so their mean is all the rebuilt pseudo-gradient needs).
 __global__ void __launch_bounds__(256) outer_states_kernel(const MatDev* __restrict__ mats, const long long* __restrict__ blk_start,
                                                            int n_mats, int K, int which) {
+  dep_begin();
   const long long blk = blockIdx.x;
   const int i = find_segment(blk_start, n_mats, blk);
   const MatDev md = mats[i];
@@ -289,6 +294,7 @@ __global__ void __launch_bounds__(256) fill_random_kernel(float* __restrict__ ou
 // The same generator for many matrices in one launch; the key of each is derived on the device.
 __global__ void __launch_bounds__(256) fill_random_grouped_kernel(const RandProblem* __restrict__ probs, int nprobs,
                                                                   unsigned long long seed, long long index) {
+  dep_begin();
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
   while (lo < hi) {
@@ -324,6 +330,7 @@ __device__ __forceinline__ void split_store4(__nv_bfloat16* dst, long long plane
 
 __global__ void __launch_bounds__(256) convert_grouped_kernel(const ConvProblem* __restrict__ probs, int nprobs, float inv_bc1, float inv_bc2,
                                                               float bc1, float bc2) {
+  dep_begin();
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
   while (lo < hi) {
@@ -354,6 +361,7 @@ __global__ void __launch_bounds__(256) convert_grouped_kernel(const ConvProblem*
 // fp64, so that what is left of the tensor cores' truncating accumulation is that of one range of k.
 // Bound by the reads of the partial products: r = 512, 16 matrices, 2 x 8 ranges in 21 us.
 __global__ void __launch_bounds__(256) gram_sum_kernel(const GramProblem* __restrict__ probs, int nprobs) {
+  dep_begin();
   __shared__ float tt[32][33];
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
@@ -401,6 +409,7 @@ __global__ void __launch_bounds__(256) gram_sum_kernel(const GramProblem* __rest
 
 // One block per 32 x 32 block of Rot, whose transpose it writes.
 __global__ void __launch_bounds__(256) rot_sum_kernel(const RotProblem* __restrict__ probs, int nprobs) {
+  dep_begin();
   __shared__ float tt[32][33];
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
@@ -438,6 +447,7 @@ __global__ void __launch_bounds__(256) rot_sum_kernel(const RotProblem* __restri
 // Sums of squares of 128 columns over kNormRows rows, in fp64. One block per 32 columns over all rows took 346 us
 // for 7 matrices of up to 5632 x 256 (and 400 us for 16 of 4096 x 512).
 __global__ void __launch_bounds__(256) colsq_kernel(const BasisProblem* __restrict__ probs, int nprobs) {
+  dep_begin();
   __shared__ double red[8][128];
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
@@ -471,6 +481,7 @@ __global__ void __launch_bounds__(256) colsq_kernel(const BasisProblem* __restri
 }
 
 __global__ void __launch_bounds__(256) commit_basis_kernel(const BasisProblem* __restrict__ probs, int nprobs) {
+  dep_begin();
   __shared__ __nv_bfloat16 tile[64][66];
   __shared__ float scale[64];
   __shared__ double part[4][64];
@@ -534,6 +545,7 @@ __global__ void __launch_bounds__(256) commit_basis_kernel(const BasisProblem* _
 
 // Device-to-device copies of many buffers in one launch (16-byte chunks).
 __global__ void __launch_bounds__(256) copy_grouped_kernel(const CopyProblem* __restrict__ probs, int nprobs) {
+  dep_begin();
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
   while (lo < hi) {
@@ -599,48 +611,48 @@ void launch_error_norms(const MatDev* mats, int n_mats, int K, int e_dt, float* 
 }
 void launch_fill_random_grouped(const RandProblem* probs, int nprobs, long long total_blocks, unsigned long long seed, long long index,
                                 cudaStream_t st) {
-  fill_random_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs, seed, index);
+  launch_dep(fill_random_grouped_kernel, dim3((unsigned)total_blocks), 256, 0, st, probs, nprobs, seed, index);
 }
 void launch_convert_grouped(const ConvProblem* probs, int nprobs, long long total_blocks, const GemmScalars& sc, cudaStream_t st) {
-  convert_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs, sc.inv_bc1, sc.inv_bc2, sc.bc1, sc.bc2);
+  launch_dep(convert_grouped_kernel, dim3((unsigned)total_blocks), 256, 0, st, probs, nprobs, sc.inv_bc1, sc.inv_bc2, sc.bc1, sc.bc2);
 }
 void launch_gram_sum(const GramProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
-  gram_sum_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+  launch_dep(gram_sum_kernel, dim3((unsigned)total_blocks), 256, 0, st, probs, nprobs);
 }
 void launch_rot_sum(const RotProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
-  rot_sum_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+  launch_dep(rot_sum_kernel, dim3((unsigned)total_blocks), 256, 0, st, probs, nprobs);
 }
 void launch_colsq(const BasisProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
-  colsq_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+  launch_dep(colsq_kernel, dim3((unsigned)total_blocks), 256, 0, st, probs, nprobs);
 }
 void launch_commit_basis(const BasisProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
-  commit_basis_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+  launch_dep(commit_basis_kernel, dim3((unsigned)total_blocks), 256, 0, st, probs, nprobs);
 }
 void launch_copy_grouped(const CopyProblem* probs, int nprobs, long long total_blocks, cudaStream_t st) {
-  copy_grouped_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(probs, nprobs);
+  launch_dep(copy_grouped_kernel, dim3((unsigned)total_blocks), 256, 0, st, probs, nprobs);
 }
 void launch_clip(const MatDev* mats, const void* const* G, const long long* chunk_start, int n_mats, int K, int g_dt, long long chunk,
                  double* partial, long long total_chunks, float rho, int scope, float* coef, double* sumsq, unsigned* tickets, unsigned* status,
                  cudaStream_t st) {
   if (g_dt == LORDO_BF16)
-    clip_kernel<true><<<(unsigned)total_chunks, 256, 0, st>>>(mats, G, chunk_start, n_mats, K, chunk, partial, rho, scope, coef, sumsq, tickets, status);
+    launch_dep(clip_kernel<true>, dim3((unsigned)total_chunks), 256, 0, st, mats, G, chunk_start, n_mats, K, chunk, partial, rho, scope, coef, sumsq, tickets, status);
   else
-    clip_kernel<false><<<(unsigned)total_chunks, 256, 0, st>>>(mats, G, chunk_start, n_mats, K, chunk, partial, rho, scope, coef, sumsq, tickets, status);
+    launch_dep(clip_kernel<false>, dim3((unsigned)total_chunks), 256, 0, st, mats, G, chunk_start, n_mats, K, chunk, partial, rho, scope, coef, sumsq, tickets, status);
 }
 void launch_fill_float(float* p, long long count, float value, cudaStream_t st) {
   fill_float_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(p, count, value);
 }
 void launch_moments(const MatDev* mats, const long long* tile_start, int n_mats, long long total_tiles, const StepScalars& sc,
                     cudaStream_t st) {
-  moments_kernel<<<(unsigned)total_tiles, dim3(32, 8), 0, st>>>(mats, tile_start, n_mats, sc);
+  launch_dep(moments_kernel, dim3((unsigned)total_tiles), 256, 0, st, mats, tile_start, n_mats, sc);
 }
 void launch_outer_weights(const MatDev* mats, const long long* blk_start, int n_mats, long long total_blocks, int K, int w_dt,
                           int outer, float eta_s, float mu_s, float delta_scale, cudaStream_t st) {
-  outer_weights_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(mats, blk_start, n_mats, K, w_dt, outer, eta_s, mu_s, delta_scale);
+  launch_dep(outer_weights_kernel, dim3((unsigned)total_blocks), 256, 0, st, mats, blk_start, n_mats, K, w_dt, outer, eta_s, mu_s, delta_scale);
 }
 void launch_outer_states(const MatDev* mats, const long long* blk_start, int n_mats, long long total_blocks, int K, int which,
                          cudaStream_t st) {
-  outer_states_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(mats, blk_start, n_mats, K, which);
+  launch_dep(outer_states_kernel, dim3((unsigned)total_blocks), 256, 0, st, mats, blk_start, n_mats, K, which);
 }
 void launch_init_weights(const MatDev* mats, const long long* blk_start, int n_mats, long long total_blocks, int K, int w_dt,
                          cudaStream_t st) {

@@ -69,6 +69,7 @@ struct Elem<false> {
 // PT16 are both written as runs of consecutive addresses.
 __global__ void __launch_bounds__(256) prep_projection_kernel(const TcPrep* __restrict__ items, const long long* __restrict__ blk_start,
                                                               int nitems) {
+  dep_begin();
   __shared__ __nv_bfloat16 tile[64][66];
   const long long blk = blockIdx.x;
   const int i = find_segment(blk_start, nitems, blk);
@@ -130,6 +131,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  dep_begin();
 
   if (warp < 8) {
     // ---------------- producers: form (cG+E)^T tiles and copy P^T tiles -----------------------
@@ -332,6 +334,8 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
     mbar_init_fence();
   }
   if (warp == kApplyEpiWarps + kApplyProdWarps) tmem_alloc(&tmem_slot, kCols);
+  __syncthreads();  // tensor memory is there before the next kernel may begin
+  dep_begin();
 
   // resident operands: rows = the strip's columns, k = rank index (zero rows beyond n)
   {
@@ -522,17 +526,17 @@ cudaError_t tc_configure(int r_n_max, int r_k_max) {
 }
 
 void launch_prep_projection(const TcPrep* items, const long long* blk_start, int nitems, long long total_blocks, cudaStream_t st) {
-  prep_projection_kernel<<<(unsigned)total_blocks, 256, 0, st>>>(items, blk_start, nitems);
+  launch_dep(prep_projection_kernel, dim3((unsigned)total_blocks), 256, 0, st, items, blk_start, nitems);
 }
 void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, const StepScalars& sc, int bf16,
                        unsigned* status, cudaStream_t st) {
-  if (bf16) project_tc_kernel<true><<<(unsigned)total_strips, kProjThreads, project_tc_smem(r_n_max), st>>>(probs, nprobs, sc, status);
-  else project_tc_kernel<false><<<(unsigned)total_strips, kProjThreads, project_tc_smem(r_n_max), st>>>(probs, nprobs, sc, status);
+  if (bf16) launch_dep(project_tc_kernel<true>, dim3((unsigned)total_strips), kProjThreads, project_tc_smem(r_n_max), st, probs, nprobs, sc, status);
+  else launch_dep(project_tc_kernel<false>, dim3((unsigned)total_strips), kProjThreads, project_tc_smem(r_n_max), st, probs, nprobs, sc, status);
 }
 void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_k_max, const StepScalars& sc, int bf16,
                      unsigned* status, cudaStream_t st) {
-  if (bf16) apply_tc_kernel<true><<<(unsigned)total_strips, kApplyThreads, apply_tc_smem(r_k_max), st>>>(probs, nprobs, sc, status);
-  else apply_tc_kernel<false><<<(unsigned)total_strips, kApplyThreads, apply_tc_smem(r_k_max), st>>>(probs, nprobs, sc, status);
+  if (bf16) launch_dep(apply_tc_kernel<true>, dim3((unsigned)total_strips), kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, status);
+  else launch_dep(apply_tc_kernel<false>, dim3((unsigned)total_strips), kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, status);
 }
 
 }  // namespace lordo

@@ -95,6 +95,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   cluster_sync();  // both CTAs' barriers exist before either reaches into the other
   tc_fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  dep_begin();
   // pair lp of a problem -> this CTA's 128 columns and its half of the rank (split problems: the two
   // halves of a column pair are neighbouring pairs)
 #define LORDO_PAIR_COORDS(pr, lp)                                                              \
@@ -339,6 +340,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  dep_begin();
   // tensor memory: columns [0,256) the low-rank operands, two bf16 per column (MODE 0: g^T then U~^T,
   // 128 columns each); [256,512) two buffers of two accumulators
 
@@ -665,13 +667,13 @@ int project_pairs(int sm_count) { return g_project_pairs > 0 ? std::min(sm_count
 void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int pairs, const TmaMatMaps* maps,
                         const TmaGradMaps* gmaps, const StepScalars& sc, unsigned* status, cudaStream_t st) {
   if (pairs <= 0) return;
-  project_tma_kernel<<<2u * (unsigned)pairs, kPThreads, kPStages * kPStageBytes + 1024, st>>>(probs, segs, start, maps, gmaps, sc, status);
+  launch_dep(project_tma_kernel, dim3(2u * (unsigned)pairs), kPThreads, kPStages * kPStageBytes + 1024, st, probs, segs, start, maps, gmaps, sc, status);
 }
 void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int ctas, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
                       const StepScalars& sc, int mode, int tr, unsigned* status, cudaStream_t st) {
   if (ctas <= 0) return;
   const size_t small = kAPStages * kAPStageBytes + kAInStages * kAInStageBytes + 1024, large = kAPStages * 65536 + kAInStages * 32768 + 1024;
-#define LORDO_APPLY(M, T, SM) apply_tma_kernel<M, T><<<(unsigned)ctas, kAThreads, SM, st>>>(probs, segs, start, maps, gmaps, sc, status)
+#define LORDO_APPLY(M, T, SM) launch_dep(apply_tma_kernel<M, T>, dim3((unsigned)ctas), kAThreads, SM, st, probs, segs, start, maps, gmaps, sc, status)
   if (!tr) {
     if (mode == 0) LORDO_APPLY(0, false, small);
     else if (mode == 1) LORDO_APPLY(1, false, large);
@@ -744,6 +746,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
   cluster_sync();  // both CTAs' barriers exist before either reaches into the other
   tc_fence_after_sync();
   const uint32_t tmem = tmem_slot;
+  dep_begin();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -922,8 +925,8 @@ void launch_sketch_tma(const SkProblem* probs, int nprobs, long long total_tiles
   long long pairs = grid / 2;
   if (g_sketch_pairs > 0 && pairs > g_sketch_pairs) pairs = g_sketch_pairs;
   const unsigned g = 2u * (unsigned)(total_tiles < pairs ? total_tiles : pairs);
-  if (big) sketch_tma_kernel<true><<<g, kSThreads, kSSmemBytes, st>>>(probs, nprobs, total_tiles, status);
-  else sketch_tma_kernel<false><<<g, kSThreads, kSSmemBytes, st>>>(probs, nprobs, total_tiles, status);
+  if (big) launch_dep(sketch_tma_kernel<true>, dim3(g), kSThreads, kSSmemBytes, st, probs, nprobs, total_tiles, status);
+  else launch_dep(sketch_tma_kernel<false>, dim3(g), kSThreads, kSSmemBytes, st, probs, nprobs, total_tiles, status);
 }
 
 }  // namespace lordo
