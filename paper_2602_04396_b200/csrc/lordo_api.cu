@@ -117,7 +117,7 @@ struct lordo_ctx {
   char* d_tc_bf16 = nullptr;  // all bf16 operand copies, zeroed once by lordo_init
   size_t tc_bf16_bytes = 0;
   long long tc_strips = 0, tc_pairs = 0, prep_blocks = 0;
-  int tc_rn_max = 0, tc_rk_max = 0;
+  int tc_rn_max = 0, tc_rk_max = 0, tc_steps_min = 0;  // largest padded ranks, fewest 64-row steps
   // TMA-fed kernels (bf16 storage): tensor maps per matrix, gradient maps re-encoded per pointer change
   bool tma = false;
   int sm_count = 0;
@@ -431,7 +431,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   for (int i = 0; i < n_mats; ++i)  // ranks above 512 (above 256 with fp32 storage) run on the fp32 path
     if (cfg.mats[i].r > (cfg.w_dtype == LORDO_BF16 ? 512 : 256) || (cfg.mats[i].side && cfg.w_dtype != LORDO_BF16)) c->tc = false;
   c->h_tc.clear(); c->h_prep.clear(); c->h_prep_start.assign(1, 0);
-  c->tc_strips = 0; c->tc_pairs = 0; c->tc_rn_max = 0; c->tc_rk_max = 0;
+  c->tc_strips = 0; c->tc_pairs = 0; c->tc_rn_max = 0; c->tc_rk_max = 0; c->tc_steps_min = 1 << 30;
   std::vector<size_t> h_prep_first(n_mats, 0);  // first entry of a matrix in h_prep
   if (c->tc) {
     auto up = [](long long x, long long q) { return (x + q - 1) / q * q; };
@@ -450,6 +450,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       float* dcol2 = nsplit == 2 ? cv.take<float>((size_t)K * md.ln) : nullptr;
       if (r_n > c->tc_rn_max) c->tc_rn_max = r_n;
       if (r_k > c->tc_rk_max) c->tc_rk_max = r_k;
+      c->tc_steps_min = std::min(c->tc_steps_min, m_k / 64);
       h_prep_first[i] = c->h_prep.size();
       for (int k = 0; k < copies; ++k) {
         TcPrep pp;
@@ -1441,12 +1442,12 @@ int lordo_inner_step(lordo_ctx* c, const void* const* G, float lr, float beta1, 
     } else {
     {
       ProfScope ps(c, st, PC_PROJECT);  // includes the moment update (fused epilogue)
-      launch_project_tc(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips, c->tc_rn_max, ss, c->cfg.w_dtype == LORDO_BF16,
+      launch_project_tc(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips, c->tc_rn_max, c->tc_steps_min, c->sm_count, ss, c->cfg.w_dtype == LORDO_BF16,
                         c->d_status, st);
     }
     {
       ProfScope ps(c, st, PC_APPLY);
-      launch_apply_tc(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips, c->tc_rk_max, ss, c->cfg.w_dtype == LORDO_BF16,
+      launch_apply_tc(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips, c->tc_rk_max, c->tc_steps_min, c->sm_count, ss, c->cfg.w_dtype == LORDO_BF16,
                       c->d_status, st);
     }
     }

@@ -8,10 +8,16 @@
 //                      resident in shared memory, swept down the m rows in steps of 64; its
 //                      epilogue is the error-feedback line and the model update of Algorithm 1.
 //
+// Both deal a strip's rows out where there are fewer strips than SMs: the projection over a cluster of CTAs that
+// exchange their partial accumulators through distributed shared memory, each finishing every S-th 16 ranks;
+// the update over independent CTAs. 2048 x 2048, r = 128, K = 4 (64 strips): projection 98 -> 42 us, update 122 -> 74 us.
+//
 // Orientation: the strip's columns (n) are the 128 lanes of tensor memory, so every epilogue
 // thread owns one column and a warp touches 32 consecutive columns of a row of G, E, W, u or v.
 // bf16 operands, fp32 accumulation. Operand tiles are written to shared memory by the kernels
 // themselves (the streamed operand has to be formed as c*G + E and transposed anyway).
+#include <algorithm>
+
 #include "lordo_kernels.h"
 #include "lordo_umma.cuh"
 
@@ -111,13 +117,15 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
   __shared__ uint64_t full_bar[2], empty_bar[2], done_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ float dsum_s[kStrip];
+  const uint32_t rank = cluster_rank(), S = cluster_size();
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long strip = blockIdx.x;
+  const long long strip = blockIdx.x / S;
   const TcProblem* __restrict__ prp = probs + find_problem(probs, nprobs, strip);
   const int m = prp->m, n = prp->n, r = prp->r, r_n = prp->r_n, m_k = prp->m_k, r_k = prp->r_k;
   const long long n0 = (strip - prp->strip_start) * kStrip;
-  const int nkb = m_k / 64;
+  // this CTA's steps of 64 rows
+  const int kb0 = (int)((long long)(m_k / 64) * rank / S), kb1 = (int)((long long)(m_k / 64) * (rank + 1) / S);
   const uint32_t a_bytes = kStrip * 128, b_bytes = (uint32_t)r_n * 128, stage_bytes = a_bytes + ((b_bytes + 1023) & ~1023u);
   const uint32_t ncols = tmem_cols_pow2((uint32_t)r_n);
 
@@ -149,8 +157,8 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
     const __nv_bfloat16* __restrict__ PT = prp->PT16;
     const int pt_chunks = r_n * 8;
     bool ok = true;
-    for (int kb = 0; kb < nkb && ok; ++kb) {
-      const int s = kb & 1, use = kb >> 1;
+    for (int kb = kb0; kb < kb1 && ok; ++kb) {
+      const int s = (kb - kb0) & 1, use = (kb - kb0) >> 1;
       pair_t rg[16], re[16];
       const int rbase = kb * 64 + kg * 16;
       if (rbase + 16 <= m) {
@@ -211,12 +219,54 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
       mbar_arrive(&full_bar[s]);
     }
 
-    // ---------------- epilogue: moments on this thread's column ------------------------------
-    if (ok) ok = mbar_wait<64>(&done_bar, 0u, status);
+  } else if (lane == 0) {
+    // ---------------- MMA issue ---------------------------------------------------------------
+    const uint32_t n_lo = r_n > 256 ? 256u : (uint32_t)r_n, n_hi = r_n > 256 ? (uint32_t)(r_n - 256) : 0u;
+    const uint32_t idesc_lo = idesc_bf16_f32(128, n_lo), idesc_hi = idesc_bf16_f32(128, n_hi);
+    bool ok = true;
+    for (int kb = kb0; kb < kb1 && ok; ++kb) {
+      const int s = (kb - kb0) & 1, use = (kb - kb0) >> 1;
+      ok = mbar_wait(&full_bar[s], (uint32_t)(use & 1), status);
+      if (!ok) break;
+      tc_fence_after_sync();
+      const uint32_t sA = smem_u32(smem + s * stage_bytes), sB = sA + a_bytes;
+#pragma unroll
+      for (int k16 = 0; k16 < 4; ++k16) {
+        const uint32_t acc = (kb > kb0 || k16 > 0) ? 1u : 0u;
+        mma_bf16(tmem, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + k16 * 32), idesc_lo, acc);
+        if (n_hi) mma_bf16(tmem + 256, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + 256 * 128 + k16 * 32), idesc_hi, acc);
+      }
+      mma_commit(&empty_bar[s]);
+    }
+    mma_commit(&done_bar);
+  }
+
+  // ---------------- partial accumulators of the ranks that other CTAs finish ---------------------
+  // exch [chunk of 16 ranks not finished here][16][128 columns], over the stages that nothing reads any more
+  float* exch = reinterpret_cast<float*>(smem);
+  const int nch = r_n / 16, q = warp & 3;
+  auto foreign = [&](int ch, int of) { return ch - (ch > of ? (ch - of + (int)S - 1) / (int)S : 0); };  // place of chunk ch in CTA `of`
+  bool done = true;
+  if (warp < 8) {
+    done = mbar_wait<64>(&done_bar, 0u, status);
     tc_fence_after_sync();
-    const int q = warp & 3, half = warp >> 2;
+    if (S > 1)
+      for (int ch = warp >> 2; ch < nch; ch += 2) {
+        if (ch % (int)S == (int)rank) continue;
+        float g[16];
+        tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 16), g);
+        float* to = exch + (size_t)foreign(ch, (int)rank) * 16 * kStrip + q * 32 + lane;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) to[i * kStrip] = g[i];
+      }
+  }
+  __syncwarp();
+  if (S > 1) cluster_sync();
+  if (warp < 8) {
+    // ---------------- epilogue: moments on this thread's column ------------------------------
+    const int half = warp >> 2;
     const long long ecol = n0 + q * 32 + lane;
-    const bool e_ok = ok && ecol < n;
+    const bool e_ok = done && ecol < n;
     const long long ecolc = ecol < n ? ecol : (long long)n - 1;
     float* __restrict__ up_ = prp->u;
     float* __restrict__ vp_ = prp->v;
@@ -225,7 +275,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
     const float b1 = sc.beta1, b2 = sc.beta2, w = sc.omega;
     const bool low = sc.form == LORDO_QHM_LOW;
     float dsum = 0.f;
-    for (int ch = half; ch < r_n / 16; ch += 2) {
+    for (int ch = (int)rank + (int)S * half; ch < nch; ch += 2 * (int)S) {
       float u[16], v[16];
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
@@ -235,6 +285,12 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
       }
       float g[16];
       tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 16), g);
+      for (uint32_t o = 0; o < S; ++o) {  // the other CTAs' partial sums
+        if (o == rank) continue;
+        const uint32_t from = cluster_addr(exch + (size_t)foreign(ch, (int)o) * 16 * kStrip + q * 32 + lane, o);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) g[i] += ld_cluster_f32(from + (uint32_t)(i * kStrip * 4));
+      }
       uint32_t gp[8], upk[8];
 #pragma unroll
       for (int i = 0; i < 16; i += 2) {
@@ -271,28 +327,21 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
     if (sc.form == LORDO_QHM_FULL) {  // mu(D): mean over the rank axis, one value per column
       if (half == 1) dsum_s[q * 32 + lane] = dsum;
       asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (half == 0 && e_ok) prp->dcol[ecol] = (dsum + dsum_s[q * 32 + lane]) / (float)r;
-    }
-  } else if (lane == 0) {
-    // ---------------- MMA issue ---------------------------------------------------------------
-    const uint32_t n_lo = r_n > 256 ? 256u : (uint32_t)r_n, n_hi = r_n > 256 ? (uint32_t)(r_n - 256) : 0u;
-    const uint32_t idesc_lo = idesc_bf16_f32(128, n_lo), idesc_hi = idesc_bf16_f32(128, n_hi);
-    bool ok = true;
-    for (int kb = 0; kb < nkb && ok; ++kb) {
-      const int s = kb & 1, use = kb >> 1;
-      ok = mbar_wait(&full_bar[s], (uint32_t)(use & 1), status);
-      if (!ok) break;
-      tc_fence_after_sync();
-      const uint32_t sA = smem_u32(smem + s * stage_bytes), sB = sA + a_bytes;
-#pragma unroll
-      for (int k16 = 0; k16 < 4; ++k16) {
-        const uint32_t acc = (kb > 0 || k16 > 0) ? 1u : 0u;
-        mma_bf16(tmem, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + k16 * 32), idesc_lo, acc);
-        if (n_hi) mma_bf16(tmem + 256, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + 256 * 128 + k16 * 32), idesc_hi, acc);
+      if (half == 0) {
+        dsum += dsum_s[q * 32 + lane];
+        if (S == 1 && e_ok) prp->dcol[ecol] = dsum / (float)r;
+        dsum_s[q * 32 + lane] = dsum;  // the cluster's first CTA adds them up below
       }
-      mma_commit(&empty_bar[s]);
     }
-    mma_commit(&done_bar);
+  }
+  if (S > 1) {
+    cluster_sync();
+    if (rank == 0 && sc.form == LORDO_QHM_FULL && tid < kStrip && n0 + tid < n) {
+      float dsum = dsum_s[tid];
+      for (uint32_t o = 1; o < S; ++o) dsum += ld_cluster_f32(cluster_addr(dsum_s + tid, o));
+      prp->dcol[n0 + tid] = dsum / (float)r;
+    }
+    cluster_sync();  // nobody leaves while its partial sums may still be read
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -304,7 +353,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
 // ---------------------------------------------------------------------------------------------
 template <bool BF16>
 __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProblem* __restrict__ probs, int nprobs, StepScalars sc,
-                                                                    unsigned* __restrict__ status) {
+                                                                    int pieces, unsigned* __restrict__ status) {
   using EL = Elem<BF16>;
   using one_t = typename EL::one;
   extern __shared__ unsigned char smem_raw[];
@@ -313,12 +362,13 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
   __shared__ uint32_t tmem_slot;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long strip = blockIdx.x;
+  const long long strip = blockIdx.x / pieces;
   const TcProblem* __restrict__ prp = probs + find_problem(probs, nprobs, strip);
   const int m = prp->m, n = prp->n, r_k = prp->r_k;
   const long long n0 = (strip - prp->strip_start) * kStrip;
   const int nkb = r_k / 64;
-  const int nsteps = (m + kApplyRows - 1) / kApplyRows;
+  const int nsteps_all = (m + kApplyRows - 1) / kApplyRows, piece = (int)(blockIdx.x % pieces);
+  const int first = nsteps_all * piece / pieces, nsteps = nsteps_all * (piece + 1) / pieces - first;  // this CTA's part of the strip
   const uint32_t x_bytes = (uint32_t)nkb * kStrip * 128;      // one resident operand (g^T or U~^T)
   const uint32_t p_bytes = (uint32_t)nkb * kApplyRows * 128;  // one ring stage of P rows
   unsigned char* sX1 = smem;
@@ -397,7 +447,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
     bool ok = true;
     for (int t = 0; t < nsteps && ok; ++t) {
       const int b = t & 1;
-      const int row0 = t * kApplyRows + grp * 16;
+      const int row0 = (first + t) * kApplyRows + grp * 16;
       const bool whole = row0 + 16 <= m;
       const size_t base = (size_t)(unsigned)min(row0, m - 1) * (size_t)n;
       one_t rg[16], re[16], rw[16];
@@ -463,7 +513,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
       const uint32_t dst = smem_u32(sP + s * p_bytes);
       for (int idx = ptid; idx < total; idx += kApplyProdWarps * 32) {
         const int row = idx / chunks_per_row, ch = idx - row * chunks_per_row;
-        const __nv_bfloat16* src = P16 + ((long long)t * kApplyRows + row) * r_k + ch * 8;
+        const __nv_bfloat16* src = P16 + ((long long)(first + t) * kApplyRows + row) * r_k + ch * 8;
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (ch >> 3) * (kApplyRows * 128) + swz_chunk(row, ch & 7)),
                      "l"(src)
                      : "memory");
@@ -506,9 +556,11 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
 // ---------------------------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------------------------
+// two stages, or the partial accumulators that a CTA of a cluster of four hands to the others
 size_t project_tc_smem(int r_n_max) {
   const size_t stage = (size_t)kStrip * 128 + (((size_t)r_n_max * 128 + 1023) & ~size_t(1023));
-  return 2 * stage + 1024;
+  const size_t nch = (size_t)r_n_max / 16;
+  return std::max(2 * stage, (nch - nch / 4) * 16 * kStrip * sizeof(float)) + 1024;
 }
 size_t apply_tc_smem(int r_k_max) {
   const size_t nkb = (size_t)r_k_max / 64;
@@ -528,15 +580,31 @@ cudaError_t tc_configure(int r_n_max, int r_k_max) {
 void launch_prep_projection(const TcPrep* items, const long long* blk_start, int nitems, long long total_blocks, cudaStream_t st) {
   launch_dep(prep_projection_kernel, dim3((unsigned)total_blocks), 256, 0, st, items, blk_start, nitems);
 }
-void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, const StepScalars& sc, int bf16,
-                       unsigned* status, cudaStream_t st) {
-  if (bf16) launch_dep(project_tc_kernel<true>, dim3((unsigned)total_strips), kProjThreads, project_tc_smem(r_n_max), st, probs, nprobs, sc, status);
-  else launch_dep(project_tc_kernel<false>, dim3((unsigned)total_strips), kProjThreads, project_tc_smem(r_n_max), st, probs, nprobs, sc, status);
+// `steps`: 64-row steps of the problem with the fewest
+void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, int steps, int sm_count, const StepScalars& sc,
+                       int bf16, unsigned* status, cudaStream_t st) {
+  // two CTAs fit an SM; each is left four steps at least
+  int c = 1;
+  while (c < 4 && total_strips * 2 * c <= 2 * (long long)sm_count && steps >= 8 * c) c *= 2;
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  lc.gridDim = dim3((unsigned)(total_strips * c), 1, 1); lc.blockDim = dim3(kProjThreads, 1, 1); lc.dynamicSmemBytes = project_tc_smem(r_n_max);
+  lc.stream = st; lc.attrs = at; lc.numAttrs = 2;
+  if (bf16) cudaLaunchKernelEx(&lc, project_tc_kernel<true>, probs, nprobs, sc, status);
+  else cudaLaunchKernelEx(&lc, project_tc_kernel<false>, probs, nprobs, sc, status);
 }
-void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_k_max, const StepScalars& sc, int bf16,
-                     unsigned* status, cudaStream_t st) {
-  if (bf16) launch_dep(apply_tc_kernel<true>, dim3((unsigned)total_strips), kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, status);
-  else launch_dep(apply_tc_kernel<false>, dim3((unsigned)total_strips), kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, status);
+void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_k_max, int steps, int sm_count, const StepScalars& sc,
+                     int bf16, unsigned* status, cudaStream_t st) {
+  // one CTA fits an SM; each is left four steps at least
+  int pieces = (int)std::min<long long>(sm_count / total_strips, steps / 4);
+  if (pieces < 1) pieces = 1;
+  const dim3 grid((unsigned)(total_strips * pieces));
+  if (bf16) launch_dep(apply_tc_kernel<true>, grid, kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, pieces, status);
+  else launch_dep(apply_tc_kernel<false>, grid, kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, pieces, status);
 }
 
 }  // namespace lordo

@@ -68,3 +68,18 @@ def test_clip_coefficients_in_one_launch(dt, mats, K, scope):
         assert ((opt.clip_coefficients().double() - ref).abs() / ref).max().item() < 1e-5
     assert opt.poll_status() == 0
     opt.close()
+
+
+@pytest.mark.parametrize("m,n,r", [(2048, 136, 16), (1096, 264, 240), (528, 1032, 144), (1032, 264, 256), (600, 72, 40), (72, 64, 8)])
+@pytest.mark.parametrize("form", [1, 2])
+def test_fp32_storage_strips_dealt_out(m, n, r, form):
+    """Register-staged kernels (fp32 storage) with a strip's rows over one, two and four CTAs, ranks that do not
+    divide evenly among them, more CTAs than chunks of 16 ranks, and the update's rows in pieces."""
+    wl = synth.Workload("t", ((m, n, r),), K=2, H=3, rounds=1, grad="gauss", clip_rho=30.0)
+    spec = RunSpec(wl, variant=0, form=form, lr=0.01, omega=0.9, check_mode=0, eps=0.05, refresh=False)
+    opt, orc = hz.run_gpu(spec), hz.run_oracle(spec)
+    st = hz.compare_states(opt, orc)
+    assert opt.poll_status() == 0
+    tol = 8 * 2.0 ** -9  # bf16 operands, as for the other fast-mode tests
+    assert st["u"] < tol and st["v"] < 2 * tol and st["E"] < tol and st["W"] < tol * 3 * 0.01 / 0.02, st
+    opt.close()
