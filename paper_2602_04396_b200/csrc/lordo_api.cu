@@ -18,7 +18,7 @@ constexpr int kMaxK = 64;
 constexpr int kMaxWorkers = 256;  // CTAs (or CTA pairs) that walk a list of work
 constexpr long long kPairs = 74;  // CTA pairs that the work of a refresh is planned for (148 SMs)
 
-enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_COLSQ = 6, ST_EIG = 7, ST_GRAM = 8, ST_BASIS = 9, ST_ROT = 10 };
+enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_COLSQ = 6, ST_EIG = 7, ST_GRAM = 8, ST_BASIS = 9, ST_ROT = 10, ST_ROTATE = 11 };
 enum Phase { PH_SUBSPACE = 0, PH_ROTATE = 1, PH_COMMIT = 2 };
 
 // One launch of the refresh / init / inner-step plans. The entries it works on are a contiguous
@@ -45,6 +45,7 @@ struct SlotBuilder {
     std::vector<ConvProblem> cv;
     std::vector<BasisProblem> bs;
     std::vector<RotProblem> rt;
+    std::vector<RotateProblem> ro;
     std::vector<EigProblem> eg;
     std::vector<GramProblem> gr;
   };
@@ -99,6 +100,7 @@ struct lordo_ctx {
   ConvProblem* d_convs = nullptr;
   BasisProblem* d_bases = nullptr;
   RotProblem* d_rots = nullptr;
+  RotateProblem* d_rotates = nullptr;
   EigProblem* d_eigs = nullptr;
   GramProblem* d_grams = nullptr;
   float* d_scratch = nullptr;
@@ -139,12 +141,13 @@ struct lordo_ctx {
   std::vector<ConvProblem> h_convs;
   std::vector<BasisProblem> h_bases;
   std::vector<RotProblem> h_rots;
+  std::vector<RotateProblem> h_rotates;
   std::vector<EigProblem> h_eigs;
   std::vector<GramProblem> h_grams;
   struct SketchBufs {
     __nv_bfloat16 *om16 = nullptr, *pn16 = nullptr, *zq16 = nullptr;
     // hi|lo planes of the tensor-core QR and rotation (null when those run in fp32)
-    __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr, *uh16 = nullptr, *wr16 = nullptr;
+    __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr;
   };
   std::vector<SketchBufs> h_skbufs;  // per matrix: bf16 right-hand sides of the sketch products (refresh scratch)
   std::vector<PlanStep> inner_proj, inner_apply;  // one launch per side present
@@ -387,15 +390,13 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       if (cfg.oversample > 0) per += 3 * rs * rs + rs * a.r;  // eigen-solver work and the truncating projector
       // bf16 right-hand sides of the tensor-core sketch products (Omega, P', Z), counted in floats
       per += (ln * a.r + (q > 0 ? pm * a.r + ln * a.r : 0)) / 2 + 64;
-      size_t states16 = 0;
       if (cfg.check_mode == 0 && cfg.w_dtype == LORDO_BF16) {
-        // bf16 planes of the tensor-core QR and rotation: X and R^-1 in three planes, P, Rot^T, its square
-        // (per batch entry) and the two moment operands of every worker in two
+        // bf16 planes of the tensor-core QR and rotation: X and R^-1 in three planes, P, Rot^T and its square in
+        // two; partial products and sums
         per += 3 * (size_t)maxd * a.r / 2 + pm * a.r + 7 * (size_t)a.r * a.r / 2 + 128;
-        states16 = 2 * (size_t)K * a.r * ln + 64;
         per += (size_t)part_matrices(pm, ln) * a.r * a.r + 2 * (size_t)((pm + kNormRows - 1) / kNormRows) * a.r + 16;
       }
-      mat_scratch[i] = nb * per + states16;
+      mat_scratch[i] = nb * per + 64;
       if (acc > 0 && acc + mat_scratch[i] > kRefreshScratchFloats) { ++grp; acc = 0; }
       group_of[i] = grp;
       acc += mat_scratch[i];
@@ -506,7 +507,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
 
   // ---------------- launch plans ----------------
   std::vector<GemmProblem>& P = c->h_probs;
-  P.clear(); c->h_chols.clear(); c->h_rands.clear(); c->h_copies.clear(); c->h_sks.clear(); c->h_convs.clear(); c->h_bases.clear(); c->h_rots.clear(); c->h_eigs.clear(); c->h_grams.clear(); c->h_diag.clear();
+  P.clear(); c->h_chols.clear(); c->h_rands.clear(); c->h_copies.clear(); c->h_sks.clear(); c->h_convs.clear(); c->h_bases.clear(); c->h_rots.clear(); c->h_rotates.clear(); c->h_eigs.clear(); c->h_grams.clear(); c->h_diag.clear();
   c->h_skbufs.assign(n_mats, lordo_ctx::SketchBufs());
   const bool tc_sketch = c->tc && c->tma && cfg.oversample == 0;  // products of the refresh on tensor cores
   c->refresh_makes_copies = tc_sketch;
@@ -551,7 +552,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         for (SkProblem& x : sl.sk) { x.tile_start = st.tiles; st.tiles += (x.M + 255) / 256; c->h_sks.push_back(x); }
       } else if (st.type == ST_CONVERT) {
         st.first = (long long)c->h_convs.size(); st.count = (int)sl.cv.size(); st.tiles = 0;
-        for (ConvProblem& x : sl.cv) { x.blk_start = st.tiles; st.tiles += (x.count + 1023) / 1024; c->h_convs.push_back(x); }
+        for (ConvProblem& x : sl.cv) { x.blk_start = st.tiles; st.tiles += (x.count + 4095) / 4096; c->h_convs.push_back(x); }
       } else if (st.type == ST_EIG) {
         st.first = (long long)c->h_eigs.size(); st.count = (int)sl.eg.size(); st.r_max = 0;
         for (const EigProblem& x : sl.eg) { if (x.w > st.r_max) st.r_max = x.w; c->h_eigs.push_back(x); }
@@ -569,6 +570,13 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           x.sq_start = sq; sq += (x.m + kNormRows - 1) / kNormRows * ((x.r + 127) / 128);
           x.tile_start = st.tiles; st.tiles += (x.m + 63) / 64 * ((x.r + 63) / 64);
           c->h_bases.push_back(x);
+        }
+      } else if (st.type == ST_ROTATE) {
+        st.first = (long long)c->h_rotates.size(); st.count = (int)sl.ro.size(); st.tiles = 0;
+        for (RotateProblem& x : sl.ro) {
+          const int strips = (x.n + 127) / 128;
+          x.item_start = st.tiles; st.tiles += x.nsplit == 2 ? strips : (strips + 1) / 2;
+          c->h_rotates.push_back(x);
         }
       } else if (st.type == ST_ROT) {
         st.first = (long long)c->h_rots.size(); st.count = (int)sl.rt.size(); st.tiles = 0;
@@ -703,7 +711,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       }
       c->h_skbufs[i].om16 = om16; c->h_skbufs[i].pn16 = pn16; c->h_skbufs[i].zq16 = zq16;
       // tensor-core QR and rotation: bf16 planes, plane p of batch entry b at index p * nb + b
-      __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr, *uh16 = nullptr, *wr16 = nullptr;
+      __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr;
       float* gpart = nullptr;   // partial sums of the Gram matrices and of Rot
       double* colsq = nullptr;  // partial sums of squares of the new basis' columns
       if (tc_sketch) {
@@ -713,24 +721,20 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         rinv16 = take16(3 * (size_t)nb * r * r / 2);
         rt16 = take16((size_t)nb * r * r);
         sq16 = take16((size_t)nb * r * r);
-        uh16 = take16((size_t)K * r * n);
-        wr16 = take16((size_t)K * r * n);
         gpart = s; s += (size_t)nb * part_matrices(m, n) * r * r;
         s = c->d_scratch + ((s - c->d_scratch + 3) & ~(ptrdiff_t)3);
         colsq = reinterpret_cast<double*>(s); s += 2 * (size_t)nb * ((m + kNormRows - 1) / kNormRows) * r;
         lordo_ctx::SketchBufs& kb = c->h_skbufs[i];
-        kb.x16 = x16; kb.rinv16 = rinv16; kb.phl = phl; kb.rt16 = rt16; kb.sq16 = sq16; kb.uh16 = uh16; kb.wr16 = wr16;
+        kb.x16 = x16; kb.rinv16 = rinv16; kb.phl = phl; kb.rt16 = rt16; kb.sq16 = sq16;
       }
       TmaMatMaps* mmi = c->d_maps + i;
-      auto conv = [&](SlotBuilder& sb, int phase, const ConvProblem& cp) { sb.next(ST_CONVERT, phase).cv.push_back(cp); };
       // C = A B as the sum of the products of np-plane split operands; planes as above. a_mn: A stored [Kd][M].
       auto sk_split = [&](SlotBuilder::Slot& sl, int a_mn, const unsigned char* map_a, int a_b, int a_nb, const unsigned char* map_b, int b_b, int b_nb,
-                          long long Mo, long long Kd, float* C, long long ldc, int c_trans, int np) {
+                          long long Mo, long long Kd, float* C, long long ldc, int np) {
         SkProblem sp;
         std::memset(&sp, 0, sizeof(sp));
         sp.M = (int)Mo; sp.Kd = (int)Kd; sp.r = r; sp.r_n = (r + 15) / 16 * 16;
         sp.a_mn = a_mn; sp.a_c2 = a_b; sp.a_pl = a_nb; sp.b_c2 = b_b; sp.b_pl = b_nb;
-        sp.c_trans = c_trans;
         // 3 planes: (0,0) (0,1) (1,0) (1,1) (0,2) (2,0); 2 planes: the first three
         sp.pa = 0x201100u; sp.pb = 0x021010u; sp.j0 = 0; sp.j1 = (np == 3 ? 6 : 3) * (int)((Kd + 63) / 64);
         sp.map_a = map_a; sp.map_b = map_b; sp.C = C; sp.ldc = ldc;
@@ -754,7 +758,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           SlotBuilder::Slot& g = sb.next(ST_SKETCH, phase);
           for (int b = 0; b < nb; ++b)
             for (int x = 0; x < 2 * ns; ++x) {  // the smaller pair of each sum first: less is truncated
-              sk_split(g, 1, x_sw, b, nb, x_sw, b, nb, r, rows, gpart + (size_t)(b * 2 * ns + x) * r * r, r, 0, 3);
+              sk_split(g, 1, x_sw, b, nb, x_sw, b, nb, r, rows, gpart + (size_t)(b * 2 * ns + x) * r * r, r, 3);
               SkProblem& sp = g.sk.back();
               sp.pa = x < ns ? 0x01u : 0x00u; sp.pb = x < ns ? 0x01u : 0x12u;
               sp.j0 = (int)((long long)steps * (x % ns) / ns); sp.j1 = (int)((long long)steps * (x % ns + 1) / ns);
@@ -776,7 +780,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           for (int b = 0; b < nb; ++b) {
             // the first pass hands its result on as planes (in place), the last one as O
             const bool to_planes = pass == 0, to_rhs = pass == 1 && !last;
-            sk_split(ap, 0, x_kb, b, nb, mmi->rinv_sw, b, nb, rows, r, to_planes || to_rhs ? nullptr : O + b * so, r, 0, 3);
+            sk_split(ap, 0, x_kb, b, nb, mmi->rinv_sw, b, nb, rows, r, to_planes || to_rhs ? nullptr : O + b * so, r, 3);
             SkProblem& sp = ap.sk.back();
             if (to_planes) { sp.C16 = x16 + (size_t)b * rows * r; sp.plane = (long long)nb * rows * r; sp.planes = 3; }
             if (to_rhs) { sp.C16 = O16 + (size_t)b * rows * r; sp.planes = 1; }
@@ -813,7 +817,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       auto convert = [&](SlotBuilder& sb, const float* src, __nv_bfloat16* dst, size_t count) {
         ConvProblem cp;
         std::memset(&cp, 0, sizeof(cp));
-        cp.mode = CONV_BF16; cp.src = src; cp.dst = dst; cp.count = (long long)count;
+        cp.src = src; cp.dst = dst; cp.count = (long long)count;
         sb.next(ST_CONVERT, PH_SUBSPACE).cv.push_back(cp);
       };
 
@@ -921,7 +925,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           SlotBuilder::Slot& g = R.next(ST_SKETCH, PH_SUBSPACE);
           for (int b = 0; b < nb; ++b)
             for (int x = 0; x < ns; ++x) {  // the smaller pairs first: less is truncated
-              sk_split(g, 1, mmi->xm_sw, b, nb, mmi->phl_sw, b, nb, r, m, gpart + (size_t)(b * ns + x) * r * r, r, 0, 2);
+              sk_split(g, 1, mmi->xm_sw, b, nb, mmi->phl_sw, b, nb, r, m, gpart + (size_t)(b * ns + x) * r * r, r, 2);
               SkProblem& sp = g.sk.back();
               sp.pa = 0x010u; sp.pb = 0x001u; sp.j0 = (int)((long long)steps * x / ns); sp.j1 = (int)((long long)steps * (x + 1) / ns);
             }
@@ -933,25 +937,14 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
             rs_.rt.push_back(rp);
           }
         }
-        {  // u^ and v^ - u^ u^ of all workers as hi|lo planes [2K][r][n]
-          ConvProblem cp;
-          std::memset(&cp, 0, sizeof(cp));
-          cp.mode = CONV_STATES; cp.src = md.u; cp.src2 = md.v; cp.count = (long long)K * r * n;
-          cp.dst = uh16; cp.dst2 = wr16; cp.plane = (long long)K * r * n; cp.planes = 2;
-          conv(R, PH_ROTATE, cp);
-        }
-        {  // (Rot u^)^T = u^^T Rot^T, stored back as [r][n] into the transient g^ area; same for the second moment
-          SlotBuilder::Slot& g = R.next(ST_SKETCH, PH_ROTATE);
-          for (int k = 0; k < K; ++k) {
-            sk_split(g, 1, mmi->uh_sw, k, K, mmi->rt_sw, local ? k : 0, nb, n, r, md.ghat + (long long)k * r * n, n, 1, 2);
-            sk_split(g, 1, mmi->wr_sw, k, K, mmi->sq_sw, local ? k : 0, nb, n, r, md.util + (long long)k * r * n, n, 1, 2);
-          }
-        }
-        {  // u = bc1 (Rot u^), v = bc2 |Rot^2 (v^ - u^ u^) + (Rot u^)^2|
-          ConvProblem cp;
-          std::memset(&cp, 0, sizeof(cp));
-          cp.mode = CONV_COMBINE; cp.src = md.ghat; cp.src2 = md.util; cp.outf = md.u; cp.outf2 = md.v; cp.count = (long long)K * r * n;
-          conv(R, PH_ROTATE, cp);
+        SlotBuilder::Slot& ro = R.next(ST_ROTATE, PH_ROTATE);
+        for (int k = 0; k < K; ++k) {
+          RotateProblem rp;
+          std::memset(&rp, 0, sizeof(rp));
+          rp.u = md.u ? md.u + (size_t)k * r * n : nullptr; rp.v = md.v ? md.v + (size_t)k * r * n : nullptr;
+          rp.map_rt = mmi->rt_32; rp.map_sq = mmi->sq_32; rp.b = local ? k : 0; rp.nb = nb;
+          rp.n = (int)n; rp.r = r; rp.r_n = (r + 15) / 16 * 16; rp.nsplit = rp.r_n > 256 ? 2 : 1;
+          ro.ro.push_back(rp);
         }
       } else {
         {  // Rot = P'^T P (always formed: it also carries the MSSV diagnostic)
@@ -1013,6 +1006,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   c->d_convs = cv.take<ConvProblem>(c->h_convs.size() + 1);
   c->d_bases = cv.take<BasisProblem>(c->h_bases.size() + 1);
   c->d_rots = cv.take<RotProblem>(c->h_rots.size() + 1);
+  c->d_rotates = cv.take<RotateProblem>(c->h_rotates.size() + 1);
   c->d_eigs = cv.take<EigProblem>(c->h_eigs.size() + 1);
   c->d_grams = cv.take<GramProblem>(c->h_grams.size() + 1);
   c->d_diag = cv.take<DiagProblem>(c->h_diag.size() + 1);
@@ -1083,7 +1077,7 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       c->launches += 1;
       return check_launch(c, "sketch");
     case ST_CONVERT:
-      launch_convert_grouped(c->d_convs + s.first, s.count, s.tiles, sc, st);
+      launch_convert_grouped(c->d_convs + s.first, s.count, s.tiles, st);
       c->launches += 1;
       return check_launch(c, "convert");
     case ST_EIG:
@@ -1098,6 +1092,10 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       launch_commit_basis(c->d_bases + s.first, s.count, s.tiles, st);
       c->launches += 1;
       return check_launch(c, "commit_basis");
+    case ST_ROTATE:
+      launch_rotate(c->d_rotates + s.first, s.count, s.tiles, c->sm_count, sc, c->d_status, st);
+      c->launches += 1;
+      return check_launch(c, "rotate");
     case ST_ROT:
       launch_rot_sum(c->d_rots + s.first, s.count, s.tiles, st);
       c->launches += 1;
@@ -1246,6 +1244,7 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
   if (!c->h_diag.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_diag, c->h_diag.data(), sizeof(DiagProblem) * c->h_diag.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_convs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_convs, c->h_convs.data(), sizeof(ConvProblem) * c->h_convs.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_bases.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_bases, c->h_bases.data(), sizeof(BasisProblem) * c->h_bases.size(), cudaMemcpyHostToDevice, st));
+  if (!c->h_rotates.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_rotates, c->h_rotates.data(), sizeof(RotateProblem) * c->h_rotates.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_rots.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_rots, c->h_rots.data(), sizeof(RotProblem) * c->h_rots.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_eigs.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_eigs, c->h_eigs.data(), sizeof(EigProblem) * c->h_eigs.size(), cudaMemcpyHostToDevice, st));
   if (!c->h_grams.empty()) INIT_CUDA(cudaMemcpyAsync(c->d_grams, c->h_grams.data(), sizeof(GramProblem) * c->h_grams.size(), cudaMemcpyHostToDevice, st));
@@ -1305,16 +1304,15 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
           good = good && encode_map3(hm[i].xn_kb, sb.x16, md.r, md.ln, 3 * nbatch, 64, 128, true);
           good = good && encode_map3(hm[i].rinv_sw, sb.rinv16, md.r, md.r, 3 * nbatch, 64, 64, true);
           good = good && encode_map3(hm[i].phl_sw, sb.phl, md.r, md.pm, 2 * nbatch, 64, 64, true);
-          good = good && encode_map3(hm[i].rt_sw, sb.rt16, md.r, md.r, 2 * nbatch, 64, 64, true);
-          good = good && encode_map3(hm[i].sq_sw, sb.sq16, md.r, md.r, 2 * nbatch, 64, 64, true);
-          good = good && encode_map3(hm[i].uh_sw, sb.uh16, md.ln, md.r, 2 * c->K, 64, 64, true);
-          good = good && encode_map3(hm[i].wr_sw, sb.wr16, md.ln, md.r, 2 * c->K, 64, 64, true);
+          good = good && encode_map3(hm[i].rt_32, sb.rt16, md.r, md.r, 2 * nbatch, 64, 32, true);
+          good = good && encode_map3(hm[i].sq_32, sb.sq16, md.r, md.r, 2 * nbatch, 64, 32, true);
         }
       }
       if (good) {
         INIT_CUDA(cudaMemcpyAsync(c->d_maps, hm.data(), sizeof(TmaMatMaps) * nm, cudaMemcpyHostToDevice, st));
         INIT_CUDA(cudaStreamSynchronize(st));
         INIT_CUDA(tma_configure());
+        INIT_CUDA(rotate_configure());
         for (int l = 0; l < 3; ++l) {
           std::vector<WorkItem> items;
           for (int x = 0; x < (int)c->h_tc.size(); ++x) {

@@ -138,8 +138,8 @@ struct alignas(128) TmaMatMaps {
   unsigned char e_st[128], w_st[128];  // stores of one row group of the update epilogue
   // refresh on tensor cores, all over hi|lo bf16 planes [2 x batch][rows][cols], 64 x 64 swizzled boxes
   // unless noted: the matrix being orthonormalised with m rows and with n rows (also as 64 x 128 boxes,
-  // rows as MMA rows), R^-1, P, Rot^T, Rot^T o Rot^T, and the moment operands u^, v^ - u^ u^ as [r][n]
-  unsigned char xm_sw[128], xm_kb[128], xn_sw[128], xn_kb[128], rinv_sw[128], phl_sw[128], rt_sw[128], sq_sw[128], uh_sw[128], wr_sw[128];
+  // rows as MMA rows), R^-1, P; 64 x 32 boxes of Rot^T and of Rot^T o Rot^T
+  unsigned char xm_sw[128], xm_kb[128], xn_sw[128], xn_kb[128], rinv_sw[128], phl_sw[128], rt_32[128], sq_32[128];
 };
 struct alignas(128) TmaGradMaps {  // re-encoded whenever the caller's gradient pointer changes
   unsigned char g_sw[128], g_kb[128];
@@ -230,26 +230,30 @@ struct CopyProblem {
 void launch_fill_random_grouped(const RandProblem* probs, int nprobs, long long total_blocks, unsigned long long seed, long long index,
                                 cudaStream_t st);
 void launch_copy_grouped(const CopyProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
-// Element-wise preparation of tensor-core operands, many buffers per launch (1024 elements per block).
-// "Split" writes a value x as `planes` bf16 planes, plane p + 1 holding the rounding residual of the
-// planes before it (x ~ p0 + p1 (+ p2)), `plane` elements apart. Products of split operands sum the
-// plane pairs (0,0), (0,1), (1,0) [two planes: 16 bits of each operand] and (1,1), (0,2), (2,0)
-// [three planes: 24 bits, the accuracy of an fp32 product].
-enum ConvMode {
-  CONV_BF16 = 0,     // dst = bf16(src)
-  CONV_STATES = 1,   // dst = split(u^ = inv_bc1 src), dst2 = split(inv_bc2 src2 - u^ u^)
-  CONV_COMBINE = 2   // outf = bc1 src, outf2 = bc2 |src2 + src src|   (rotated moments from the two products)
-};
+// fp32 -> bf16 copies (rounded to nearest) of many buffers, 4096 elements per block.
 struct ConvProblem {
   const float* src;
-  const float* src2;
-  __nv_bfloat16 *dst, *dst2;
-  float *outf, *outf2;
+  __nv_bfloat16* dst;
   long long count, blk_start;  // count is a multiple of 8
-  long long plane;             // elements between the planes of dst and of dst2
-  int mode, planes;
 };
-void launch_convert_grouped(const ConvProblem* probs, int nprobs, long long total_blocks, const GemmScalars& sc, cudaStream_t st);
+void launch_convert_grouped(const ConvProblem* probs, int nprobs, long long total_blocks, cudaStream_t st);
+
+// "Planes": a value x as bf16 numbers p0, p1 (, p2), each the rounding residual of the ones before it, stored as
+// arrays of their own a fixed distance apart. Products of such operands sum pairs of planes: (0,0), (0,1), (1,0) with
+// two planes (16 bits of each operand), (1,1), (0,2), (2,0) as well with three (24 bits, the accuracy of an fp32
+// product).
+
+// Moments of one worker in a new basis (lordo_rotate.cu), in place. map_rt, map_sq: 64 x 32 swizzled boxes over the two planes of
+// Rot^T and of its square, entry b of nb. Items are what a CTA pair works on at a time: two strips of 128
+// columns, or one when nsplit = 2 (r > 256).
+struct RotateProblem {
+  float *u, *v;               // [r][n]
+  const void *map_rt, *map_sq;
+  long long item_start;       // first item of this problem within the launch
+  int n, r, r_n, b, nb, nsplit;
+};
+cudaError_t rotate_configure();
+void launch_rotate(const RotateProblem* probs, int nprobs, long long items, int sm_count, const GemmScalars& sc, unsigned* status, cudaStream_t st);
 
 // Gram matrix of a tensor-core QR from its partial products: gram = sum_s S_s + sum_s (T_s + T_s^T), the S
 // and T of `ns` ranges of k each, all r x r, S first. With X ~ p0 + p1 + p2, S = p1^T p1 + p0^T p0 and
@@ -306,7 +310,6 @@ struct SkProblem {
   unsigned pa, pb;
   int j0, j1;
   int a_pl, b_pl;            // third-coordinate distance between the planes of A and of B
-  int c_trans, pad;          // 1: C is stored transposed, C[col * ldc + row]
   const void* map_a;         // 64 x 64 swizzled boxes (a_mn) or 64 x 128 swizzled boxes
   const void* map_e;         // same shape over E, or null
   const void* map_b;         // 64 x 64 swizzled boxes over B [batch][Kd][r]

@@ -891,14 +891,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
               if (ch * 16 + 8 < r) *reinterpret_cast<uint4*>(d + 8) = make_uint4(w[4], w[5], w[6], w[7]);
             }
           }
-        } else if (row_ok && !pr->c_trans) {
+        } else if (row_ok) {
 #pragma unroll
           for (int j = 0; j < 16; j += 4)
             if (ch * 16 + j < r) *reinterpret_cast<float4*>(crow + ch * 16 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-        } else if (row_ok) {  // transposed: the warp's lanes write 32 neighbouring floats of each output row
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (ch * 16 + j < r) pr->C[(long long)(ch * 16 + j) * pr->ldc + row] = v[j];
         }
       }
       tc_fence_before_sync();

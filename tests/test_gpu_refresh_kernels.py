@@ -43,3 +43,19 @@ def test_cholesky_panels_and_clusters(r, count):
         q = q * torch.sign(torch.diagonal(t))
         assert ((opt.P[i].double() - q).norm() / q.norm()).item() < 1e-5
     opt.close()
+
+
+@pytest.mark.parametrize("mats,K", [(((72, 64, 8),), 1), (((136, 264, 40), (264, 392, 136)), 3), (((520, 648, 256), (600, 1032, 264)), 2),
+                                    (((1032, 1544, 512),), 2), (((64, 40, 8), (64, 2056, 24)), 2)])
+@pytest.mark.parametrize("variant,side", [(0, 0), (1, 0), (1, 1)])
+def test_rotation_in_place(mats, K, variant, side):
+    """Rotated moments against the oracle's rotation lines on the bases of the CUDA path: ranks below one stage of
+    32, ragged stages, above and below 256 in one launch (pairs that share a strip and pairs that do not), an odd
+    number of strips, one basis and one per worker."""
+    mats = tuple((n, m, r) if side else (m, n, r) for m, n, r in mats)
+    wl = synth.Workload("t", mats, K=K, H=2, rounds=2, grad="gauss", clip_rho=30.0, w_dtype="bf16", g_dtype="bf16", e_dtype="bf16",
+                        sides=(side,) * len(mats))
+    opt, _, w = hz.run_lockstep_refresh(RunSpec(wl, variant=variant, form=1, lr=0.01, check_mode=0, eps=0.05), rounded_signal=True)
+    assert opt.poll_status() == 0
+    opt.close()
+    assert w["rot_u"] < ROT_TOL and w["rot_v"] < 2 * ROT_TOL, w
