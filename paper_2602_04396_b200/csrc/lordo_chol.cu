@@ -17,7 +17,8 @@
 // and per panel one trip to L2 for the newest columns, the small products and the barrier; for few CTAs per matrix
 // the fp64 products. One CTA per matrix with a thread per row took 2200 us for r = 512 and 16 matrices, 580 us
 // for r = 256 and 7, 197 us for r = 128 and 56; clusters that summed a whole panel at its turn 654, 131 and 62 us;
-// this one 392, 117 and 60 us.
+// this one 325, 86 and 46 us. (Scaling the block so that rsqrt.approx needs no care, and handing the factoring warp
+// its block summed, both made the column chain slower: 98 us at r = 256.)
 #include "lordo_kernels.h"
 
 namespace lordo {
@@ -184,9 +185,14 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
 
   double c[4][4][2];  // a product warp's sum, begun one panel ahead
   clear(c);
-  if (warp == 0)
+  auto stage_diag = [&](int k) {
+    float t[kB];  // all loads before the first store (one after the other they took half a panel's time)
 #pragma unroll
-    for (int j = 0; j < kB; ++j) ga[j * kB + lane] = a_diag(0, j);
+    for (int j = 0; j < kB; ++j) t[j] = a_diag(k, j);
+#pragma unroll
+    for (int j = 0; j < kB; ++j) ga[j * kB + lane] = t[j];
+  };
+  if (warp == 0) stage_diag(0);
 
 #pragma unroll 1
   for (int k = 0; k < nb; ++k) {
@@ -361,9 +367,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
     }
     // the panel is in memory for every CTA of the cluster
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    if (warp == 0 && k + 1 < nb)
-#pragma unroll
-      for (int j = 0; j < kB; ++j) ga[j * kB + lane] = a_diag(k + 1, j);
+    if (warp == 0 && k + 1 < nb) stage_diag(k + 1);
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
 }
@@ -382,12 +386,12 @@ static cudaLaunchConfig_t chol_launch(cudaLaunchAttribute* at, int nprobs, int c
 }
 
 // CTAs per problem: as many, up to the portable cluster size, as leave every problem a place on the device at
-// once (sixteen clusters of eight do not fit 148 SMs and would take two turns) and
-// every CTA at least two row blocks.
+// once (fifteen clusters of seven or eight fit, 22 of six: r = 512, 16 problems 375 us with four CTAs each, 325 with
+// six) and every CTA about two row blocks.
 void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, unsigned* status, cudaStream_t st) {
   const int panels = (r_max + kB - 1) / kB;
-  int c = 1;
-  while (c < 8 && 2 * c <= panels && nprobs <= g_clusters[2 * c]) c *= 2;
+  int c = 8;
+  while (c > 1 && (2 * c > panels + 1 || nprobs > g_clusters[c])) --c;
   cudaLaunchAttribute at[2];
   const cudaLaunchConfig_t lc = chol_launch(at, nprobs, c, st);
   cudaLaunchKernelEx(&lc, chol_inverse_kernel, probs, status);
@@ -395,7 +399,7 @@ void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, unsign
 
 cudaError_t chol_configure() {
   cudaError_t e = cudaFuncSetAttribute(chol_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCholSmem);
-  for (int c = 2; c <= 8 && e == cudaSuccess; c *= 2) {
+  for (int c = 2; c <= 8 && e == cudaSuccess; ++c) {
     cudaLaunchAttribute at[2];
     cudaLaunchConfig_t lc = chol_launch(at, 256, c, nullptr);
     lc.numAttrs = 1;  // the cluster size alone
