@@ -27,6 +27,7 @@ struct PlanStep {
   int type = ST_GEMM, phase = PH_SUBSPACE;
   int atrans = 0, dual = 0, a_square = 0;  // gemm
   int r_max = 0;                           // chol, eig: largest size; gemm: longest contraction
+  int with_e = 0;                          // sketch: the problems' A is c G + E
   int p0 = 0;                              // random: 1 = initial projection (draw index 0), 0 = sketch (index = refresh count)
   long long first = 0, tiles = 0;          // tiles: gemm tiles or 256-thread blocks
   int count = 0;
@@ -145,7 +146,7 @@ struct lordo_ctx {
   std::vector<EigProblem> h_eigs;
   std::vector<GramProblem> h_grams;
   struct SketchBufs {
-    __nv_bfloat16 *om16 = nullptr, *pn16 = nullptr, *zq16 = nullptr;
+    __nv_bfloat16 *om16 = nullptr, *pn16 = nullptr, *zq16 = nullptr, *s16 = nullptr;
     // hi|lo planes of the tensor-core QR and rotation (null when those run in fp32)
     __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr;
   };
@@ -377,6 +378,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   auto part_matrices = [&](long long pm, long long ln) { return std::max(2 * std::max(gram_ranges(pm), gram_ranges(ln)), rot_ranges(pm)); };
   std::vector<int> group_of(n_mats);
   size_t scratch_floats = 0;
+  const bool keep_signal = local && cfg.error_feedback && 2 * q + (warm ? 0 : 1) > 1;  // see `sketch` below
   {
     size_t acc = 0;
     int grp = 0;
@@ -394,6 +396,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         // bf16 planes of the tensor-core QR and rotation: X and R^-1 in three planes, P, Rot^T and its square in
         // two; partial products and sums
         per += 3 * (size_t)maxd * a.r / 2 + pm * a.r + 7 * (size_t)a.r * a.r / 2 + 128;
+        if (keep_signal) per += (size_t)a.m * a.n / 2 + 64;
         per += (size_t)part_matrices(pm, ln) * a.r * a.r + 2 * (size_t)((pm + kNormRows - 1) / kNormRows) * a.r + 16;
       }
       mat_scratch[i] = nb * per + 64;
@@ -548,6 +551,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         for (RandProblem& x : sl.rn) { x.blk_start = st.tiles; st.tiles += (x.count + 2047) / 2048; c->h_rands.push_back(x); }  // 8 per thread
       } else if (st.type == ST_SKETCH) {
         st.first = (long long)c->h_sks.size(); st.count = (int)sl.sk.size(); st.tiles = 0;
+        st.with_e = !sl.sk.empty() && sl.sk[0].cptr != nullptr;
         // the kernel runs as CTA pairs: tiles of 256 rows, 128 per CTA
         for (SkProblem& x : sl.sk) { x.tile_start = st.tiles; st.tiles += (x.M + 255) / 256; c->h_sks.push_back(x); }
       } else if (st.type == ST_CONVERT) {
@@ -725,6 +729,10 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         s = c->d_scratch + ((s - c->d_scratch + 3) & ~(ptrdiff_t)3);
         colsq = reinterpret_cast<double*>(s); s += 2 * (size_t)nb * ((m + kNormRows - 1) / kNormRows) * r;
         lordo_ctx::SketchBufs& kb = c->h_skbufs[i];
+        if (keep_signal) {
+          s = c->d_scratch + ((s - c->d_scratch + 63) & ~(ptrdiff_t)63);
+          kb.s16 = take16((size_t)nb * md.m * md.n / 2);
+        }
         kb.x16 = x16; kb.rinv16 = rinv16; kb.phl = phl; kb.rt16 = rt16; kb.sq16 = sq16;
       }
       TmaMatMaps* mmi = c->d_maps + i;
@@ -792,6 +800,11 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         if (tc_sketch) cholqr2_tc(sb, phase, O, so, O16, rows, last);
         else cholqr2(sb, phase, X, sx, T, st, O, so, rows, w, nb, gram, lw, rinv);
       };
+      // Local rule with error feedback and more than one product: the first one keeps the signal it forms, c G + E in
+      // bf16, for the others, which then read half as much and need no transform (4096 x 11008, r = 512, K = 16: 0.8 to 0.9
+      // ms a product that forms it, 0.6 to 0.7 one that reads it)
+      __nv_bfloat16* s16 = c->h_skbufs[i].s16;
+      bool s16_made = false;
       // S * B on tensor cores, into the three planes of x16: a_mn = 0 -> S rows are the output rows (Y = S B), 1 -> S^T B
       auto sketch = [&](SlotBuilder& sb, int a_mn, unsigned char* map_b, long long Mo, long long Kd) {
         SlotBuilder::Slot& sl = sb.next(ST_SKETCH, PH_SUBSPACE);
@@ -803,8 +816,11 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           sp.a_mn = st_mn; sp.a_c2 = local ? b : 0; sp.b_c2 = b;
           TmaMatMaps* mm = c->d_maps + i;
           TmaGradMaps* gm = c->d_gmaps + i;
-          if (local) {
+          if (s16 && s16_made) {
+            sp.map_a = st_mn ? mm->s_sw : mm->s_kb;
+          } else if (local) {
             sp.map_a = st_mn ? gm->g_sw : gm->g_kb;
+            if (s16) { sp.S16 = s16 + (size_t)b * md.m * md.n; sp.S_rows = (int)md.m; sp.S_cols = (int)md.n; }
             if (cfg.error_feedback) { sp.map_e = st_mn ? mm->e_sw : mm->e_kb; sp.cptr = c->d_coef + (size_t)i * K + b; }
           } else {
             sp.map_a = st_mn ? mm->d_sw : mm->d_kb;
@@ -813,6 +829,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
           sp.C16 = x16 + (size_t)b * Mo * r; sp.plane = (long long)nb * Mo * r; sp.planes = 3;
           sl.sk.push_back(sp);
         }
+        s16_made = true;
       };
       auto convert = [&](SlotBuilder& sb, const float* src, __nv_bfloat16* dst, size_t count) {
         ConvProblem cp;
@@ -1073,7 +1090,7 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       c->launches += 1;
       return check_launch(c, "fill_random");
     case ST_SKETCH:
-      launch_sketch_tma(c->d_sks + s.first, s.count, s.tiles, c->sm_count, c->tc_rn_max > 256, c->d_status, st);
+      launch_sketch_tma(c->d_sks + s.first, s.count, s.tiles, c->sm_count, c->tc_rn_max > 256, s.with_e, c->d_status, st);
       c->launches += 1;
       return check_launch(c, "sketch");
     case ST_CONVERT:
@@ -1304,6 +1321,10 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
           good = good && encode_map3(hm[i].xn_kb, sb.x16, md.r, md.ln, 3 * nbatch, 64, 128, true);
           good = good && encode_map3(hm[i].rinv_sw, sb.rinv16, md.r, md.r, 3 * nbatch, 64, 64, true);
           good = good && encode_map3(hm[i].phl_sw, sb.phl, md.r, md.pm, 2 * nbatch, 64, 64, true);
+          if (sb.s16) {
+            good = good && encode_map3(hm[i].s_sw, sb.s16, md.n, md.m, c->K, 64, 64, true);
+            good = good && encode_map3(hm[i].s_kb, sb.s16, md.n, md.m, c->K, 64, 128, true);
+          }
           good = good && encode_map3(hm[i].rt_32, sb.rt16, md.r, md.r, 2 * nbatch, 64, 32, true);
           good = good && encode_map3(hm[i].sq_32, sb.sq16, md.r, md.r, 2 * nbatch, 64, 32, true);
         }

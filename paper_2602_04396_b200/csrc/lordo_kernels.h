@@ -140,6 +140,7 @@ struct alignas(128) TmaMatMaps {
   // unless noted: the matrix being orthonormalised with m rows and with n rows (also as 64 x 128 boxes,
   // rows as MMA rows), R^-1, P; 64 x 32 boxes of Rot^T and of Rot^T o Rot^T
   unsigned char xm_sw[128], xm_kb[128], xn_sw[128], xn_kb[128], rinv_sw[128], phl_sw[128], rt_32[128], sq_32[128];
+  unsigned char s_sw[128], s_kb[128];  // the Local signal c G + E in bf16, [K][m][n], as 64 x 64 and as 64 x 128 boxes
 };
 struct alignas(128) TmaGradMaps {  // re-encoded whenever the caller's gradient pointer changes
   unsigned char g_sw[128], g_kb[128];
@@ -318,9 +319,13 @@ struct SkProblem {
   long long ldc;             // C16 may be A's own storage: a tile reads no rows of A but those it writes, and has read them all
   __nv_bfloat16* C16;
   long long plane;
-  int planes, pad2;
+  int planes;
+  // with map_e: where c G + E is kept in bf16, as stored [S_rows][S_cols], for the products that follow; or null
+  int S_rows, S_cols, pad2;
+  __nv_bfloat16* S16;
 };
-void launch_sketch_tma(const SkProblem* probs, int nprobs, long long total_tiles, int grid, int big, unsigned* status, cudaStream_t st);
+// with_e: map_e and cptr are set in every problem of the launch, else in none
+void launch_sketch_tma(const SkProblem* probs, int nprobs, long long total_tiles, int grid, int big, int with_e, unsigned* status, cudaStream_t st);
 
 // streaming kernels
 // tickets: n_mats * K + K counters, zero before the first launch (every launch leaves them at zero)

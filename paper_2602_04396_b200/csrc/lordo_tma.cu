@@ -705,8 +705,8 @@ void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* star
 namespace lordo {
 using namespace umma;
 namespace {
-constexpr int kSMaxStages = 4;
-constexpr uint32_t kSSmemBytes = 196608 + 1024;  // 4 stages of A 16 KB | E 16 KB | B 16 KB, or 3 with 32 KB of B
+constexpr int kSMaxStages = 6;
+constexpr uint32_t kSSmemBytes = 196608 + 1024;  // stages of A 16 KB [| E 16 KB] | B 16 KB, or 32 KB for r > 256
 constexpr int kSThreads = (2 + 4 + 8) * 32;  // TMA, MMA, 4 transform warps, 8 epilogue warps
 constexpr uint32_t kIdescBMajorMN = 1u << 16;
 
@@ -720,13 +720,16 @@ __device__ __forceinline__ int find_sk(const SkProblem* __restrict__ probs, int 
 }
 }  // namespace
 
-template <bool BIG>
+// BIG: ranks above 256. WITH_E: the problems' A is c G + E, formed from two tiles; without, the stage is a third or a
+// quarter smaller and the pipeline one or two stages deeper.
+template <bool BIG, bool WITH_E>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
     sketch_tma_kernel(const SkProblem* __restrict__ probs, int nprobs, long long total_tiles, unsigned* __restrict__ status) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr int ST = BIG ? 3 : 4;
-  constexpr uint32_t SB = BIG ? 65536u : 49152u;  // A 16 KB | E 16 KB | this CTA's columns of B: up to 2 (+ 2) boxes of 8 KB
+  constexpr uint32_t BOFF = WITH_E ? 32768u : 16384u;
+  constexpr uint32_t SB = BOFF + (BIG ? 32768u : 16384u);  // A 16 KB | E 16 KB | this CTA's columns of B: up to 2 (+ 2) boxes of 8 KB
+  constexpr int ST = 196608 / SB;
   static_assert(ST * SB + 1024 <= kSSmemBytes, "stages do not fit the shared memory asked for");
   // xform_bar and acc_empty are waited on by the MMA thread of the pair's first CTA only and fed by the
   // warps of both CTAs; empty_bar and acc_full are signalled in both CTAs by that thread's commits
@@ -760,8 +763,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
         const int n_lo = pr->r_n < 256 ? pr->r_n : 256, n_hi = pr->r_n - n_lo;
         const int c_lo = (int)rank * (n_lo / 2), c_hi = 256 + (int)rank * (n_hi / 2);
         const int nbox_lo = (n_lo / 2 + 63) / 64, nbox_hi = (n_hi / 2 + 63) / 64;
-        const bool has_e = pr->map_e != nullptr;
-        const uint32_t tx = 16384u + (has_e ? 16384u : 0u) + (uint32_t)(nbox_lo + nbox_hi) * 8192u;
+        const uint32_t tx = 16384u + (WITH_E ? 16384u : 0u) + (uint32_t)(nbox_lo + nbox_hi) * 8192u;
         const int j1 = pr->j1;
         int seg = pr->j0 / nkb1, kb = pr->j0 - seg * nkb1;
         for (int j = pr->j0; j < j1; ++j, ++it, ++kb) {
@@ -775,16 +777,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
           if (pr->a_mn) {  // S stored [Kd][M]: two boxes of 64 k-rows x 64 columns
             tma_load_3d(base, pr->map_a, m0, kb * 64, a_c2, &full_bar[s]);
             tma_load_3d(base + 8192, pr->map_a, m0 + 64, kb * 64, a_c2, &full_bar[s]);
-            if (has_e) {
+            if (WITH_E) {
               tma_load_3d(base + 16384, pr->map_e, m0, kb * 64, a_c2, &full_bar[s]);
               tma_load_3d(base + 24576, pr->map_e, m0 + 64, kb * 64, a_c2, &full_bar[s]);
             }
           } else {         // S stored [M][Kd]: one box of 128 rows x 64 k
             tma_load_3d(base, pr->map_a, kb * 64, m0, a_c2, &full_bar[s]);
-            if (has_e) tma_load_3d(base + 16384, pr->map_e, kb * 64, m0, a_c2, &full_bar[s]);
+            if (WITH_E) tma_load_3d(base + 16384, pr->map_e, kb * 64, m0, a_c2, &full_bar[s]);
           }
-          for (int x = 0; x < nbox_lo; ++x) tma_load_3d(base + 32768 + x * 8192, pr->map_b, c_lo + x * 64, kb * 64, b_c2, &full_bar[s]);
-          for (int x = 0; x < nbox_hi; ++x) tma_load_3d(base + 49152 + x * 8192, pr->map_b, c_hi + x * 64, kb * 64, b_c2, &full_bar[s]);
+          for (int x = 0; x < nbox_lo; ++x) tma_load_3d(base + BOFF + x * 8192, pr->map_b, c_lo + x * 64, kb * 64, b_c2, &full_bar[s]);
+          for (int x = 0; x < nbox_hi; ++x) tma_load_3d(base + BOFF + 16384 + x * 8192, pr->map_b, c_hi + x * 64, kb * 64, b_c2, &full_bar[s]);
         }
       }
     }
@@ -810,7 +812,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
           ok = mbar_wait(&xform_bar[s], (it / ST) & 1u, status);
           if (!ok) break;
           tc_fence_after_sync();
-          const uint32_t sA = smem_u32(smem + s * SB), sB = sA + 32768;
+          const uint32_t sA = smem_u32(smem + s * SB), sB = sA + BOFF;
 #pragma unroll
           for (int k16 = 0; k16 < 4; ++k16) {
             const uint64_t ad = a_mn ? smem_desc_mn128(sA + k16 * 2048) : smem_desc_k128(sA + k16 * 32);
@@ -830,13 +832,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
     for (long long tile = tile_first; tile < total_tiles && ok; tile += tile_step) {
       const SkProblem* __restrict__ pr = probs + find_sk(probs, nprobs, tile);
       const int nkb = pr->j1 - pr->j0;
-      const bool has_e = pr->map_e != nullptr;
-      const float c = pr->cptr ? *pr->cptr : 1.f;
+      const float c = WITH_E ? *pr->cptr : 1.f;
+      __nv_bfloat16* S16 = WITH_E ? pr->S16 : nullptr;
+      const bool a_mn = pr->a_mn != 0;
+      const int m0 = (2 * (int)(tile - pr->tile_start) + (int)rank) * 128;
       for (int kb = 0; kb < nkb; ++kb, ++it) {
         const int s = it % ST;
         ok = mbar_wait(&full_bar[s], (it / ST) & 1u, status);
         if (!ok) break;
-        if (has_e) {
+        if (WITH_E) {
           uint4* G = reinterpret_cast<uint4*>(smem + s * SB);
           const uint4* E = G + 1024;
 #pragma unroll
@@ -849,6 +853,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
             a.z = pack2_bf16(fmaf(c, bf_lo(g.z), bf_lo(e.z)), fmaf(c, bf_hi(g.z), bf_hi(e.z)));
             a.w = pack2_bf16(fmaf(c, bf_lo(g.w), bf_lo(e.w)), fmaf(c, bf_hi(g.w), bf_hi(e.w)));
             G[idx] = a;
+            if (S16) {  // every tile passes here once: eight lanes hold 128 neighbouring bytes of a stored row
+              const int in_box = a_mn ? (idx >> 3) & 63 : idx >> 3, c8 = ((idx & 7) ^ (in_box & 7)) * 8;
+              const int row = (a_mn ? kb * 64 : m0) + in_box, col = (a_mn ? m0 + (idx >> 9) * 64 : kb * 64) + c8;
+              if (row < pr->S_rows && col < pr->S_cols) *reinterpret_cast<uint4*>(S16 + (size_t)row * pr->S_cols + col) = a;
+            }
           }
           fence_async_smem();
         }
@@ -909,20 +918,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
 }
 
 cudaError_t sketch_configure() {
-  cudaError_t e = cudaFuncSetAttribute(sketch_tma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(sketch_tma_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(sketch_tma_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(sketch_tma_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(sketch_tma_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmemBytes);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(sketch_tma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmemBytes);
-  if (e != cudaSuccess) return e;
-  return max_resident_pairs(sketch_tma_kernel<true>, kSThreads, kSSmemBytes, &g_sketch_pairs);
+  return max_resident_pairs(sketch_tma_kernel<true, true>, kSThreads, kSSmemBytes, &g_sketch_pairs);
 }
 // total_tiles counts tiles of 256 rows (tile_start in `probs` does too); a CTA pair per SM pair.
-void launch_sketch_tma(const SkProblem* probs, int nprobs, long long total_tiles, int grid, int big, unsigned* status, cudaStream_t st) {
+void launch_sketch_tma(const SkProblem* probs, int nprobs, long long total_tiles, int grid, int big, int with_e, unsigned* status, cudaStream_t st) {
   if (total_tiles <= 0 || grid < 2) return;
   long long pairs = grid / 2;
   if (g_sketch_pairs > 0 && pairs > g_sketch_pairs) pairs = g_sketch_pairs;
   const unsigned g = 2u * (unsigned)(total_tiles < pairs ? total_tiles : pairs);
-  if (big) launch_dep(sketch_tma_kernel<true>, dim3(g), kSThreads, kSSmemBytes, st, probs, nprobs, total_tiles, status);
-  else launch_dep(sketch_tma_kernel<false>, dim3(g), kSThreads, kSSmemBytes, st, probs, nprobs, total_tiles, status);
+#define LORDO_SKETCH(B, E) launch_dep(sketch_tma_kernel<B, E>, dim3(g), kSThreads, kSSmemBytes, st, probs, nprobs, total_tiles, status)
+  if (big && with_e) LORDO_SKETCH(true, true);
+  else if (big) LORDO_SKETCH(true, false);
+  else if (with_e) LORDO_SKETCH(false, true);
+  else LORDO_SKETCH(false, false);
+#undef LORDO_SKETCH
 }
 
 }  // namespace lordo

@@ -59,3 +59,21 @@ def test_rotation_in_place(mats, K, variant, side):
     assert opt.poll_status() == 0
     opt.close()
     assert w["rot_u"] < ROT_TOL and w["rot_v"] < 2 * ROT_TOL, w
+
+
+@pytest.mark.parametrize("shape", [(136, 72, 16), (520, 1032, 40), (648, 776, 264)])
+@pytest.mark.parametrize("q,warm,side", [(1, False, 0), (2, False, 1), (1, True, 0), (2, True, 1)])
+def test_signal_kept_for_later_products(shape, q, warm, side):
+    """Local rule with several products per refresh: c G + E is formed once, by a product of either orientation,
+    with ragged edges in both directions. Signal of rank r plus 0.5 % noise, as in the tests of the subspace angle."""
+    m, n, r = shape
+    if side:
+        m, n = n, m
+    wl = synth.Workload("t", ((m, n, r),), K=2, H=2, rounds=2, grad="lowrank", signal_rank=r, noise=0.005, clip_rho=30.0, power_iters=q,
+                        w_dtype="bf16", g_dtype="bf16", e_dtype="bf16", sides=(side,))
+    spec = RunSpec(wl, variant=1, form=1, lr=0.01, check_mode=0, eps=0.05, warm_start=warm)
+    opt, _, w = hz.run_lockstep_refresh(spec, rounded_signal=True)
+    assert opt.poll_status() == 0
+    opt.close()
+    assert w["P_orth"] < ORTH_TOL and w["rot_u"] < ROT_TOL and w["rot_v"] < 2 * ROT_TOL, w
+    assert w["P_angle_bf16rhs"] < (5e-3 if warm else ANGLE_TOL), w  # warm: from the first columns of the identity
