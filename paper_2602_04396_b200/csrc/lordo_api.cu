@@ -110,11 +110,11 @@ struct lordo_ctx {
   // tensor-core path of the inner step (check_mode == 0 and every r <= 256)
   bool tc = false;
   TcProblem* d_tc_probs = nullptr;
-  // TMA-fed kernels: who does what, [0] projection, [1] update of the problems stored as they are projected,
-  // [2] of the ones stored transposed (matrices projected from the right)
-  TcSeg* d_segs[3] = {nullptr, nullptr, nullptr};
-  int* d_seg_start[3] = {nullptr, nullptr, nullptr};
-  int seg_workers[3] = {0, 0, 0};
+  // TMA-fed kernels: who does what, [0] projection, [1] update
+  TcSeg* d_segs[2] = {nullptr, nullptr};
+  int* d_seg_start[2] = {nullptr, nullptr};
+  int seg_workers[2] = {0, 0};
+  int tma_side = 0;  // 0: no matrix is projected from the right, 1: every one is, 2: some are
   TcPrep* d_tc_prep = nullptr;
   long long* d_prep_start = nullptr;
   char* d_tc_bf16 = nullptr;  // all bf16 operand copies, zeroed once by lordo_init
@@ -496,7 +496,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
     c->d_tc_probs = cv.take<TcProblem>(c->h_tc.size());
     c->tma = cfg.w_dtype == LORDO_BF16;
     if (c->tma)
-      for (int l = 0; l < 3; ++l) {
+      for (int l = 0; l < 2; ++l) {
         c->d_segs[l] = cv.take<TcSeg>((size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers));
         c->d_seg_start[l] = cv.take<int>(kMaxWorkers + 1);
       }
@@ -1334,11 +1334,13 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
         INIT_CUDA(cudaStreamSynchronize(st));
         INIT_CUDA(tma_configure());
         INIT_CUDA(rotate_configure());
-        for (int l = 0; l < 3; ++l) {
+        int right = 0;
+        for (const lordo_mat& a : c->mats) right += a.side;
+        c->tma_side = right == 0 ? 0 : right == nm ? 1 : 2;
+        for (int l = 0; l < 2; ++l) {
           std::vector<WorkItem> items;
           for (int x = 0; x < (int)c->h_tc.size(); ++x) {
             const TcProblem& tp = c->h_tc[x];
-            if (l > 0 && tp.tr != l - 1) continue;
             const int steps = tp.m_k / 64, strips = (tp.n + 127) / 128;
             if (l == 0) {  // the longer of the two chains, k steps and moment update (16 ranks about as long as half a step)
               const int half = tp.r_n < 256 ? tp.r_n : 256;
@@ -1347,7 +1349,6 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
               for (int s2 = 0; s2 < strips; ++s2) items.push_back({x, s2, steps, (double)steps});
             }
           }
-          if (items.empty()) continue;
           std::vector<TcSeg> list;
           std::vector<int> start;
           long long steps = 0;
@@ -1447,14 +1448,11 @@ int lordo_inner_step(lordo_ctx* c, const void* const* G, float lr, float beta1, 
       }
       {
         ProfScope ps(c, st, PC_APPLY);
-        for (int side = 0; side < 2; ++side) {  // problems stored as projected, then the ones stored transposed
-          if (c->seg_workers[1 + side] == 0) continue;
-          // 256 < r <= 512: the error-feedback sweep, then the model-update sweep; else one sweep does both
-          for (int mode = big ? (c->cfg.error_feedback ? 1 : 2) : 0; mode <= (big ? 2 : 0); ++mode) {
-            launch_apply_tma(c->d_tc_probs, c->d_segs[1 + side], c->d_seg_start[1 + side], c->seg_workers[1 + side], c->d_maps, c->d_gmaps, ss,
-                             mode, side, c->d_status, st);
-            c->launches += 1;
-          }
+        // 256 < r <= 512: the error-feedback sweep, then the model-update sweep; else one sweep does both
+        for (int mode = big ? (c->cfg.error_feedback ? 1 : 2) : 0; mode <= (big ? 2 : 0); ++mode) {
+          launch_apply_tma(c->d_tc_probs, c->d_segs[1], c->d_seg_start[1], c->seg_workers[1], c->d_maps, c->d_gmaps, ss, mode, c->tma_side,
+                           c->d_status, st);
+          c->launches += 1;
         }
       }
       c->launches -= 1;  // the common tail below counts one update launch

@@ -4,12 +4,13 @@
 
 namespace lordo {
 
-// Elements per partial sum of squares: small enough that a step with few gradients still has a few thousand
-// threads in flight on every SM, and no smaller. Never below 2048 (256 threads of 8).
+// Elements per partial sum of squares: 32768, or less where that leaves less than a wave of blocks (eight fit an SM),
+// then about one wave, down to 2048 (256 threads of 8). Smaller blocks cost more in counters and exits than they
+// balance (five ragged matrices, 15 million elements: blocks of 2048 29 us, 1038 blocks 13 us), larger ones end apart
+// (4096 x 11008, K = 4: blocks of 131072 70 us, of 32768 58 us).
 inline long long sq_chunk(long long elements) {
-  long long c = 32768;
-  while (c > 2048 && elements / c < 4 * 148) c /= 2;
-  return c;
+  const long long c = (elements / (8 * 148) + 2047) / 2048 * 2048;
+  return c < 2048 ? 2048 : c > 32768 ? 32768 : c;
 }
 
 // Launch of a kernel that calls dep_begin() in every thread before it touches anything that another kernel writes. Its
@@ -173,10 +174,10 @@ cudaError_t tma_configure();
 int project_pairs(int sm_count);  // CTA pairs of the projection that the device holds at once
 void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int pairs, const TmaMatMaps* maps,
                         const TmaGradMaps* gmaps, const StepScalars& sc, unsigned* status, cudaStream_t st);
-// mode 0: r <= 256, one sweep; modes 1 and 2: the two sweeps for 256 < r <= 512. A launch covers problems of one
-// side only: tr = 0 stored as the problem, tr = 1 transposed.
+// mode 0: r <= 256, one sweep; modes 1 and 2: the two sweeps for 256 < r <= 512. side 0: every problem is stored as it
+// is (tr = 0), 1: every one transposed, 2: some of either.
 void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int ctas, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
-                      const StepScalars& sc, int mode, int tr, unsigned* status, cudaStream_t st);
+                      const StepScalars& sc, int mode, int side, unsigned* status, cudaStream_t st);
 
 void launch_selftest_wait(unsigned* status, cudaStream_t st);
 

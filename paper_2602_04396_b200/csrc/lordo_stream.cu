@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
   const long long end = begin + chunk < elems ? begin + chunk : elems;
   constexpr int kBytes = BF16 ? 2 : 4;
   const char* g = reinterpret_cast<const char*>(G[i]) + (long long)k * elems * kBytes;
-  float acc = 0.f;
+  float sum[4] = {0.f, 0.f, 0.f, 0.f};  // of at most 128 squares each
   for (long long e = begin + 8ll * t; e < end; e += 4 * 8 * 256) {  // elems is a multiple of 8
     uint4 x[4][BF16 ? 1 : 2];
 #pragma unroll
@@ -62,15 +62,15 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
         for (int j = 0; j < 4; ++j) {
           if (BF16) {
             const float lo = __uint_as_float(w[j] << 16), hi = __uint_as_float(w[j] & 0xFFFF0000u);
-            acc += lo * lo + hi * hi;
+            sum[u] += lo * lo + hi * hi;
           } else {
             const float v = __uint_as_float(w[j]);
-            acc += v * v;
+            sum[u] += v * v;
           }
         }
       }
   }
-  double d = (double)acc;
+  double d = ((double)sum[0] + (double)sum[1]) + ((double)sum[2] + (double)sum[3]);
   for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
   if ((t & 31) == 0) red[t >> 5] = d;
   __syncthreads();

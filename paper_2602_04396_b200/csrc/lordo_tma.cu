@@ -301,11 +301,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
 // MODE 0: r <= 256, both products in one sweep. For 256 < r <= 512 one low-rank operand alone fills
 // 256 columns of tensor memory, so the update is two sweeps of the same kernel: MODE 1 does the
 // error-feedback line (operand g^T, tiles G and E), MODE 2 the model update (operand U~^T, tiles G, W).
-// TR: the problems of this launch are matrices projected from the right, whose W, G, E are stored
+// SIDE 1: the problems of this launch are matrices projected from the right, whose W, G, E are stored
 // transposed with respect to the problem: a strip is 128 stored rows, a step 64 stored columns, and the
 // accumulator tile (lane = strip element, column = step element) already lies the way the tiles are
-// stored, so a thread works on 16 neighbouring stored columns of its own row.
-template <int MODE, bool TR>
+// stored, so a thread works on 16 neighbouring stored columns of its own row. SIDE 2: both kinds, told apart piece by
+// piece; as two launches, each with its own start and end, five ragged matrices took 28 + 31 us, as one 46 us.
+template <int MODE, int SIDE>
 __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem* __restrict__ probs, const TcSeg* __restrict__ segs,
                                                                  const int* __restrict__ start, const TmaMatMaps* __restrict__ maps,
                                                                  const TmaGradMaps* __restrict__ gmaps, StepScalars sc,
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
           unsigned char* base = sIn + is * ISB;
           const bool ld_e = DO_E && ef;
           mbar_expect_tx(&in_full[is], 16384u + (ld_e ? 16384u : 0u) + (DO_W ? 16384u : 0u));
-          if (TR) {  // one box of 128 stored rows x 64 stored columns per tile
+          if (SIDE == 1 || (SIDE == 2 && pr->tr)) {  // one box of 128 stored rows x 64 stored columns per tile
             tma_load_3d(base, gm->g_kb, t * kARows, n0, rep, &in_full[is]);
             if (ld_e) tma_load_3d(base + EOFF, mm->e_kb, t * kARows, n0, rep, &in_full[is]);
             if (DO_W) tma_load_3d(base + WOFF, mm->w_kb, t * kARows, n0, rep, &in_full[is]);
@@ -439,7 +440,6 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
     // 2(t%4), +1, +8, +9 of its row group: 8-byte accesses to the swizzled tiles, free of conflicts.
     const int ew = warp - 2;
     const int q = warp & 3, grp = ew >> 2;  // lane quarter (fixed by the hardware), row group 0..3
-    const int colq = TR ? q * 32 + lane : q * 32 + 4 * (lane & 7) + (lane >> 3);  // strip element this lane's operands belong to
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     const int tb = lane >> 2, tr = lane & 3;
     const int ecol0 = q * 32 + 4 * tb;  // first of this thread's four epilogue columns
@@ -463,13 +463,15 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
       const int n0 = sg.strip * kStrip;
       const TmaMatMaps* mm = maps + pr->mat;
       const int rep = pr->replica;
+      const bool tr_p = SIDE == 1 || (SIDE == 2 && pr->tr);
+      const int colq = tr_p ? q * 32 + lane : q * 32 + 4 * (lane & 7) + (lane >> 3);  // strip element this lane's operands belong to
       const long long col = (long long)n0 + colq;
       const float c = *pr->cptr;
       float cd[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        // TR: one strip element per thread (its own row); else the four columns of the thread's epilogue block
-        const long long ec = TR ? col : (long long)n0 + ecol0 + j;
+        // right side: one strip element per thread (its own row); else the four columns of the thread's epilogue block
+        const long long ec = tr_p ? col : (long long)n0 + ecol0 + j;
         const long long ecc = ec < n ? ec : (long long)n - 1;
         cd[j] = full ? (1.f - om) * c / (pr->dcol[ecc] + (pr->dcol2 ? pr->dcol2[ecc] : 0.f)) : 0.f;
       }
@@ -506,7 +508,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
         if (ok) ok = mbar_wait<32>(&acc_full[b], (jt >> 1) & 1u, status);
         if (!ok) break;
         tc_fence_after_sync();
-        if constexpr (TR) {
+        if (tr_p) {
           // this thread: stored row 32q + lane of the strip, stored columns 16 grp .. +15 of the step
           const int row = q * 32 + lane;
           const uint32_t o0 = swz_chunk(row, 2 * grp), o1 = swz_chunk(row, 2 * grp + 1);
@@ -545,7 +547,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
           }
           // the four warps that share 32 stored rows hand them to the TMA engine on their own
           fence_async_smem();
-          asm volatile("bar.sync %0, 128;" ::"r"(2 + q) : "memory");
+          asm volatile("bar.sync %0, 128;" ::"r"(6 + q) : "memory");
           if (grp == 0 && lane == 0) {
             if (n0 + q * 32 < n) {
               if (DO_E && ef) tma_store_3d(mm->e_st32, t * kARows, n0 + q * 32, rep, base + EOFF + q * 4096);
@@ -617,7 +619,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
         }
       }
     }
-    if ((TR ? grp == 0 : (ew & 3) == 0) && lane == 0) tma_store_wait_all();
+    if ((grp == 0 || (ew & 3) == 0) && lane == 0) tma_store_wait_all();
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -649,17 +651,12 @@ cudaError_t tma_configure() {
   e = max_resident_pairs(project_tma_kernel, kPThreads, kPStages * kPStageBytes + 1024, &g_project_pairs);
   if (e != cudaSuccess) return e;
   const int smem = (int)(kAPStages * 65536 + kAInStages * 32768 + 1024);  // the largest of the three modes
-  e = cudaFuncSetAttribute(apply_tma_kernel<0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(apply_tma_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(apply_tma_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(apply_tma_kernel<0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(apply_tma_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(apply_tma_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const void* kernels[9] = {(const void*)apply_tma_kernel<0, 0>, (const void*)apply_tma_kernel<1, 0>, (const void*)apply_tma_kernel<2, 0>,
+                            (const void*)apply_tma_kernel<0, 1>, (const void*)apply_tma_kernel<1, 1>, (const void*)apply_tma_kernel<2, 1>,
+                            (const void*)apply_tma_kernel<0, 2>, (const void*)apply_tma_kernel<1, 2>, (const void*)apply_tma_kernel<2, 2>};
+  for (const void* k : kernels)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return e;
 }
 
 int project_pairs(int sm_count) { return g_project_pairs > 0 ? std::min(sm_count / 2, g_project_pairs) : sm_count / 2; }
@@ -670,19 +667,18 @@ void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* st
   launch_dep(project_tma_kernel, dim3(2u * (unsigned)pairs), kPThreads, kPStages * kPStageBytes + 1024, st, probs, segs, start, maps, gmaps, sc, status);
 }
 void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int ctas, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
-                      const StepScalars& sc, int mode, int tr, unsigned* status, cudaStream_t st) {
+                      const StepScalars& sc, int mode, int side, unsigned* status, cudaStream_t st) {
   if (ctas <= 0) return;
   const size_t small = kAPStages * kAPStageBytes + kAInStages * kAInStageBytes + 1024, large = kAPStages * 65536 + kAInStages * 32768 + 1024;
 #define LORDO_APPLY(M, T, SM) launch_dep(apply_tma_kernel<M, T>, dim3((unsigned)ctas), kAThreads, SM, st, probs, segs, start, maps, gmaps, sc, status)
-  if (!tr) {
-    if (mode == 0) LORDO_APPLY(0, false, small);
-    else if (mode == 1) LORDO_APPLY(1, false, large);
-    else LORDO_APPLY(2, false, large);
-  } else {
-    if (mode == 0) LORDO_APPLY(0, true, small);
-    else if (mode == 1) LORDO_APPLY(1, true, large);
-    else LORDO_APPLY(2, true, large);
-  }
+#define LORDO_APPLY_SIDE(T)                    \
+  if (mode == 0) LORDO_APPLY(0, T, small);      \
+  else if (mode == 1) LORDO_APPLY(1, T, large); \
+  else LORDO_APPLY(2, T, large)
+  if (side == 0) { LORDO_APPLY_SIDE(0); }
+  else if (side == 1) { LORDO_APPLY_SIDE(1); }
+  else { LORDO_APPLY_SIDE(2); }
+#undef LORDO_APPLY_SIDE
 #undef LORDO_APPLY
 }
 
