@@ -578,6 +578,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       } else if (st.type == ST_ROTATE) {
         st.first = (long long)c->h_rotates.size(); st.count = (int)sl.ro.size(); st.tiles = 0;
         for (RotateProblem& x : sl.ro) {
+          st.r_max = std::max(st.r_max, x.r_n);
           const int strips = (x.n + 127) / 128;
           x.item_start = st.tiles; st.tiles += x.nsplit == 2 ? strips : (strips + 1) / 2;
           c->h_rotates.push_back(x);
@@ -1110,7 +1111,7 @@ int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t 
       c->launches += 1;
       return check_launch(c, "commit_basis");
     case ST_ROTATE:
-      launch_rotate(c->d_rotates + s.first, s.count, s.tiles, c->sm_count, sc, c->d_status, st);
+      launch_rotate(c->d_rotates + s.first, s.count, s.tiles, s.r_max, c->sm_count, sc, c->d_status, st);
       c->launches += 1;
       return check_launch(c, "rotate");
     case ST_ROT:

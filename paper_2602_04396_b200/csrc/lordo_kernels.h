@@ -255,7 +255,7 @@ struct RotateProblem {
   int n, r, r_n, b, nb, nsplit;
 };
 cudaError_t rotate_configure();
-void launch_rotate(const RotateProblem* probs, int nprobs, long long items, int sm_count, const GemmScalars& sc, unsigned* status, cudaStream_t st);
+void launch_rotate(const RotateProblem* probs, int nprobs, long long items, int r_max, int sm_count, const GemmScalars& sc, unsigned* status, cudaStream_t st);
 
 // Gram matrix of a tensor-core QR from its partial products: gram = sum_s S_s + sum_s (T_s + T_s^T), the S
 // and T of `ns` ranges of k each, all r x r, S first. With X ~ p0 + p1 + p2, S = p1^T p1 + p0^T p0 and
