@@ -21,7 +21,7 @@ __device__ __forceinline__ Source resolve(const Operand& op) {
   Source s;
   const void* base = op.p0_ind ? *op.p0_ind : op.p0;
   s.p0 = reinterpret_cast<const char*>(base) + op.p0_off * (op.dt0 == LORDO_F32 ? 4 : 2);
-  s.p1 = op.p1; s.ld = op.ld; s.s0 = op.s0_ptr ? *op.s0_ptr : 1.f; s.dt0 = op.dt0; s.dt1 = op.dt1; s.kind = op.kind;
+  s.p1 = op.p1; s.ld = op.ld; s.s0 = 1.f; s.dt0 = op.dt0; s.dt1 = op.dt1; s.kind = op.kind;
   return s;
 }
 
@@ -144,9 +144,23 @@ __device__ __forceinline__ void partials_of(const double* p, unsigned rank, doub
 // distributed shared memory, every CTA finishing its share of the tile's rows (see launch_gemm for the size).
 // CARRY = 1: slice sums carried across k-slices in fp64 (parity mode). CARRY = 0: plain fp32
 // accumulation, half the registers (the fp32 work of the fast mode: QR and moment rotation).
+// With two products twice the threads of half the columns: 256 threads held so many sums (190 to 250 registers) that an SM
+// had eight warps to cover the loads with. Three ragged matrices with three workers, r up to 136: update 175 -> 145 us.
+template <int DUAL>
+constexpr int kGemmThreads = DUAL ? 512 : 256;
+
+__device__ __forceinline__ void load_columns(float (&x)[4], const float* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+}
+__device__ __forceinline__ void load_columns(float (&x)[2], const float* p) {
+  const float2 v = *reinterpret_cast<const float2*>(p);
+  x[0] = v.x; x[1] = v.y;
+}
+
 template <int ATRANS, int DUAL, int CARRY>
-__global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
-  dep_begin();
+__global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
+  constexpr int NT = kGemmThreads<DUAL>, CN = BN * BM / 4 / NT;  // threads, output columns per thread (rows: four)
   __shared__ __align__(16) float sA[2][BK][BM + PADS];
   __shared__ __align__(16) float sB[2][BK][BN + PADS];
   __shared__ __align__(16) float sB2[2][DUAL ? BK : 1][BN + PADS];
@@ -168,21 +182,28 @@ __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(c
   const int M = pr.M, N = pr.N, Kd = pr.Kd;
   const long long m0 = (long long)tile_m * BM, n0 = (long long)tile_n * BN;
 
-  const Source A = resolve(pr.A), B = resolve(pr.B), B2 = resolve(DUAL ? pr.B2 : pr.B);
+  Source A = resolve(pr.A), B = resolve(pr.B);
+  const Source B2 = resolve(DUAL ? pr.B2 : pr.B);
+  dep_begin();  // the tables are constant, and gradient pointers are copied in front of the kernel before this one
+  if (pr.A.s0_ptr) A.s0 = *pr.A.s0_ptr;
+  if (pr.B.s0_ptr) B.s0 = *pr.B.s0_ptr;
 
   const int t = threadIdx.x;
-  const int tx = t & 15, ty = t >> 4;
-  // B tile loader: one float4 per thread, row kk = t/16, columns (t%16)*4
-  const int bk = t >> 4, bc = (t & 15) * 4;
-  // A tile loader. ATRANS: as B (stored [Kd][M]). Otherwise stored [M][Kd]: row t/4, k (t%4)*4.
-  const int ar = ATRANS ? (t >> 4) : (t >> 2), ac = ATRANS ? (t & 15) * 4 : (t & 3) * 4;
+  const int tx = t % (BN / CN), ty = t / (BN / CN);
+  // loaders, one float4 of a slice each. One product: every thread A and B. Two: the first 256 threads A, the others B and B2.
+  const bool load_a = !DUAL || t < 256, load_b = !DUAL || t >= 256;
+  const int lt = t & 255;
+  // B: row kk = lt/16, columns (lt%16)*4
+  const int bk = lt >> 4, bc = (lt & 15) * 4;
+  // A. ATRANS: as B (stored [Kd][M]). Otherwise stored [M][Kd]: row lt/4, k (lt%4)*4.
+  const int ar = ATRANS ? (lt >> 4) : (lt >> 2), ac = ATRANS ? (lt & 15) * 4 : (lt & 3) * 4;
 
-  float acc[4][4], acc2[DUAL ? 4 : 1][4];
-  double tot[CARRY ? 4 : 1][4], tot2[(CARRY && DUAL) ? 4 : 1][4];
+  float acc[4][CN], acc2[DUAL ? 4 : 1][CN];
+  double tot[CARRY ? 4 : 1][CN], tot2[(CARRY && DUAL) ? 4 : 1][CN];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < CN; ++j) {
       acc[i][j] = 0.f;
       if constexpr (CARRY) tot[i][j] = 0.0;
       if constexpr (DUAL) {
@@ -193,23 +214,28 @@ __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(c
 
   // Two slices of k are on their way in registers while a third, in one of two buffers, is multiplied.
   struct Slice {
-    Raw a, b, b2;
+    Raw x, y;  // one product: A and B; two: A and nothing, or B and B2
   };
-  auto fetch = [&](Slice& x, int k0) {
-    if (ATRANS) x.a = source_load(A, k0 + ar, m0 + ac, Kd, M);
-    else x.a = source_load(A, m0 + ar, k0 + ac, M, Kd);
-    x.b = source_load(B, k0 + bk, n0 + bc, Kd, N);
-    if constexpr (DUAL) x.b2 = source_load(B2, k0 + bk, n0 + bc, Kd, N);
-  };
-  auto stash = [&](const Slice& x, int buf) {
-    const float4 v = source_value(A, x.a, sc);
-    if (ATRANS) {
-      *reinterpret_cast<float4*>(&sA[buf][ar][ac]) = v;
-    } else {
-      sA[buf][ac + 0][ar] = v.x; sA[buf][ac + 1][ar] = v.y; sA[buf][ac + 2][ar] = v.z; sA[buf][ac + 3][ar] = v.w;
+  auto fetch = [&](Slice& s, int k0) {
+    if (load_a) s.x = ATRANS ? source_load(A, k0 + ar, m0 + ac, Kd, M) : source_load(A, m0 + ar, k0 + ac, M, Kd);
+    if (load_b) {
+      (DUAL ? s.x : s.y) = source_load(B, k0 + bk, n0 + bc, Kd, N);
+      if constexpr (DUAL) s.y = source_load(B2, k0 + bk, n0 + bc, Kd, N);
     }
-    *reinterpret_cast<float4*>(&sB[buf][bk][bc]) = source_value(B, x.b, sc);
-    if constexpr (DUAL) *reinterpret_cast<float4*>(&sB2[buf][bk][bc]) = source_value(B2, x.b2, sc);
+  };
+  auto stash = [&](const Slice& s, int buf) {
+    if (load_a) {
+      const float4 v = source_value(A, s.x, sc);
+      if (ATRANS) {
+        *reinterpret_cast<float4*>(&sA[buf][ar][ac]) = v;
+      } else {
+        sA[buf][ac + 0][ar] = v.x; sA[buf][ac + 1][ar] = v.y; sA[buf][ac + 2][ar] = v.z; sA[buf][ac + 3][ar] = v.w;
+      }
+    }
+    if (load_b) {
+      *reinterpret_cast<float4*>(&sB[buf][bk][bc]) = source_value(B, DUAL ? s.x : s.y, sc);
+      if constexpr (DUAL) *reinterpret_cast<float4*>(&sB2[buf][bk][bc]) = source_value(B2, s.y, sc);
+    }
   };
 
   // this CTA's range of k
@@ -225,21 +251,20 @@ __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(c
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
       const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][kk][ty * 4]);
-      const float4 b4 = *reinterpret_cast<const float4*>(&sB[buf][kk][tx * 4]);
       const float a[4] = {a4.x, a4.y, a4.z, a4.w};
-      const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+      float b[CN], c[CN];
+      load_columns(b, &sB[buf][kk][tx * CN]);
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < CN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
       if constexpr (DUAL) {
-        const float4 c4 = *reinterpret_cast<const float4*>(&sB2[buf][kk][tx * 4]);
-        const float c[4] = {c4.x, c4.y, c4.z, c4.w};
+        load_columns(c, &sB2[buf][kk][tx * CN]);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float a2 = sc.a_square ? a[i] * a[i] : a[i];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc2[i][j] = fmaf(a2, c[j], acc2[i][j]);
+          for (int j = 0; j < CN; ++j) acc2[i][j] = fmaf(a2, c[j], acc2[i][j]);
         }
       }
     }
@@ -247,7 +272,7 @@ __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(c
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < CN; ++j) {
           tot[i][j] += (double)acc[i][j];
           acc[i][j] = 0.f;
           if constexpr (DUAL) { tot2[i][j] += (double)acc2[i][j]; acc2[i][j] = 0.f; }
@@ -269,25 +294,21 @@ __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(c
     if (k0 + BK < kend) turn(k0 + BK, x1, x0);
   }
   const Epilogue& ep = pr.epi;
-  if (csize > 1) {
+  if (DUAL || csize > 1) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      double v[4], v2[4];
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if constexpr (CARRY) v[j] = tot[i][j]; else v[j] = (double)acc[i][j];
-        if constexpr (CARRY && DUAL) v2[j] = tot2[i][j]; else v2[j] = (double)acc2[DUAL ? i : 0][j];
+      for (int j = 0; j < CN; j += 2) {
+        double* o = part + (ty * 4 + i) * BN + tx * CN + j;
+        if constexpr (CARRY) *reinterpret_cast<double2*>(o) = make_double2(tot[i][j], tot[i][j + 1]);
+        else *reinterpret_cast<double2*>(o) = make_double2((double)acc[i][j], (double)acc[i][j + 1]);
+        if constexpr (CARRY && DUAL) *reinterpret_cast<double2*>(o + BM * BN) = make_double2(tot2[i][j], tot2[i][j + 1]);
+        else if constexpr (DUAL) *reinterpret_cast<double2*>(o + BM * BN) = make_double2((double)acc2[i][j], (double)acc2[i][j + 1]);
       }
-      double2* o = reinterpret_cast<double2*>(part + (ty * 4 + i) * BN + tx * 4);
-      o[0] = make_double2(v[0], v[1]); o[1] = make_double2(v[2], v[3]);
-      if constexpr (DUAL) {
-        double2* o2 = o + BM * BN / 2;
-        o2[0] = make_double2(v2[0], v2[1]); o2[1] = make_double2(v2[2], v2[3]);
-      }
-    }
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
     const int rows = BM / (int)csize;
-    for (int e = t; e < rows * (BN / 4); e += 256) {
+    for (int e = t; e < rows * (BN / 4); e += NT) {
       const int lr = (int)rank * rows + e / (BN / 4), lc = (e % (BN / 4)) * 4;
       const long long row = m0 + lr, col = n0 + lc;
       if (row >= M || col >= N) continue;
@@ -307,26 +328,23 @@ __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(c
       gemm_epilogue<DUAL>(ep, sc, N, row, col, a1, a2);
     }
     // nobody leaves while its partial sums may still be read
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     return;
   }
-  if constexpr (CARRY) {
+  if constexpr (!DUAL) {
+    // each thread owns rows m0+ty*4.., columns n0+tx*4..+3
+    const long long col = n0 + tx * 4;
+    if (col >= N) return;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) {
+      const long long row = m0 + ty * 4 + i;
+      if (row >= M) break;
+      if constexpr (CARRY) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        acc[i][j] = (float)tot[i][j];
-        if constexpr (DUAL) acc2[i][j] = (float)tot2[i][j];
+        for (int j = 0; j < 4; ++j) acc[i][j] = (float)tot[i][j];
       }
-  }
-  // each thread owns rows m0+ty*4.., columns n0+tx*4..+3
-  const long long col = n0 + tx * 4;
-  if (col >= N) return;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const long long row = m0 + ty * 4 + i;
-    if (row >= M) break;
-    gemm_epilogue<DUAL>(ep, sc, N, row, col, acc[i], acc2[DUAL ? i : 0]);
+      gemm_epilogue<0>(ep, sc, N, row, col, acc[i], acc[i]);
+    }
   }
 }
 
@@ -336,7 +354,7 @@ __global__ void __launch_bounds__(256, DUAL && CARRY ? 1 : 2) gemm_ffma_kernel(c
 // and r up to 136 in 14 CTAs 105 us, in 112 17.
 void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
                  const GemmScalars& sc, cudaStream_t st) {
-  const long long room = (long long)sm_count * (dual && carry ? 1 : 2);  // by registers
+  const long long room = (long long)sm_count * (dual ? 1 : 2);  // by registers
   const int slices = (kd_max + BK - 1) / BK;
   int c = 1;
   while (c < 8 && total_tiles * 2 * c <= room && slices >= 4 * c) c *= 2;
@@ -346,8 +364,8 @@ void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, in
   at[0].val.clusterDim.x = (unsigned)c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(256, 1, 1); lc.stream = st;
-  lc.dynamicSmemBytes = c > 1 ? sizeof(double) * BM * BN * (dual ? 2 : 1) : 0;
+  lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(dual ? kGemmThreads<1> : kGemmThreads<0>, 1, 1); lc.stream = st;
+  lc.dynamicSmemBytes = c > 1 || dual ? sizeof(double) * BM * BN * (dual ? 2 : 1) : 0;
   lc.attrs = at; lc.numAttrs = 2;
 #define LORDO_GEMM(A, B, C) cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, C>, probs, nprobs, sc)
   if (carry) {

@@ -29,13 +29,13 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
                                                    const long long* __restrict__ chunk_start, int n_mats, int K, long long chunk, double* partial,
                                                    float rho, int scope, float* __restrict__ coef, double* sumsq, unsigned* __restrict__ tickets,
                                                    unsigned* __restrict__ status) {
-  dep_begin();
   __shared__ double red[256];
   __shared__ bool last_s;
   const int t = threadIdx.x;
   const long long blk = blockIdx.x;
-  const int i = find_segment(chunk_start, n_mats, blk);
+  const int i = find_segment(chunk_start, n_mats, blk);  // the tables are constant
   const long long elems = mats[i].m * mats[i].n;
+  dep_begin();
   const unsigned chunks = (unsigned)((elems + chunk - 1) / chunk);
   const unsigned local = (unsigned)(blk - chunk_start[i]);
   const int k = (int)(local / chunks);
@@ -120,11 +120,11 @@ __global__ void fill_float_kernel(float* __restrict__ p, long long count, float 
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) moments_kernel(const MatDev* __restrict__ mats, const long long* __restrict__ tile_start,
                                                       int n_mats, StepScalars sc) {
-  dep_begin();
   const int lane = threadIdx.x & 31, wrow = threadIdx.x >> 5;
   const long long blk = blockIdx.x;
-  const int i = find_segment(tile_start, n_mats, blk);
+  const int i = find_segment(tile_start, n_mats, blk);  // the tables are constant
   const MatDev md = mats[i];
+  dep_begin();
   const long long n = md.ln;  // columns of the low-rank arrays
   const int r = md.r;
   const long long ctiles = (n + 127) / 128;
