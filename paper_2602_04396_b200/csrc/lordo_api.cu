@@ -276,7 +276,7 @@ void prefix_arrays(const lordo_config& cfg, std::vector<long long>& chunk_start,
     const long long elems = a.m * a.n;
     chunk_start[i + 1] = chunk_start[i] + (long long)K * ((elems + chunk - 1) / chunk);
     const long long ln = a.side ? a.m : a.n;  // columns of the low-rank arrays
-    mom_start[i + 1] = mom_start[i] + (long long)K * ((ln + 127) / 128);
+    mom_start[i + 1] = mom_start[i] + (long long)K * ((ln + kMomCols - 1) / kMomCols);
     wblk[i + 1] = wblk[i] + (elems + 1023) / 1024;
     sblk[i + 1] = sblk[i] + ((long long)a.r * ln + 1023) / 1024;
   }

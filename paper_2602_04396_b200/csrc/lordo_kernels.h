@@ -334,6 +334,7 @@ void launch_clip(const MatDev* mats, const void* const* G, const long long* chun
                  double* partial, long long total_chunks, float rho, int scope, float* coef, double* sumsq, unsigned* tickets, unsigned* status,
                  cudaStream_t st);
 void launch_fill_float(float* p, long long count, float value, cudaStream_t st);
+constexpr int kMomCols = 32;  // columns of the low-rank arrays per block of the moment update
 void launch_moments(const MatDev* mats, const long long* tile_start, int n_mats, long long total_tiles, const StepScalars& sc,
                     cudaStream_t st);
 void launch_outer_weights(const MatDev* mats, const long long* blk_start, int n_mats, long long total_blocks, int K, int w_dt,

@@ -116,28 +116,32 @@ __global__ void fill_float_kernel(float* __restrict__ p, long long count, float 
 //   u <- b1 u + (1-b1) g ; v <- b2 v + (1-b2) g*g ; u^ = u/(1-b1^s) ; v^ = v/(1-b2^s)
 //   D = sqrt(v^) + eps ; U~ = u^/D (no / full-rank QHM) or (w u^ + (1-w) g)/D (low-rank QHM)
 //   full-rank QHM also needs mu(D) = mean over the rank axis, one value per column.
-// One block = 128 columns of one (matrix, replica); its warps stride over the r rows.
+// One block = kMomCols columns of one (matrix, replica), eight lanes across and 32 rows of ranks down: bound by latency
+// at the sizes of check mode (a rank's loads, square root and division take about a microsecond), so a thread has few ranks
+// and a full line per row of a block is all the width that the loads need. With 128 columns a block three ragged
+// matrices with three workers (r up to 136) took 20 us, now 9; 256 columns, r = 16, two workers 5.3, now 4.5 us.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) moments_kernel(const MatDev* __restrict__ mats, const long long* __restrict__ tile_start,
                                                       int n_mats, StepScalars sc) {
-  const int lane = threadIdx.x & 31, wrow = threadIdx.x >> 5;
+  constexpr int LANES = kMomCols / 4, ROWS = 256 / LANES;
+  const int lane = threadIdx.x % LANES, row = threadIdx.x / LANES;
   const long long blk = blockIdx.x;
   const int i = find_segment(tile_start, n_mats, blk);  // the tables are constant
   const MatDev md = mats[i];
   dep_begin();
   const long long n = md.ln;  // columns of the low-rank arrays
   const int r = md.r;
-  const long long ctiles = (n + 127) / 128;
+  const long long ctiles = (n + kMomCols - 1) / kMomCols;
   const long long local = blk - tile_start[i];
   const int k = (int)(local / ctiles);
-  const long long col = (local - (long long)k * ctiles) * 128 + 4ll * lane;
+  const long long col = (local - (long long)k * ctiles) * kMomCols + 4ll * lane;
   const bool active = col < n;
   const long long base = (long long)k * r * n + col;
   const float b1 = sc.beta1, b2 = sc.beta2, w = sc.omega;
   float dsum0 = 0.f, dsum1 = 0.f, dsum2 = 0.f, dsum3 = 0.f;
   if (active) {
 #pragma unroll 2
-    for (int a = wrow; a < r; a += 8) {
+    for (int a = row; a < r; a += ROWS) {
       const long long idx = base + (long long)a * n;
       const float4 g = *reinterpret_cast<const float4*>(md.ghat + idx);
       float4 u = *reinterpret_cast<const float4*>(md.u + idx);
@@ -167,11 +171,19 @@ __global__ void __launch_bounds__(256) moments_kernel(const MatDev* __restrict__
     }
   }
   if (sc.form == LORDO_QHM_FULL) {  // uniform over the grid
-    __shared__ float4 red[8][32];
-    red[wrow][lane] = make_float4(dsum0, dsum1, dsum2, dsum3);
+    // the four rows of a warp, then the warps, in a fixed order
+    __shared__ float4 red[8][LANES];
+    float4 s = make_float4(dsum0, dsum1, dsum2, dsum3);
+#pragma unroll
+    for (int o = LANES; o < 32; o <<= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, o); s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+      s.z += __shfl_xor_sync(0xffffffffu, s.z, o); s.w += __shfl_xor_sync(0xffffffffu, s.w, o);
+    }
+    if ((threadIdx.x & 31) < LANES) red[threadIdx.x >> 5][lane] = s;
     __syncthreads();
-    if (wrow == 0 && active) {
-      float4 s = red[0][lane];
+    if (row == 0 && active) {
+      s = red[0][lane];
+#pragma unroll
       for (int y = 1; y < 8; ++y) {
         const float4 t = red[y][lane];
         s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
