@@ -80,7 +80,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   // fed by the warps of both; empty_bar and acc_full are signalled in both CTAs by that thread's commits
   __shared__ uint64_t full_a[kMaxStages], full_b[kMaxStages], empty_bar[kMaxStages], acc_full, acc_empty, peer_read;
   __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const uint32_t rank = cluster_rank();
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(&full_a[s], kCtas * kFormWarps); mbar_init(&full_b[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -124,7 +124,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issue --------------------------------------------------------------------
-    if (lane == 0 && (!PAIR || rank == 0)) {
+    if (!PAIR || rank == 0) {
+      const uint32_t one = elect_one();
       uint32_t it = 0, si = 0;
       bool ok = true;
       const uint32_t eb0 = cluster_addr(&empty_bar[0], 0), eb1 = cluster_addr(&empty_bar[0], 1);
@@ -134,11 +135,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int r_lo = pr->nsplit == 2 ? (int)rank * 256 : 0, n_h = min(pr->r_n - r_lo, 256);
         const int nkb = (pr->r + kRows - 1) / kRows;
         const uint32_t idesc = idesc_bf16_f32(128 * kCtas, (uint32_t)n_h) | kIdescAMajorMN | (1u << 16);  // both operands MN-major
-        ok = mbar_wait(&acc_empty, (si & 1u) ^ 1u, status);
+        ok = mbar_wait_warp(&acc_empty, (si & 1u) ^ 1u, status);
         for (int kb = 0; kb < nkb && ok; ++kb, ++it) {
           const int s = it % kStages;
-          if (!PAIR) ok = mbar_wait(&full_b[s], (it / kStages) & 1u, status);
-          if (ok) ok = mbar_wait(&full_a[s], (it / kStages) & 1u, status);
+          if (!PAIR) ok = mbar_wait_warp(&full_b[s], (it / kStages) & 1u, status);
+          if (ok) ok = mbar_wait_warp(&full_a[s], (it / kStages) & 1u, status);
           if (!ok) break;
           tc_fence_after_sync();
           const uint32_t a = smem_u32(smem + s * kStage), b = a + 4 * kPlaneA;
@@ -149,19 +150,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               const uint32_t ah = a + 2 * d * kPlaneA + k16 * 2048, bh = b + 2 * d * kPlaneB + k16 * 2048, acc = tmem + 256 * d;
               const uint32_t more = (kb > 0 || k16 > 0) ? 1u : 0u;
               if (PAIR) {
-                mma_bf16_pair(acc, desc_mn_rows32(ah), desc_mn_rows32(bh + kPlaneB), idesc, more);
-                mma_bf16_pair(acc, desc_mn_rows32(ah + kPlaneA), desc_mn_rows32(bh), idesc, 1u);
-                mma_bf16_pair(acc, desc_mn_rows32(ah), desc_mn_rows32(bh), idesc, 1u);
+                mma_bf16_pair(acc, desc_mn_rows32(ah), desc_mn_rows32(bh + kPlaneB), idesc, more, one);
+                mma_bf16_pair(acc, desc_mn_rows32(ah + kPlaneA), desc_mn_rows32(bh), idesc, 1u, one);
+                mma_bf16_pair(acc, desc_mn_rows32(ah), desc_mn_rows32(bh), idesc, 1u, one);
               } else {
-                mma_bf16(acc, desc_mn_rows32(ah), desc_mn_rows32(bh + kPlaneB), idesc, more);
-                mma_bf16(acc, desc_mn_rows32(ah + kPlaneA), desc_mn_rows32(bh), idesc, 1u);
-                mma_bf16(acc, desc_mn_rows32(ah), desc_mn_rows32(bh), idesc, 1u);
+                mma_bf16(acc, desc_mn_rows32(ah), desc_mn_rows32(bh + kPlaneB), idesc, more, one);
+                mma_bf16(acc, desc_mn_rows32(ah + kPlaneA), desc_mn_rows32(bh), idesc, 1u, one);
+                mma_bf16(acc, desc_mn_rows32(ah), desc_mn_rows32(bh), idesc, 1u, one);
               }
             }
-          if (PAIR) { mma_commit_pair(eb0 + 8u * s); mma_commit_pair(eb1 + 8u * s); }
-          else mma_commit(&empty_bar[s]);
+          if (one) {
+            if (PAIR) { mma_commit_pair(eb0 + 8u * s); mma_commit_pair(eb1 + 8u * s); }
+            else mma_commit(&empty_bar[s]);
+          }
         }
-        if (ok) {
+        if (ok && one) {
           if (PAIR) { mma_commit_pair(af0); mma_commit_pair(af1); }
           else mma_commit(&acc_full);
         }

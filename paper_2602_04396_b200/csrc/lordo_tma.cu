@@ -80,7 +80,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
   __shared__ uint32_t tmem_slot;
   __shared__ float dsum_s[3][kStrip];
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const bool ef = sc.ef != 0;
   const uint32_t rank = cluster_rank();
   const int seg_begin = start[blockIdx.x >> 1], seg_end = start[(blockIdx.x >> 1) + 1];
@@ -141,7 +141,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issue ---------------------------------------------------------------
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
+      const uint32_t one = elect_one();
       uint32_t it = 0, si = 0;
       bool ok = true;
       // the barriers the commits arrive on, in this CTA and in the other (8 bytes apart within an array)
@@ -155,21 +156,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
         const bool tr = pr->tr != 0;  // the tile then lies as [128 strip elements][64 k]: a K-major operand
         const uint32_t idesc = idesc_bf16_f32(256, n_h) | (tr ? 0u : kIdescAMajorMN);
         const uint32_t buf = si & 1u;
-        ok = mbar_wait(&acc_empty[buf], ((si >> 1) & 1u) ^ 1u, status);
+        ok = mbar_wait_warp(&acc_empty[buf], ((si >> 1) & 1u) ^ 1u, status);
         if (!ok) break;
         for (int kb = 0; kb < nkb; ++kb, ++it) {
           const int s = it % ST;
-          ok = mbar_wait(&xform_bar[s], (it / ST) & 1u, status);
+          ok = mbar_wait_warp(&xform_bar[s], (it / ST) & 1u, status);
           if (!ok) break;
           tc_fence_after_sync();
           const uint32_t sA = smem_u32(smem + s * SB), sB = sA + 32768;
 #pragma unroll
           for (int k16 = 0; k16 < 4; ++k16)
             mma_bf16_pair(tmem + buf * 256, tr ? smem_desc_k128(sA + k16 * 32) : smem_desc_mn128(sA + k16 * 2048), smem_desc_k128(sB + k16 * 32),
-                          idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
-          mma_commit_pair(eb0 + 8u * s); mma_commit_pair(eb1 + 8u * s);
+                          idesc, (kb > 0 || k16 > 0) ? 1u : 0u, one);
+          if (one) { mma_commit_pair(eb0 + 8u * s); mma_commit_pair(eb1 + 8u * s); }
         }
-        if (ok) { mma_commit_pair(af0 + 8u * buf); mma_commit_pair(af1 + 8u * buf); }
+        if (ok && one) { mma_commit_pair(af0 + 8u * buf); mma_commit_pair(af1 + 8u * buf); }
       }
     }
   } else if (warp < 2 + kPXformWarps) {
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
   __shared__ uint64_t p_full[kAPStages], p_empty[kAPStages], in_full[kAInStages], in_free[kAInStages], acc_full[2], acc_empty[2], x_ready;
   __shared__ uint32_t tmem_slot;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const bool ef = sc.ef != 0;
   const int seg_begin = start[blockIdx.x], seg_end = start[blockIdx.x + 1];
 
@@ -399,21 +400,21 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
     }
   } else if (warp == 1) {
     // ---------------- MMA issue: A operands from tensor memory ----------------------------------
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16_f32(128, kARows);
+    {
+      const uint32_t idesc = idesc_bf16_f32(128, kARows), one = elect_one();
       uint32_t jt = 0, si = 0;
       bool ok = true;
       for (int e = seg_begin; e < seg_end && ok; ++e, ++si) {
         const TcSeg sg = segs[e];
         const TcProblem* __restrict__ pr = probs + sg.prob;
         const int nkb = pr->r_k / 64;
-        ok = mbar_wait(&x_ready, si & 1u, status);
+        ok = mbar_wait_warp(&x_ready, si & 1u, status);
         if (!ok) break;
         for (int t = sg.t0; t < sg.t1; ++t, ++jt) {
           const int ps = jt % kAPStages;
           const uint32_t b = jt & 1u;
-          ok = mbar_wait(&p_full[ps], (jt / kAPStages) & 1u, status);
-          if (ok) ok = mbar_wait(&acc_empty[b], ((jt >> 1) & 1u) ^ 1u, status);
+          ok = mbar_wait_warp(&p_full[ps], (jt / kAPStages) & 1u, status);
+          if (ok) ok = mbar_wait_warp(&acc_empty[b], ((jt >> 1) & 1u) ^ 1u, status);
           if (!ok) break;
           tc_fence_after_sync();
           const uint32_t pbase = smem_u32(sP + ps * PSB);
@@ -424,12 +425,14 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
               const uint32_t acc = (kb > 0 || k16 > 0) ? 1u : 0u;
               const uint64_t bd = smem_desc_k128(pbase + kb * 8192 + k16 * 32);
               const uint32_t acol = (uint32_t)(kb * 4 + k16) * 8;
-              if (DO_E) mma_bf16_ts(d1, tmem + acol, bd, idesc, acc);
-              if (DO_W) mma_bf16_ts(d2, tmem + A2COL + acol, bd, idesc, acc);
+              if (DO_E) mma_bf16_ts(d1, tmem + acol, bd, idesc, acc, one);
+              if (DO_W) mma_bf16_ts(d2, tmem + A2COL + acol, bd, idesc, acc, one);
             }
           }
-          mma_commit(&p_empty[ps]);
-          mma_commit(&acc_full[b]);
+          if (one) {
+            mma_commit(&p_empty[ps]);
+            mma_commit(&acc_full[b]);
+          }
         }
       }
     }
@@ -731,7 +734,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
   // warps of both CTAs; empty_bar and acc_full are signalled in both CTAs by that thread's commits
   __shared__ uint64_t full_bar[kSMaxStages], xform_bar[kSMaxStages], empty_bar[kSMaxStages], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const uint32_t rank = cluster_rank();
   const long long tile_first = blockIdx.x >> 1, tile_step = gridDim.x >> 1;  // tiles of 256 rows, one per pair
 
@@ -787,7 +790,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
+      const uint32_t one = elect_one();
       uint32_t it = 0, si = 0;
       bool ok = true;
       // the barriers the commits arrive on, in this CTA and in the other (8 bytes apart within an array)
@@ -801,23 +805,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
         const uint32_t majors = kIdescBMajorMN | (a_mn ? kIdescAMajorMN : 0u);
         const uint32_t idesc = idesc_bf16_f32(256, n_lo) | majors, idesc_hi = idesc_bf16_f32(256, n_hi ? n_hi : 16u) | majors;
         const uint32_t buf = BIG ? 0u : (si & 1u);
-        ok = mbar_wait(&acc_empty[buf], ((BIG ? si : (si >> 1)) & 1u) ^ 1u, status);
+        ok = mbar_wait_warp(&acc_empty[buf], ((BIG ? si : (si >> 1)) & 1u) ^ 1u, status);
         if (!ok) break;
         for (int kb = 0; kb < nkb; ++kb, ++it) {
           const int s = it % ST;
-          ok = mbar_wait(&xform_bar[s], (it / ST) & 1u, status);
+          ok = mbar_wait_warp(&xform_bar[s], (it / ST) & 1u, status);
           if (!ok) break;
           tc_fence_after_sync();
           const uint32_t sA = smem_u32(smem + s * SB), sB = sA + BOFF;
 #pragma unroll
           for (int k16 = 0; k16 < 4; ++k16) {
             const uint64_t ad = a_mn ? smem_desc_mn128(sA + k16 * 2048) : smem_desc_k128(sA + k16 * 32);
-            mma_bf16_pair(tmem + buf * 256, ad, smem_desc_mn128(sB + k16 * 2048), idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
-            if (BIG && n_hi) mma_bf16_pair(tmem + 256, ad, smem_desc_mn128(sB + 2 * 8192 + k16 * 2048), idesc_hi, (kb > 0 || k16 > 0) ? 1u : 0u);
+            mma_bf16_pair(tmem + buf * 256, ad, smem_desc_mn128(sB + k16 * 2048), idesc, (kb > 0 || k16 > 0) ? 1u : 0u, one);
+            if (BIG && n_hi) mma_bf16_pair(tmem + 256, ad, smem_desc_mn128(sB + 2 * 8192 + k16 * 2048), idesc_hi, (kb > 0 || k16 > 0) ? 1u : 0u, one);
           }
-          mma_commit_pair(eb0 + 8u * s); mma_commit_pair(eb1 + 8u * s);
+          if (one) { mma_commit_pair(eb0 + 8u * s); mma_commit_pair(eb1 + 8u * s); }
         }
-        if (ok) { mma_commit_pair(af0 + 8u * buf); mma_commit_pair(af1 + 8u * buf); }
+        if (ok && one) { mma_commit_pair(af0 + 8u * buf); mma_commit_pair(af1 + 8u * buf); }
       }
     }
   } else if (warp < 6) {

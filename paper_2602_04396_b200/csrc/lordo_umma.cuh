@@ -54,6 +54,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsign
   return true;
 }
 
+// The MMA warp's loop runs in all 32 lanes with one elected for the instructions themselves: what every lane agrees on (stage,
+// addresses, descriptors) then stays in uniform registers, which is where tcgen05.mma takes them from. In a loop of
+// one lane each of them has to be carried over for every instruction, which made the issue the longest chain of several
+// kernels: update of 4096 x 11008, r = 512, K = 4 592 -> 450 us, of 14 layers of 2048 (r = 256, K = 8) 1468 -> 1419 us, projection of
+// 7 matrices of 768 92 -> 82 us, of five ragged ones 49 -> 42 us.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, unsigned* timed_out) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, timed_out));
+}
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t one;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(one));
+  return one;
+}
+
 // Generic-proxy writes to shared memory (st.shared) become visible to the tensor core / bulk-copy
 // engine (async proxy) only after this fence, executed by the writing thread before it signals.
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -94,10 +108,10 @@ __device__ __forceinline__ uint32_t idesc_bf16_f32(uint32_t M, uint32_t N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T for one 16-deep k-step; issued by a single thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
-               "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+// D[tmem] (+)= A[smem] * B[smem]^T for one 16-deep k-step; issued by a single thread: the one whose `one` is set.
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate, uint32_t one = 1u) {
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+               "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(one)
                : "memory");
 }
 // Arrives on `bar` once every MMA issued so far by this thread has completed.
@@ -135,9 +149,9 @@ constexpr uint32_t kIdescAMajorMN = 1u << 15;
 
 // Same MMA with the A operand in tensor memory: lane = row, two bf16 k-elements per 32-bit column,
 // 8 columns per 16-deep k-step.
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d_tmem),
-               "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate, uint32_t one) {
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d_tmem),
+               "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(one)
                : "memory");
 }
 // 8 consecutive 32-bit columns of this thread's lane.
@@ -246,9 +260,9 @@ __device__ __forceinline__ void tmem_free_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 // Both operands in shared memory: 128 rows of A and N/2 rows (or columns, MN-major) of B per CTA, M = 256.
-__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
-               "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+__device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate, uint32_t one) {
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+               "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(one)
                : "memory");
 }
 // Arrives on one barrier (of either CTA) once every MMA issued so far by this thread has completed.
