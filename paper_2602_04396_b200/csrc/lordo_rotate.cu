@@ -100,7 +100,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const long long first = blockIdx.x >> 1, step = gridDim.x >> 1;
   if (warp == 0) {
     // ---------------- TMA producer: planes of Rot^T and of its square -----------------------------
-    if (lane == 0) {
+    {
+      const uint32_t one = elect_one();
       uint32_t it = 0;
       bool ok = true;
       for (long long item = first; item < items && ok; item += step) {
@@ -111,14 +112,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int nbox = (cols + 63) / 64, nkb = (pr->r + kRows - 1) / kRows;
         for (int kb = 0; kb < nkb; ++kb, ++it) {
           const int s = it % kStages;
-          ok = mbar_wait(&empty_bar[s], ((it / kStages) & 1u) ^ 1u, status);
+          ok = mbar_wait_warp(&empty_bar[s], ((it / kStages) & 1u) ^ 1u, status);
           if (!ok) break;
           unsigned char* base = smem + s * kStage + 4 * kPlaneA;
-          mbar_expect_tx(&full_b[s], 4u * (uint32_t)nbox * 4096u);
+          mbar_expect_tx(&full_b[s], 4u * (uint32_t)nbox * 4096u, one);
           for (int p = 0; p < 4; ++p)  // Rot^T hi, lo, square hi, lo
             for (int x = 0; x < nbox; ++x)
               tma_load_3d(base + p * kPlaneB + x * 4096, p < 2 ? pr->map_rt : pr->map_sq, c0 + x * 64, kb * kRows, (p & 1) * pr->nb + pr->b,
-                          &full_b[s]);
+                          &full_b[s], one);
         }
       }
     }

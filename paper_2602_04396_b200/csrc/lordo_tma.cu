@@ -104,7 +104,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
 
   if (warp == 0) {
     // ---------------- TMA producer ------------------------------------------------------------
-    if (lane == 0) {
+    {
+      const uint32_t one = elect_one();
       uint32_t it = 0;
       bool ok = true;
       for (int e = seg_begin; e < seg_end && ok; ++e) {
@@ -120,22 +121,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
         const uint32_t tx = 16384u + (ef ? 16384u : 0u) + (uint32_t)pt_rows * 128u;
         for (int kb = 0; kb < nkb; ++kb, ++it) {
           const int s = it % ST;
-          ok = mbar_wait(&empty_bar[s], ((it / ST) & 1u) ^ 1u, status);
+          ok = mbar_wait_warp(&empty_bar[s], ((it / ST) & 1u) ^ 1u, status);
           if (!ok) break;
           unsigned char* base = smem + s * SB;
-          mbar_expect_tx(&full_bar[s], tx);
+          mbar_expect_tx(&full_bar[s], tx, one);
           if (pr->tr) {  // stored transposed: the strip's 128 elements are stored rows, the k-block 64 stored columns
-            tma_load_3d(base, gm->g_kb, kb * 64, n0, rep, &full_bar[s]);
-            if (ef) tma_load_3d(base + 16384, mm->e_kb, kb * 64, n0, rep, &full_bar[s]);
+            tma_load_3d(base, gm->g_kb, kb * 64, n0, rep, &full_bar[s], one);
+            if (ef) tma_load_3d(base + 16384, mm->e_kb, kb * 64, n0, rep, &full_bar[s], one);
           } else {
-            tma_load_3d(base, gm->g_sw, n0, kb * 64, rep, &full_bar[s]);
-            tma_load_3d(base + 8192, gm->g_sw, n0 + 64, kb * 64, rep, &full_bar[s]);
+            tma_load_3d(base, gm->g_sw, n0, kb * 64, rep, &full_bar[s], one);
+            tma_load_3d(base + 8192, gm->g_sw, n0 + 64, kb * 64, rep, &full_bar[s], one);
             if (ef) {
-              tma_load_3d(base + 16384, mm->e_sw, n0, kb * 64, rep, &full_bar[s]);
-              tma_load_3d(base + 24576, mm->e_sw, n0 + 64, kb * 64, rep, &full_bar[s]);
+              tma_load_3d(base + 16384, mm->e_sw, n0, kb * 64, rep, &full_bar[s], one);
+              tma_load_3d(base + 24576, mm->e_sw, n0 + 64, kb * 64, rep, &full_bar[s], one);
             }
           }
-          tma_load_3d(base + 32768, mm->pt, kb * 64, pt_row0, pc, &full_bar[s]);  // rows past r_n arrive as zeros
+          tma_load_3d(base + 32768, mm->pt, kb * 64, pt_row0, pc, &full_bar[s], one);  // rows past r_n arrive as zeros
         }
       }
     }
@@ -348,7 +349,8 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
 
   if (warp == 0) {
     // ---------------- TMA producer: tiles of G, E, W ---------------------------------------------
-    if (lane == 0) {
+    {
+      const uint32_t one = elect_one();
       uint32_t jt = 0;
       bool ok = true;
       for (int e = seg_begin; e < seg_end && ok; ++e) {
@@ -360,20 +362,20 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
         const int rep = pr->replica;
         for (int t = sg.t0; t < sg.t1; ++t, ++jt) {
           const int is = jt % INST;
-          ok = mbar_wait(&in_free[is], ((jt / INST) & 1u) ^ 1u, status);
+          ok = mbar_wait_warp(&in_free[is], ((jt / INST) & 1u) ^ 1u, status);
           if (!ok) break;
           unsigned char* base = sIn + is * ISB;
           const bool ld_e = DO_E && ef;
-          mbar_expect_tx(&in_full[is], 16384u + (ld_e ? 16384u : 0u) + (DO_W ? 16384u : 0u));
+          mbar_expect_tx(&in_full[is], 16384u + (ld_e ? 16384u : 0u) + (DO_W ? 16384u : 0u), one);
           if (SIDE == 1 || (SIDE == 2 && pr->tr)) {  // one box of 128 stored rows x 64 stored columns per tile
-            tma_load_3d(base, gm->g_kb, t * kARows, n0, rep, &in_full[is]);
-            if (ld_e) tma_load_3d(base + EOFF, mm->e_kb, t * kARows, n0, rep, &in_full[is]);
-            if (DO_W) tma_load_3d(base + WOFF, mm->w_kb, t * kARows, n0, rep, &in_full[is]);
+            tma_load_3d(base, gm->g_kb, t * kARows, n0, rep, &in_full[is], one);
+            if (ld_e) tma_load_3d(base + EOFF, mm->e_kb, t * kARows, n0, rep, &in_full[is], one);
+            if (DO_W) tma_load_3d(base + WOFF, mm->w_kb, t * kARows, n0, rep, &in_full[is], one);
           } else {
             for (int hh = 0; hh < 2; ++hh) {  // two 64-column halves per tile, 8 KB each
-              tma_load_3d(base + hh * 8192, gm->g_sw, n0 + hh * 64, t * kARows, rep, &in_full[is]);
-              if (ld_e) tma_load_3d(base + EOFF + hh * 8192, mm->e_sw, n0 + hh * 64, t * kARows, rep, &in_full[is]);
-              if (DO_W) tma_load_3d(base + WOFF + hh * 8192, mm->w_sw, n0 + hh * 64, t * kARows, rep, &in_full[is]);
+              tma_load_3d(base + hh * 8192, gm->g_sw, n0 + hh * 64, t * kARows, rep, &in_full[is], one);
+              if (ld_e) tma_load_3d(base + EOFF + hh * 8192, mm->e_sw, n0 + hh * 64, t * kARows, rep, &in_full[is], one);
+              if (DO_W) tma_load_3d(base + WOFF + hh * 8192, mm->w_sw, n0 + hh * 64, t * kARows, rep, &in_full[is], one);
             }
           }
         }
@@ -381,7 +383,8 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
     }
   } else if (warp == 2 + kAEpiWarps) {
     // ---------------- TMA producer: rows of P ---------------------------------------------------
-    if (lane == 0) {
+    {
+      const uint32_t one = elect_one();
       uint32_t jt = 0;
       bool ok = true;
       for (int e = seg_begin; e < seg_end && ok; ++e) {
@@ -391,10 +394,10 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
         const int nkb = pr->r_k / 64, pc = pr->pcopy;
         for (int t = sg.t0; t < sg.t1; ++t, ++jt) {
           const int ps = jt % kAPStages;
-          ok = mbar_wait(&p_empty[ps], ((jt / kAPStages) & 1u) ^ 1u, status);
+          ok = mbar_wait_warp(&p_empty[ps], ((jt / kAPStages) & 1u) ^ 1u, status);
           if (!ok) break;
-          mbar_expect_tx(&p_full[ps], (uint32_t)nkb * 8192u);
-          for (int kb = 0; kb < nkb; ++kb) tma_load_3d(sP + ps * PSB + kb * 8192, mm->p16, kb * 64, t * kARows, pc, &p_full[ps]);
+          mbar_expect_tx(&p_full[ps], (uint32_t)nkb * 8192u, one);
+          for (int kb = 0; kb < nkb; ++kb) tma_load_3d(sP + ps * PSB + kb * 8192, mm->p16, kb * 64, t * kARows, pc, &p_full[ps], one);
         }
       }
     }
@@ -751,7 +754,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
   dep_begin();
 
   if (warp == 0) {
-    if (lane == 0) {
+    {
+      const uint32_t one = elect_one();
       uint32_t it = 0;
       bool ok = true;
       for (long long tile = tile_first; tile < total_tiles && ok; tile += tile_step) {
@@ -769,23 +773,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
           if (kb == nkb1) { kb = 0; ++seg; }
           const int a_c2 = pr->a_c2 + (int)((pr->pa >> (4 * seg)) & 15u) * pr->a_pl, b_c2 = pr->b_c2 + (int)((pr->pb >> (4 * seg)) & 15u) * pr->b_pl;
           const int s = it % ST;
-          ok = mbar_wait(&empty_bar[s], ((it / ST) & 1u) ^ 1u, status);
+          ok = mbar_wait_warp(&empty_bar[s], ((it / ST) & 1u) ^ 1u, status);
           if (!ok) break;
           unsigned char* base = smem + s * SB;
-          mbar_expect_tx(&full_bar[s], tx);
+          mbar_expect_tx(&full_bar[s], tx, one);
           if (pr->a_mn) {  // S stored [Kd][M]: two boxes of 64 k-rows x 64 columns
-            tma_load_3d(base, pr->map_a, m0, kb * 64, a_c2, &full_bar[s]);
-            tma_load_3d(base + 8192, pr->map_a, m0 + 64, kb * 64, a_c2, &full_bar[s]);
+            tma_load_3d(base, pr->map_a, m0, kb * 64, a_c2, &full_bar[s], one);
+            tma_load_3d(base + 8192, pr->map_a, m0 + 64, kb * 64, a_c2, &full_bar[s], one);
             if (WITH_E) {
-              tma_load_3d(base + 16384, pr->map_e, m0, kb * 64, a_c2, &full_bar[s]);
-              tma_load_3d(base + 24576, pr->map_e, m0 + 64, kb * 64, a_c2, &full_bar[s]);
+              tma_load_3d(base + 16384, pr->map_e, m0, kb * 64, a_c2, &full_bar[s], one);
+              tma_load_3d(base + 24576, pr->map_e, m0 + 64, kb * 64, a_c2, &full_bar[s], one);
             }
           } else {         // S stored [M][Kd]: one box of 128 rows x 64 k
-            tma_load_3d(base, pr->map_a, kb * 64, m0, a_c2, &full_bar[s]);
-            if (WITH_E) tma_load_3d(base + 16384, pr->map_e, kb * 64, m0, a_c2, &full_bar[s]);
+            tma_load_3d(base, pr->map_a, kb * 64, m0, a_c2, &full_bar[s], one);
+            if (WITH_E) tma_load_3d(base + 16384, pr->map_e, kb * 64, m0, a_c2, &full_bar[s], one);
           }
-          for (int x = 0; x < nbox_lo; ++x) tma_load_3d(base + BOFF + x * 8192, pr->map_b, c_lo + x * 64, kb * 64, b_c2, &full_bar[s]);
-          for (int x = 0; x < nbox_hi; ++x) tma_load_3d(base + BOFF + 16384 + x * 8192, pr->map_b, c_hi + x * 64, kb * 64, b_c2, &full_bar[s]);
+          for (int x = 0; x < nbox_lo; ++x) tma_load_3d(base + BOFF + x * 8192, pr->map_b, c_lo + x * 64, kb * 64, b_c2, &full_bar[s], one);
+          for (int x = 0; x < nbox_hi; ++x) tma_load_3d(base + BOFF + 16384 + x * 8192, pr->map_b, c_hi + x * 64, kb * 64, b_c2, &full_bar[s], one);
         }
       }
     }

@@ -164,13 +164,15 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 
 // TMA: 3-d tiled load into shared memory completing on an mbarrier, 3-d tiled store from shared
 // memory in a bulk group. Every load goes to the issuing CTA's shared memory alone. `map` is a 128-byte tensor map in global memory.
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+// `one`: whether this thread is the one that does it (see elect_one).
+__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes, uint32_t one) {
+  asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(smem_u32(bar)), "r"(bytes), "r"(one) : "memory");
 }
-__device__ __forceinline__ void tma_load_3d(void* smem_dst, const void* map, int c0, int c1, int c2, uint64_t* bar) {
-  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+__device__ __forceinline__ void tma_load_3d(void* smem_dst, const void* map, int c0, int c1, int c2, uint64_t* bar, uint32_t one) {
+  asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n"
+               "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n}" ::"r"(
                    smem_u32(smem_dst)),
-               "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
+               "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar)), "r"(one)
                : "memory");
 }
 __device__ __forceinline__ void tma_store_3d(const void* map, int c0, int c1, int c2, const void* smem_src) {
