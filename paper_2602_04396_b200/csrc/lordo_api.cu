@@ -791,6 +791,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
             const bool to_planes = pass == 0, to_rhs = pass == 1 && !last;
             sk_split(ap, 0, x_kb, b, nb, mmi->rinv_sw, b, nb, rows, r, to_planes || to_rhs ? nullptr : O + b * so, r, 3);
             SkProblem& sp = ap.sk.back();
+            sp.tri = 1;
             if (to_planes) { sp.C16 = x16 + (size_t)b * rows * r; sp.plane = (long long)nb * rows * r; sp.planes = 3; }
             if (to_rhs) { sp.C16 = O16 + (size_t)b * rows * r; sp.planes = 1; }
           }

@@ -322,7 +322,8 @@ struct SkProblem {
   long long plane;
   int planes;
   // with map_e: where c G + E is kept in bf16, as stored [S_rows][S_cols], for the products that follow; or null
-  int S_rows, S_cols, pad2;
+  int S_rows, S_cols;
+  int tri;                   // B is upper triangular (used above r = 256)
   __nv_bfloat16* S16;
 };
 // with_e: map_e and cptr are set in every problem of the launch, else in none

@@ -722,6 +722,24 @@ __device__ __forceinline__ int find_sk(const SkProblem* __restrict__ probs, int 
 }
 }  // namespace
 
+namespace {
+// Columns of B that take part in the 64-deep step kb: of the first n_lo all but skip_lo, of the other n_hi all but skip_hi. With
+// an upper triangular B (R^-1) the columns below 64 kb are zero there and cost neither loads nor MMAs; the first step of a
+// pair of planes has them all, so it may overwrite the accumulator. r = 512, 16 workers: 11008 rows 385 -> 301 us, 4096 rows
+// 160 -> 125 us. For r <= 256 the table's word is not looked at: widths that change from step to step cost every launch a
+// microsecond, and at r = 128 the products with R^-1 gain nothing (41.5 -> 42.7 us; r = 256 26.0 -> 24.3 us).
+struct SkCols {
+  int lo, hi, skip_lo, skip_hi;
+  __device__ __forceinline__ SkCols(int n_lo, int n_hi, int tri, int kb) {
+    const int skip = tri ? kb * 64 : 0;
+    skip_lo = skip < n_lo ? skip : n_lo;
+    skip_hi = skip > 256 ? skip - 256 : 0;
+    lo = n_lo - skip_lo;
+    hi = n_hi - skip_hi;
+  }
+};
+}  // namespace
+
 // BIG: ranks above 256. WITH_E: the problems' A is c G + E, formed from two tiles; without, the stage is a third or a
 // quarter smaller and the pipeline one or two stages deeper.
 template <bool BIG, bool WITH_E>
@@ -764,19 +782,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
         const int nkb1 = (pr->Kd + 63) / 64;
         // this CTA's columns of B: half of the first 256 (one MMA) and half of the rest (a second MMA)
         const int n_lo = pr->r_n < 256 ? pr->r_n : 256, n_hi = pr->r_n - n_lo;
-        const int c_lo = (int)rank * (n_lo / 2), c_hi = 256 + (int)rank * (n_hi / 2);
-        const int nbox_lo = (n_lo / 2 + 63) / 64, nbox_hi = (n_hi / 2 + 63) / 64;
-        const uint32_t tx = 16384u + (WITH_E ? 16384u : 0u) + (uint32_t)(nbox_lo + nbox_hi) * 8192u;
-        const int j1 = pr->j1;
+        const int j1 = pr->j1, tri = BIG ? pr->tri : 0;
         int seg = pr->j0 / nkb1, kb = pr->j0 - seg * nkb1;
         for (int j = pr->j0; j < j1; ++j, ++it, ++kb) {
           if (kb == nkb1) { kb = 0; ++seg; }
           const int a_c2 = pr->a_c2 + (int)((pr->pa >> (4 * seg)) & 15u) * pr->a_pl, b_c2 = pr->b_c2 + (int)((pr->pb >> (4 * seg)) & 15u) * pr->b_pl;
           const int s = it % ST;
+          const SkCols cols(n_lo, n_hi, tri, kb);
+          const int c_lo = cols.skip_lo + (int)rank * (cols.lo / 2), c_hi = 256 + cols.skip_hi + (int)rank * (cols.hi / 2);
+          const int nbox_lo = (cols.lo / 2 + 63) / 64, nbox_hi = (cols.hi / 2 + 63) / 64;
           ok = mbar_wait_warp(&empty_bar[s], ((it / ST) & 1u) ^ 1u, status);
           if (!ok) break;
           unsigned char* base = smem + s * SB;
-          mbar_expect_tx(&full_bar[s], tx, one);
+          mbar_expect_tx(&full_bar[s], 16384u + (WITH_E ? 16384u : 0u) + (uint32_t)(nbox_lo + nbox_hi) * 8192u, one);
           if (pr->a_mn) {  // S stored [Kd][M]: two boxes of 64 k-rows x 64 columns
             tma_load_3d(base, pr->map_a, m0, kb * 64, a_c2, &full_bar[s], one);
             tma_load_3d(base + 8192, pr->map_a, m0 + 64, kb * 64, a_c2, &full_bar[s], one);
@@ -805,14 +823,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
         const SkProblem* __restrict__ pr = probs + find_sk(probs, nprobs, tile);
         const int nkb = pr->j1 - pr->j0;
         const bool a_mn = pr->a_mn != 0;
-        const uint32_t n_lo = pr->r_n < 256 ? (uint32_t)pr->r_n : 256u, n_hi = (uint32_t)pr->r_n - n_lo;
+        const int n_lo = pr->r_n < 256 ? pr->r_n : 256, n_hi = pr->r_n - n_lo, tri = BIG ? pr->tri : 0, nkb1 = (pr->Kd + 63) / 64;
         const uint32_t majors = kIdescBMajorMN | (a_mn ? kIdescAMajorMN : 0u);
-        const uint32_t idesc = idesc_bf16_f32(256, n_lo) | majors, idesc_hi = idesc_bf16_f32(256, n_hi ? n_hi : 16u) | majors;
+        int kk = pr->j0 % nkb1;  // 64-deep step within a pair of planes
         const uint32_t buf = BIG ? 0u : (si & 1u);
         ok = mbar_wait_warp(&acc_empty[buf], ((BIG ? si : (si >> 1)) & 1u) ^ 1u, status);
         if (!ok) break;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        for (int kb = 0; kb < nkb; ++kb, ++it, ++kk) {
+          if (kk == nkb1) kk = 0;
           const int s = it % ST;
+          const SkCols cols(n_lo, n_hi, tri, kk);
+          const uint32_t idesc = idesc_bf16_f32(256, cols.lo ? (uint32_t)cols.lo : 16u) | majors, idesc_hi = idesc_bf16_f32(256, cols.hi ? (uint32_t)cols.hi : 16u) | majors;
           ok = mbar_wait_warp(&xform_bar[s], (it / ST) & 1u, status);
           if (!ok) break;
           tc_fence_after_sync();
@@ -820,8 +841,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSThreads, 1)
 #pragma unroll
           for (int k16 = 0; k16 < 4; ++k16) {
             const uint64_t ad = a_mn ? smem_desc_mn128(sA + k16 * 2048) : smem_desc_k128(sA + k16 * 32);
-            mma_bf16_pair(tmem + buf * 256, ad, smem_desc_mn128(sB + k16 * 2048), idesc, (kb > 0 || k16 > 0) ? 1u : 0u, one);
-            if (BIG && n_hi) mma_bf16_pair(tmem + 256, ad, smem_desc_mn128(sB + 2 * 8192 + k16 * 2048), idesc_hi, (kb > 0 || k16 > 0) ? 1u : 0u, one);
+            if (!BIG || cols.lo) mma_bf16_pair(tmem + buf * 256 + cols.skip_lo, ad, smem_desc_mn128(sB + k16 * 2048), idesc, (kb > 0 || k16 > 0) ? 1u : 0u, one);
+            if (BIG && cols.hi) mma_bf16_pair(tmem + 256 + cols.skip_hi, ad, smem_desc_mn128(sB + 2 * 8192 + k16 * 2048), idesc_hi, (kb > 0 || k16 > 0) ? 1u : 0u, one);
           }
           if (one) { mma_commit_pair(eb0 + 8u * s); mma_commit_pair(eb1 + 8u * s); }
         }
