@@ -358,7 +358,6 @@ __device__ __forceinline__ void split_store4(__nv_bfloat16* dst, long long plane
 
 // Four vectors per thread in flight: 7 matrices of 2048 (51 million elements) 84 -> 40 us.
 __global__ void __launch_bounds__(256) convert_grouped_kernel(const ConvProblem* __restrict__ probs, int nprobs) {
-  dep_begin();
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
   while (lo < hi) {
@@ -366,6 +365,7 @@ __global__ void __launch_bounds__(256) convert_grouped_kernel(const ConvProblem*
     if (probs[mid].blk_start <= blk) lo = mid; else hi = mid - 1;
   }
   const ConvProblem pb = probs[lo];
+  dep_begin();  // the tables are constant
   const long long e = (blk - pb.blk_start) * 4096 + threadIdx.x * 4;
   float4 v[4];
 #pragma unroll
@@ -377,14 +377,15 @@ __global__ void __launch_bounds__(256) convert_grouped_kernel(const ConvProblem*
 }
 
 // One block per 32 x 32 block on or below the diagonal, which it also mirrors; the partial products meet in
-// fp64, so that what is left of the tensor cores' truncating accumulation is that of one range of k.
-// Bound by the reads of the partial products: r = 512, 16 matrices, 2 x 8 ranges in 21 us.
+// fp64, so that what is left of the tensor cores' truncating accumulation is that of one range of k. The mirrored
+// block of T is summed as it lies and turned over once, in fp64, so the ranges' loads wait for nothing.
+// Bound by the reads of the partial products: 56 matrices of r = 128 14.5 -> 10.5 us, 7 of r = 256 20 -> 12.6 us, six launches
+// over 16 matrices of r = 512 283 -> 246 us, against two barriers a range
 __global__ void __launch_bounds__(256) gram_sum_kernel(const GramProblem* __restrict__ probs, int nprobs) {
-  dep_begin();
-  __shared__ float tt[32][33];
+  __shared__ double tt[32][33];
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
-  while (lo < hi) {
+  while (lo < hi) {  // the tables are constant
     const int mid = (lo + hi + 1) >> 1;
     if (probs[mid].blk_start <= blk) lo = mid; else hi = mid - 1;
   }
@@ -395,40 +396,48 @@ __global__ void __launch_bounds__(256) gram_sum_kernel(const GramProblem* __rest
   while (rest > bi) rest -= ++bi;  // block row bi has bi + 1 blocks
   const int bj = rest;
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  double acc[4] = {0.0, 0.0, 0.0, 0.0}, mir[4] = {0.0, 0.0, 0.0, 0.0};
+  size_t at[4], am[4];  // elements outside the matrix: its first one, summed and not used
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = bi * 32 + y + 8 * q, j = bj * 32 + x, i2 = bj * 32 + y + 8 * q, j2 = bi * 32 + x;
+    at[q] = i < r && j < r ? (size_t)i * r + j : 0;
+    am[q] = i2 < r && j2 < r ? (size_t)i2 * r + j2 : 0;
+  }
+  dep_begin();
+#pragma unroll 2
   for (int s = 0; s < pb.ns; ++s) {
     const float* S = pb.part + s * rr;
     const float* T = pb.part + (pb.ns + s) * rr;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int i = bj * 32 + y + 8 * q, j = bi * 32 + x;  // the mirrored block of T
-      tt[y + 8 * q][x] = (i < r && j < r) ? T[(size_t)i * r + j] : 0.f;
+      acc[q] += (double)S[at[q]] + (double)T[at[q]];
+      mir[q] += (double)T[am[q]];
     }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = bi * 32 + y + 8 * q, j = bj * 32 + x;
-      if (i < r && j < r) acc[q] += (double)S[(size_t)i * r + j] + ((double)T[(size_t)i * r + j] + (double)tt[x][y + 8 * q]);
-    }
-    __syncthreads();
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) tt[y + 8 * q][x] = mir[q];
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) acc[q] += tt[x][y + 8 * q];
+  __syncthreads();
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = bi * 32 + y + 8 * q, j = bj * 32 + x;
-    tt[y + 8 * q][x] = (float)acc[q];
+    tt[y + 8 * q][x] = acc[q];
     if (i < r && j < r && (bi != bj || j <= i)) pb.gram[(size_t)i * r + j] = (float)acc[q];
   }
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = bj * 32 + y + 8 * q, j = bi * 32 + x;
-    if (i < r && j < r && (bi != bj || j > i)) pb.gram[(size_t)i * r + j] = tt[x][y + 8 * q];
+    if (i < r && j < r && (bi != bj || j > i)) pb.gram[(size_t)i * r + j] = (float)tt[x][y + 8 * q];
   }
 }
 
-// One block per 32 x 32 block of Rot, whose transpose it writes.
+// One block per 32 x 32 block of Rot, whose transpose it writes. Sixteen loads of a thread are in
+// flight: 7 matrices of r = 256 22.7 us with one row after the other, now 12.7.
 __global__ void __launch_bounds__(256) rot_sum_kernel(const RotProblem* __restrict__ probs, int nprobs) {
-  dep_begin();
   __shared__ float tt[32][33];
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
@@ -440,15 +449,23 @@ __global__ void __launch_bounds__(256) rot_sum_kernel(const RotProblem* __restri
   const int r = pb.r, nb = (r + 31) / 32;
   const int bi = (int)(blk - pb.blk_start) / nb, bj = (int)(blk - pb.blk_start) - bi * nb;
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  size_t at[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = bi * 32 + y + 8 * q, j = bj * 32 + x;
-    if (i < r && j < r) {
-      double a = 0.0;
-      for (int s = 0; s < pb.ns; ++s) a += (double)pb.part[(size_t)s * r * r + (size_t)i * r + j];
-      pb.rot[(size_t)i * r + j] = (float)a;
-      tt[y + 8 * q][x] = (float)a;
-    }
+    at[q] = i < r && j < r ? (size_t)i * r + j : 0;
+  }
+  dep_begin();
+#pragma unroll 4
+  for (int s = 0; s < pb.ns; ++s) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] += (double)pb.part[(size_t)s * r * r + at[q]];
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (bi * 32 + y + 8 * q < r && bj * 32 + x < r) pb.rot[at[q]] = (float)a[q];
+    tt[y + 8 * q][x] = (float)a[q];
   }
   __syncthreads();
   for (int e = threadIdx.x; e < 256; e += 256) {  // four neighbouring elements of a row of Rot^T per thread
@@ -466,7 +483,6 @@ __global__ void __launch_bounds__(256) rot_sum_kernel(const RotProblem* __restri
 // Sums of squares of 128 columns over kNormRows rows, in fp64. One block per 32 columns over all rows took 346 us
 // for 7 matrices of up to 5632 x 256 (and 400 us for 16 of 4096 x 512).
 __global__ void __launch_bounds__(256) colsq_kernel(const BasisProblem* __restrict__ probs, int nprobs) {
-  dep_begin();
   __shared__ double red[8][128];
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
@@ -476,6 +492,7 @@ __global__ void __launch_bounds__(256) colsq_kernel(const BasisProblem* __restri
   }
   const BasisProblem pb = probs[lo];
   const int nc = (pb.r + 127) / 128;
+  dep_begin();  // the tables are constant
   const long long chunk = (blk - pb.sq_start) / nc;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c0 = (int)(blk - pb.sq_start - chunk * nc) * 128;
   const int col = c0 + 4 * lane;
@@ -564,7 +581,6 @@ __global__ void __launch_bounds__(256) commit_basis_kernel(const BasisProblem* _
 
 // Device-to-device copies of many buffers in one launch (16-byte chunks).
 __global__ void __launch_bounds__(256) copy_grouped_kernel(const CopyProblem* __restrict__ probs, int nprobs) {
-  dep_begin();
   const long long blk = blockIdx.x;
   int lo = 0, hi = nprobs - 1;
   while (lo < hi) {
@@ -572,6 +588,7 @@ __global__ void __launch_bounds__(256) copy_grouped_kernel(const CopyProblem* __
     if (probs[mid].blk_start <= blk) lo = mid; else hi = mid - 1;
   }
   const CopyProblem pb = probs[lo];
+  dep_begin();  // the tables are constant
   const long long c = ((blk - pb.blk_start) * 256 + threadIdx.x) * 4;
   const uint4* __restrict__ src = reinterpret_cast<const uint4*>(pb.src);
   uint4* __restrict__ dst = reinterpret_cast<uint4*>(pb.dst);
