@@ -17,8 +17,10 @@
 // and per panel one trip to L2 for the newest columns, the small products and the barrier; for few CTAs per matrix
 // the fp64 products. One CTA per matrix with a thread per row took 2200 us for r = 512 and 16 matrices, 580 us
 // for r = 256 and 7, 197 us for r = 128 and 56; clusters that summed a whole panel at its turn 654, 131 and 62 us;
-// this one 325, 86 and 46 us. (Scaling the block so that rsqrt.approx needs no care, and handing the factoring warp
-// its block summed, both made the column chain slower: 98 us at r = 256.)
+// clusters that sum a panel ahead
+// 360, 99 and 56 us (first launch of a stream), with the next diagonal block staged by the inverting warp and the pivots worked
+// out by every lane 359, 90 and 53 us. (Scaling the block so that rsqrt.approx needs no care, and handing the factoring
+// warp its block summed, both made the column chain slower.)
 #include "lordo_kernels.h"
 
 namespace lordo {
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
   double* dinv = Lc + kB * kB;                       // [kB] 1 / its diagonal
   double* Li = dinv + kB;                            // [kB][kLd] inverse of the diagonal block
   __shared__ float wmax[kCholWarps];
-  __shared__ float ga[kB * kB];                      // the Gram matrix' diagonal block of the coming panel, for warp 0
+  __shared__ float ga[2 * kB * kB];                  // the Gram matrix' diagonal blocks of this panel and the next, for warp 0
 
   const uint32_t rank = cluster_ctarank(), csize = cluster_nctarank();
   const CholProblem pb = probs[blockIdx.x / csize];
@@ -190,7 +192,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
 #pragma unroll
     for (int j = 0; j < kB; ++j) t[j] = a_diag(k, j);
 #pragma unroll
-    for (int j = 0; j < kB; ++j) ga[j * kB + lane] = t[j];
+    for (int j = 0; j < kB; ++j) ga[((k & 1) * kB + j) * kB + lane] = t[j];
   };
   if (warp == 0) stage_diag(0);
 
@@ -217,44 +219,54 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
     }
 
     if (warp == 0) {
-      // Factor of the diagonal block: lane i holds row i of what is left of the block. The next pivot is kept up to
-      // date by its own lane (dg), so that the chain from column to column is a shuffle, a reciprocal square root
-      // (one Newton step in fp64 on rsqrtf's 22 bits: 44 bits) and two multiply-adds; the update of the columns
-      // behind the next one fills its gaps.
+      // Factor of the diagonal block: lane i holds row i of what is left of the block. Every lane works out every pivot d
+      // for itself, from the element b beside the pivot before it and the diagonal element D that were handed round a column
+      // earlier: D - b b / d. With r0 = 1/d to 20 bits and e = 1 - d r0 that is D - b b r0 (1 + e + e e), 60 bits, and the next
+      // column's elements are worked out likewise; the square root, the column of L and the update of the columns behind
+      // the next one fill the gaps. (No chain is what is left: a column is some 70 instructions of one warp, which issues one
+      // every four clocks. Handing two elements round and updating the columns behind one column late: slower, registers.)
       asm volatile("bar.sync 1, 128;" ::: "memory");
-      double a[kB], dg = 1.0, fl = 0.0;
+      const float* gk = ga + (k & 1) * kB * kB;
+      double a[kB], dg = 1.0;
 #pragma unroll
       for (int j = 0; j < kB; ++j) {
         const double* q = dpart + j * kLd + lane;  // symmetric too
-        const float ga_j = ga[j * kB + lane];
-        a[j] = (double)ga_j - ((q[0] + q[kPartDoubles]) + (q[2 * kPartDoubles] + q[3 * kPartDoubles]));
-        if (lane == j) {
-          dg = a[j];
-          if (j < kw) fl = (double)fmaxf(kBreakdown * ga_j, abs_floor);
-        }
+        a[j] = (double)gk[j * kB + lane] - ((q[0] + q[kPartDoubles]) + (q[2 * kPartDoubles] + q[3 * kPartDoubles]));
+        if (lane == j) dg = a[j];
       }
       bool broke = false;
-      double d, y;
-      auto pivot = [&](int j) {  // every lane offers its own; !(x > y) also catches NaN
-        const bool low = !(dg > fl);
-        if (lane == j) broke |= low;
-        d = __shfl_sync(0xffffffffu, low ? fl : dg, j);
-        const double y0 = (double)rsqrtf((float)d);
-        y = fma(0.5 * y0, fma(-d * y0, y0, 1.0), y0);  // 1 / L_jj
+      auto pivot = [&](double x, int j) {  // x, or the floor where it is not above it (NaN neither)
+        const double fl = j < kw ? (double)fmaxf(kBreakdown * gk[j * kB + j], abs_floor) : 0.0;
+        const int h = __double2hiint(x);
+        const bool low = !(h > __double2hiint(fl) && h < 0x7FF00000);
+        broke |= low;
+        return low ? fl : x;
       };
-      pivot(0);
+      double d = pivot(__shfl_sync(0xffffffffu, dg, 0), 0);
+      double b = __shfl_sync(0xffffffffu, a[0], 1), D = __shfl_sync(0xffffffffu, dg, 1);
 #pragma unroll
       for (int j = 0; j < kB; ++j) {
-        const double l = lane == j ? d * y : (lane > j ? a[j] * y : 0.0);
-        dg -= l * l;
+        double r0, y0, dn = 1.0;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
+        const double e0 = fma(-d, r0, 1.0), e = fma(e0, e0, e0), aj = a[j];
+        auto minus = [&](double x, double pq) { const double p = pq * r0; return fma(-p, e, x - p); };  // x - pq / d
+        if (j + 1 < kB) {
+          dn = minus(D, b * b);
+          a[j + 1] = minus(a[j + 1], aj * b);  // rows from j on; those above are done with
+          dg = minus(dg, aj * aj);
+        }
+        if (j + 2 < kB) {
+          b = __shfl_sync(0xffffffffu, a[j + 1], j + 2);
+          D = __shfl_sync(0xffffffffu, dg, j + 2);
+        }
+        const double f = fma(-d * y0, y0, 1.0), y = fma(y0 * f, fma(0.375, f, 0.5), y0);  // 1 / L_jj, 58 bits
+        const double l = lane == j ? d * y : (lane > j ? aj * y : 0.0);
         Lc[j * kB + lane] = l;
         if (lane == 0) dinv[j] = y;
+        if (j + 1 < kB) d = pivot(dn, j + 1);
         __syncwarp();
         if (j % 8 == 7) asm volatile("bar.arrive %0, 64;" ::"r"(2 + j / 8) : "memory");  // eight more columns for the inverse
-        if (j + 1 < kB) {
-          a[j + 1] -= l * Lc[j * kB + j + 1];
-          pivot(j + 1);
-        }
 #pragma unroll
         for (int j2 = (j + 2) & ~1; j2 < kB; j2 += 2) {
           const double2 v = *reinterpret_cast<const double2*>(Lc + j * kB + j2);
@@ -262,13 +274,14 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
           a[j2 + 1] -= l * v.y;
         }
       }
-      if (broke && rank == 0) atomicOr(status, LORDO_FLAG_QR_BREAKDOWN);
+      if (broke && rank == 0 && lane == 0) atomicOr(status, LORDO_FLAG_QR_BREAKDOWN);
       clear(c);  // not held in registers meanwhile
     } else if (warp < 3) {
       asm volatile("bar.arrive 1, 128;" ::: "memory");
       if (k + 1 < nb) block_sum(c, L, k0 + kB, L, k0 + kB, r, warp - 1, k, 2);
     } else if (warp == 4) {
       asm volatile("bar.arrive 1, 128;" ::: "memory");
+      if (k + 1 < nb) stage_diag(k + 1);  // before the first columns are there
       // inverse of the diagonal block, column `lane`, eight columns of the factor behind warp 0
       double x[kB];
 #pragma unroll
@@ -367,7 +380,6 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
     }
     // the panel is in memory for every CTA of the cluster
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    if (warp == 0 && k + 1 < nb) stage_diag(k + 1);
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
 }
