@@ -19,7 +19,7 @@
 // for r = 256 and 7, 197 us for r = 128 and 56; clusters that summed a whole panel at its turn 654, 131 and 62 us;
 // clusters that sum a panel ahead
 // 360, 99 and 56 us (first launch of a stream), with the next diagonal block staged by the inverting warp and the pivots worked
-// out by every lane 359, 90 and 53 us. (Scaling the block so that rsqrt.approx needs no care, and handing the factoring
+// out by every lane 345, 88 and 53 us. (Scaling the block so that rsqrt.approx needs no care, and handing the factoring
 // warp its block summed, both made the column chain slower.)
 #include "lordo_kernels.h"
 
@@ -39,7 +39,11 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
 
 // Sums of products of rows: lane l of a warp holds rows l/4 + 8i of both 32-row blocks (rows from r on read as
 // zeros). The columns may be dealt to the lanes in any order as long as it is the same on both sides.
+// DIAG: both blocks are the same one, so its rows are fetched once and only the 8 x 8 tiles on and above the diagonal are
+// multiplied (every CTA of a cluster sums the diagonal block for itself: r = 512, 16 matrices
+// 359 -> 345 us, r = 256, 7 matrices 90 -> 88 us).
 // c += X_cols L_cols^T over 8 columns from `col` on.
+template <bool DIAG>
 __device__ __forceinline__ void block_cols(double (&c)[4][4][2], const float* X, int xr, const float* L, int lr, int r, int col) {
   const int lane = threadIdx.x & 31, row = lane >> 2, kc = col + (lane & 3) * 2;
   float2 a[4], b[4];
@@ -48,16 +52,18 @@ __device__ __forceinline__ void block_cols(double (&c)[4][4][2], const float* X,
     const int ra = xr + row + 8 * i, rb = lr + row + 8 * i;
     a[i] = b[i] = make_float2(0.f, 0.f);
     if (ra < r) a[i] = *reinterpret_cast<const float2*>(X + (size_t)ra * r + kc);
-    if (rb < r) b[i] = *reinterpret_cast<const float2*>(L + (size_t)rb * r + kc);
+    if (DIAG) b[i] = a[i];
+    else if (rb < r) b[i] = *reinterpret_cast<const float2*>(L + (size_t)rb * r + kc);
   }
 #pragma unroll
   for (int t = 0; t < 2; ++t)
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int n = 0; n < 4; ++n) dmma(c[i][n][0], c[i][n][1], (double)(t ? a[i].y : a[i].x), (double)(t ? b[n].y : b[n].x));
+      for (int n = DIAG ? i : 0; n < 4; ++n) dmma(c[i][n][0], c[i][n][1], (double)(t ? a[i].y : a[i].x), (double)(t ? b[n].y : b[n].x));
 }
 
+template <bool DIAG>
 __device__ __forceinline__ void fetch16(float4 (&a)[4], float4 (&b)[4], const float* X, int xr, const float* L, int lr, int r, int col) {
   const int lane = threadIdx.x & 31, row = lane >> 2, kc = col + (lane & 3) * 4;
 #pragma unroll
@@ -65,34 +71,39 @@ __device__ __forceinline__ void fetch16(float4 (&a)[4], float4 (&b)[4], const fl
     const int ra = xr + row + 8 * i, rb = lr + row + 8 * i;
     a[i] = b[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (ra < r) a[i] = *reinterpret_cast<const float4*>(X + (size_t)ra * r + kc);
-    if (rb < r) b[i] = *reinterpret_cast<const float4*>(L + (size_t)rb * r + kc);
+    if (!DIAG && rb < r) b[i] = *reinterpret_cast<const float4*>(L + (size_t)rb * r + kc);
   }
 }
+template <bool DIAG>
 __device__ __forceinline__ void mma16(double (&c)[4][4][2], const float4 (&a)[4], const float4 (&b)[4]) {
 #pragma unroll
   for (int t = 0; t < 4; ++t) {
     double bv[4];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) bv[n] = (double)(t == 0 ? b[n].x : t == 1 ? b[n].y : t == 2 ? b[n].z : b[n].w);
+    for (int n = 0; n < 4; ++n) {
+      const float4& v = DIAG ? a[n] : b[n];
+      bv[n] = (double)(t == 0 ? v.x : t == 1 ? v.y : t == 2 ? v.z : v.w);
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const double av = (double)(t == 0 ? a[i].x : t == 1 ? a[i].y : t == 2 ? a[i].z : a[i].w);
+      const double av = DIAG ? bv[i] : (double)(t == 0 ? a[i].x : t == 1 ? a[i].y : t == 2 ? a[i].z : a[i].w);
 #pragma unroll
-      for (int n = 0; n < 4; ++n) dmma(c[i][n][0], c[i][n][1], av, bv[n]);
+      for (int n = DIAG ? i : 0; n < 4; ++n) dmma(c[i][n][0], c[i][n][1], av, bv[n]);
     }
   }
 }
 // c += X_j L_j^T over the 32-column blocks j = j0, j0 + dj, ... < j1, 16 columns on their way while 16 are multiplied.
+template <bool DIAG>
 __device__ __forceinline__ void block_sum(double (&c)[4][4][2], const float* X, int xr, const float* L, int lr, int r, int j0, int j1, int dj) {
   if (j0 >= j1) return;
   float4 a0[4], b0[4], a1[4], b1[4];
-  fetch16(a0, b0, X, xr, L, lr, r, j0 * kB);
+  fetch16<DIAG>(a0, b0, X, xr, L, lr, r, j0 * kB);
 #pragma unroll 1
   for (int j = j0; j < j1; j += dj) {
-    fetch16(a1, b1, X, xr, L, lr, r, j * kB + 16);
-    mma16(c, a0, b0);
-    if (j + dj < j1) fetch16(a0, b0, X, xr, L, lr, r, (j + dj) * kB);
-    mma16(c, a1, b1);
+    fetch16<DIAG>(a1, b1, X, xr, L, lr, r, j * kB + 16);
+    mma16<DIAG>(c, a0, b0);
+    if (j + dj < j1) fetch16<DIAG>(a0, b0, X, xr, L, lr, r, (j + dj) * kB);
+    mma16<DIAG>(c, a1, b1);
   }
 }
 
@@ -205,15 +216,15 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
     // ---- the newest 32 columns (or, without a head start, all of them) and the sums to shared memory
     if (u == kUnits) {
       const int w = warp == 4 ? 3 : warp;
-      if (k > 0) block_cols(c, L, k0, L, k0, r, k0 - kB + w * 8);
+      if (k > 0) block_cols<true>(c, L, k0, L, k0, r, k0 - kB + w * 8);
       store_part(dpart + w * kPartDoubles, c);
       clear(c);
     } else if (u < first * slices(first)) {
       const int s = slices(first), b = tile_block(k, u / s), sl = u % s;
       const float* X = b > k ? L : Z;
-      if (!ahead) block_sum(c, X, b * kB, L, k0, r, (b > k ? 0 : b) + sl, k, s);
+      if (!ahead) block_sum<false>(c, X, b * kB, L, k0, r, (b > k ? 0 : b) + sl, k, s);
       else if (k > 0)
-        for (int h = sl; h < 4; h += s) block_cols(c, X, b * kB, L, k0, r, k0 - kB + h * 8);
+        for (int h = sl; h < 4; h += s) block_cols<false>(c, X, b * kB, L, k0, r, k0 - kB + h * 8);
       store_part(part + u * kPartDoubles, c);
       clear(c);
     }
@@ -278,7 +289,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
       clear(c);  // not held in registers meanwhile
     } else if (warp < 3) {
       asm volatile("bar.arrive 1, 128;" ::: "memory");
-      if (k + 1 < nb) block_sum(c, L, k0 + kB, L, k0 + kB, r, warp - 1, k, 2);
+      if (k + 1 < nb) block_sum<true>(c, L, k0 + kB, L, k0 + kB, r, warp - 1, k, 2);
     } else if (warp == 4) {
       asm volatile("bar.arrive 1, 128;" ::: "memory");
       if (k + 1 < nb) stage_diag(k + 1);  // before the first columns are there
@@ -303,7 +314,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
       const int n1 = tiles(k + 1), s = slices(n1);
       if (u < n1 * s) {
         const int b = tile_block(k + 1, u / s), sl = u % s;
-        block_sum(c, b > k + 1 ? L : Z, b * kB, L, k0 + kB, r, (b > k + 1 ? 0 : b) + sl, k, s);
+        block_sum<false>(c, b > k + 1 ? L : Z, b * kB, L, k0 + kB, r, (b > k + 1 ? 0 : b) + sl, k, s);
       }
     }
 
@@ -323,7 +334,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
         __syncthreads();  // the batch before is done with its sums
         if (u < cnt * s) {
           const int b = tile_block(k, base + u / s);
-          block_sum(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + u % s, k, s);
+          block_sum<false>(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + u % s, k, s);
           store_part(part + u * kPartDoubles, c);
           clear(c);
         }
