@@ -158,6 +158,27 @@ __device__ __forceinline__ void load_columns(float (&x)[2], const float* p) {
   x[0] = v.x; x[1] = v.y;
 }
 
+// Two fp32 multiply-adds in one instruction, each rounded like fmaf. The main loop is bound by the issue of instructions
+// (16 multiply-adds, two loads from shared memory): rows in pairs and columns doubled up make 14 of 18
+// (three ragged matrices with three workers, projection 84 -> 78 us).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pair_of(float lo, float hi) {
+  f32x2 p;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(lo), "f"(hi));
+  return p;
+}
+__device__ __forceinline__ void unpair(f32x2 p, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 square2(f32x2 a) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %1;" : "=l"(d) : "l"(a));
+  return d;
+}
+
 template <int ATRANS, int DUAL, int CARRY>
 __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
   constexpr int NT = kGemmThreads<DUAL>, CN = BN * BM / 4 / NT;  // threads, output columns per thread (rows: four)
@@ -198,16 +219,16 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
   // A. ATRANS: as B (stored [Kd][M]). Otherwise stored [M][Kd]: row lt/4, k (lt%4)*4.
   const int ar = ATRANS ? (lt >> 4) : (lt >> 2), ac = ATRANS ? (lt & 15) * 4 : (lt & 3) * 4;
 
-  float acc[4][CN], acc2[DUAL ? 4 : 1][CN];
+  f32x2 acc[2][CN], acc2[DUAL ? 2 : 1][CN];  // rows in pairs
   double tot[CARRY ? 4 : 1][CN], tot2[(CARRY && DUAL) ? 4 : 1][CN];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < CN; ++j) {
-      acc[i][j] = 0.f;
+      acc[i / 2][j] = 0ull;
       if constexpr (CARRY) tot[i][j] = 0.0;
       if constexpr (DUAL) {
-        acc2[i][j] = 0.f;
+        acc2[i / 2][j] = 0ull;
         if constexpr (CARRY) tot2[i][j] = 0.0;
       }
     }
@@ -251,31 +272,40 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
       const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][kk][ty * 4]);
-      const float a[4] = {a4.x, a4.y, a4.z, a4.w};
+      const f32x2 a[2] = {pair_of(a4.x, a4.y), pair_of(a4.z, a4.w)};
       float b[CN], c[CN];
       load_columns(b, &sB[buf][kk][tx * CN]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < CN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      for (int j = 0; j < CN; ++j) {
+        const f32x2 bb = pair_of(b[j], b[j]);
+        acc[0][j] = fma2(a[0], bb, acc[0][j]);
+        acc[1][j] = fma2(a[1], bb, acc[1][j]);
+      }
       if constexpr (DUAL) {
         load_columns(c, &sB2[buf][kk][tx * CN]);
+        const f32x2 a2[2] = {sc.a_square ? square2(a[0]) : a[0], sc.a_square ? square2(a[1]) : a[1]};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float a2 = sc.a_square ? a[i] * a[i] : a[i];
-#pragma unroll
-          for (int j = 0; j < CN; ++j) acc2[i][j] = fmaf(a2, c[j], acc2[i][j]);
+        for (int j = 0; j < CN; ++j) {
+          const f32x2 cc = pair_of(c[j], c[j]);
+          acc2[0][j] = fma2(a2[0], cc, acc2[0][j]);
+          acc2[1][j] = fma2(a2[1], cc, acc2[1][j]);
         }
       }
     }
     if constexpr (CARRY) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int p = 0; p < 2; ++p)
 #pragma unroll
         for (int j = 0; j < CN; ++j) {
-          tot[i][j] += (double)acc[i][j];
-          acc[i][j] = 0.f;
-          if constexpr (DUAL) { tot2[i][j] += (double)acc2[i][j]; acc2[i][j] = 0.f; }
+          float lo, hi;
+          unpair(acc[p][j], lo, hi);
+          tot[2 * p][j] += (double)lo; tot[2 * p + 1][j] += (double)hi;
+          acc[p][j] = 0ull;
+          if constexpr (DUAL) {
+            unpair(acc2[p][j], lo, hi);
+            tot2[2 * p][j] += (double)lo; tot2[2 * p + 1][j] += (double)hi;
+            acc2[p][j] = 0ull;
+          }
         }
     }
   };
@@ -293,6 +323,16 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
     turn(k0, x0, x1);
     if (k0 + BK < kend) turn(k0 + BK, x1, x0);
   }
+  float out[4][CN], out2[DUAL ? 4 : 1][CN];  // without the carry: the sums
+  if constexpr (!CARRY) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int j = 0; j < CN; ++j) {
+        unpair(acc[p][j], out[2 * p][j], out[2 * p + 1][j]);
+        if constexpr (DUAL) unpair(acc2[p][j], out2[2 * p][j], out2[2 * p + 1][j]);
+      }
+  }
   const Epilogue& ep = pr.epi;
   if (DUAL || csize > 1) {
 #pragma unroll
@@ -301,9 +341,9 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
       for (int j = 0; j < CN; j += 2) {
         double* o = part + (ty * 4 + i) * BN + tx * CN + j;
         if constexpr (CARRY) *reinterpret_cast<double2*>(o) = make_double2(tot[i][j], tot[i][j + 1]);
-        else *reinterpret_cast<double2*>(o) = make_double2((double)acc[i][j], (double)acc[i][j + 1]);
+        else *reinterpret_cast<double2*>(o) = make_double2((double)out[i][j], (double)out[i][j + 1]);
         if constexpr (CARRY && DUAL) *reinterpret_cast<double2*>(o + BM * BN) = make_double2(tot2[i][j], tot2[i][j + 1]);
-        else if constexpr (DUAL) *reinterpret_cast<double2*>(o + BM * BN) = make_double2((double)acc2[i][j], (double)acc2[i][j + 1]);
+        else if constexpr (DUAL) *reinterpret_cast<double2*>(o + BM * BN) = make_double2((double)out2[i][j], (double)out2[i][j + 1]);
       }
     if (csize > 1) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     else __syncthreads();
@@ -341,9 +381,9 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
       if (row >= M) break;
       if constexpr (CARRY) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = (float)tot[i][j];
+        for (int j = 0; j < 4; ++j) out[i][j] = (float)tot[i][j];
       }
-      gemm_epilogue<0>(ep, sc, N, row, col, acc[i], acc[i]);
+      gemm_epilogue<0>(ep, sc, N, row, col, out[i], out[i]);
     }
   }
 }
