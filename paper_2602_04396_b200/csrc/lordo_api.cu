@@ -518,7 +518,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
     GemmProblem g;
     std::memset(&g, 0, sizeof(g));
     g.M = M; g.N = N; g.Kd = Kd;
-    g.tiles_n = (N + 63) / 64;
+    g.tiles_n = (N + gemm_columns(B2 != nullptr) - 1) / gemm_columns(B2 != nullptr);
     g.A = A; g.B = B;
     if (B2) g.B2 = *B2; else g.B2 = B;
     g.epi = ep;

@@ -1,14 +1,14 @@
 // Grouped fp32 FFMA GEMM with fused operand formation and epilogues: the fp32-accurate ("check
 // mode") realisation of every contraction of the path -- P^T(cG+E), P g, P U~, the sketch and
 // subspace-iteration products, Gram matrices, R^-1 application, Rot = P'^T P and the rotation of
-// the moments. 64 x 64 output tile, 16-deep k-slices, 256 threads, 4 x 4 outputs per thread.
+// the moments. 64 x 64 output tile (64 x 32 with two products), 16-deep k-slices, 256 threads, 16 outputs per thread.
 // Products are formed and summed in fp32 inside a k-slice; the slice sums are carried across slices
 // in fp64, so a result is accurate to fp32 rounding whatever the contraction length.
 #include "lordo_kernels.h"
 
 namespace lordo {
 
-constexpr int BM = 64, BN = 64, BK = 16, PADS = 4;
+constexpr int BM = 64, BK = 16, PADS = 4;
 
 // An operand as the main loop reads it, resolved once per tile.
 struct Source {
@@ -144,10 +144,10 @@ __device__ __forceinline__ void partials_of(const double* p, unsigned rank, doub
 // distributed shared memory, every CTA finishing its share of the tile's rows (see launch_gemm for the size).
 // CARRY = 1: slice sums carried across k-slices in fp64 (parity mode). CARRY = 0: plain fp32
 // accumulation, half the registers (the fp32 work of the fast mode: QR and moment rotation).
-// With two products twice the threads of half the columns: 256 threads held so many sums (190 to 250 registers) that an SM
-// had eight warps to cover the loads with. Three ragged matrices with three workers, r up to 136: update 175 -> 145 us.
-template <int DUAL>
-constexpr int kGemmThreads = DUAL ? 512 : 256;
+// With two products a tile is half as wide (gemm_columns): a thread then holds two columns of each, two CTAs fit an SM and the
+// loads of one's epilogue (G, E, W) run under the other's products. Three ragged matrices with three workers, r up to 136: update
+// 175 us with 256 threads of 4 x 4 outputs, 146 with 512 threads of 4 x 2, now 120.
+constexpr int kGemmThreads = 256;
 
 __device__ __forceinline__ void load_columns(float (&x)[4], const float* p) {
   const float4 v = *reinterpret_cast<const float4*>(p);
@@ -180,8 +180,8 @@ __device__ __forceinline__ f32x2 square2(f32x2 a) {
 }
 
 template <int ATRANS, int DUAL, int CARRY>
-__global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
-  constexpr int NT = kGemmThreads<DUAL>, CN = BN * BM / 4 / NT;  // threads, output columns per thread (rows: four)
+__global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
+  constexpr int NT = kGemmThreads, BN = gemm_columns(DUAL), CN = BN * BM / 4 / NT;  // threads, output columns per thread (rows: four)
   __shared__ __align__(16) float sA[2][BK][BM + PADS];
   __shared__ __align__(16) float sB[2][BK][BN + PADS];
   __shared__ __align__(16) float sB2[2][DUAL ? BK : 1][BN + PADS];
@@ -211,13 +211,14 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
 
   const int t = threadIdx.x;
   const int tx = t % (BN / CN), ty = t / (BN / CN);
-  // loaders, one float4 of a slice each. One product: every thread A and B. Two: the first 256 threads A, the others B and B2.
-  const bool load_a = !DUAL || t < 256, load_b = !DUAL || t >= 256;
-  const int lt = t & 255;
-  // B: row kk = lt/16, columns (lt%16)*4
-  const int bk = lt >> 4, bc = (lt & 15) * 4;
+  // loaders, a float4 of a slice each: every thread A; one product: every thread B, two: half of them B and the others B2.
+  const bool second = DUAL && t >= NT / 2;
+  const int lt = DUAL ? t & (NT / 2 - 1) : t;
+  // B: row kk, columns four at a time
+  const int bk = lt / (BN / 4), bc = lt % (BN / 4) * 4;
+  const Source Bm = second ? B2 : B;
   // A. ATRANS: as B (stored [Kd][M]). Otherwise stored [M][Kd]: row lt/4, k (lt%4)*4.
-  const int ar = ATRANS ? (lt >> 4) : (lt >> 2), ac = ATRANS ? (lt & 15) * 4 : (lt & 3) * 4;
+  const int ar = ATRANS ? (t >> 4) : (t >> 2), ac = ATRANS ? (t & 15) * 4 : (t & 3) * 4;
 
   f32x2 acc[2][CN], acc2[DUAL ? 2 : 1][CN];  // rows in pairs
   double tot[CARRY ? 4 : 1][CN], tot2[(CARRY && DUAL) ? 4 : 1][CN];
@@ -235,28 +236,20 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
 
   // Two slices of k are on their way in registers while a third, in one of two buffers, is multiplied.
   struct Slice {
-    Raw x, y;  // one product: A and B; two: A and nothing, or B and B2
+    Raw x, y;
   };
   auto fetch = [&](Slice& s, int k0) {
-    if (load_a) s.x = ATRANS ? source_load(A, k0 + ar, m0 + ac, Kd, M) : source_load(A, m0 + ar, k0 + ac, M, Kd);
-    if (load_b) {
-      (DUAL ? s.x : s.y) = source_load(B, k0 + bk, n0 + bc, Kd, N);
-      if constexpr (DUAL) s.y = source_load(B2, k0 + bk, n0 + bc, Kd, N);
-    }
+    s.x = ATRANS ? source_load(A, k0 + ar, m0 + ac, Kd, M) : source_load(A, m0 + ar, k0 + ac, M, Kd);
+    s.y = source_load(Bm, k0 + bk, n0 + bc, Kd, N);
   };
   auto stash = [&](const Slice& s, int buf) {
-    if (load_a) {
-      const float4 v = source_value(A, s.x, sc);
-      if (ATRANS) {
-        *reinterpret_cast<float4*>(&sA[buf][ar][ac]) = v;
-      } else {
-        sA[buf][ac + 0][ar] = v.x; sA[buf][ac + 1][ar] = v.y; sA[buf][ac + 2][ar] = v.z; sA[buf][ac + 3][ar] = v.w;
-      }
+    const float4 v = source_value(A, s.x, sc);
+    if (ATRANS) {
+      *reinterpret_cast<float4*>(&sA[buf][ar][ac]) = v;
+    } else {
+      sA[buf][ac + 0][ar] = v.x; sA[buf][ac + 1][ar] = v.y; sA[buf][ac + 2][ar] = v.z; sA[buf][ac + 3][ar] = v.w;
     }
-    if (load_b) {
-      *reinterpret_cast<float4*>(&sB[buf][bk][bc]) = source_value(B, DUAL ? s.x : s.y, sc);
-      if constexpr (DUAL) *reinterpret_cast<float4*>(&sB2[buf][bk][bc]) = source_value(B2, s.y, sc);
-    }
+    *reinterpret_cast<float4*>(second ? &sB2[buf][DUAL ? bk : 0][bc] : &sB[buf][bk][bc]) = source_value(Bm, s.y, sc);
   };
 
   // this CTA's range of k
@@ -394,7 +387,7 @@ __global__ void __launch_bounds__(kGemmThreads<DUAL>, DUAL ? 1 : 2) gemm_ffma_ke
 // and r up to 136 in 14 CTAs 105 us, in 112 17.
 void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
                  const GemmScalars& sc, cudaStream_t st) {
-  const long long room = (long long)sm_count * (dual ? 1 : 2);  // by registers
+  const long long room = (long long)sm_count * 2;  // by registers
   const int slices = (kd_max + BK - 1) / BK;
   int c = 1;
   while (c < 8 && total_tiles * 2 * c <= room && slices >= 4 * c) c *= 2;
@@ -404,8 +397,8 @@ void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, in
   at[0].val.clusterDim.x = (unsigned)c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(dual ? kGemmThreads<1> : kGemmThreads<0>, 1, 1); lc.stream = st;
-  lc.dynamicSmemBytes = c > 1 || dual ? sizeof(double) * BM * BN * (dual ? 2 : 1) : 0;
+  lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(kGemmThreads, 1, 1); lc.stream = st;
+  lc.dynamicSmemBytes = c > 1 || dual ? sizeof(double) * BM * gemm_columns(dual) * (dual ? 2 : 1) : 0;
   lc.attrs = at; lc.numAttrs = 2;
 #define LORDO_GEMM(A, B, C) cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, C>, probs, nprobs, sc)
   if (carry) {
@@ -424,7 +417,7 @@ void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, in
 
 // With its partial sums a CTA exceeds the 48 KB of shared memory that a launch may ask for unannounced.
 cudaError_t gemm_configure() {
-  const int one = (int)(sizeof(double) * BM * BN), two = 2 * one;
+  const int one = (int)(sizeof(double) * BM * gemm_columns(0)), two = (int)(2 * sizeof(double) * BM * gemm_columns(1));
   cudaError_t e = cudaSuccess;
   auto set = [&](const void* kernel, int smem) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -74,6 +74,8 @@ struct Epilogue {
   long long ldt;
 };
 
+// Columns of an output tile of the fp32 products (rows: 64), with one product or two.
+__host__ __device__ constexpr int gemm_columns(int dual) { return dual ? 32 : 64; }
 struct GemmProblem {
   int M, N, Kd, tiles_n;
   long long tile_start;  // first tile of this problem within its launch
