@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
   __shared__ float dsum_s[kStrip];
   const uint32_t rank = cluster_rank(), S = cluster_size();
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const long long strip = blockIdx.x / S;
   const TcProblem* __restrict__ prp = probs + find_problem(probs, nprobs, strip);
   const int m = prp->m, n = prp->n, r = prp->r, r_n = prp->r_n, m_k = prp->m_k, r_k = prp->r_k;
@@ -219,26 +219,27 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
       mbar_arrive(&full_bar[s]);
     }
 
-  } else if (lane == 0) {
+  } else {
     // ---------------- MMA issue ---------------------------------------------------------------
+    const uint32_t one = elect_one();
     const uint32_t n_lo = r_n > 256 ? 256u : (uint32_t)r_n, n_hi = r_n > 256 ? (uint32_t)(r_n - 256) : 0u;
     const uint32_t idesc_lo = idesc_bf16_f32(128, n_lo), idesc_hi = idesc_bf16_f32(128, n_hi);
     bool ok = true;
     for (int kb = kb0; kb < kb1 && ok; ++kb) {
       const int s = (kb - kb0) & 1, use = (kb - kb0) >> 1;
-      ok = mbar_wait(&full_bar[s], (uint32_t)(use & 1), status);
+      ok = mbar_wait_warp(&full_bar[s], (uint32_t)(use & 1), status);
       if (!ok) break;
       tc_fence_after_sync();
       const uint32_t sA = smem_u32(smem + s * stage_bytes), sB = sA + a_bytes;
 #pragma unroll
       for (int k16 = 0; k16 < 4; ++k16) {
         const uint32_t acc = (kb > kb0 || k16 > 0) ? 1u : 0u;
-        mma_bf16(tmem, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + k16 * 32), idesc_lo, acc);
-        if (n_hi) mma_bf16(tmem + 256, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + 256 * 128 + k16 * 32), idesc_hi, acc);
+        mma_bf16(tmem, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + k16 * 32), idesc_lo, acc, one);
+        if (n_hi) mma_bf16(tmem + 256, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + 256 * 128 + k16 * 32), idesc_hi, acc, one);
       }
-      mma_commit(&empty_bar[s]);
+      if (one) mma_commit(&empty_bar[s]);
     }
-    mma_commit(&done_bar);
+    if (one) mma_commit(&done_bar);
   }
 
   // ---------------- partial accumulators of the ranks that other CTAs finish ---------------------
@@ -361,7 +362,7 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
   __shared__ uint64_t p_full[2], p_empty[2], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_slot;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const long long strip = blockIdx.x / pieces;
   const TcProblem* __restrict__ prp = probs + find_problem(probs, nprobs, strip);
   const int m = prp->m, n = prp->n, r_k = prp->r_k;
@@ -444,60 +445,51 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
     const one_t* __restrict__ Gc = Gp + colc;
     one_t* __restrict__ Ec = Ep + colc;
     one_t* __restrict__ Wc = Wp + colc;
-    bool ok = true;
-    for (int t = 0; t < nsteps && ok; ++t) {
-      const int b = t & 1;
-      const int row0 = (first + t) * kApplyRows + grp * 16;
-      const bool whole = row0 + 16 <= m;
+    // Half a step's rows are loaded while the other half is worked on (2048 x 2048, r = 128, K = 4: 73 -> 71 us, all 16 at
+    // once left the loads idle in between).
+    struct Rows {
+      one_t g[8], e[8], w[8];
+    };
+    auto load = [&](int t, int h, Rows& x) {
+      const int row0 = (first + t) * kApplyRows + grp * 16 + h * 8;
       const size_t base = (size_t)(unsigned)min(row0, m - 1) * (size_t)n;
-      one_t rg[16], re[16], rw[16];
-      if (whole) {
+      const bool whole = row0 + 8 <= m;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const size_t off = base + (size_t)(unsigned)(j * n);
-          rg[j] = Gc[off];
-          re[j] = Ec[off];
-          rw[j] = Wc[off];
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const size_t off = (size_t)(unsigned)min(row0 + j, m - 1) * (size_t)n;
-          rg[j] = Gc[off];
-          re[j] = Ec[off];
-          rw[j] = Wc[off];
-        }
+      for (int j = 0; j < 8; ++j) {
+        const size_t off = whole ? base + (size_t)(unsigned)(j * n) : (size_t)(unsigned)min(row0 + j, m - 1) * (size_t)n;
+        x.g[j] = Gc[off];
+        x.e[j] = Ec[off];
+        x.w[j] = Wc[off];
       }
-      ok = mbar_wait<40>(&acc_full[b], (uint32_t)((t >> 1) & 1), status);
-      if (!ok) break;
+    };
+    auto finish = [&](int t, int h, const Rows& x) {
+      const int row0 = (first + t) * kApplyRows + grp * 16 + h * 8, b = t & 1;
+      const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 128 + grp * 16 + h * 8);
+      float a1[8], a2[8];
+      tmem_ld8x2(taddr, taddr + 64, a1, a2);  // (P g)^T, (P U~)^T
+      if (h == 1) {
+        tc_fence_before_sync();
+        mbar_arrive(&acc_empty[b]);
+      }
+      if (!col_ok) return;
+      const size_t base = (size_t)(unsigned)min(row0, m - 1) * (size_t)n;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (row0 + j >= m) break;
+        const size_t off = base + (size_t)(unsigned)(j * n);
+        if (ef) Ec[off] = EL::pack((c * EL::cvt(x.g[j]) + EL::cvt(x.e[j])) - a1[j]);
+        Wc[off] = EL::pack(EL::cvt(x.w[j]) - lr * (cd * EL::cvt(x.g[j]) + a2w * a2[j]));
+      }
+    };
+    Rows x0, x1;
+    if (nsteps > 0) load(0, 0, x0);
+    for (int t = 0; t < nsteps; ++t) {
+      load(t, 1, x1);
+      if (!mbar_wait<40>(&acc_full[t & 1], (uint32_t)((t >> 1) & 1), status)) break;
       tc_fence_after_sync();
-      const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 128 + grp * 16);
-      float acc[16];
-      tmem_ld16(taddr, acc);  // (P g)^T
-      if (ef && col_ok) {
-        if (whole) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) Ec[base + (size_t)(unsigned)(j * n)] = EL::pack((c * EL::cvt(rg[j]) + EL::cvt(re[j])) - acc[j]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (row0 + j < m) Ec[base + (size_t)(unsigned)(j * n)] = EL::pack((c * EL::cvt(rg[j]) + EL::cvt(re[j])) - acc[j]);
-        }
-      }
-      tmem_ld16(taddr + 64, acc);  // (P U~)^T
-      tc_fence_before_sync();
-      mbar_arrive(&acc_empty[b]);
-      if (col_ok) {
-        if (whole) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            Wc[base + (size_t)(unsigned)(j * n)] = EL::pack(EL::cvt(rw[j]) - lr * (cd * EL::cvt(rg[j]) + a2w * acc[j]));
-        } else {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (row0 + j < m) Wc[base + (size_t)(unsigned)(j * n)] = EL::pack(EL::cvt(rw[j]) - lr * (cd * EL::cvt(rg[j]) + a2w * acc[j]));
-        }
-      }
+      finish(t, 0, x0);
+      if (t + 1 < nsteps) load(t + 1, 0, x0);
+      finish(t, 1, x1);
     }
   } else if (warp < kApplyEpiWarps + kApplyProdWarps) {
     // ---------------- producers: rows of P for the next step (asynchronous 16-byte copies) -----
@@ -523,15 +515,16 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
       fence_async_smem();
       mbar_arrive(&p_full[s]);
     }
-  } else if (lane == 0) {
+  } else {
     // ---------------- MMA issue ---------------------------------------------------------------
+    const uint32_t one = elect_one();
     const uint32_t idesc = idesc_bf16_f32(128, kApplyRows);
     const uint32_t x1 = smem_u32(sX1), x2 = smem_u32(sX2);
     bool ok = true;
     for (int t = 0; t < nsteps && ok; ++t) {
       const int s = t & 1;
-      ok = mbar_wait(&p_full[s], (uint32_t)((t >> 1) & 1), status);
-      if (ok) ok = mbar_wait(&acc_empty[s], (uint32_t)(((t >> 1) & 1) ^ 1), status);
+      ok = mbar_wait_warp(&p_full[s], (uint32_t)((t >> 1) & 1), status);
+      if (ok) ok = mbar_wait_warp(&acc_empty[s], (uint32_t)(((t >> 1) & 1) ^ 1), status);
       if (!ok) break;
       tc_fence_after_sync();
       const uint32_t pbase = smem_u32(sP + s * p_bytes);
@@ -540,12 +533,14 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
         for (int k16 = 0; k16 < 4; ++k16) {
           const uint32_t acc = (kb > 0 || k16 > 0) ? 1u : 0u;
           const uint64_t bd = smem_desc_k128(pbase + kb * (kApplyRows * 128) + k16 * 32);
-          mma_bf16(tmem + s * 128, smem_desc_k128(x1 + kb * (kStrip * 128) + k16 * 32), bd, idesc, acc);
-          mma_bf16(tmem + s * 128 + 64, smem_desc_k128(x2 + kb * (kStrip * 128) + k16 * 32), bd, idesc, acc);
+          mma_bf16(tmem + s * 128, smem_desc_k128(x1 + kb * (kStrip * 128) + k16 * 32), bd, idesc, acc, one);
+          mma_bf16(tmem + s * 128 + 64, smem_desc_k128(x2 + kb * (kStrip * 128) + k16 * 32), bd, idesc, acc, one);
         }
       }
-      mma_commit(&p_empty[s]);
-      mma_commit(&acc_full[s]);
+      if (one) {
+        mma_commit(&p_empty[s]);
+        mma_commit(&acc_full[s]);
+      }
     }
   }
   tc_fence_before_sync();
