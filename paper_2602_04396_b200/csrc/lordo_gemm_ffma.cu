@@ -381,16 +381,21 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
   }
 }
 
-// CTAs per output tile: doubled, up to the portable cluster size, while all of them have a place on the device at
-// once and each is left two slices of k. A product with few tiles is a chain of slices, each about a trip to
-// memory long: 256 x 256, r = 16, two replicas, P^T (c G + E) in 8 CTAs 44 us, in 64 10.5; Gram matrices of 1000 rows
-// and r up to 136 in 14 CTAs 105 us, in 112 17.
+// CTAs per output tile, up to the portable cluster size: the count whose turns of CTAs on the device (two fit an SM) times
+// the slices of k of each, with about three more for its start and end, are least; each is left two slices. A product
+// with few tiles is a chain of slices, each about a trip to memory long: 256 x 256, r = 16, two replicas, P^T (c G + E) in
+// 8 CTAs 44 us, in 64 10.5; Gram matrices of 1000 rows and r up to 136 in 14 CTAs 105 us, in 112 17; 198 tiles of up to 63 slices
+// in 198 CTAs 78 us, in 792 74.
 void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
                  const GemmScalars& sc, cudaStream_t st) {
   const long long room = (long long)sm_count * 2;  // by registers
   const int slices = (kd_max + BK - 1) / BK;
   int c = 1;
-  while (c < 8 && total_tiles * 2 * c <= room && slices >= 4 * c) c *= 2;
+  long long best = -1;
+  for (int x = 1; x <= 8 && (x == 1 || slices >= 2 * x); x *= 2) {
+    const long long cost = ((total_tiles * x + room - 1) / room) * ((slices + x - 1) / x + 3);
+    if (best < 0 || cost < best) { best = cost; c = x; }
+  }
   cudaLaunchConfig_t lc = {};
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
