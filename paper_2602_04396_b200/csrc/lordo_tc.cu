@@ -581,14 +581,14 @@ void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strip
   // two CTAs fit an SM; each is left four steps at least
   int c = 1;
   while (c < 4 && total_strips * 2 * c <= 2 * (long long)sm_count && steps >= 8 * c) c *= 2;
+  // Begun under the end of the kernel before it (as launch_dep does), or as clusters of one, its CTAs are not spread over the SMs
+  // but land two to an SM while others idle: four ragged matrices, r up to 256, 54 strips, step 355 us, plainly launched 285 us.
   cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
-  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
   lc.gridDim = dim3((unsigned)(total_strips * c), 1, 1); lc.blockDim = dim3(kProjThreads, 1, 1); lc.dynamicSmemBytes = project_tc_smem(r_n_max);
-  lc.stream = st; lc.attrs = at; lc.numAttrs = 2;
+  lc.stream = st; lc.attrs = &at; lc.numAttrs = c > 1 ? 1 : 0;
   if (bf16) cudaLaunchKernelEx(&lc, project_tc_kernel<true>, probs, nprobs, sc, status);
   else cudaLaunchKernelEx(&lc, project_tc_kernel<false>, probs, nprobs, sc, status);
 }
@@ -598,8 +598,19 @@ void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips,
   int pieces = (int)std::min<long long>(sm_count / total_strips, steps / 4);
   if (pieces < 1) pieces = 1;
   const dim3 grid((unsigned)(total_strips * pieces));
-  if (bf16) launch_dep(apply_tc_kernel<true>, grid, kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, pieces, status);
-  else launch_dep(apply_tc_kernel<false>, grid, kApplyThreads, apply_tc_smem(r_k_max), st, probs, nprobs, sc, pieces, status);
+  const size_t smem = apply_tc_smem(r_k_max);
+  // CTAs that begin under the end of the projection gain 3 us where all of them fit the device, but where they run in
+  // several turns the early ones take places in the wrong order: 448 strips, r = 256, step 806 us, plainly launched 693 us.
+  const bool early = (long long)grid.x <= sm_count;
+#define LORDO_APPLY_TC(B)                                                                                          \
+  if (early) launch_dep(apply_tc_kernel<B>, grid, kApplyThreads, smem, st, probs, nprobs, sc, pieces, status);      \
+  else apply_tc_kernel<B><<<grid, kApplyThreads, smem, st>>>(probs, nprobs, sc, pieces, status)
+  if (bf16) {
+    LORDO_APPLY_TC(true);
+  } else {
+    LORDO_APPLY_TC(false);
+  }
+#undef LORDO_APPLY_TC
 }
 
 }  // namespace lordo
