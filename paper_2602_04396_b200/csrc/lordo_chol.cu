@@ -13,7 +13,7 @@
 // While one warp factors the diagonal block of panel k, the others already sum panel k + 1 over the panels
 // before k, so that a panel waits for the newest 32 columns only.
 //
-// What bounds it: the chain of r columns, 200 to 350 clocks each (shuffle, reciprocal square root, multiply-adds),
+// What bounds it: the r columns of the diagonal blocks, 300 clocks each (some 70 instructions of one warp),
 // and per panel one trip to L2 for the newest columns, the small products and the barrier; for few CTAs per matrix
 // the fp64 products. One CTA per matrix with a thread per row took 2200 us for r = 512 and 16 matrices, 580 us
 // for r = 256 and 7, 197 us for r = 128 and 56; clusters that summed a whole panel at its turn 654, 131 and 62 us;
