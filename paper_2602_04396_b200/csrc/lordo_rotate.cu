@@ -78,13 +78,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   constexpr int kStages = 196608 / kStage, kCtas = PAIR ? 2 : 1;  // CTAs behind one MMA
   // PAIR: full_a (here: A and B of both CTAs) and acc_empty are waited on by the MMA thread of the pair's first CTA only and
   // fed by the warps of both; empty_bar and acc_full are signalled in both CTAs by that thread's commits
-  __shared__ uint64_t full_a[kMaxStages], full_b[kMaxStages], empty_bar[kMaxStages], acc_full, acc_empty, peer_read;
+  // peer_read: two barriers in turn, one per split strip. The other CTA arrives for a strip as soon as all warps here have arrived
+  // for the one before it, whether or not each of them has seen that phase complete; on a single barrier a warp that
+  // polls late would find the parity of the phase after it. Nobody arrives for the strip after the next before
+  // every warp here has arrived for the next, hence has seen this one.
+  __shared__ uint64_t full_a[kMaxStages], full_b[kMaxStages], empty_bar[kMaxStages], acc_full, acc_empty, peer_read[2];
   __shared__ uint32_t tmem_slot;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const uint32_t rank = cluster_rank();
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(&full_a[s], kCtas * kFormWarps); mbar_init(&full_b[s], 1); mbar_init(&empty_bar[s], 1); }
-    mbar_init(&acc_full, 1); mbar_init(&acc_empty, kCtas * kEpiWarps); mbar_init(&peer_read, kEpiWarps);
+    mbar_init(&acc_full, 1); mbar_init(&acc_empty, kCtas * kEpiWarps); for (int b = 0; b < 2; ++b) mbar_init(&peer_read[b], kEpiWarps);
     mbar_init_fence();
   }
   if (warp == 1) {
@@ -238,7 +242,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   } else {
     // ---------------- the rotated moments out of tensor memory ---------------------------------------
     const int q = warp & 3, half = (warp - (2 + kFormWarps)) >> 2;
-    const uint32_t peer = cluster_addr(&peer_read, rank ^ 1u), drained = cluster_addr(&acc_empty, 0);
+    const uint32_t peer = cluster_addr(&peer_read[0], rank ^ 1u), drained = cluster_addr(&acc_empty, 0);
     uint32_t si = 0, split_items = 0;
     bool ok = true;
     for (long long item = first; item < items && ok; item += step, ++si) {
@@ -254,8 +258,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       tc_fence_after_sync();
       if (split) {  // the other CTA has read this strip too
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(peer);
-        ok = mbar_wait<32>(&peer_read, split_items++ & 1u, status);
+        if (lane == 0) mbar_arrive_cluster(peer + 8u * (split_items & 1u));
+        ok = mbar_wait<32>(&peer_read[split_items & 1u], (split_items >> 1) & 1u, status);
+        ++split_items;
         if (!ok) break;
       }
       for (int ch = half; ch < n_h / 16; ch += 2) {

@@ -46,12 +46,12 @@ def test_cholesky_panels_and_clusters(r, count):
 
 
 @pytest.mark.parametrize("mats,K", [(((72, 64, 8),), 1), (((136, 264, 40), (264, 392, 136)), 3), (((520, 648, 256), (600, 1032, 264)), 2),
-                                    (((1032, 1544, 512),), 2), (((64, 40, 8), (64, 2056, 24)), 2)])
+                                    (((1032, 1544, 512),), 2), (((64, 40, 8), (64, 2056, 24)), 2), (((392, 1288, 264),), 16)])
 @pytest.mark.parametrize("variant,side", [(0, 0), (1, 0), (1, 1)])
 def test_rotation_in_place(mats, K, variant, side):
     """Rotated moments against the oracle's rotation lines on the bases of the CUDA path: ranks below one stage of
     32, ragged stages, above and below 256 in one launch (pairs that share a strip and pairs that do not), an odd
-    number of strips, one basis and one per worker."""
+    number of strips, several shared strips one after the other in a pair (176 strips), one basis and one per worker."""
     mats = tuple((n, m, r) if side else (m, n, r) for m, n, r in mats)
     wl = synth.Workload("t", mats, K=K, H=2, rounds=2, grad="gauss", clip_rho=30.0, w_dtype="bf16", g_dtype="bf16", e_dtype="bf16",
                         sides=(side,) * len(mats))
