@@ -599,9 +599,13 @@ void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips,
   if (pieces < 1) pieces = 1;
   const dim3 grid((unsigned)(total_strips * pieces));
   const size_t smem = apply_tc_smem(r_k_max);
-  // CTAs that begin under the end of the projection gain 3 us where all of them fit the device, but where they run in
+  // CTAs that begin under the end of the projection gain 2 to 5 us where all of them fit the device, but where they run in
   // several turns the early ones take places in the wrong order: 448 strips, r = 256, step 806 us, plainly launched 693 us.
-  const bool early = (long long)grid.x <= sm_count;
+  // In one turn too they take the SMs in the order in which the projection leaves them and not in the device's own. At
+  // r_k = 256, where a step pulls 32 KB of P out of L2, the same strips then last a third longer by their own clocks (144
+  // strips of three lengths, one to an SM either way: 66 instead of 49 us, step 159 instead of 139 us; 98 strips 284 and
+  // 241 us; 128 equal strips 312 and 287 us); r_k <= 192 is within 2 % for mixed strips and gains 3 us for equal ones.
+  const bool early = (long long)grid.x <= sm_count && r_k_max < 256;
 #define LORDO_APPLY_TC(B)                                                                                          \
   if (early) launch_dep(apply_tc_kernel<B>, grid, kApplyThreads, smem, st, probs, nprobs, sc, pieces, status);      \
   else apply_tc_kernel<B><<<grid, kApplyThreads, smem, st>>>(probs, nprobs, sc, pieces, status)
