@@ -9,6 +9,7 @@
 #include <cuda.h>
 
 #include "lordo_kernels.h"
+#include "lordo_plan.h"
 
 using namespace lordo;
 
@@ -357,24 +358,12 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   std::vector<size_t> mat_scratch(n_mats);
   // Ranges of k that the two sums of a tensor-core Gram matrix are dealt out in (`gram_sum_kernel` adds them).
   // A Gram matrix has only ceil(r / 256) output tiles, so without ranges a launch over few matrices leaves most
-  // of the CTA pairs idle (7 matrices of r = 256: 265 us in 7 pairs, 30 us in 70): the count with the shortest
-  // last wave is taken, a range costing about four steps of 64 k on top of its own (start of the pipeline,
-  // epilogue). A range is also kept below 64 steps, because the tensor cores' fp32 accumulation truncates and
-  // the ranges meet in fp64.
+  // of the CTA pairs idle (7 matrices of r = 256: 265 us in 7 pairs, 30 us in 70).
   long long gram_tiles = 0;
   for (int i = 0; i < n_mats; ++i) gram_tiles += 2ll * (local ? K : 1) * ((cfg.mats[i].r + 255) / 256);
-  auto ranges = [&](long long tiles, long long steps, long long most) {
-    int best = 1;
-    long long best_cost = -1;
-    for (int ns = (int)((steps + 63) / 64); ns <= most && (ns == 1 || steps / ns >= 4); ++ns) {
-      const long long cost = ((tiles * ns + kPairs - 1) / kPairs) * ((steps + ns - 1) / ns + 4);
-      if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = ns; }
-    }
-    return best;
-  };
-  auto gram_ranges = [&](long long rows) { return ranges(gram_tiles, 2 * ((rows + 63) / 64), 32); };
+  auto gram_ranges = [&](long long rows) { return k_ranges(gram_tiles, 2 * ((rows + 63) / 64), 32, kPairs); };
   // Rot has half the tiles and three pairs of planes; its partial products share the Gram matrices' buffer
-  auto rot_ranges = [&](long long rows) { return ranges(gram_tiles / 2, 3 * ((rows + 63) / 64), 64); };
+  auto rot_ranges = [&](long long rows) { return k_ranges(gram_tiles / 2, 3 * ((rows + 63) / 64), 64, kPairs); };
   auto part_matrices = [&](long long pm, long long ln) { return std::max(2 * std::max(gram_ranges(pm), gram_ranges(ln)), rot_ranges(pm)); };
   std::vector<int> group_of(n_mats);
   size_t scratch_floats = 0;

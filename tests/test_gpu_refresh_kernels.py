@@ -29,6 +29,16 @@ def test_gram_in_ranges_of_k(shape):
     assert w["rot_u"] < ROT_TOL and w["rot_v"] < 2 * ROT_TOL, w
 
 
+@pytest.mark.parametrize("shape,q", [((70000, 64, 8), 0), ((64, 70000, 8), 1), ((90048, 72, 40), 0)])
+def test_gram_of_a_vocabulary_sized_matrix(shape, q):
+    """More rows (or, with an iteration, columns) than 32 ranges of 64 steps hold; Rot above 64 ranges of 64 steps. Signal of
+    rank r plus 0.5 % noise, so that the iteration's span is well conditioned; tolerances as above."""
+    kw = dict(grad="lowrank", signal_rank=shape[2], noise=0.005) if q else {}
+    w = _refresh(*shape, q=q, **kw)
+    assert w["P_orth"] < ORTH_TOL and w["rot_u"] < ROT_TOL and w["rot_v"] < 2 * ROT_TOL, w
+    assert w["P_angle_bf16rhs"] < ANGLE_TOL, w
+
+
 @pytest.mark.parametrize("r,count", [(8, 1), (32, 1), (40, 3), (256, 2), (264, 40), (504, 1), (296, 80), (512, 75)])
 def test_cholesky_panels_and_clusters(r, count):
     """The factorisation behind P_0 = Q of a 2r x r integer matrix, against a QR in fp64: one panel, whole and
