@@ -22,6 +22,7 @@
 // out by every lane 345, 88 and 53 us. (Scaling the block so that rsqrt.approx needs no care, and handing the factoring
 // warp its block summed, both made the column chain slower.)
 #include "lordo_kernels.h"
+#include "lordo_recip.cuh"
 
 namespace lordo {
 namespace {
@@ -232,9 +233,8 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
     if (warp == 0) {
       // Factor of the diagonal block: lane i holds row i of what is left of the block. Every lane works out every pivot d
       // for itself, from the element b beside the pivot before it and the diagonal element D that were handed round a column
-      // earlier: D - b b / d. With r0 = 1/d to 20 bits and e = 1 - d r0 that is D - b b r0 (1 + e + e e), 60 bits, and the next
-      // column's elements are worked out likewise; the square root, the column of L and the update of the columns behind
-      // the next one fill the gaps. (No chain is what is left: a column is some 70 instructions of one warp, which issues one
+      // earlier: D - b b / d = D - b b r0 (1 + e), see lordo_recip.cuh, and the next column's elements likewise; the square
+      // root, the column of L and the update of the columns behind the next one fill the gaps. (No chain is what is left: a column is some 70 instructions of one warp, which issues one
       // every four clocks. Handing two elements round and updating the columns behind one column late: slower, registers.)
       asm volatile("bar.sync 1, 128;" ::: "memory");
       const float* gk = ga + (k & 1) * kB * kB;
@@ -257,10 +257,9 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
       double b = __shfl_sync(0xffffffffu, a[0], 1), D = __shfl_sync(0xffffffffu, dg, 1);
 #pragma unroll
       for (int j = 0; j < kB; ++j) {
-        double r0, y0, dn = 1.0;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
-        const double e0 = fma(-d, r0, 1.0), e = fma(e0, e0, e0), aj = a[j];
+        double r0, e, dn = 1.0;
+        recip_parts(d, r0, e);
+        const double aj = a[j];
         auto minus = [&](double x, double pq) { const double p = pq * r0; return fma(-p, e, x - p); };  // x - pq / d
         if (j + 1 < kB) {
           dn = minus(D, b * b);
@@ -271,7 +270,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
           b = __shfl_sync(0xffffffffu, a[j + 1], j + 2);
           D = __shfl_sync(0xffffffffu, dg, j + 2);
         }
-        const double f = fma(-d * y0, y0, 1.0), y = fma(y0 * f, fma(0.375, f, 0.5), y0);  // 1 / L_jj, 58 bits
+        const double y = recip_sqrt(d);  // 1 / L_jj
         const double l = lane == j ? d * y : (lane > j ? aj * y : 0.0);
         Lc[j * kB + lane] = l;
         if (lane == 0) dinv[j] = y;

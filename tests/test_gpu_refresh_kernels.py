@@ -1,7 +1,11 @@
 """Edges of the kernels of the tensor-core refresh, against the oracle on the CUDA path's own state."""
+import ctypes as C
+import subprocess
+
 import pytest
 import torch
 
+from paper_2602_04396_b200 import build as lbuild
 from paper_2602_04396_b200 import lordo, synth
 from tests import harness as hz
 from tests.harness import RunSpec
@@ -53,6 +57,46 @@ def test_cholesky_panels_and_clusters(r, count):
         q = q * torch.sign(torch.diagonal(t))
         assert ((opt.P[i].double() - q).norm() / q.norm()).item() < 1e-5
     opt.close()
+
+
+RECIP = """
+#include "lordo_recip.cuh"
+__global__ void kernel(const double* d, double* out, int n) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  double r0, e;
+  lordo::recip_parts(d[i], r0, e);
+  out[i] = fma(r0, e, r0);
+  out[n + i] = lordo::recip_sqrt(d[i]);
+  out[2 * n + i] = 1.0 / d[i];
+  out[3 * n + i] = 1.0 / sqrt(d[i]);
+}
+extern "C" int run(const double* d, double* out, int n) {
+  kernel<<<(n + 255) / 256, 256>>>(d, out, n);
+  return (int)cudaDeviceSynchronize();
+}
+"""
+
+
+def test_reciprocals_of_the_pivots(tmp_path):
+    """lordo_recip.cuh against CUDA's division and square root: both sides are within 2^-52 of the exact value (the
+    header's bound; half an ulp for the division, an ulp for the root and the division behind it), so they differ by 2^-51 at
+    most. Every exponent that a pivot of an fp32 Gram matrix can have, powers of two and their neighbours, and pivots at
+    the two floors."""
+    src, so = tmp_path / "recip.cu", tmp_path / "recip.so"
+    src.write_text(RECIP)
+    subprocess.run(["/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-shared", "-Xcompiler", "-fPIC",
+                    "-I", lbuild.CSRC, "-o", str(so), str(src)], check=True)
+    gen = torch.Generator().manual_seed(1)
+    exps = torch.arange(-190, 130, dtype=torch.float64)
+    mant = torch.cat([1 + torch.rand(4000, generator=gen, dtype=torch.float64), torch.tensor([1.0, 1 + 2.0 ** -52, 2 - 2.0 ** -52, 1.5])])
+    d = (2.0 ** exps[:, None] * mant).flatten()
+    diag = torch.rand(4000, generator=gen) * 1e3
+    d = torch.cat([d, (3e-5 * diag).double(), (1e-12 * diag).double().clamp_min(1e-30), torch.ones(1, dtype=torch.float64)]).cuda()
+    out = torch.empty(4, d.numel(), device="cuda", dtype=torch.float64)
+    assert C.CDLL(str(so)).run(C.c_void_p(d.data_ptr()), C.c_void_p(out.data_ptr()), d.numel()) == 0
+    for mine, cuda in ((out[0], out[2]), (out[1], out[3])):
+        assert ((mine - cuda).abs() / cuda).max().item() <= 2.0 ** -51
 
 
 @pytest.mark.parametrize("mats,K", [(((72, 64, 8),), 1), (((136, 264, 40), (264, 392, 136)), 3), (((520, 648, 256), (600, 1032, 264)), 2),
