@@ -338,6 +338,11 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   const bool warm = cfg.warm_start != 0;  // start the subspace iteration from the previous P instead of a random sketch
   const int q = (warm && cfg.power_iters < 1) ? 1 : cfg.power_iters;
   Carver cv(ws);
+  c->tc = cfg.check_mode == 0 && cfg.g_dtype == cfg.w_dtype && (!cfg.error_feedback || cfg.e_dtype == cfg.w_dtype);
+  for (int i = 0; i < n_mats; ++i)  // ranks above 512 (above 256 with fp32 storage) run on the fp32 path
+    if (cfg.mats[i].r > (cfg.w_dtype == LORDO_BF16 ? 512 : 256) || (cfg.mats[i].side && cfg.w_dtype != LORDO_BF16)) c->tc = false;
+  c->tma = c->tc && cfg.w_dtype == LORDO_BF16;
+  const bool tc_sketch = c->tma && cfg.oversample == 0;  // products of the refresh on tensor cores
 
   c->d_mats = cv.take<MatDev>(n_mats);
   c->d_chunk_start = cv.take<long long>(n_mats + 1);
@@ -368,6 +373,12 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   std::vector<int> group_of(n_mats);
   size_t scratch_floats = 0;
   const bool keep_signal = local && cfg.error_feedback && 2 * q + (warm ? 0 : 1) > 1;  // see `sketch` below
+  // Floats per basis of what takes turns in one place on the tensor-core path: the fp32 work of P_0 (Global, lordo_init only);
+  // the kept signal, until the last product that reads it; the new basis as the QR leaves it and the planes of the old one.
+  auto shared_floats = [&](const lordo_mat& a) {
+    const size_t pm = a.side ? a.n : a.m, maxd = a.m > a.n ? a.m : a.n, r = a.r;
+    return std::max(std::max(2 * pm * r, local ? 0 : (pm + maxd) * r), keep_signal ? (size_t)a.m * a.n / 2 : 0) + 64;
+  };
   {
     size_t acc = 0;
     int grp = 0;
@@ -377,16 +388,17 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       const size_t pm = a.side ? a.n : a.m, ln = a.side ? a.m : a.n;  // rows of P, columns of the low-rank arrays
       const size_t nb = local ? K : 1;
       const size_t rs = (size_t)a.r + cfg.oversample;  // columns of the sketch and of everything up to the truncation
-      size_t per = ln * rs + 2 * pm * rs + (size_t)maxd * rs + ((q > 0 || cfg.oversample > 0) ? 2 * ln * rs : 0) + 4 * rs * rs;
-      if (cfg.oversample > 0) per += 3 * rs * rs + rs * a.r;  // eigen-solver work and the truncating projector
+      size_t per = 4 * rs * rs;
       // bf16 right-hand sides of the tensor-core sketch products (Omega, P', Z), counted in floats
       per += (ln * a.r + (q > 0 ? pm * a.r + ln * a.r : 0)) / 2 + 64;
-      if (cfg.check_mode == 0 && cfg.w_dtype == LORDO_BF16) {
-        // bf16 planes of the tensor-core QR and rotation: X and R^-1 in three planes, P, Rot^T and its square in
-        // two; partial products and sums
-        per += 3 * (size_t)maxd * a.r / 2 + pm * a.r + 7 * (size_t)a.r * a.r / 2 + 128;
-        if (keep_signal) per += (size_t)a.m * a.n / 2 + 64;
+      if (tc_sketch) {
+        // bf16 planes of the tensor-core QR and rotation: X and R^-1 in three planes, Rot^T and its square in two;
+        // partial products and sums
+        per += shared_floats(a) + 3 * (size_t)maxd * a.r / 2 + 7 * (size_t)a.r * a.r / 2 + 128;
         per += (size_t)part_matrices(pm, ln) * a.r * a.r + 2 * (size_t)((pm + kNormRows - 1) / kNormRows) * a.r + 16;
+      } else {
+        per += ln * rs + 2 * pm * rs + (size_t)maxd * rs + ((q > 0 || cfg.oversample > 0) ? 2 * ln * rs : 0);
+        if (cfg.oversample > 0) per += 3 * rs * rs + rs * a.r;  // eigen-solver work and the truncating projector
       }
       mat_scratch[i] = nb * per + 64;
       if (acc > 0 && acc + mat_scratch[i] > kRefreshScratchFloats) { ++grp; acc = 0; }
@@ -407,8 +419,8 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
     MatDev& md = c->h_mats[i];
     md.m = a.m; md.n = a.n; md.r = a.r; md.side = a.side; md.Delta16 = nullptr;
     md.pm = a.side ? a.n : a.m; md.ln = a.side ? a.m : a.n;
-    md.ghat = cv.take<float>((size_t)K * a.r * md.ln);
-    md.util = cv.take<float>((size_t)K * a.r * md.ln);
+    md.ghat = tc_sketch ? nullptr : cv.take<float>((size_t)K * a.r * md.ln);  // check mode, and rotations on the fp32 path
+    md.util = tc_sketch ? nullptr : cv.take<float>((size_t)K * a.r * md.ln);
     md.dcol = cv.take<float>((size_t)K * md.ln);
     md.T = cfg.time_buffer ? cv.take<float>((size_t)K * a.r * md.ln) : nullptr;
     md.p_stride = local ? md.pm * a.r : 0;
@@ -420,9 +432,6 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   c->d_scratch = cv.take<float>(scratch_floats);
 
   // ---------------- tensor-core operand copies and problem table ----------------
-  c->tc = cfg.check_mode == 0 && cfg.g_dtype == cfg.w_dtype && (!cfg.error_feedback || cfg.e_dtype == cfg.w_dtype);
-  for (int i = 0; i < n_mats; ++i)  // ranks above 512 (above 256 with fp32 storage) run on the fp32 path
-    if (cfg.mats[i].r > (cfg.w_dtype == LORDO_BF16 ? 512 : 256) || (cfg.mats[i].side && cfg.w_dtype != LORDO_BF16)) c->tc = false;
   c->h_tc.clear(); c->h_prep.clear(); c->h_prep_start.assign(1, 0);
   c->tc_strips = 0; c->tc_pairs = 0; c->tc_rn_max = 0; c->tc_rk_max = 0; c->tc_steps_min = 1 << 30;
   std::vector<size_t> h_prep_first(n_mats, 0);  // first entry of a matrix in h_prep
@@ -483,7 +492,6 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
     c->tc_bf16_bytes = cv.off - bf16_begin;
     c->prep_blocks = c->h_prep_start.back();
     c->d_tc_probs = cv.take<TcProblem>(c->h_tc.size());
-    c->tma = cfg.w_dtype == LORDO_BF16;
     if (c->tma)
       for (int l = 0; l < 2; ++l) {
         c->d_segs[l] = cv.take<TcSeg>((size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers));
@@ -501,7 +509,6 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   std::vector<GemmProblem>& P = c->h_probs;
   P.clear(); c->h_chols.clear(); c->h_rands.clear(); c->h_copies.clear(); c->h_sks.clear(); c->h_convs.clear(); c->h_bases.clear(); c->h_rots.clear(); c->h_rotates.clear(); c->h_eigs.clear(); c->h_grams.clear(); c->h_diag.clear();
   c->h_skbufs.assign(n_mats, lordo_ctx::SketchBufs());
-  const bool tc_sketch = c->tc && c->tma && cfg.oversample == 0;  // products of the refresh on tensor cores
   c->refresh_makes_copies = tc_sketch;
   auto gemm_prob = [&](int M, int N, int Kd, const Operand& A, const Operand& B, const Operand* B2, const Epilogue& ep) {
     GemmProblem g;
@@ -685,12 +692,21 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       goff += mat_scratch[i];
       const bool rr = cfg.oversample > 0;  // oversampled sketch, Rayleigh-Ritz truncation back to r columns
       const int rs = r + cfg.oversample;   // equals r on the tensor-core path
-      float* Om = s; s += (size_t)nb * n * rs;
-      float* Ya = s; s += (size_t)nb * m * rs;
-      float* Pn = s; s += (size_t)nb * m * rs;
-      float* Yb = s; s += (size_t)nb * maxd * rs;
-      float *Za = nullptr, *Zq = nullptr;
-      if (q > 0 || rr) { Za = s; s += (size_t)nb * n * rs; Zq = s; s += (size_t)nb * n * rs; }
+      float *Om = nullptr, *Ya = nullptr, *Pn = nullptr, *Yb = nullptr, *Za = nullptr, *Zq = nullptr;
+      __nv_bfloat16 *phl = nullptr, *s16 = nullptr;  // planes of the old basis; the kept signal
+      if (tc_sketch) {  // see shared_floats
+        s = c->d_scratch + ((s - c->d_scratch + 63) & ~(ptrdiff_t)63);
+        if (!local) { Ya = s; Yb = s + m * r; }
+        if (keep_signal) s16 = reinterpret_cast<__nv_bfloat16*>(s);
+        Pn = s; phl = reinterpret_cast<__nv_bfloat16*>(s + (size_t)nb * m * r);
+        s += (size_t)nb * (shared_floats(cfg.mats[i]) - 64);
+      } else {
+        Om = s; s += (size_t)nb * n * rs;
+        Ya = s; s += (size_t)nb * m * rs;
+        Pn = s; s += (size_t)nb * m * rs;
+        Yb = s; s += (size_t)nb * maxd * rs;
+        if (q > 0 || rr) { Za = s; s += (size_t)nb * n * rs; Zq = s; s += (size_t)nb * n * rs; }
+      }
       float* gram = s; s += (size_t)nb * rs * rs;
       float* lw = s; s += (size_t)nb * rs * rs;
       float* rinv = s; s += (size_t)nb * rs * rs;
@@ -705,13 +721,12 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       }
       c->h_skbufs[i].om16 = om16; c->h_skbufs[i].pn16 = pn16; c->h_skbufs[i].zq16 = zq16;
       // tensor-core QR and rotation: bf16 planes, plane p of batch entry b at index p * nb + b
-      __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *phl = nullptr, *rt16 = nullptr, *sq16 = nullptr;
+      __nv_bfloat16 *x16 = nullptr, *rinv16 = nullptr, *rt16 = nullptr, *sq16 = nullptr;
       float* gpart = nullptr;   // partial sums of the Gram matrices and of Rot
       double* colsq = nullptr;  // partial sums of squares of the new basis' columns
       if (tc_sketch) {
         auto take16 = [&](size_t floats) { __nv_bfloat16* p16 = reinterpret_cast<__nv_bfloat16*>(s); s += floats + 16; return p16; };
         x16 = take16(3 * (size_t)nb * maxd * r / 2);
-        phl = take16((size_t)nb * m * r);
         rinv16 = take16(3 * (size_t)nb * r * r / 2);
         rt16 = take16((size_t)nb * r * r);
         sq16 = take16((size_t)nb * r * r);
@@ -719,11 +734,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
         s = c->d_scratch + ((s - c->d_scratch + 3) & ~(ptrdiff_t)3);
         colsq = reinterpret_cast<double*>(s); s += 2 * (size_t)nb * ((m + kNormRows - 1) / kNormRows) * r;
         lordo_ctx::SketchBufs& kb = c->h_skbufs[i];
-        if (keep_signal) {
-          s = c->d_scratch + ((s - c->d_scratch + 63) & ~(ptrdiff_t)63);
-          kb.s16 = take16((size_t)nb * md.m * md.n / 2);
-        }
-        kb.x16 = x16; kb.rinv16 = rinv16; kb.phl = phl; kb.rt16 = rt16; kb.sq16 = sq16;
+        kb.x16 = x16; kb.rinv16 = rinv16; kb.phl = phl; kb.rt16 = rt16; kb.sq16 = sq16; kb.s16 = s16;
       }
       TmaMatMaps* mmi = c->d_maps + i;
       // C = A B as the sum of the products of np-plane split operands; planes as above. a_mn: A stored [Kd][M].
@@ -794,7 +805,6 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       // Local rule with error feedback and more than one product: the first one keeps the signal it forms, c G + E in
       // bf16, for the others, which then read half as much and need no transform (4096 x 11008, r = 512, K = 16: 0.8 to 0.9
       // ms a product that forms it, 0.6 to 0.7 one that reads it)
-      __nv_bfloat16* s16 = c->h_skbufs[i].s16;
       bool s16_made = false;
       // S * B on tensor cores, into the three planes of x16: a_mn = 0 -> S rows are the output rows (Y = S B), 1 -> S^T B
       auto sketch = [&](SlotBuilder& sb, int a_mn, unsigned char* map_b, long long Mo, long long Kd) {

@@ -45,3 +45,17 @@ def test_workspace_holds_the_ranges_of_tall_matrices():
         return lordo.query_workspace(cfg)
     for m in (65536, 87360, 128256):
         assert size(m) < size(m + 64)
+
+
+def test_workspace_of_the_kept_signal():
+    """Local rule with iterations: the signal c G + E kept in bf16 lies where the new and the old basis are put after it, and nothing that
+    only the fp32 path uses is set aside: at large ranks the workspace stays below 4.88 and 39.04 GB, what it took before the
+    signal was kept; at small ones the signal's own 2 bytes per weight-replica are all that it adds."""
+    def size(mats, K, q, ef=True):
+        cfg, _keep = lordo.make_config(mats, K, 1, w_dtype=lordo.BF16, g_dtype=lordo.BF16, e_dtype=lordo.BF16, check_mode=0, variant=lordo.LOCAL,
+                                       power_iters=q, error_feedback=ef)
+        return lordo.query_workspace(cfg)
+    big = (4096, 11008, 512)
+    assert size([big], 16, 2) <= 4.88e9 and size([big] * 8, 16, 2) <= 39.04e9
+    for m, n, r, K in ((2048, 2048, 64, 8), (7504, 3888, 168, 2), (200, 1112, 8, 1), (2048, 2048, 256, 8)):
+        assert size([(m, n, r)], K, 1) - size([(m, n, r)], K, 1, ef=False) <= 2 * K * m * n
