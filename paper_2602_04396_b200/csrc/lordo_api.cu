@@ -9,7 +9,6 @@
 #include <cuda.h>
 
 #include "lordo_kernels.h"
-#include "lordo_plan.h"
 
 using namespace lordo;
 
@@ -280,52 +279,6 @@ void prefix_arrays(const lordo_config& cfg, std::vector<long long>& chunk_start,
     mom_start[i + 1] = mom_start[i] + (long long)K * ((ln + kMomCols - 1) / kMomCols);
     wblk[i + 1] = wblk[i] + (elems + 1023) / 1024;
     sblk[i + 1] = sblk[i] + ((long long)a.r * ln + 1023) / 1024;
-  }
-}
-
-// Deals the work of the TMA-fed kernels out, longest pieces first, each to the worker with the least so far.
-// An item is a strip (or a pair of strips) of `len` steps that costs `cost`; `lists` comes back with every worker's
-// pieces, `start` with their offsets. With `split` a strip that would take its worker past the even share is cut
-// there and the rest dealt on, so that all workers end together; a piece costs `head` on top of its steps (its
-// operands are fetched anew; about four steps) and has at least kMinPiece. Strips dealt round the grid ended apart
-// wherever they were few or of different lengths: 7 layers of 768 (r = 128, K = 8) update 183 us, dealt out 137 us.
-constexpr int kMinPiece = 8;
-struct WorkItem {
-  int prob, strip, len;
-  double cost;
-};
-void deal_out(std::vector<WorkItem> items, int workers, bool split, double head, std::vector<TcSeg>& list, std::vector<int>& start) {
-  std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.cost > b.cost; });
-  double total = 0.0;
-  for (const WorkItem& it : items) total += it.cost + head;
-  const double share = std::max(total / workers + (split ? head / 2 : 0.0), split ? kMinPiece + head : 0.0);
-  std::vector<std::vector<TcSeg>> lists(workers);
-  typedef std::pair<double, int> Load;  // what a worker has, the worker
-  std::vector<Load> heap;
-  for (int w = 0; w < workers; ++w) heap.push_back(Load(0.0, w));
-  const auto later = [](const Load& a, const Load& b) { return a > b; };
-  for (const WorkItem& it : items) {
-    int t0 = 0;
-    while (t0 < it.len) {
-      std::pop_heap(heap.begin(), heap.end(), later);
-      Load& ld = heap.back();
-      int n = it.len - t0;
-      if (split) {
-        const int room = (int)(share - ld.first - head + 0.5);
-        if (n > room) n = std::min(n, std::max(room, kMinPiece));
-        if (it.len - t0 - n < kMinPiece) n = it.len - t0;
-      }
-      lists[ld.second].push_back({it.prob, it.strip, t0, t0 + n});
-      ld.first += it.cost * n / it.len + head;
-      t0 += n;
-      std::push_heap(heap.begin(), heap.end(), later);
-    }
-  }
-  list.clear();
-  start.assign(1, 0);
-  for (const std::vector<TcSeg>& l : lists) {
-    list.insert(list.end(), l.begin(), l.end());
-    start.push_back((int)list.size());
   }
 }
 
@@ -1354,11 +1307,12 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
           std::vector<int> start;
           long long steps = 0;
           for (const WorkItem& it : items) steps += it.len;
+          // SMs whose update keeps the memory busy; two sweeps (r > 256) are bound by what an SM pulls out of L2
+          const int busy = c->tc_rn_max > 256 ? c->sm_count : c->sm_count * 7 / 9;
           // no more workers than there are pieces
           const int most = l == 0 ? std::min(project_pairs(c->sm_count), (int)items.size())
                                   : (int)std::min<long long>(c->sm_count, std::max<long long>((long long)items.size(), steps / kMinPiece));
-          deal_out(std::move(items), std::min(most, kMaxWorkers), l > 0, l > 0 ? 4.0 : 0.0, list, start);
-          while (start.size() > 1 && start[start.size() - 2] == (int)list.size()) start.pop_back();  // workers without work
+          deal_out(std::move(items), std::min(most, kMaxWorkers), l > 0, l > 0 ? kPieceHead : 0, busy, list, start);
           c->seg_workers[l] = (int)start.size() - 1;
           if (list.size() > (size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers)) return bail(LORDO_ERR_NOMEM);
           INIT_CUDA(cudaMemcpyAsync(c->d_segs[l], list.data(), sizeof(TcSeg) * list.size(), cudaMemcpyHostToDevice, st));

@@ -1,6 +1,7 @@
 // Internal interface between the host layer (lordo_api.cu) and the kernel files.
 #pragma once
 #include "lordo_common.cuh"
+#include "lordo_plan.h"
 
 namespace lordo {
 
@@ -166,12 +167,6 @@ void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips,
                      int bf16, unsigned* status, cudaStream_t st);
 
 // TMA-fed persistent kernels for bf16 storage (lordo_tma.cu).
-// A piece of work of one CTA (update) or CTA pair (projection): steps [t0, t1) of 64 rows of one strip, or one
-// pair of strips. Workers walk their own part of a list, [start[w], start[w + 1]), dealt out by lordo_init so
-// that all of them end together.
-struct TcSeg {
-  int prob, strip, t0, t1;
-};
 cudaError_t tma_configure();
 int project_pairs(int sm_count);  // CTA pairs of the projection that the device holds at once
 void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int pairs, const TmaMatMaps* maps,

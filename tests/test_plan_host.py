@@ -10,6 +10,18 @@ from paper_2602_04396_b200 import lordo
 
 WRAPPER = """
 #include "lordo_plan.h"
+extern "C" int deal(int n, const int* len, int workers, int split, int busy, int* seg, int* start, int* starts) {
+  std::vector<lordo::WorkItem> items;
+  for (int i = 0; i < n; ++i) items.push_back({i, i, len[i], (double)len[i]});
+  std::vector<lordo::TcSeg> list;
+  std::vector<int> st;
+  lordo::deal_out(items, workers, split != 0, split ? lordo::kPieceHead : 0, busy, list, st);
+  if ((int)list.size() > n + workers || (int)st.size() > workers + 1) return -1;
+  for (size_t i = 0; i < list.size(); ++i) { seg[3 * i] = list[i].prob; seg[3 * i + 1] = list[i].t0; seg[3 * i + 2] = list[i].t1; }
+  for (size_t i = 0; i < st.size(); ++i) start[i] = st[i];
+  *starts = (int)st.size();
+  return (int)list.size();
+}
 extern "C" int ranges(long long tiles, long long steps, long long most, long long pairs) { return lordo::k_ranges(tiles, steps, most, pairs); }
 """
 
@@ -23,7 +35,41 @@ def plan(tmp_path_factory):
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", lbuild.CSRC, "-o", so, src], check=True)
     lib = C.CDLL(so)
     lib.ranges.argtypes = [C.c_longlong] * 4
+    lib.deal.argtypes = [C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
     return lib
+
+
+MIN_PIECE, HEAD = 8, 4
+
+
+# strips (count, 64-row steps); on 148 SMs: are strips cut, and the longest worker over the mean. One long strip, few long ones, two halves
+# each, most of the SMs busy with whole strips, one turn and a bit, several turns, too short to cut, ragged
+@pytest.mark.parametrize("strips,cut,most", [([(1, 2004)], True, 1.1), ([(6, 500)], True, 1.1), ([(1, 172)], True, 1.4), ([(74, 32)], True, 1.01),
+                                             ([(40, 64)], True, 1.1), ([(110, 64)], False, 1.4), ([(128, 64)], False, 1.2), ([(156, 64)], True, 1.15),
+                                             ([(2432, 32), (256, 88)], False, 1.05), ([(1, 7)], False, 1.0), ([(1, 15)], False, 1.0),
+                                             ([(149, 9)], False, 2.0), ([(576, 12), (48, 48)], False, 1.1),
+                                             ([(33, 16), (48, 9), (72, 8), (27, 11), (51, 3)], False, 1.25)])
+@pytest.mark.parametrize("sms", [148, 40])
+@pytest.mark.parametrize("split", [1, 0])
+def test_strips_dealt_out(plan, strips, cut, most, sms, split):
+    """Every step of every strip once, no piece below the shortest, at most strips + workers pieces (the room that the table has), and
+    on 148 SMs the longest worker at most `most` times the mean, heads of pieces counted."""
+    lens = [ln for count, ln in strips for _ in range(count)]
+    workers = min(sms, max(len(lens), sum(lens) // MIN_PIECE))
+    seg, start, starts = (C.c_int * (3 * (len(lens) + workers)))(), (C.c_int * (workers + 1))(), C.c_int()
+    pieces = plan.deal(len(lens), (C.c_int * len(lens))(*lens), workers, split, sms * 7 // 9, seg, start, C.byref(starts))
+    assert 0 < pieces <= len(lens) + workers
+    got = [(seg[3 * i], seg[3 * i + 1], seg[3 * i + 2]) for i in range(pieces)]
+    at = [0] * len(lens)
+    for prob, t0, t1 in sorted(got):
+        assert t0 == at[prob] and t1 - t0 >= min(MIN_PIECE, lens[prob])
+        at[prob] = t1
+    assert at == lens and (split or pieces == len(lens))
+    starts = list(start)[:starts.value]
+    assert starts[0] == 0 and starts[-1] == pieces and starts == sorted(starts)
+    if split and sms == 148:
+        loads = [sum(t1 - t0 + HEAD for _, t0, t1 in got[a:b]) for a, b in zip(starts, starts[1:])]
+        assert max(loads) <= most * sum(loads) / workers and (pieces > len(lens)) == cut
 
 
 @pytest.mark.parametrize("rows", [8, 64, 520, 4096, 65536, 65600, 70000, 87424, 128256, 151936, 1 << 20])
