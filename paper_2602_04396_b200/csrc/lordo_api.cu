@@ -16,7 +16,6 @@ namespace {
 
 constexpr int kMaxK = 64;
 constexpr int kMaxWorkers = 256;  // CTAs (or CTA pairs) that walk a list of work
-constexpr long long kPairs = 74;  // CTA pairs that the work of a refresh is planned for (148 SMs)
 
 enum StepType { ST_GEMM = 0, ST_CHOL = 1, ST_RANDOM = 2, ST_COPY = 3, ST_SKETCH = 4, ST_CONVERT = 5, ST_COLSQ = 6, ST_EIG = 7, ST_GRAM = 8, ST_BASIS = 9, ST_ROT = 10, ST_ROTATE = 11 };
 enum Phase { PH_SUBSPACE = 0, PH_ROTATE = 1, PH_COMMIT = 2 };
@@ -319,9 +318,9 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   // of the CTA pairs idle (7 matrices of r = 256: 265 us in 7 pairs, 30 us in 70).
   long long gram_tiles = 0;
   for (int i = 0; i < n_mats; ++i) gram_tiles += 2ll * (local ? K : 1) * ((cfg.mats[i].r + 255) / 256);
-  auto gram_ranges = [&](long long rows) { return k_ranges(gram_tiles, 2 * ((rows + 63) / 64), 32, kPairs); };
+  auto gram_ranges = [&](long long rows) { return k_ranges(gram_tiles, 2 * ((rows + 63) / 64), 32, kPlannedSms / 2); };
   // Rot has half the tiles and three pairs of planes; its partial products share the Gram matrices' buffer
-  auto rot_ranges = [&](long long rows) { return k_ranges(gram_tiles / 2, 3 * ((rows + 63) / 64), 64, kPairs); };
+  auto rot_ranges = [&](long long rows) { return k_ranges(gram_tiles / 2, 3 * ((rows + 63) / 64), 64, kPlannedSms / 2); };
   auto part_matrices = [&](long long pm, long long ln) { return std::max(2 * std::max(gram_ranges(pm), gram_ranges(ln)), rot_ranges(pm)); };
   std::vector<int> group_of(n_mats);
   size_t scratch_floats = 0;

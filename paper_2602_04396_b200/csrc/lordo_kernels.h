@@ -10,7 +10,7 @@ namespace lordo {
 // balance (five ragged matrices, 15 million elements: blocks of 2048 29 us, 1038 blocks 13 us), larger ones end apart
 // (4096 x 11008, K = 4: blocks of 131072 70 us, of 32768 58 us).
 inline long long sq_chunk(long long elements) {
-  const long long c = (elements / (8 * 148) + 2047) / 2048 * 2048;
+  const long long c = (elements / (8 * kPlannedSms) + 2047) / 2048 * 2048;
   return c < 2048 ? 2048 : c > 32768 ? 32768 : c;
 }
 

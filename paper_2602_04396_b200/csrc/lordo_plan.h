@@ -6,6 +6,10 @@
 
 namespace lordo {
 
+// SMs that sizes in the workspace are planned for: lordo_query_workspace makes no CUDA call and lordo_init has to agree with it. With
+// fewer at hand the same ranges and chunks take more waves. Lists that lordo_init alone makes go by the device's own count.
+constexpr int kPlannedSms = 148;
+
 // Ranges of k that a product of the refresh with few output tiles is dealt out in: the count with the shortest last wave on
 // `pairs` CTA pairs, a range costing about four steps of 64 k on top of its own (start of the pipeline, epilogue), and
 // left four steps at least. A range has at most 64 steps, whatever their count: the tensor cores' fp32 accumulation truncates, and

@@ -726,8 +726,9 @@ namespace {
 // Columns of B that take part in the 64-deep step kb: of the first n_lo all but skip_lo, of the other n_hi all but skip_hi. With
 // an upper triangular B (R^-1) the columns below 64 kb are zero there and cost neither loads nor MMAs; the first step of a
 // pair of planes has them all, so it may overwrite the accumulator. r = 512, 16 workers: 11008 rows 385 -> 301 us, 4096 rows
-// 160 -> 125 us. For r <= 256 the table's word is not looked at: widths that change from step to step cost every launch a
-// microsecond, and at r = 128 the products with R^-1 gain nothing (41.5 -> 42.7 us; r = 256 26.0 -> 24.3 us).
+// 160 -> 125 us. For r <= 256 the table's word is not looked at: the products with R^-1 of r = 256 gain 2 us each, but widths that may change
+// from step to step cost each of a refresh's other launches up to a microsecond. Whole refreshes with the word looked at everywhere: 7
+// matrices of 768, r = 128 507 -> 511 us; of 2048, r = 192 493 -> 495 us, r = 256 600 -> 597 us; two iterations of r = 256 1042 -> 1032 us.
 struct SkCols {
   int lo, hi, skip_lo, skip_hi;
   __device__ __forceinline__ SkCols(int n_lo, int n_hi, int tri, int kb) {
