@@ -46,12 +46,12 @@ HYPER = {
 LR = 0.004
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture summarised in the named
-# file under profiles/ (taken on 2 of the 24 layers and scaled by 12: traffic grows with the layers).
+# file under profiles/ (taken on 1 of the 24 layers and scaled by 24: traffic grows with the layers).
 # An entry is removed when its kernel changes, until the counters have been taken again.
 NCU_TRAFFIC = {
-    "cfg4_1B_r256:global:fast:apply": (102849540000, "profiles/ncu_project_tma_apply_tma_cfg4_first2layers.md"),
-    "cfg4_1B_r256:global:fast:project": (60545076000, "profiles/ncu_project_tma_apply_tma_cfg4_first2layers.md"),
-    "cfg4_1B_r256:local:fast:apply": (102849540000, "profiles/ncu_project_tma_apply_tma_cfg4_first2layers.md"),
+    "cfg4_1B_r256:global:fast:apply": (102737640000, "profiles/ncu_step_and_outer_2048_layer.md"),
+    "cfg4_1B_r256:global:fast:project": (59758200000, "profiles/ncu_step_and_outer_2048_layer.md"),
+    "cfg4_1B_r256:local:fast:apply": (102737640000, "profiles/ncu_step_and_outer_2048_layer.md"),
 }
 
 
