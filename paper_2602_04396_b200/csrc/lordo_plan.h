@@ -37,34 +37,41 @@ struct WorkItem {  // a strip (or a pair of strips) of `len` steps that costs `c
 constexpr int kMinPiece = 8;   // steps of a piece of a cut strip
 constexpr int kPieceHead = 4;  // steps that a piece costs on top of its own: its operands are fetched anew
 
-// Deals items out, longest first, each to the worker with the least so far. With `split` no worker gets more than `share`: a
-// strip that would take its worker past it is cut there and the rest dealt on, a remainder that would be too short being
-// made long enough at the cost of the piece before it. False where something has no place.
-// A worker is cut at most once: it is left with less room than a piece needs. So there are at most items + workers pieces.
-inline bool deal_within(const std::vector<WorkItem>& items, bool split, int head, double share, std::vector<std::vector<TcSeg>>& lists) {
+// Deals items out, longest first, each to the worker with the least so far. Returns the longest worker's.
+//   WHOLE  strips are not cut
+//   EVEN   a strip that would take its worker past `share` is cut there and the rest dealt on; what finds no room is dealt on
+//          top, in the shortest pieces, and a remainder that would be too short stays with the piece before it
+//   WITHIN no worker gets more than `share`: a remainder that would be too short is made long enough at the cost of the piece
+//          before it. Returns -1 where something has no place. A worker is cut at most once, being left with less room
+//          than a piece needs, so there are at most items + workers pieces.
+enum Dealing { WHOLE, EVEN, WITHIN };
+inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, double share, std::vector<std::vector<TcSeg>>& lists) {
   typedef std::pair<double, int> Load;  // what a worker has, the worker
   std::vector<Load> heap;
   for (int w = 0; w < (int)lists.size(); ++w) { lists[w].clear(); heap.push_back(Load(0.0, w)); }
   const auto later = [](const Load& a, const Load& b) { return a > b; };
+  double longest = 0.0;
   for (const WorkItem& it : items) {
     for (int t0 = 0; t0 < it.len;) {
       std::pop_heap(heap.begin(), heap.end(), later);
       Load& ld = heap.back();
-      int n = it.len - t0;
-      if (split) {
-        const int room = (int)(share - ld.first) - head;
-        if (n > room) {
-          n = std::min(room, n - kMinPiece);
-          if (n < kMinPiece) return false;
-        }
+      const int rest = it.len - t0, room = (int)(share - ld.first - head + 0.5);
+      int n = rest;
+      if (how == EVEN && n > room) {
+        n = std::min(n, std::max(room, kMinPiece));
+        if (rest - n < kMinPiece) n = rest;
+      } else if (how == WITHIN && n > room) {
+        n = std::min(room, rest - kMinPiece);
+        if (n < kMinPiece) return -1;
       }
       lists[ld.second].push_back({it.prob, it.strip, t0, t0 + n});
-      ld.first += it.cost * n / it.len + head;
+      ld.first += how == WHOLE ? it.cost + head : n + head;
+      longest = std::max(longest, ld.first);
       t0 += n;
       std::push_heap(heap.begin(), heap.end(), later);
     }
   }
-  return true;
+  return (int)(longest + 0.5);
 }
 
 // How long the workers of a cut or uncut list take, in steps of a worker that has the memory to itself: up to `busy` of them run at that
@@ -85,23 +92,34 @@ inline double time_of(const std::vector<std::vector<TcSeg>>& lists, int head, in
   return t;
 }
 
-// `list` comes back with every worker's pieces, `start` with their offsets; workers at the end without work are left out. The
-// share is the smallest, in steps of 2 %, in which everything has a place. Strips dealt round the grid ended apart wherever
-// they were few or of different lengths: 7 layers of 768 (r = 128, K = 8) update 183 us, dealt out 137 us.
-// Strips are cut only where that ends sooner by time_of: with most of the SMs at work the memory is busy anyway, and every
-// piece fetches its operands. Update of 4096 rows, r = 256: 40 strips 83 us whole, 43 us cut; 110 strips 101 and 110 us,
-// 128 strips 114 and 127 us, 156 strips 199 and 147 us, 256 strips 241 and 245 us.
+// `list` comes back with every worker's pieces, `start` with their offsets; workers at the end without work are left out. Strips dealt
+// round the grid ended apart wherever they were few or of different lengths: 7 layers of 768 (r = 128, K = 8) update 183 us,
+// dealt out 137 us.
+// With `split` strips are dealt out by EVEN, with half a head of slack per worker. Where cuts cost more than that (few long strips: one
+// of 2004 steps ended with a longest worker of 1.75 times the mean), the smallest share that WITHIN finds a place for is better, and where
+// most SMs have a whole strip the memory is busy anyway and WHOLE is, since every piece fetches its operands. Either is taken where
+// it ends sooner than EVEN by a tenth by time_of, which is about how well that tells: update of 4096 rows, r = 256, EVEN, WHOLE and WITHIN:
+// 40 strips 50, 83, 43 us; 120 strips 122, 107, 121 us; 256 strips 241, 241, 245 us; mixes that it called 4 to 8 % better were 2 to 5 % slower.
 inline void deal_out(std::vector<WorkItem> items, int workers, bool split, int head, int busy, std::vector<TcSeg>& list, std::vector<int>& start) {
   std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.cost > b.cost; });
   std::vector<std::vector<TcSeg>> lists(workers);
-  deal_within(items, false, head, 0.0, lists);
+  const int longest = deal(items, WHOLE, head, 0.0, lists);
   if (split) {
-    std::vector<std::vector<TcSeg>> cut(workers);
     double total = 0.0;
     for (const WorkItem& it : items) total += it.cost + head;
-    double share = std::max(total / workers, (double)(kMinPiece + head));
-    while (!deal_within(items, true, head, share, cut)) share += std::max(0.02 * share, 0.5);
-    if (time_of(cut, head, busy) < time_of(lists, head, busy)) lists.swap(cut);
+    std::vector<std::vector<TcSeg>> even(workers), cut(workers), within;
+    deal(items, EVEN, head, std::max(total / workers + head / 2.0, (double)(kMinPiece + head)), even);
+    size_t pieces = 0;
+    for (const std::vector<TcSeg>& l : even) pieces += l.size();
+    int least = std::max((int)(total / workers), kMinPiece + head) - 1, share = longest;  // nothing below, everything at WHOLE's longest
+    while (share - least > 1) {
+      const int mid = least + (share - least) / 2;
+      if (deal(items, WITHIN, head, mid, cut) < 0) least = mid;
+      else { share = mid; within.swap(cut); cut.resize(workers); }
+    }
+    if (!within.empty() && time_of(within, head, busy) < time_of(lists, head, busy)) lists.swap(within);
+    const bool fits = pieces <= items.size() + workers;  // the room that the table has; either of the others does
+    if (fits && time_of(lists, head, busy) > 0.9 * time_of(even, head, busy)) lists.swap(even);
   }
   list.clear();
   start.assign(1, 0);

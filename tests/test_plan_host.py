@@ -45,9 +45,9 @@ MIN_PIECE, HEAD = 8, 4
 # strips (count, 64-row steps); on 148 SMs: are strips cut, and the longest worker over the mean. One long strip, few long ones, two halves
 # each, most of the SMs busy with whole strips, one turn and a bit, several turns, too short to cut, ragged
 @pytest.mark.parametrize("strips,cut,most", [([(1, 2004)], True, 1.1), ([(6, 500)], True, 1.1), ([(1, 172)], True, 1.4), ([(74, 32)], True, 1.01),
-                                             ([(40, 64)], True, 1.1), ([(110, 64)], False, 1.4), ([(128, 64)], False, 1.2), ([(156, 64)], True, 1.15),
-                                             ([(2432, 32), (256, 88)], False, 1.05), ([(1, 7)], False, 1.0), ([(1, 15)], False, 1.0),
-                                             ([(149, 9)], False, 2.0), ([(576, 12), (48, 48)], False, 1.1),
+                                             ([(40, 64)], True, 1.1), ([(100, 64)], True, 1.25), ([(120, 64)], False, 1.25), ([(128, 64)], False, 1.2),
+                                             ([(156, 64)], True, 1.15), ([(64, 63)], True, 1.2), ([(2432, 32), (256, 88)], False, 1.05),
+                                             ([(1, 7)], False, 1.0), ([(1, 15)], False, 1.0), ([(149, 9)], False, 2.0), ([(576, 12), (48, 48)], False, 1.1),
                                              ([(33, 16), (48, 9), (72, 8), (27, 11), (51, 3)], False, 1.25)])
 @pytest.mark.parametrize("sms", [148, 40])
 @pytest.mark.parametrize("split", [1, 0])
