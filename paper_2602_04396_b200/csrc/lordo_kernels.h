@@ -160,11 +160,11 @@ struct TcPrep {
 
 cudaError_t tc_configure(int r_n_max, int r_k_max);
 void launch_prep_projection(const TcPrep* items, const long long* blk_start, int nitems, long long total_blocks, cudaStream_t st);
-// fp32 storage of G, E and W, r <= 256 (mixed storage and larger ranks run on the fp32 path)
+// bf16 != 0: G, E, W are all bf16; else all fp32 (mixed storage runs on the fp32 path).
 void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, int steps, int sm_count, const StepScalars& sc,
-                       unsigned* status, cudaStream_t st);
+                       int bf16, unsigned* status, cudaStream_t st);
 void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_k_max, int steps, int sm_count, const StepScalars& sc,
-                     unsigned* status, cudaStream_t st);
+                     int bf16, unsigned* status, cudaStream_t st);
 
 // TMA-fed persistent kernels for bf16 storage (lordo_tma.cu).
 cudaError_t tma_configure();

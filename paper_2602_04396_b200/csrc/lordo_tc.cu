@@ -1,4 +1,4 @@
-// Tensor-core (tcgen05 + tensor memory) kernels of the inner step, "fast mode", for fp32 storage of G, E and W and r <= 256:
+// Tensor-core (tcgen05 + tensor memory) kernels of the inner step, "fast mode":
 //
 //   project_tc_kernel  g^T = (cG+E)^T P  for one 128-column strip of one (matrix, worker), swept
 //                      down the m rows; the low-rank moment update (Algorithm 1: u, v lines and the
@@ -42,6 +42,30 @@ __device__ __forceinline__ int find_problem(const TcProblem* __restrict__ probs,
   return lo;
 }
 
+// Storage type of G, E and W inside the tensor-core kernels: all bf16 or all fp32. Loads are kept
+// as raw values in registers (no use before the whole batch has been issued), converted afterwards.
+template <bool BF16>
+struct Elem;
+template <>
+struct Elem<true> {
+  using one = unsigned short;
+  using pair = uint32_t;
+  static __device__ __forceinline__ float cvt(one x) { return __uint_as_float(((uint32_t)x) << 16); }
+  static __device__ __forceinline__ float2 cvt2(pair x) { return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u)); }
+  static __device__ __forceinline__ one pack(float v) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(v);
+    return *reinterpret_cast<const unsigned short*>(&h);
+  }
+};
+template <>
+struct Elem<false> {
+  using one = float;
+  using pair = float2;
+  static __device__ __forceinline__ float cvt(one x) { return x; }
+  static __device__ __forceinline__ float2 cvt2(pair x) { return x; }
+  static __device__ __forceinline__ one pack(float v) { return v; }
+};
+
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -82,8 +106,12 @@ __global__ void __launch_bounds__(256) prep_projection_kernel(const TcPrep* __re
 // ---------------------------------------------------------------------------------------------
 // project + moments
 // ---------------------------------------------------------------------------------------------
+template <bool BF16>
 __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcProblem* __restrict__ probs, int nprobs, StepScalars sc,
                                                                      unsigned* __restrict__ status) {
+  using EL = Elem<BF16>;
+  using one_t = typename EL::one;
+  using pair_t = typename EL::pair;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t full_bar[2], empty_bar[2], done_bar;
@@ -119,11 +147,11 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
     const long long col = n0 + 2 * cp;
     const bool col_ok = col < n;
     const long long colc = col_ok ? col : (long long)n - 2;  // loads stay in bounds, results are masked
-    const float* __restrict__ Gp = reinterpret_cast<const float*>(*prp->G_ind) + prp->G_off;
+    const one_t* __restrict__ Gp = reinterpret_cast<const one_t*>(*prp->G_ind) + prp->G_off;
     const bool have_e = sc.ef != 0;
-    const float* __restrict__ Ep = have_e ? reinterpret_cast<const float*>(prp->E) : Gp;
-    const float* __restrict__ Gc = Gp + colc;
-    const float* __restrict__ Ec = Ep + colc;
+    const one_t* __restrict__ Ep = have_e ? reinterpret_cast<const one_t*>(prp->E) : Gp;
+    const one_t* __restrict__ Gc = Gp + colc;
+    const one_t* __restrict__ Ec = Ep + colc;
     const float c = *prp->cptr;
     const float es = have_e ? 1.f : 0.f;
     const __nv_bfloat16* __restrict__ PT = prp->PT16;
@@ -131,21 +159,21 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
     bool ok = true;
     for (int kb = kb0; kb < kb1 && ok; ++kb) {
       const int s = (kb - kb0) & 1, use = (kb - kb0) >> 1;
-      float2 rg[16], re[16];
+      pair_t rg[16], re[16];
       const int rbase = kb * 64 + kg * 16;
       if (rbase + 16 <= m) {
         const size_t base = (size_t)rbase * (size_t)n;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          rg[j] = *reinterpret_cast<const float2*>(Gc + base + (size_t)(unsigned)(j * n));
-          re[j] = *reinterpret_cast<const float2*>(Ec + base + (size_t)(unsigned)(j * n));
+          rg[j] = *reinterpret_cast<const pair_t*>(Gc + base + (size_t)(unsigned)(j * n));
+          re[j] = *reinterpret_cast<const pair_t*>(Ec + base + (size_t)(unsigned)(j * n));
         }
       } else {
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           const size_t off = (size_t)(unsigned)min(rbase + j, m - 1) * (size_t)n;
-          rg[j] = *reinterpret_cast<const float2*>(Gc + off);
-          re[j] = *reinterpret_cast<const float2*>(Ec + off);
+          rg[j] = *reinterpret_cast<const pair_t*>(Gc + off);
+          re[j] = *reinterpret_cast<const pair_t*>(Ec + off);
         }
       }
       uint4 pt[8];
@@ -158,7 +186,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
       float2 a[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const float2 g = rg[j], e = re[j];
+        const float2 g = EL::cvt2(rg[j]), e = EL::cvt2(re[j]);
         const float live = (col_ok && rbase + j < m) ? 1.f : 0.f;
         a[j] = make_float2(live * (c * g.x + es * e.x), live * (c * g.y + es * e.y));
       }
@@ -181,6 +209,12 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
         const int idx = tid + t * 256;
         if (idx < pt_chunks) *reinterpret_cast<uint4*>(sB + swz_chunk(idx >> 3, idx & 7)) = pt[t];
       }
+      if (r_n > 256) {  // rows 256.. of the P^T tile (r up to 512)
+        for (int idx = 2048 + tid; idx < pt_chunks; idx += 256) {
+          const uint4 v = *reinterpret_cast<const uint4*>(PT + (long long)(idx >> 3) * m_k + kb * 64 + (idx & 7) * 8);
+          *reinterpret_cast<uint4*>(sB + swz_chunk(idx >> 3, idx & 7)) = v;
+        }
+      }
       fence_async_smem();
       mbar_arrive(&full_bar[s]);
     }
@@ -188,7 +222,8 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
   } else {
     // ---------------- MMA issue ---------------------------------------------------------------
     const uint32_t one = elect_one();
-    const uint32_t idesc = idesc_bf16_f32(128, (uint32_t)r_n);
+    const uint32_t n_lo = r_n > 256 ? 256u : (uint32_t)r_n, n_hi = r_n > 256 ? (uint32_t)(r_n - 256) : 0u;
+    const uint32_t idesc_lo = idesc_bf16_f32(128, n_lo), idesc_hi = idesc_bf16_f32(128, n_hi);
     bool ok = true;
     for (int kb = kb0; kb < kb1 && ok; ++kb) {
       const int s = (kb - kb0) & 1, use = (kb - kb0) >> 1;
@@ -199,7 +234,8 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
 #pragma unroll
       for (int k16 = 0; k16 < 4; ++k16) {
         const uint32_t acc = (kb > kb0 || k16 > 0) ? 1u : 0u;
-        mma_bf16(tmem, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + k16 * 32), idesc, acc, one);
+        mma_bf16(tmem, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + k16 * 32), idesc_lo, acc, one);
+        if (n_hi) mma_bf16(tmem + 256, smem_desc_k128(sA + k16 * 32), smem_desc_k128(sB + 256 * 128 + k16 * 32), idesc_hi, acc, one);
       }
       if (one) mma_commit(&empty_bar[s]);
     }
@@ -316,8 +352,11 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
 // ---------------------------------------------------------------------------------------------
 // back-projection + error feedback + model update
 // ---------------------------------------------------------------------------------------------
+template <bool BF16>
 __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProblem* __restrict__ probs, int nprobs, StepScalars sc,
                                                                     int pieces, unsigned* __restrict__ status) {
+  using EL = Elem<BF16>;
+  using one_t = typename EL::one;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t p_full[2], p_empty[2], acc_full[2], acc_empty[2];
@@ -394,22 +433,22 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
     const long long col = n0 + q * 32 + lane;
     const bool col_ok = col < n;
     const long long colc = col_ok ? col : (long long)n - 1;
-    const float* __restrict__ Gp = reinterpret_cast<const float*>(*prp->G_ind) + prp->G_off;
-    float* __restrict__ Wp = reinterpret_cast<float*>(prp->W);
+    const one_t* __restrict__ Gp = reinterpret_cast<const one_t*>(*prp->G_ind) + prp->G_off;
+    one_t* __restrict__ Wp = reinterpret_cast<one_t*>(prp->W);
     const bool ef = sc.ef != 0;
-    float* __restrict__ Ep = ef ? reinterpret_cast<float*>(prp->E) : Wp;
+    one_t* __restrict__ Ep = ef ? reinterpret_cast<one_t*>(prp->E) : Wp;
     const float c = *prp->cptr;
     const float lr = sc.lr, om = sc.omega;
     const bool full = sc.form == LORDO_QHM_FULL;
     const float cd = full ? (1.f - om) * c / prp->dcol[colc] : 0.f;
     const float a2w = full ? om : 1.f;
-    const float* __restrict__ Gc = Gp + colc;
-    float* __restrict__ Ec = Ep + colc;
-    float* __restrict__ Wc = Wp + colc;
+    const one_t* __restrict__ Gc = Gp + colc;
+    one_t* __restrict__ Ec = Ep + colc;
+    one_t* __restrict__ Wc = Wp + colc;
     // Half a step's rows are loaded while the other half is worked on (2048 x 2048, r = 128, K = 4: 73 -> 71 us, all 16 at
     // once left the loads idle in between).
     struct Rows {
-      float g[8], e[8], w[8];
+      one_t g[8], e[8], w[8];
     };
     auto load = [&](int t, int h, Rows& x) {
       const int row0 = (first + t) * kApplyRows + grp * 16 + h * 8;
@@ -438,8 +477,8 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProb
       for (int j = 0; j < 8; ++j) {
         if (row0 + j >= m) break;
         const size_t off = base + (size_t)(unsigned)(j * n);
-        if (ef) Ec[off] = (c * x.g[j] + x.e[j]) - a1[j];
-        Wc[off] = x.w[j] - lr * (cd * x.g[j] + a2w * a2[j]);
+        if (ef) Ec[off] = EL::pack((c * EL::cvt(x.g[j]) + EL::cvt(x.e[j])) - a1[j]);
+        Wc[off] = EL::pack(EL::cvt(x.w[j]) - lr * (cd * EL::cvt(x.g[j]) + a2w * a2[j]));
       }
     };
     Rows x0, x1;
@@ -524,9 +563,13 @@ size_t apply_tc_smem(int r_k_max) {
 }
 
 cudaError_t tc_configure(int r_n_max, int r_k_max) {
-  const cudaError_t e = cudaFuncSetAttribute(project_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
+  cudaError_t e = cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(apply_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_tc_smem(r_k_max));
+  e = cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(apply_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_tc_smem(r_k_max));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(apply_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_tc_smem(r_k_max));
 }
 
 void launch_prep_projection(const TcPrep* items, const long long* blk_start, int nitems, long long total_blocks, cudaStream_t st) {
@@ -534,7 +577,7 @@ void launch_prep_projection(const TcPrep* items, const long long* blk_start, int
 }
 // `steps`: 64-row steps of the problem with the fewest
 void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, int steps, int sm_count, const StepScalars& sc,
-                       unsigned* status, cudaStream_t st) {
+                       int bf16, unsigned* status, cudaStream_t st) {
   // two CTAs fit an SM; each is left four steps at least
   int c = 1;
   while (c < 4 && total_strips * 2 * c <= 2 * (long long)sm_count && steps >= 8 * c) c *= 2;
@@ -546,10 +589,11 @@ void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strip
   at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
   lc.gridDim = dim3((unsigned)(total_strips * c), 1, 1); lc.blockDim = dim3(kProjThreads, 1, 1); lc.dynamicSmemBytes = project_tc_smem(r_n_max);
   lc.stream = st; lc.attrs = &at; lc.numAttrs = c > 1 ? 1 : 0;
-  cudaLaunchKernelEx(&lc, project_tc_kernel, probs, nprobs, sc, status);
+  if (bf16) cudaLaunchKernelEx(&lc, project_tc_kernel<true>, probs, nprobs, sc, status);
+  else cudaLaunchKernelEx(&lc, project_tc_kernel<false>, probs, nprobs, sc, status);
 }
 void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_k_max, int steps, int sm_count, const StepScalars& sc,
-                     unsigned* status, cudaStream_t st) {
+                     int bf16, unsigned* status, cudaStream_t st) {
   // one CTA fits an SM; each is left four steps at least
   int pieces = (int)std::min<long long>(sm_count / total_strips, steps / 4);
   if (pieces < 1) pieces = 1;
@@ -562,8 +606,15 @@ void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips,
   // strips of three lengths, one to an SM either way: 66 instead of 49 us, step 159 instead of 139 us; 98 strips 284 and
   // 241 us; 128 equal strips 312 and 287 us); r_k <= 192 is within 2 % for mixed strips and gains 3 us for equal ones.
   const bool early = (long long)grid.x <= sm_count && r_k_max < 256;
-  if (early) launch_dep(apply_tc_kernel, grid, kApplyThreads, smem, st, probs, nprobs, sc, pieces, status);
-  else apply_tc_kernel<<<grid, kApplyThreads, smem, st>>>(probs, nprobs, sc, pieces, status);
+#define LORDO_APPLY_TC(B)                                                                                          \
+  if (early) launch_dep(apply_tc_kernel<B>, grid, kApplyThreads, smem, st, probs, nprobs, sc, pieces, status);      \
+  else apply_tc_kernel<B><<<grid, kApplyThreads, smem, st>>>(probs, nprobs, sc, pieces, status)
+  if (bf16) {
+    LORDO_APPLY_TC(true);
+  } else {
+    LORDO_APPLY_TC(false);
+  }
+#undef LORDO_APPLY_TC
 }
 
 }  // namespace lordo
