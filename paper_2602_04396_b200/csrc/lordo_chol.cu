@@ -13,14 +13,14 @@
 // While one warp factors the diagonal block of panel k, the others already sum panel k + 1 over the panels
 // before k, so that a panel waits for the newest 32 columns only.
 //
-// What bounds it: the r columns of the diagonal blocks, 300 clocks each (some 70 instructions of one warp),
-// and per panel one trip to L2 for the newest columns, the small products and the barrier; for few CTAs per matrix
-// the fp64 products. One CTA per matrix with a thread per row took 2200 us for r = 512 and 16 matrices, 580 us
-// for r = 256 and 7, 197 us for r = 128 and 56; clusters that summed a whole panel at its turn 654, 131 and 62 us;
-// clusters that sum a panel ahead
-// 360, 99 and 56 us (first launch of a stream), with the next diagonal block staged by the inverting warp and the pivots worked
-// out by every lane 345, 88 and 53 us. (Scaling the block so that rsqrt.approx needs no care, and handing the factoring
-// warp its block summed, both made the column chain slower.)
+// What bounds it: the r columns of the diagonal blocks, 165 to 200 clocks each (some 45 instructions of one warp), and per panel one trip
+// to L2 for the newest columns, the small products and the barrier (14 thousand clocks a panel at r = 256, 17 with 270 clocks a
+// column); for few CTAs per matrix the fp64 products. r = 512 and 16 matrices, r = 256 and 7, r = 128 and 56, us: one CTA per matrix
+// with a thread per row 2200, 580, 197; clusters that summed a whole panel at its turn 654, 131, 62; that sum a panel ahead 312, 77, 46;
+// with the factor free of roots, the diagonal block handed to it summed, units by the panels they have, and a unit instead of
+// the inverse on the factor's scheduler (products of all four units on three schedulers: 296) 265, 66, 43. Every block's sum as
+// quarters of 16 x 16 on four warps was slower (four sums in flight a warp instead of sixteen; 354, 86, 48), and so were units that hand steps
+// to one another (registers; 346, 80, 55).
 #include "lordo_kernels.h"
 #include "lordo_recip.cuh"
 
@@ -32,7 +32,7 @@ constexpr int kCholWarps = 8;                // 255 registers a thread: with 168
 constexpr int kUnits = 4;                    // partial sums of 32 x 32 blocks in flight, one per warp
 constexpr int kLd = 36;                      // row stride of the partial sums and of the inverse: 8 rows x 4 columns meet no bank twice
 constexpr int kPartDoubles = kB * kLd;
-constexpr size_t kCholSmem = sizeof(double) * (size_t)((4 + kUnits) * kPartDoubles + kB * kB + kB + kB * kLd);
+constexpr size_t kCholSmem = sizeof(double) * (size_t)((5 + kUnits) * kPartDoubles + 2 * kB * kB + 3 * kB);
 
 __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b) {
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1},{%2},{%3},{%0,%1};" : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
@@ -108,6 +108,23 @@ __device__ __forceinline__ void block_sum(double (&c)[4][4][2], const float* X, 
   }
 }
 
+// c += X_cols L_cols^T over the quarters slice, slice + of, ... of the 32 columns from `col` on, all loads before the first product.
+__device__ __forceinline__ void newest(double (&c)[4][4][2], const float* X, int xr, const float* L, int lr, int r, int col, int slice, int of) {
+  if (of == 1) {
+    float4 a0[4], b0[4], a1[4], b1[4];
+    fetch16<false>(a0, b0, X, xr, L, lr, r, col);
+    fetch16<false>(a1, b1, X, xr, L, lr, r, col + 16);
+    mma16<false>(c, a0, b0);
+    mma16<false>(c, a1, b1);
+  } else if (of == 2) {
+    float4 a0[4], b0[4];
+    fetch16<false>(a0, b0, X, xr, L, lr, r, col + 16 * slice);
+    mma16<false>(c, a0, b0);
+  } else {
+    for (int h = slice; h < 4; h += of) block_cols<false>(c, X, xr, L, lr, r, col + h * 8);
+  }
+}
+
 __device__ __forceinline__ void clear(double (&c)[4][4][2]) {
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -123,6 +140,13 @@ __device__ __forceinline__ void store_part(double* p, const double (&c)[4][4][2]
     for (int n = 0; n < 4; ++n)
       *reinterpret_cast<double2*>(p + (8 * i + (lane >> 2)) * kLd + 8 * n + 2 * (lane & 3)) = make_double2(c[i][n][0], c[i][n][1]);
 }
+
+// Which unit sums what. Of the t-th block: its place in the matrix, its first unit and the number of its units. Of unit x: its block (the
+// number among the CTA's, -1: none) and its place among the block's units.
+struct Plan {
+  int block[kUnits], first[kUnits], of[kUnits];
+  int tile[kUnits], slice[kUnits];
+};
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t x;
@@ -142,19 +166,23 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
   extern __shared__ __align__(16) double csm[];
   double* dpart = csm;                               // [4] parts of the diagonal block's sum
   double* part = dpart + 4 * kPartDoubles;           // [kUnits] partial sums of the other blocks
-  double* Lc = part + kUnits * kPartDoubles;         // [kB][kB] columns of the diagonal block of L
-  double* dinv = Lc + kB * kB;                       // [kB] 1 / its diagonal
-  double* Li = dinv + kB;                            // [kB][kLd] inverse of the diagonal block
+  double* Xs = part + kUnits * kPartDoubles;         // [kB][kB] columns of the diagonal block's factor, not divided by their pivots
+  double* Ts = Xs + kB * kB;                         // ... and divided
+  double* piv = Ts + kB * kB;                        // [kB] pivots
+  double* floors = piv + kB;                         // [2][kB] least pivots of this panel and the next
+  double* Li = floors + 2 * kB;                      // [kB][kLd] inverse of the diagonal block of L
   __shared__ float wmax[kCholWarps];
+  __shared__ Plan plans[3], late;                    // of this panel, the next and the one after it; of blocks that find no unit at first
   __shared__ float ga[2 * kB * kB];                  // the Gram matrix' diagonal blocks of this panel and the next, for warp 0
 
-  const uint32_t rank = cluster_ctarank(), csize = cluster_nctarank();
+  // handed round, so that the compiler sees that the lanes of a warp agree on what depends on them
+  const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0), csize = __shfl_sync(0xffffffffu, cluster_nctarank(), 0);
   const CholProblem pb = probs[blockIdx.x / csize];
   const int r = pb.r, nb = (r + kB - 1) / kB;
   const float* A = pb.gram;
   float* L = pb.lwork;   // [r][r], blocks below the diagonal
   float* Z = pb.rinv;    // [r][r], upper triangle
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   constexpr int nt = kCholWarps * 32;
 
   // zeros below the diagonal of rinv (this CTA's row blocks), largest diagonal element
@@ -182,16 +210,41 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
   constexpr float kBreakdown = 3e-5f;
   const float abs_floor = md > 0.f ? md * 1e-12f : 1.f;
 
-  // Warps 0 and 4 (one scheduler's fp64 pipe, kept free of the products) factor and invert the diagonal block,
-  // warps 1 and 2 sum the diagonal block, the other four the row blocks.
-  const int u = warp == 3 ? 0 : warp > 4 ? warp - 4 : kUnits;
+  // Warp 0 factors the diagonal block, warp 7 inverts it, warps 1 and 2 sum it, the other four are the units that sum the row blocks. The
+  // factor shares its scheduler with the last unit, which is idle first.
+  const int u = warp == 3 ? 0 : warp == 5 ? 1 : warp == 6 ? 2 : warp == 4 ? 3 : kUnits;
   const int own = (int)rank < nb ? (nb - 1 - (int)rank) / (int)csize + 1 : 0;  // this CTA's row blocks: rank, rank + csize, ...
-  const bool ahead = own <= kUnits;  // every block of a panel has a warp of its own, so its sum may begin early
+  const bool ahead = own <= kUnits;  // every block of a panel has a unit of its own, so its sum may begin early
   auto has = [&](int k) { return k % (int)csize == (int)rank; };
   auto tiles = [&](int k) { return own - (has(k) ? 1 : 0); };                  // ... without the block of the diagonal
   auto tile_block = [&](int k, int t) { return (int)rank + (int)csize * ((has(k) && t >= k / (int)csize) ? t + 1 : t); };
-  // slices of the summation index per block, so that a batch of `cnt` blocks has work for every warp
-  auto slices = [&](int cnt) { return cnt > 0 && cnt <= kUnits ? kUnits / cnt : 1; };
+  // The panels behind the blocks' sums, dealt out to the units (a block above the diagonal has panels from itself on): every block has
+  // a unit, those left over go, one after the other, to the block with the most panels a unit. With as many units for each
+  // block one was idle with three blocks, and a block of two panels had as many as one of fourteen. Laid down by one thread two panels
+  // ahead.
+  auto lay_out = [&](Plan& pl, int k, int t0, int cnt) {
+    int n[kUnits], of[kUnits];
+    for (int t = 0; t < kUnits; ++t) {
+      const int b = t < cnt ? tile_block(k, t0 + t) : 0;
+      pl.block[t] = b;
+      n[t] = b > k ? k : k - b;
+      of[t] = t < cnt ? 1 : 0;
+    }
+    for (int left = cnt > 0 ? kUnits - cnt : 0; left > 0; --left) {
+      int best = 0;
+      for (int t = 1; t < cnt; ++t)
+        if (n[t] * of[best] > n[best] * of[t]) best = t;
+      ++of[best];
+    }
+    for (int t = 0, at = 0; t < kUnits; ++t) {
+      pl.first[t] = at;
+      pl.of[t] = of[t];
+      for (int x = 0; x < of[t]; ++x) { pl.tile[at + x] = t; pl.slice[at + x] = x; }
+      at += of[t];
+    }
+    if (cnt == 0)
+      for (int x = 0; x < kUnits; ++x) pl.tile[x] = -1;
+  };
   auto a_diag = [&](int k, int j) {  // element (lane, j) of the Gram matrix' diagonal block; A is symmetric
     const int k0 = k * kB, kw = r - k0 < kB ? r - k0 : kB;
     return lane < kw && j < kw ? A[(size_t)(k0 + j) * r + k0 + lane] : (lane == j ? 1.f : 0.f);
@@ -204,9 +257,14 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
 #pragma unroll
     for (int j = 0; j < kB; ++j) t[j] = a_diag(k, j);
 #pragma unroll
-    for (int j = 0; j < kB; ++j) ga[((k & 1) * kB + j) * kB + lane] = t[j];
+    for (int j = 0; j < kB; ++j) {
+      ga[((k & 1) * kB + j) * kB + lane] = t[j];
+      if (lane == j) floors[(k & 1) * kB + j] = k * kB + j < r ? (double)fmaxf(kBreakdown * t[j], abs_floor) : 0.0;
+    }
   };
   if (warp == 0) stage_diag(0);
+  if (warp > 1 && warp < 4 && lane == 0 && warp - 2 < nb) lay_out(plans[warp - 2], warp - 2, 0, min(tiles(warp - 2), kUnits));
+  __syncthreads();
 
 #pragma unroll 1
   for (int k = 0; k < nb; ++k) {
@@ -216,176 +274,201 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
 
     // ---- the newest 32 columns (or, without a head start, all of them) and the sums to shared memory
     if (u == kUnits) {
-      const int w = warp == 4 ? 3 : warp;
+      const int w = warp == 7 ? 3 : warp;
       if (k > 0) block_cols<true>(c, L, k0, L, k0, r, k0 - kB + w * 8);
       store_part(dpart + w * kPartDoubles, c);
       clear(c);
-    } else if (u < first * slices(first)) {
-      const int s = slices(first), b = tile_block(k, u / s), sl = u % s;
-      const float* X = b > k ? L : Z;
-      if (!ahead) block_sum<false>(c, X, b * kB, L, k0, r, (b > k ? 0 : b) + sl, k, s);
-      else if (k > 0)
-        for (int h = sl; h < 4; h += s) block_cols<false>(c, X, b * kB, L, k0, r, k0 - kB + h * 8);
-      store_part(part + u * kPartDoubles, c);
-      clear(c);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {  // what is left of the diagonal block, for warp 0: eight columns each
+        const double* q = dpart + (w * 8 + j) * kLd + lane;  // symmetric too
+        Ts[(w * 8 + j) * kB + lane] =
+            (double)ga[((k & 1) * kB + w * 8 + j) * kB + lane] - ((q[0] + q[kPartDoubles]) + (q[2 * kPartDoubles] + q[3 * kPartDoubles]));
+      }
+      if (warp == 0) asm volatile("bar.sync 10, 128;" ::: "memory");
+      else asm volatile("bar.arrive 10, 128;" ::: "memory");
+    } else {
+      const Plan& pl = plans[k % 3];
+      const int t = pl.tile[u];
+      if (t >= 0) {
+        const int b = pl.block[t], sl = pl.slice[u], of = pl.of[t];
+        const float* X = b > k ? L : Z;
+        if (!ahead) block_sum<false>(c, X, b * kB, L, k0, r, (b > k ? 0 : b) + sl, k, of);
+        else if (k > 0) newest(c, X, b * kB, L, k0, r, k0 - kB, sl, of);
+        store_part(part + u * kPartDoubles, c);
+        clear(c);
+      }
     }
 
     if (warp == 0) {
-      // Factor of the diagonal block: lane i holds row i of what is left of the block. Every lane works out every pivot d
-      // for itself, from the element b beside the pivot before it and the diagonal element D that were handed round a column
-      // earlier: D - b b / d = D - b b r0 (1 + e), see lordo_recip.cuh, and the next column's elements likewise; the square
-      // root, the column of L and the update of the columns behind the next one fill the gaps. (No chain is what is left: a column is some 70 instructions of one warp, which issues one
-      // every four clocks. Handing two elements round and updating the columns behind one column late: slower, registers.)
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      const float* gk = ga + (k & 1) * kB * kB;
+      // Factor X D^-1 X^T of the diagonal block: lane i holds row i of what is left of the block, X_j its column j, d_j the pivot. Every lane
+      // works out every pivot for itself, from the element b beside the pivot before it and the diagonal element D that were
+      // handed round a column earlier: D - b b / d = D - b b r0 (1 + e), see lordo_recip.cuh. Nothing here is scaled by a root: the
+      // columns behind X_j need X_j, which is in shared memory before its pivot is known, and X_j / d_j. With the roots on the way a column
+      // took 270 clocks, now 165: some 45 instructions of one warp.
+      const double* fl = floors + (k & 1) * kB;
       double a[kB], dg = 1.0;
 #pragma unroll
       for (int j = 0; j < kB; ++j) {
-        const double* q = dpart + j * kLd + lane;  // symmetric too
-        a[j] = (double)gk[j * kB + lane] - ((q[0] + q[kPartDoubles]) + (q[2 * kPartDoubles] + q[3 * kPartDoubles]));
+        a[j] = Ts[j * kB + lane];
         if (lane == j) dg = a[j];
       }
+      Xs[lane] = a[0];
+      __syncwarp();
       bool broke = false;
-      auto pivot = [&](double x, int j) {  // x, or the floor where it is not above it (NaN neither)
-        const double fl = j < kw ? (double)fmaxf(kBreakdown * gk[j * kB + j], abs_floor) : 0.0;
+      auto pivot = [&](double x, double least) {  // x, or the floor where it is not above it (NaN neither)
         const int h = __double2hiint(x);
-        const bool low = !(h > __double2hiint(fl) && h < 0x7FF00000);
+        const bool low = !(h > __double2hiint(least) && h < 0x7FF00000);
         broke |= low;
-        return low ? fl : x;
+        return low ? least : x;
       };
-      double d = pivot(__shfl_sync(0xffffffffu, dg, 0), 0);
+      double d = pivot(__shfl_sync(0xffffffffu, dg, 0), fl[0]);
       double b = __shfl_sync(0xffffffffu, a[0], 1), D = __shfl_sync(0xffffffffu, dg, 1);
 #pragma unroll
       for (int j = 0; j < kB; ++j) {
         double r0, e, dn = 1.0;
         recip_parts(d, r0, e);
-        const double aj = a[j];
-        auto minus = [&](double x, double pq) { const double p = pq * r0; return fma(-p, e, x - p); };  // x - pq / d
+        const double t0 = a[j] * r0, t = fma(t0, e, t0);  // X_j / d_j
         if (j + 1 < kB) {
-          dn = minus(D, b * b);
-          a[j + 1] = minus(a[j + 1], aj * b);  // rows from j on; those above are done with
-          dg = minus(dg, aj * aj);
+          const double p = (b * b) * r0;
+          dn = fma(-p, e, D - p);
+          a[j + 1] = fma(-t, b, a[j + 1]);
+          dg = fma(-t, a[j], dg);
+          Xs[(j + 1) * kB + lane] = a[j + 1];
         }
         if (j + 2 < kB) {
           b = __shfl_sync(0xffffffffu, a[j + 1], j + 2);
           D = __shfl_sync(0xffffffffu, dg, j + 2);
         }
-        const double y = recip_sqrt(d);  // 1 / L_jj
-        const double l = lane == j ? d * y : (lane > j ? aj * y : 0.0);
-        Lc[j * kB + lane] = l;
-        if (lane == 0) dinv[j] = y;
-        if (j + 1 < kB) d = pivot(dn, j + 1);
+        Ts[j * kB + lane] = t;
+        if (lane == 0) piv[j] = d;
+        if (j + 1 < kB) d = pivot(dn, fl[j + 1]);
         __syncwarp();
-        if (j % 8 == 7) asm volatile("bar.arrive %0, 64;" ::"r"(2 + j / 8) : "memory");  // eight more columns for the inverse
+        if (j % 4 == 3) asm volatile("bar.arrive %0, 64;" ::"r"(2 + j / 4) : "memory");  // four more columns for the inverse
 #pragma unroll
         for (int j2 = (j + 2) & ~1; j2 < kB; j2 += 2) {
-          const double2 v = *reinterpret_cast<const double2*>(Lc + j * kB + j2);
-          if (j2 > j + 1) a[j2] -= l * v.x;
-          a[j2 + 1] -= l * v.y;
+          const double2 v = *reinterpret_cast<const double2*>(Xs + j * kB + j2);
+          if (j2 > j + 1) a[j2] = fma(-t, v.x, a[j2]);
+          a[j2 + 1] = fma(-t, v.y, a[j2 + 1]);
         }
       }
       if (broke && rank == 0 && lane == 0) atomicOr(status, LORDO_FLAG_QR_BREAKDOWN);
       clear(c);  // not held in registers meanwhile
     } else if (warp < 3) {
-      asm volatile("bar.arrive 1, 128;" ::: "memory");
+      if (warp == 2 && k + 1 < nb) stage_diag(k + 1);
+      if (warp == 1 && lane == 0 && k + 2 < nb) lay_out(plans[(k + 2) % 3], k + 2, 0, min(tiles(k + 2), kUnits));
+      __syncwarp();
       if (k + 1 < nb) block_sum<true>(c, L, k0 + kB, L, k0 + kB, r, warp - 1, k, 2);
-    } else if (warp == 4) {
-      asm volatile("bar.arrive 1, 128;" ::: "memory");
-      if (k + 1 < nb) stage_diag(k + 1);  // before the first columns are there
-      // inverse of the diagonal block, column `lane`, eight columns of the factor behind warp 0
-      double x[kB];
+    } else if (warp == 7) {
+      // inverse of the diagonal block, column `lane`, four columns of the factor behind warp 0; its rows are divided by the pivots' roots
+      double x[kB], y = 0.0;
 #pragma unroll
       for (int i = 0; i < kB; ++i) x[i] = lane == i ? 1.0 : 0.0;
 #pragma unroll
       for (int p = 0; p < kB; ++p) {
-        if (p % 8 == 0) asm volatile("bar.sync %0, 64;" ::"r"(2 + p / 8) : "memory");
-        x[p] *= dinv[p];
-        Li[p * kLd + lane] = x[p];
+        if (p % 4 == 0) {
+          asm volatile("bar.sync %0, 64;" ::"r"(2 + p / 4) : "memory");
+          y = recip_sqrt(piv[p + (lane & 3)]);
+        }
+        Li[p * kLd + lane] = x[p] * __shfl_sync(0xffffffffu, y, p & 3);
 #pragma unroll
         for (int i = (p + 1) & ~1; i < kB; i += 2) {
-          const double2 v = *reinterpret_cast<const double2*>(Lc + p * kB + i);
-          if (i > p) x[i] -= v.x * x[p];
-          x[i + 1] -= v.y * x[p];
+          const double2 v = *reinterpret_cast<const double2*>(Ts + p * kB + i);
+          if (i > p) x[i] = fma(-v.x, x[p], x[i]);
+          x[i + 1] = fma(-v.y, x[p], x[i + 1]);
         }
       }
       clear(c);
     } else if (ahead && k + 1 < nb) {
-      const int n1 = tiles(k + 1), s = slices(n1);
-      if (u < n1 * s) {
-        const int b = tile_block(k + 1, u / s), sl = u % s;
-        block_sum<false>(c, b > k + 1 ? L : Z, b * kB, L, k0 + kB, r, (b > k + 1 ? 0 : b) + sl, k, s);
+      const Plan& pl = plans[(k + 1) % 3];
+      const int t = pl.tile[u];
+      if (t >= 0) {
+        const int b = pl.block[t];
+        block_sum<false>(c, b > k + 1 ? L : Z, b * kB, L, k0 + kB, r, (b > k + 1 ? 0 : b) + pl.slice[u], k, pl.of[t]);
       }
     }
 
-    // ---- Z_k = M Lkk^-T, eight rows of a block per warp and turn; the panel's own rows of rinv with the first batch
+    // ---- Z_k = M Lkk^-T, eight rows of a block per warp and turn; the panel's own rows of rinv are Lkk^-T itself
     const int lr = lane >> 2, lc = lane & 3;
     auto gram_init = [&](int b, int row, float (&g)[8]) {  // below the diagonal k0 + 32 <= row, so the columns exist
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) g[kk] = b > k && row < r ? A[(size_t)row * r + k0 + kk * 4 + lc] : 0.f;
     };
-    float g[8];
-    if (warp < first * 4) gram_init(tile_block(k, warp >> 2), tile_block(k, warp >> 2) * kB + (warp & 3) * 8 + lr, g);
-    __syncthreads();  // the inverse of the diagonal block and the sums of the first batch are there
-    for (int base = 0; base < ntiles || base == 0; base += kUnits) {
-      const int cnt = ntiles - base < kUnits ? ntiles - base : kUnits;
-      const int s = slices(cnt);
-      if (base > 0) {
-        __syncthreads();  // the batch before is done with its sums
-        if (u < cnt * s) {
-          const int b = tile_block(k, base + u / s);
-          block_sum<false>(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + u % s, k, s);
-          store_part(part + u * kPartDoubles, c);
-          clear(c);
+    auto put = [&](int b, int row, int col, float x, float y) {
+      *reinterpret_cast<float2*>((b > k ? L : Z) + (size_t)row * r + k0 + col) = make_float2(x, y);
+      if (b <= k && pb.rinv16) {
+        __nv_bfloat16* o16 = pb.rinv16 + (size_t)row * r + k0 + col;
+#pragma unroll
+        for (int p = 0; p < 3; ++p, o16 += pb.plane) {
+          const uint32_t w = pack_bf16x2(x, y);
+          *reinterpret_cast<uint32_t*>(o16) = w;
+          x -= __uint_as_float(w << 16);
+          y -= __uint_as_float(w & 0xFFFF0000u);
         }
-        __syncthreads();
       }
-      const int strips = cnt * 4 + (base == 0 && has_k ? 4 : 0);
-      for (int q = warp; q < strips; q += kCholWarps) {
-        const int t = q >> 2, r8 = (q & 3) * 8;
-        const bool diag = t == cnt;
-        const int b = diag ? k : tile_block(k, base + t);
-        const int row = b * kB + r8 + lr;
-        if (!diag && (q != warp || base > 0)) gram_init(b, row, g);
-        double z[4][2];
+    };
+    // The 32 columns are summed in two halves side by side: a product waits 26 clocks for the one before it in its sum.
+    auto finish = [&](const Plan& pl, int t, int r8, const float (&g)[8]) {
+      const int b = pl.block[t], of = pl.of[t];
+      double z[2][4][2], m[8];
 #pragma unroll
-        for (int n = 0; n < 4; ++n) z[n][0] = z[n][1] = 0.0;
+      for (int n = 0; n < 8; ++n) z[n >> 2][n & 3][0] = z[n >> 2][n & 3][1] = 0.0;
+      const double* q0 = part + pl.first[t] * kPartDoubles + (r8 + lr) * kLd + lc;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const int col = kk * 4 + lc;
-          double m;
-          if (diag) {
-            m = r8 + lr == col ? 1.0 : 0.0;
-          } else {
-            const double* q0 = part + (size_t)t * s * kPartDoubles + (r8 + lr) * kLd + col;
-            double sum = 0.0;
+      for (int kk = 0; kk < 8; ++kk) m[kk] = (double)g[kk];
 #pragma unroll
-            for (int sl = 0; sl < kUnits; ++sl)
-              if (sl < s) sum += q0[(size_t)sl * kPartDoubles];
-            m = (double)g[kk] - sum;
-          }
+      for (int sl = 0; sl < kUnits; ++sl)
+        if (sl < of) {
 #pragma unroll
-          for (int n = 0; n < 4; ++n) dmma(z[n][0], z[n][1], m, Li[(8 * n + lr) * kLd + col]);
+          for (int kk = 0; kk < 8; ++kk) m[kk] -= q0[(size_t)sl * kPartDoubles + kk * 4];
         }
-        if (row < r) {
-          float* out = (b > k ? L : Z) + (size_t)row * r + k0;
 #pragma unroll
-          for (int n = 0; n < 4; ++n) {
-            const int col = 8 * n + 2 * lc;
-            if (col >= kw) continue;
-            float x = (float)z[n][0], y = (float)z[n][1];
-            *reinterpret_cast<float2*>(out + col) = make_float2(x, y);
-            if (b <= k && pb.rinv16) {
-              __nv_bfloat16* o16 = pb.rinv16 + (size_t)row * r + k0 + col;
+      for (int kk = 0; kk < 8; ++kk)
 #pragma unroll
-              for (int p = 0; p < 3; ++p, o16 += pb.plane) {
-                const uint32_t w = pack_bf16x2(x, y);
-                *reinterpret_cast<uint32_t*>(o16) = w;
-                x -= __uint_as_float(w << 16);
-                y -= __uint_as_float(w & 0xFFFF0000u);
-              }
-            }
-          }
+        for (int n = kk / 2; n < 4; ++n) dmma(z[kk & 1][n][0], z[kk & 1][n][1], m[kk], Li[(8 * n + lr) * kLd + kk * 4 + lc]);  // zeros right of its diagonal
+      const int row = b * kB + r8 + lr;
+      if (row < r) {
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          const int col = 8 * n + 2 * lc;
+          if (col < kw) put(b, row, col, (float)(z[0][n][0] + z[1][n][0]), (float)(z[0][n][1] + z[1][n][1]));
         }
+      }
+    };
+    float g[2][8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (warp + 8 * h < first * 4) {
+        const int b = plans[k % 3].block[(warp + 8 * h) >> 2];
+        gram_init(b, b * kB + (warp & 3) * 8 + lr, g[h]);
+      }
+    __syncthreads();  // the inverse of the diagonal block and the sums of the first blocks are there
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (warp + 8 * h < first * 4) finish(plans[k % 3], (warp + 8 * h) >> 2, (warp & 3) * 8, g[h]);
+    if (has_k) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = warp * 4 + 2 * h + (lane >> 4), col = 2 * (lane & 15);
+        if (row < kw && col < kw) put(k, k0 + row, col, (float)Li[col * kLd + row], (float)Li[(col + 1) * kLd + row]);
+      }
+    }
+    for (int base = kUnits; base < ntiles; base += kUnits) {
+      const int cnt = ntiles - base < kUnits ? ntiles - base : kUnits;
+      __syncthreads();  // the blocks before are done with their sums
+      if (tid == 0) lay_out(late, k, base, cnt);
+      __syncthreads();
+      if (u < kUnits) {
+        const int t = late.tile[u], b = late.block[t];
+        block_sum<false>(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + late.slice[u], k, late.of[t]);
+        store_part(part + u * kPartDoubles, c);
+        clear(c);
+      }
+      __syncthreads();
+      for (int q = warp; q < cnt * 4; q += kCholWarps) {
+        const int b = late.block[q >> 2];
+        gram_init(b, b * kB + (q & 3) * 8 + lr, g[0]);
+        finish(late, q >> 2, (q & 3) * 8, g[0]);
       }
     }
     // the panel is in memory for every CTA of the cluster
