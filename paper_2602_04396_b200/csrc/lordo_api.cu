@@ -119,9 +119,9 @@ struct lordo_ctx {
   char* d_tc_bf16 = nullptr;  // all bf16 operand copies, zeroed once by lordo_init
   size_t tc_bf16_bytes = 0;
   long long tc_strips = 0, tc_pairs = 0, prep_blocks = 0;
-  int tc_rn_max = 0, tc_rk_max = 0, tc_steps_min = 0;  // largest padded ranks, fewest 64-row steps
+  int tc_rn_max = 0, tc_steps_min = 0;  // largest padded rank, fewest 64-row steps
   // TMA-fed kernels (bf16 storage): tensor maps per matrix, gradient maps re-encoded per pointer change
-  bool tma = false;
+  bool tma = false;              // bf16 storage: projection and refresh too; with fp32 storage the update alone is fed by TMA
   int sm_count = 0;
   TmaMatMaps* d_maps = nullptr;
   TmaGradMaps* d_gmaps = nullptr;
@@ -156,7 +156,7 @@ struct lordo_ctx {
 
   // pinned host staging
   const void** h_Gtab = nullptr;  // pinned, two slots of n_mats entries
-  unsigned* h_status = nullptr;   // pinned
+  unsigned* h_status = nullptr;   // pinned (this and h_gmaps: in h_Gtab's block)
   std::vector<const void*> last_G;
   cudaEvent_t g_slot_ev[2] = {nullptr, nullptr};  // behind the last copy out of each staging slot
   bool g_slot_used[2] = {false, false};
@@ -197,16 +197,16 @@ tmap_encode_fn tmap_encoder() {
   return fn;
 }
 
-// bf16 tensor [d2][d1][d0] (d0 contiguous), box b0 x b1 x 1, written into 128 bytes at `out`.
-bool encode_map3(unsigned char* out, const void* base, long long d0, long long d1, long long d2, int b0, int b1, bool swizzle) {
+// bf16 (or fp32) tensor [d2][d1][d0] (d0 contiguous), box b0 x b1 x 1, written into 128 bytes at `out`.
+bool encode_map3(unsigned char* out, const void* base, long long d0, long long d1, long long d2, int b0, int b1, bool swizzle, bool f32 = false) {
   tmap_encode_fn fn = tmap_encoder();
   if (!fn) return false;
   alignas(64) CUtensorMap tm;
   const cuuint64_t dims[3] = {(cuuint64_t)d0, (cuuint64_t)d1, (cuuint64_t)d2};
-  const cuuint64_t strides[2] = {(cuuint64_t)d0 * 2, (cuuint64_t)d0 * (cuuint64_t)d1 * 2};
+  const cuuint64_t size = f32 ? 4 : 2, strides[2] = {(cuuint64_t)d0 * size, (cuuint64_t)d0 * (cuuint64_t)d1 * size};
   const cuuint32_t box[3] = {(cuuint32_t)b0, (cuuint32_t)b1, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = fn(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+  const CUresult r = fn(&tm, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return false;
@@ -385,7 +385,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
 
   // ---------------- tensor-core operand copies and problem table ----------------
   c->h_tc.clear(); c->h_prep.clear(); c->h_prep_start.assign(1, 0);
-  c->tc_strips = 0; c->tc_pairs = 0; c->tc_rn_max = 0; c->tc_rk_max = 0; c->tc_steps_min = 1 << 30;
+  c->tc_strips = 0; c->tc_pairs = 0; c->tc_rn_max = 0; c->tc_steps_min = 1 << 30;
   std::vector<size_t> h_prep_first(n_mats, 0);  // first entry of a matrix in h_prep
   if (c->tc) {
     auto up = [](long long x, long long q) { return (x + q - 1) / q * q; };
@@ -403,7 +403,6 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       const int nsplit = (cfg.w_dtype == LORDO_BF16 && r_n > 256) ? 2 : 1;  // TMA-fed projection: one strip per half of the rank
       float* dcol2 = nsplit == 2 ? cv.take<float>((size_t)K * md.ln) : nullptr;
       if (r_n > c->tc_rn_max) c->tc_rn_max = r_n;
-      if (r_k > c->tc_rk_max) c->tc_rk_max = r_k;
       c->tc_steps_min = std::min(c->tc_steps_min, m_k / 64);
       h_prep_first[i] = c->h_prep.size();
       for (int k = 0; k < copies; ++k) {
@@ -444,8 +443,8 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
     c->tc_bf16_bytes = cv.off - bf16_begin;
     c->prep_blocks = c->h_prep_start.back();
     c->d_tc_probs = cv.take<TcProblem>(c->h_tc.size());
-    if (c->tma)
-      for (int l = 0; l < 2; ++l) {
+    for (int l = 0; l < 2; ++l)
+      if (c->tma || l > 0) {  // fp32 storage: the update alone is fed by TMA
         c->d_segs[l] = cv.take<TcSeg>((size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers));
         c->d_seg_start[l] = cv.take<int>(kMaxWorkers + 1);
       }
@@ -1098,17 +1097,19 @@ int set_gradients(lordo_ctx* c, const void* const* G, cudaStream_t st) {
   const int slot = c->g_slot ^ 1;
   if (c->g_slot_used[slot]) CUDA_OK(c, cudaEventSynchronize(c->g_slot_ev[slot]));
   const void** tab = c->h_Gtab + (size_t)slot * c->n_mats;
-  TmaGradMaps* gm = c->tma ? c->h_gmaps + (size_t)slot * c->n_mats : nullptr;
-  if (c->tma) {
+  TmaGradMaps* gm = c->tc ? c->h_gmaps + (size_t)slot * c->n_mats : nullptr;
+  if (c->tc) {
     for (int i = 0; i < c->n_mats; ++i) {
       const lordo_mat& a = c->mats[i];
-      if (!encode_map3(gm[i].g_sw, G[i], a.n, a.m, c->K, 64, 64, true) || !encode_map3(gm[i].g_kb, G[i], a.n, a.m, c->K, 64, 128, true))
+      const bool good = !c->tma ? encode_map3(gm[i].g_kb, G[i], a.n, a.m, c->K, 128, 32, false, true)
+                                : encode_map3(gm[i].g_sw, G[i], a.n, a.m, c->K, 64, 64, true) && encode_map3(gm[i].g_kb, G[i], a.n, a.m, c->K, 64, 128, true);
+      if (!good)
         return fail(c, LORDO_ERR_CUDA, "tensor map encoding failed for a gradient");
     }
   }
   for (int i = 0; i < c->n_mats; ++i) tab[i] = G[i];
   cudaError_t e = cudaMemcpyAsync(c->d_Gtab, tab, sizeof(void*) * c->n_mats, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && c->tma) e = cudaMemcpyAsync(c->d_gmaps, gm, sizeof(TmaGradMaps) * c->n_mats, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && c->tc) e = cudaMemcpyAsync(c->d_gmaps, gm, sizeof(TmaGradMaps) * c->n_mats, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaEventRecord(c->g_slot_ev[slot], st);
   if (e != cudaSuccess) {
     // the device tables may be half written: force the next call to write them again
@@ -1192,10 +1193,14 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
   if (need > workspace_bytes) { delete c; return LORDO_ERR_NOMEM; }
 
   auto bail = [&](int code) { lordo_destroy(c); return code; };
-  if (cudaHostAlloc((void**)&c->h_Gtab, 2 * sizeof(void*) * c->n_mats, cudaHostAllocDefault) != cudaSuccess) return bail(LORDO_ERR_NOMEM);
+  {  // one pinned block: an allocation takes some 80 us
+    const size_t status_at = (2 * sizeof(void*) * c->n_mats + 255) & ~size_t(255), maps_at = status_at + 256;
+    if (cudaHostAlloc((void**)&c->h_Gtab, maps_at + (c->tc ? 2 * sizeof(TmaGradMaps) * c->n_mats : 0), cudaHostAllocDefault) != cudaSuccess) return bail(LORDO_ERR_NOMEM);
+    c->h_status = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(c->h_Gtab) + status_at);
+    if (c->tc) c->h_gmaps = reinterpret_cast<TmaGradMaps*>(reinterpret_cast<char*>(c->h_Gtab) + maps_at);
+  }
   for (int sl = 0; sl < 2; ++sl)
     if (cudaEventCreateWithFlags(&c->g_slot_ev[sl], cudaEventDisableTiming) != cudaSuccess) return bail(LORDO_ERR_CUDA);
-  if (cudaHostAlloc((void**)&c->h_status, 256, cudaHostAllocDefault) != cudaSuccess) return bail(LORDO_ERR_NOMEM);
 
   std::vector<long long> cs, ms, wb, sb;
   prefix_arrays(c->cfg, cs, ms, wb, sb);
@@ -1228,13 +1233,13 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
     INIT_CUDA(chol_configure());
   }
   if (c->tc) {
-    if (!c->tma) INIT_CUDA(tc_configure(c->tc_rn_max, c->tc_rk_max));  // register-staged kernels (fp32 storage)
+    if (!c->tma) INIT_CUDA(tc_configure(c->tc_rn_max));  // register-staged kernels (fp32 storage)
     INIT_CUDA(cudaMemsetAsync(c->d_tc_bf16, 0, c->tc_bf16_bytes, st));
     INIT_CUDA(cudaMemcpyAsync(c->d_tc_probs, c->h_tc.data(), sizeof(TcProblem) * c->h_tc.size(), cudaMemcpyHostToDevice, st));
     INIT_CUDA(cudaMemcpyAsync(c->d_tc_prep, c->h_prep.data(), sizeof(TcPrep) * c->h_prep.size(), cudaMemcpyHostToDevice, st));
     INIT_CUDA(cudaMemcpyAsync(c->d_prep_start, c->h_prep_start.data(), 8 * c->h_prep_start.size(), cudaMemcpyHostToDevice, st));
-    if (c->tma) {
-      if (c->sm_count < 2) return bail(LORDO_ERR_UNSUPPORTED);  // the projection and the refresh products run as CTA pairs
+    {
+      if (c->tma && c->sm_count < 2) return bail(LORDO_ERR_UNSUPPORTED);  // the projection and the refresh products run as CTA pairs
       std::vector<TmaMatMaps> hm(nm);
       bool good = tmap_encoder() != nullptr;
       const bool loc = c->cfg.variant == LORDO_LOCAL;
@@ -1243,6 +1248,13 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
         const TcProblem& tp = c->h_tc[(size_t)i * c->K];  // worker 0 of matrix i: base pointers of the copies
         const int copies = loc ? c->K : 1;
         std::memset(&hm[i], 0, sizeof(TmaMatMaps));
+        if (!c->tma) {  // fp32 storage: tiles of 32 rows x 128 columns, as they are, handed back eight rows at a time
+          good = good && encode_map3(hm[i].w_kb, md.W, md.n, md.m, c->K, 128, 32, false, true) && encode_map3(hm[i].w_st, md.W, md.n, md.m, c->K, 128, 8, false, true);
+          if (c->cfg.error_feedback)
+            good = good && encode_map3(hm[i].e_kb, md.E, md.n, md.m, c->K, 128, 32, false, true) && encode_map3(hm[i].e_st, md.E, md.n, md.m, c->K, 128, 8, false, true);
+          good = good && encode_map3(hm[i].p16, tp.P16, tp.r_k, tp.m_k, copies, 64, 32, true);
+          continue;
+        }
         if (md.E) {
           good = good && encode_map3(hm[i].e_sw, md.E, md.n, md.m, c->K, 64, 64, true);
           good = good && encode_map3(hm[i].e_st, md.E, md.n, md.m, c->K, 64, 16, true);
@@ -1284,17 +1296,18 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
       }
       if (good) {
         INIT_CUDA(cudaMemcpyAsync(c->d_maps, hm.data(), sizeof(TmaMatMaps) * nm, cudaMemcpyHostToDevice, st));
-        INIT_CUDA(cudaStreamSynchronize(st));
-        INIT_CUDA(tma_configure());
-        INIT_CUDA(rotate_configure());
+        INIT_CUDA(c->tma ? tma_configure() : tma_configure_f32());
+        if (c->tma) INIT_CUDA(rotate_configure());
         int right = 0;
         for (const lordo_mat& a : c->mats) right += a.side;
         c->tma_side = right == 0 ? 0 : right == nm ? 1 : 2;
-        for (int l = 0; l < 2; ++l) {
+        std::vector<TcSeg> seg_list[2];
+        std::vector<int> seg_start[2];
+        for (int l = c->tma ? 0 : 1; l < 2; ++l) {
           std::vector<WorkItem> items;
           for (int x = 0; x < (int)c->h_tc.size(); ++x) {
             const TcProblem& tp = c->h_tc[x];
-            const int steps = tp.m_k / 64, strips = (tp.n + 127) / 128;
+            const int steps = l > 0 && !c->tma ? (tp.m + 31) / 32 : tp.m_k / 64, strips = (tp.n + 127) / 128;  // fp32 storage: half the rows a step
             if (l == 0) {  // the longer of the two chains, k steps and moment update (16 ranks about as long as half a step)
               const int half = tp.r_n < 256 ? tp.r_n : 256;
               for (int s2 = 0; s2 < tp.nsplit * ((strips + 1) / 2); ++s2) items.push_back({x, s2, 1, std::max((double)steps, half / 32.0) + 1.0});
@@ -1302,8 +1315,8 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
               for (int s2 = 0; s2 < strips; ++s2) items.push_back({x, s2, steps, (double)steps});
             }
           }
-          std::vector<TcSeg> list;
-          std::vector<int> start;
+          std::vector<TcSeg>& list = seg_list[l];
+          std::vector<int>& start = seg_start[l];
           long long steps = 0;
           for (const WorkItem& it : items) steps += it.len;
           // SMs whose update keeps the memory busy; two sweeps (r > 256) are bound by what an SM pulls out of L2
@@ -1316,9 +1329,8 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
           if (list.size() > (size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers)) return bail(LORDO_ERR_NOMEM);
           INIT_CUDA(cudaMemcpyAsync(c->d_segs[l], list.data(), sizeof(TcSeg) * list.size(), cudaMemcpyHostToDevice, st));
           INIT_CUDA(cudaMemcpyAsync(c->d_seg_start[l], start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, st));
-          INIT_CUDA(cudaStreamSynchronize(st));
         }
-        if (cudaHostAlloc((void**)&c->h_gmaps, 2 * sizeof(TmaGradMaps) * nm, cudaHostAllocDefault) != cudaSuccess) return bail(LORDO_ERR_NOMEM);
+        INIT_CUDA(cudaStreamSynchronize(st));  // the tables above leave the host's stack
       } else {
         return bail(LORDO_ERR_CUDA);  // tensor maps could not be encoded (driver without cuTensorMapEncodeTiled?)
       }
@@ -1404,7 +1416,7 @@ int lordo_inner_step(lordo_ctx* c, const void* const* G, float lr, float beta1, 
         ProfScope ps(c, st, PC_APPLY);
         // 256 < r <= 512: the error-feedback sweep, then the model-update sweep; else one sweep does both
         for (int mode = big ? (c->cfg.error_feedback ? 1 : 2) : 0; mode <= (big ? 2 : 0); ++mode) {
-          launch_apply_tma(c->d_tc_probs, c->d_segs[1], c->d_seg_start[1], c->seg_workers[1], c->d_maps, c->d_gmaps, ss, mode, c->tma_side,
+          launch_apply_tma(c->d_tc_probs, c->d_segs[1], c->d_seg_start[1], c->seg_workers[1], c->d_maps, c->d_gmaps, ss, 0, mode, c->tma_side,
                            c->d_status, st);
           c->launches += 1;
         }
@@ -1418,8 +1430,7 @@ int lordo_inner_step(lordo_ctx* c, const void* const* G, float lr, float beta1, 
     }
     {
       ProfScope ps(c, st, PC_APPLY);
-      launch_apply_tc(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips, c->tc_rk_max, c->tc_steps_min, c->sm_count, ss, c->cfg.w_dtype == LORDO_BF16,
-                      c->d_status, st);
+      launch_apply_tma(c->d_tc_probs, c->d_segs[1], c->d_seg_start[1], c->seg_workers[1], c->d_maps, c->d_gmaps, ss, 1, 0, 0, c->d_status, st);
     }
     }
     c->launches += 2;
@@ -1663,8 +1674,6 @@ const char* lordo_last_error(const lordo_ctx* c) { return c ? c->err.c_str() : "
 int lordo_destroy(lordo_ctx* c) {
   if (!c) return LORDO_ERR_INVALID_ARG;
   if (c->h_Gtab) cudaFreeHost(c->h_Gtab);
-  if (c->h_status) cudaFreeHost(c->h_status);
-  if (c->h_gmaps) cudaFreeHost(c->h_gmaps);
   for (int sl = 0; sl < 2; ++sl)
     if (c->g_slot_ev[sl]) cudaEventDestroy(c->g_slot_ev[sl]);
   for (const lordo_ctx::Span& sp : c->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }

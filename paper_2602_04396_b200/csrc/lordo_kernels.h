@@ -106,9 +106,9 @@ struct TcProblem {
   const __nv_bfloat16* PT16;   // [r_n][m_k]  P^T, zero padded
   const __nv_bfloat16* P16;    // [m_k][r_k]  P, zero padded
   // Low-rank gradient and normalised low-rank update U~, transposed, private to the projection and
-  // update kernels of one path. Register-staged kernels: [n][r_k]. TMA-fed kernels:
+  // update kernels:
   // [strip][r_k/8][128 columns][8], i.e. the 16-byte pieces of one k-chunk of a strip's columns lie
-  // side by side and a warp moves 512 contiguous bytes. Room for ceil(n/128)*128 columns either way.
+  // side by side and a warp moves 512 contiguous bytes.
   __nv_bfloat16* gT16;
   __nv_bfloat16* uT16;
   float* u;                    // [r][n] of this worker
@@ -158,23 +158,21 @@ struct TcPrep {
   int r, r_k, m_k, pad;
 };
 
-cudaError_t tc_configure(int r_n_max, int r_k_max);
+cudaError_t tc_configure(int r_n_max);
 void launch_prep_projection(const TcPrep* items, const long long* blk_start, int nitems, long long total_blocks, cudaStream_t st);
 // bf16 != 0: G, E, W are all bf16; else all fp32 (mixed storage runs on the fp32 path).
 void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, int steps, int sm_count, const StepScalars& sc,
                        int bf16, unsigned* status, cudaStream_t st);
-void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_k_max, int steps, int sm_count, const StepScalars& sc,
-                     int bf16, unsigned* status, cudaStream_t st);
-
 // TMA-fed persistent kernels for bf16 storage (lordo_tma.cu).
-cudaError_t tma_configure();
+cudaError_t tma_configure();      // bf16 storage
+cudaError_t tma_configure_f32();  // fp32 storage
 int project_pairs(int sm_count);  // CTA pairs of the projection that the device holds at once
 void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int pairs, const TmaMatMaps* maps,
                         const TmaGradMaps* gmaps, const StepScalars& sc, unsigned* status, cudaStream_t st);
-// mode 0: r <= 256, one sweep; modes 1 and 2: the two sweeps for 256 < r <= 512. side 0: every problem is stored as it
-// is (tr = 0), 1: every one transposed, 2: some of either.
+// f32: fp32 storage. mode 0: r <= 256, one sweep; modes 1 and 2: the two sweeps for 256 < r <= 512. side 0: every problem is
+// stored as it is (tr = 0), 1: every one transposed, 2: some of either. With fp32 storage mode and side are 0.
 void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int ctas, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
-                      const StepScalars& sc, int mode, int side, unsigned* status, cudaStream_t st);
+                      const StepScalars& sc, int f32, int mode, int side, unsigned* status, cudaStream_t st);
 
 void launch_selftest_wait(unsigned* status, cudaStream_t st);
 

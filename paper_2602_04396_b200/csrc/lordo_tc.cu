@@ -1,16 +1,12 @@
-// Tensor-core (tcgen05 + tensor memory) kernels of the inner step, "fast mode":
+// Tensor-core (tcgen05 + tensor memory) projection of the inner step with fp32 storage, "fast mode":
 //
 //   project_tc_kernel  g^T = (cG+E)^T P  for one 128-column strip of one (matrix, worker), swept
 //                      down the m rows; the low-rank moment update (Algorithm 1: u, v lines and the
 //                      bracket of the update cases) runs in its epilogue straight out of tensor
 //                      memory, so the low-rank gradient never goes to global memory in fp32.
-//   apply_tc_kernel    (P g)^T and (P U~)^T for the same strip with the two low-rank operands
-//                      resident in shared memory, swept down the m rows in steps of 64; its
-//                      epilogue is the error-feedback line and the model update of Algorithm 1.
 //
-// Both deal a strip's rows out where there are fewer strips than SMs: the projection over a cluster of CTAs that
-// exchange their partial accumulators through distributed shared memory, each finishing every S-th 16 ranks;
-// the update over independent CTAs. 2048 x 2048, r = 128, K = 4 (64 strips): projection 98 -> 42 us, update 122 -> 74 us.
+// Where there are fewer strips than SMs, the rows of a strip are dealt out over a cluster of CTAs that exchange their partial
+// accumulators through distributed shared memory, each finishing every S-th 16 ranks: 2048 x 2048, r = 128, K = 4 (64 strips) 98 -> 42 us.
 //
 // Orientation: the strip's columns (n) are the 128 lanes of tensor memory, so every epilogue
 // thread owns one column and a warp touches 32 consecutive columns of a row of G, E, W, u or v.
@@ -29,9 +25,6 @@ namespace {
 
 constexpr int kStrip = 128;        // columns per strip = MMA M
 constexpr int kProjThreads = 288;  // 8 producer/epilogue warps + 1 MMA warp
-constexpr int kApplyEpiWarps = 16, kApplyProdWarps = 2;
-constexpr int kApplyThreads = (kApplyEpiWarps + kApplyProdWarps + 1) * 32;
-constexpr int kApplyRows = 64;     // rows of W per sweep step = MMA N
 
 __device__ __forceinline__ int find_problem(const TcProblem* __restrict__ probs, int nprobs, long long strip) {
   int lo = 0, hi = nprobs - 1;
@@ -271,8 +264,9 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
     const long long ecolc = ecol < n ? ecol : (long long)n - 1;
     float* __restrict__ up_ = prp->u;
     float* __restrict__ vp_ = prp->v;
-    __nv_bfloat16* __restrict__ gT = prp->gT16 + ecolc * r_k;
-    __nv_bfloat16* __restrict__ uT = prp->uT16 + ecolc * r_k;
+    const size_t lr_off = (size_t)(n0 / kStrip) * (size_t)r_k * kStrip + (size_t)(q * 32 + lane) * 8;  // this column's 16-byte pieces
+    __nv_bfloat16* __restrict__ gT = prp->gT16 + lr_off;
+    __nv_bfloat16* __restrict__ uT = prp->uT16 + lr_off;
     const float b1 = sc.beta1, b2 = sc.beta2, w = sc.omega;
     const bool low = sc.form == LORDO_QHM_LOW;
     float dsum = 0.f;
@@ -319,10 +313,10 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
         upk[i >> 1] = pack2_bf16(o[0], o[1]);
       }
       if (e_ok) {
-        uint4* gd = reinterpret_cast<uint4*>(gT + ch * 16);
-        uint4* ud = reinterpret_cast<uint4*>(uT + ch * 16);
-        gd[0] = make_uint4(gp[0], gp[1], gp[2], gp[3]); gd[1] = make_uint4(gp[4], gp[5], gp[6], gp[7]);
-        ud[0] = make_uint4(upk[0], upk[1], upk[2], upk[3]); ud[1] = make_uint4(upk[4], upk[5], upk[6], upk[7]);
+        uint4* gd = reinterpret_cast<uint4*>(gT + (size_t)ch * 2048);  // k-chunks 2 ch and 2 ch + 1, 128 pieces apart
+        uint4* ud = reinterpret_cast<uint4*>(uT + (size_t)ch * 2048);
+        gd[0] = make_uint4(gp[0], gp[1], gp[2], gp[3]); gd[128] = make_uint4(gp[4], gp[5], gp[6], gp[7]);
+        ud[0] = make_uint4(upk[0], upk[1], upk[2], upk[3]); ud[128] = make_uint4(upk[4], upk[5], upk[6], upk[7]);
       }
     }
     if (sc.form == LORDO_QHM_FULL) {  // mu(D): mean over the rank axis, one value per column
@@ -350,205 +344,6 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
 }
 
 // ---------------------------------------------------------------------------------------------
-// back-projection + error feedback + model update
-// ---------------------------------------------------------------------------------------------
-template <bool BF16>
-__global__ void __launch_bounds__(kApplyThreads, 1) apply_tc_kernel(const TcProblem* __restrict__ probs, int nprobs, StepScalars sc,
-                                                                    int pieces, unsigned* __restrict__ status) {
-  using EL = Elem<BF16>;
-  using one_t = typename EL::one;
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t p_full[2], p_empty[2], acc_full[2], acc_empty[2];
-  __shared__ uint32_t tmem_slot;
-
-  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-  const long long strip = blockIdx.x / pieces;
-  const TcProblem* __restrict__ prp = probs + find_problem(probs, nprobs, strip);
-  const int m = prp->m, n = prp->n, r_k = prp->r_k;
-  const long long n0 = (strip - prp->strip_start) * kStrip;
-  const int nkb = r_k / 64;
-  const int nsteps_all = (m + kApplyRows - 1) / kApplyRows, piece = (int)(blockIdx.x % pieces);
-  const int first = nsteps_all * piece / pieces, nsteps = nsteps_all * (piece + 1) / pieces - first;  // this CTA's part of the strip
-  const uint32_t x_bytes = (uint32_t)nkb * kStrip * 128;      // one resident operand (g^T or U~^T)
-  const uint32_t p_bytes = (uint32_t)nkb * kApplyRows * 128;  // one ring stage of P rows
-  unsigned char* sX1 = smem;
-  unsigned char* sX2 = smem + x_bytes;
-  unsigned char* sP = smem + 2 * x_bytes;
-  constexpr uint32_t kCols = 256;  // 2 buffers x (2 accumulators x 64 rows)
-
-  if (tid == 0) {
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&p_full[s], kApplyProdWarps * 32); mbar_init(&p_empty[s], 1);
-      mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], kApplyEpiWarps * 32);
-    }
-    mbar_init_fence();
-  }
-  if (warp == kApplyEpiWarps + kApplyProdWarps) tmem_alloc(&tmem_slot, kCols);
-  __syncthreads();  // tensor memory is there before the next kernel may begin
-  dep_begin();
-
-  // resident operands: rows = the strip's columns, k = rank index (zero rows beyond n)
-  {
-    const int chunks_per_row = r_k / 8;
-    const int per_op = kStrip * chunks_per_row;
-    const int total = 2 * per_op;
-    const __nv_bfloat16* __restrict__ g16 = prp->gT16;
-    const __nv_bfloat16* __restrict__ u16 = prp->uT16;
-    for (int base = tid; base < total; base += 4 * kApplyThreads) {
-      uint4 v[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        int idx = base + t * kApplyThreads;
-        idx = idx < total ? idx : total - 1;
-        const int which = idx >= per_op;
-        const int rem = idx - which * per_op;
-        const int row = rem / chunks_per_row, ch = rem - row * chunks_per_row;
-        long long grow = n0 + row;
-        grow = grow < n ? grow : (long long)n - 1;
-        v[t] = *reinterpret_cast<const uint4*>((which ? u16 : g16) + grow * r_k + ch * 8);
-      }
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int idx = base + t * kApplyThreads;
-        if (idx < total) {
-          const int which = idx >= per_op;
-          const int rem = idx - which * per_op;
-          const int row = rem / chunks_per_row, ch = rem - row * chunks_per_row;
-          const uint4 val = (n0 + row < n) ? v[t] : make_uint4(0u, 0u, 0u, 0u);
-          *reinterpret_cast<uint4*>((which ? sX2 : sX1) + (ch >> 3) * (kStrip * 128) + swz_chunk(row, ch & 7)) = val;
-        }
-      }
-    }
-  }
-  fence_async_smem();
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = tmem_slot;
-
-  if (warp < kApplyEpiWarps) {
-    // ---------------- epilogue: one column per thread, 16 rows per step -----------------------
-    const int q = warp & 3, grp = warp >> 2;
-    const long long col = n0 + q * 32 + lane;
-    const bool col_ok = col < n;
-    const long long colc = col_ok ? col : (long long)n - 1;
-    const one_t* __restrict__ Gp = reinterpret_cast<const one_t*>(*prp->G_ind) + prp->G_off;
-    one_t* __restrict__ Wp = reinterpret_cast<one_t*>(prp->W);
-    const bool ef = sc.ef != 0;
-    one_t* __restrict__ Ep = ef ? reinterpret_cast<one_t*>(prp->E) : Wp;
-    const float c = *prp->cptr;
-    const float lr = sc.lr, om = sc.omega;
-    const bool full = sc.form == LORDO_QHM_FULL;
-    const float cd = full ? (1.f - om) * c / prp->dcol[colc] : 0.f;
-    const float a2w = full ? om : 1.f;
-    const one_t* __restrict__ Gc = Gp + colc;
-    one_t* __restrict__ Ec = Ep + colc;
-    one_t* __restrict__ Wc = Wp + colc;
-    // Half a step's rows are loaded while the other half is worked on (2048 x 2048, r = 128, K = 4: 73 -> 71 us, all 16 at
-    // once left the loads idle in between).
-    struct Rows {
-      one_t g[8], e[8], w[8];
-    };
-    auto load = [&](int t, int h, Rows& x) {
-      const int row0 = (first + t) * kApplyRows + grp * 16 + h * 8;
-      const size_t base = (size_t)(unsigned)min(row0, m - 1) * (size_t)n;
-      const bool whole = row0 + 8 <= m;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const size_t off = whole ? base + (size_t)(unsigned)(j * n) : (size_t)(unsigned)min(row0 + j, m - 1) * (size_t)n;
-        x.g[j] = Gc[off];
-        x.e[j] = Ec[off];
-        x.w[j] = Wc[off];
-      }
-    };
-    auto finish = [&](int t, int h, const Rows& x) {
-      const int row0 = (first + t) * kApplyRows + grp * 16 + h * 8, b = t & 1;
-      const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * 128 + grp * 16 + h * 8);
-      float a1[8], a2[8];
-      tmem_ld8x2(taddr, taddr + 64, a1, a2);  // (P g)^T, (P U~)^T
-      if (h == 1) {
-        tc_fence_before_sync();
-        mbar_arrive(&acc_empty[b]);
-      }
-      if (!col_ok) return;
-      const size_t base = (size_t)(unsigned)min(row0, m - 1) * (size_t)n;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (row0 + j >= m) break;
-        const size_t off = base + (size_t)(unsigned)(j * n);
-        if (ef) Ec[off] = EL::pack((c * EL::cvt(x.g[j]) + EL::cvt(x.e[j])) - a1[j]);
-        Wc[off] = EL::pack(EL::cvt(x.w[j]) - lr * (cd * EL::cvt(x.g[j]) + a2w * a2[j]));
-      }
-    };
-    Rows x0, x1;
-    if (nsteps > 0) load(0, 0, x0);
-    for (int t = 0; t < nsteps; ++t) {
-      load(t, 1, x1);
-      if (!mbar_wait<40>(&acc_full[t & 1], (uint32_t)((t >> 1) & 1), status)) break;
-      tc_fence_after_sync();
-      finish(t, 0, x0);
-      if (t + 1 < nsteps) load(t + 1, 0, x0);
-      finish(t, 1, x1);
-    }
-  } else if (warp < kApplyEpiWarps + kApplyProdWarps) {
-    // ---------------- producers: rows of P for the next step (asynchronous 16-byte copies) -----
-    const int ptid = tid - kApplyEpiWarps * 32;
-    const int chunks_per_row = r_k / 8;
-    const int total = kApplyRows * chunks_per_row;
-    const __nv_bfloat16* __restrict__ P16 = prp->P16;
-    bool ok = true;
-    for (int t = 0; t < nsteps && ok; ++t) {
-      const int s = t & 1;
-      ok = mbar_wait(&p_empty[s], (uint32_t)(((t >> 1) & 1) ^ 1), status);
-      if (!ok) break;
-      const uint32_t dst = smem_u32(sP + s * p_bytes);
-      for (int idx = ptid; idx < total; idx += kApplyProdWarps * 32) {
-        const int row = idx / chunks_per_row, ch = idx - row * chunks_per_row;
-        const __nv_bfloat16* src = P16 + ((long long)(first + t) * kApplyRows + row) * r_k + ch * 8;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (ch >> 3) * (kApplyRows * 128) + swz_chunk(row, ch & 7)),
-                     "l"(src)
-                     : "memory");
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      fence_async_smem();
-      mbar_arrive(&p_full[s]);
-    }
-  } else {
-    // ---------------- MMA issue ---------------------------------------------------------------
-    const uint32_t one = elect_one();
-    const uint32_t idesc = idesc_bf16_f32(128, kApplyRows);
-    const uint32_t x1 = smem_u32(sX1), x2 = smem_u32(sX2);
-    bool ok = true;
-    for (int t = 0; t < nsteps && ok; ++t) {
-      const int s = t & 1;
-      ok = mbar_wait_warp(&p_full[s], (uint32_t)((t >> 1) & 1), status);
-      if (ok) ok = mbar_wait_warp(&acc_empty[s], (uint32_t)(((t >> 1) & 1) ^ 1), status);
-      if (!ok) break;
-      tc_fence_after_sync();
-      const uint32_t pbase = smem_u32(sP + s * p_bytes);
-      for (int kb = 0; kb < nkb; ++kb) {
-#pragma unroll
-        for (int k16 = 0; k16 < 4; ++k16) {
-          const uint32_t acc = (kb > 0 || k16 > 0) ? 1u : 0u;
-          const uint64_t bd = smem_desc_k128(pbase + kb * (kApplyRows * 128) + k16 * 32);
-          mma_bf16(tmem + s * 128, smem_desc_k128(x1 + kb * (kStrip * 128) + k16 * 32), bd, idesc, acc, one);
-          mma_bf16(tmem + s * 128 + 64, smem_desc_k128(x2 + kb * (kStrip * 128) + k16 * 32), bd, idesc, acc, one);
-        }
-      }
-      if (one) {
-        mma_commit(&p_empty[s]);
-        mma_commit(&acc_full[s]);
-      }
-    }
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  if (warp == kApplyEpiWarps + kApplyProdWarps) tmem_free(tmem, kCols);
-}
-
-// ---------------------------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------------------------
 // two stages, or the partial accumulators that a CTA of a cluster of four hands to the others
@@ -557,19 +352,10 @@ size_t project_tc_smem(int r_n_max) {
   const size_t nch = (size_t)r_n_max / 16;
   return std::max(2 * stage, (nch - nch / 4) * 16 * kStrip * sizeof(float)) + 1024;
 }
-size_t apply_tc_smem(int r_k_max) {
-  const size_t nkb = (size_t)r_k_max / 64;
-  return 2 * nkb * kStrip * 128 + 2 * nkb * kApplyRows * 128 + 1024;
-}
-
-cudaError_t tc_configure(int r_n_max, int r_k_max) {
+cudaError_t tc_configure(int r_n_max) {
   cudaError_t e = cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(apply_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_tc_smem(r_k_max));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(apply_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_tc_smem(r_k_max));
+  return cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
 }
 
 void launch_prep_projection(const TcPrep* items, const long long* blk_start, int nitems, long long total_blocks, cudaStream_t st) {
@@ -592,29 +378,4 @@ void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strip
   if (bf16) cudaLaunchKernelEx(&lc, project_tc_kernel<true>, probs, nprobs, sc, status);
   else cudaLaunchKernelEx(&lc, project_tc_kernel<false>, probs, nprobs, sc, status);
 }
-void launch_apply_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_k_max, int steps, int sm_count, const StepScalars& sc,
-                     int bf16, unsigned* status, cudaStream_t st) {
-  // one CTA fits an SM; each is left four steps at least
-  int pieces = (int)std::min<long long>(sm_count / total_strips, steps / 4);
-  if (pieces < 1) pieces = 1;
-  const dim3 grid((unsigned)(total_strips * pieces));
-  const size_t smem = apply_tc_smem(r_k_max);
-  // CTAs that begin under the end of the projection gain 2 to 5 us where all of them fit the device, but where they run in
-  // several turns the early ones take places in the wrong order: 448 strips, r = 256, step 806 us, plainly launched 693 us.
-  // In one turn too they take the SMs in the order in which the projection leaves them and not in the device's own. At
-  // r_k = 256, where a step pulls 32 KB of P out of L2, the same strips then last a third longer by their own clocks (144
-  // strips of three lengths, one to an SM either way: 66 instead of 49 us, step 159 instead of 139 us; 98 strips 284 and
-  // 241 us; 128 equal strips 312 and 287 us); r_k <= 192 is within 2 % for mixed strips and gains 3 us for equal ones.
-  const bool early = (long long)grid.x <= sm_count && r_k_max < 256;
-#define LORDO_APPLY_TC(B)                                                                                          \
-  if (early) launch_dep(apply_tc_kernel<B>, grid, kApplyThreads, smem, st, probs, nprobs, sc, pieces, status);      \
-  else apply_tc_kernel<B><<<grid, kApplyThreads, smem, st>>>(probs, nprobs, sc, pieces, status)
-  if (bf16) {
-    LORDO_APPLY_TC(true);
-  } else {
-    LORDO_APPLY_TC(false);
-  }
-#undef LORDO_APPLY_TC
-}
-
 }  // namespace lordo

@@ -1,4 +1,4 @@
-// TMA-fed, persistent tensor-core kernels of the inner step for bf16 storage of G, E and W.
+// TMA-fed, persistent tensor-core kernels of the inner step: the projection for bf16 storage of G, E and W, the update for either.
 //
 //   project_tma_kernel  The streamed operand never passes through registers as single elements:
 //                       TMA brings 64-row tiles of G, E (and of P^T) into 128B-swizzled shared
@@ -40,8 +40,8 @@ constexpr int kPXformWarps = 4, kPEpiWarps = 16;
 constexpr int kPThreads = (2 + kPXformWarps + kPEpiWarps) * 32;  // 704
 
 // ---- update -------------------------------------------------------------------------------------
-constexpr int kARows = 64;                // rows of W per step = MMA N
-constexpr int kAInStages = 3;             // G | E | W tiles, 16 KB each
+constexpr int kARows = 64, kARows32 = 32; // rows of W per step = MMA N, with bf16 and with fp32 storage
+constexpr int kAInStages = 3, kAInStages32 = 4;  // G | E | W tiles, 16 KB each
 constexpr uint32_t kAInStageBytes = 49152;
 constexpr int kAPStages = 2;              // rows of P, up to 32 KB
 constexpr uint32_t kAPStageBytes = 32768;
@@ -308,15 +308,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPThreads, 1)
 // accumulator tile (lane = strip element, column = step element) already lies the way the tiles are
 // stored, so a thread works on 16 neighbouring stored columns of its own row. SIDE 2: both kinds, told apart piece by
 // piece; as two launches, each with its own start and end, five ragged matrices took 28 + 31 us, as one 46 us.
-template <int MODE, int SIDE>
+// F32: fp32 storage. A step is half as many rows, so a tile is as large and the accumulator half; tiles lie unswizzled, a row of 512 bytes
+// after the other, and a thread works on one column. The rows of P take half the room, which gives a fourth stage of tiles. Bound by HBM and,
+// where strips are few, by what an SM can have on its way. The kernel before it loaded G, E and W into registers itself, half of a step ahead:
+// whole steps of 2048 x 2048, r = 128, K = 4 131 -> 120 us, 2048 x 5632, r = 256, K = 4 488 -> 412, seven matrices of 768 with two workers
+// (strips of 12 and of 48 steps, all cut in the same number of parts) 354 -> 208, one 64 x 64 21.0 -> 21.1.
+template <int MODE, int SIDE, bool F32>
 __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem* __restrict__ probs, const TcSeg* __restrict__ segs,
                                                                  const int* __restrict__ start, const TmaMatMaps* __restrict__ maps,
                                                                  const TmaGradMaps* __restrict__ gmaps, StepScalars sc,
                                                                  unsigned* __restrict__ status) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr uint32_t PSB = MODE ? 65536u : kAPStageBytes;  // one stage of rows of P
-  constexpr int INST = kAInStages;
+  static_assert(!F32 || (MODE == 0 && SIDE == 0), "fp32 storage: ranks up to 256, matrices projected from the left");
+  constexpr int ROWS = F32 ? kARows32 : kARows;
+  constexpr uint32_t PSB = MODE ? 65536u : F32 ? kAPStageBytes / 2 : kAPStageBytes;  // one stage of rows of P
+  constexpr int INST = F32 ? kAInStages32 : kAInStages;
   constexpr bool DO_E = MODE != 2, DO_W = MODE != 1;
   constexpr uint32_t A2COL = MODE ? 0u : 128u;             // first column of the U~^T operand
   // a stage holds the tiles the mode works on: G | E | W (MODE 0), G | E (MODE 1), G | W (MODE 2)
@@ -324,7 +331,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
   constexpr uint32_t EOFF = 16384u, WOFF = MODE == 2 ? 16384u : 32768u;
   unsigned char* sP = smem;                      // kAPStages stages of rows of P
   unsigned char* sIn = smem + kAPStages * PSB;   // INST stages of tiles
-  __shared__ uint64_t p_full[kAPStages], p_empty[kAPStages], in_full[kAInStages], in_free[kAInStages], acc_full[2], acc_empty[2], x_ready;
+  __shared__ uint64_t p_full[kAPStages], p_empty[kAPStages], in_full[INST], in_free[INST], acc_full[2], acc_empty[2], x_ready;
   __shared__ uint32_t tmem_slot;
 
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -367,15 +374,19 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
           unsigned char* base = sIn + is * ISB;
           const bool ld_e = DO_E && ef;
           mbar_expect_tx(&in_full[is], 16384u + (ld_e ? 16384u : 0u) + (DO_W ? 16384u : 0u), one);
-          if (SIDE == 1 || (SIDE == 2 && pr->tr)) {  // one box of 128 stored rows x 64 stored columns per tile
-            tma_load_3d(base, gm->g_kb, t * kARows, n0, rep, &in_full[is], one);
-            if (ld_e) tma_load_3d(base + EOFF, mm->e_kb, t * kARows, n0, rep, &in_full[is], one);
-            if (DO_W) tma_load_3d(base + WOFF, mm->w_kb, t * kARows, n0, rep, &in_full[is], one);
+          if (F32) {  // one box of 32 rows x 128 columns per tile
+            tma_load_3d(base, gm->g_kb, n0, t * ROWS, rep, &in_full[is], one);
+            if (ld_e) tma_load_3d(base + EOFF, mm->e_kb, n0, t * ROWS, rep, &in_full[is], one);
+            tma_load_3d(base + WOFF, mm->w_kb, n0, t * ROWS, rep, &in_full[is], one);
+          } else if (SIDE == 1 || (SIDE == 2 && pr->tr)) {  // one box of 128 stored rows x 64 stored columns per tile
+            tma_load_3d(base, gm->g_kb, t * ROWS, n0, rep, &in_full[is], one);
+            if (ld_e) tma_load_3d(base + EOFF, mm->e_kb, t * ROWS, n0, rep, &in_full[is], one);
+            if (DO_W) tma_load_3d(base + WOFF, mm->w_kb, t * ROWS, n0, rep, &in_full[is], one);
           } else {
             for (int hh = 0; hh < 2; ++hh) {  // two 64-column halves per tile, 8 KB each
-              tma_load_3d(base + hh * 8192, gm->g_sw, n0 + hh * 64, t * kARows, rep, &in_full[is], one);
-              if (ld_e) tma_load_3d(base + EOFF + hh * 8192, mm->e_sw, n0 + hh * 64, t * kARows, rep, &in_full[is], one);
-              if (DO_W) tma_load_3d(base + WOFF + hh * 8192, mm->w_sw, n0 + hh * 64, t * kARows, rep, &in_full[is], one);
+              tma_load_3d(base + hh * 8192, gm->g_sw, n0 + hh * 64, t * ROWS, rep, &in_full[is], one);
+              if (ld_e) tma_load_3d(base + EOFF + hh * 8192, mm->e_sw, n0 + hh * 64, t * ROWS, rep, &in_full[is], one);
+              if (DO_W) tma_load_3d(base + WOFF + hh * 8192, mm->w_sw, n0 + hh * 64, t * ROWS, rep, &in_full[is], one);
             }
           }
         }
@@ -396,15 +407,15 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
           const int ps = jt % kAPStages;
           ok = mbar_wait_warp(&p_empty[ps], ((jt / kAPStages) & 1u) ^ 1u, status);
           if (!ok) break;
-          mbar_expect_tx(&p_full[ps], (uint32_t)nkb * 8192u, one);
-          for (int kb = 0; kb < nkb; ++kb) tma_load_3d(sP + ps * PSB + kb * 8192, mm->p16, kb * 64, t * kARows, pc, &p_full[ps], one);
+          mbar_expect_tx(&p_full[ps], (uint32_t)nkb * (ROWS * 128u), one);
+          for (int kb = 0; kb < nkb; ++kb) tma_load_3d(sP + ps * PSB + kb * (ROWS * 128), mm->p16, kb * 64, t * ROWS, pc, &p_full[ps], one);
         }
       }
     }
   } else if (warp == 1) {
     // ---------------- MMA issue: A operands from tensor memory ----------------------------------
     {
-      const uint32_t idesc = idesc_bf16_f32(128, kARows), one = elect_one();
+      const uint32_t idesc = idesc_bf16_f32(128, ROWS), one = elect_one();
       uint32_t jt = 0, si = 0;
       bool ok = true;
       for (int e = seg_begin; e < seg_end && ok; ++e, ++si) {
@@ -426,7 +437,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
 #pragma unroll
             for (int k16 = 0; k16 < 4; ++k16) {
               const uint32_t acc = (kb > 0 || k16 > 0) ? 1u : 0u;
-              const uint64_t bd = smem_desc_k128(pbase + kb * 8192 + k16 * 32);
+              const uint64_t bd = smem_desc_k128(pbase + kb * (ROWS * 128) + k16 * 32);
               const uint32_t acol = (uint32_t)(kb * 4 + k16) * 8;
               if (DO_E) mma_bf16_ts(d1, tmem + acol, bd, idesc, acc, one);
               if (DO_W) mma_bf16_ts(d2, tmem + A2COL + acol, bd, idesc, acc, one);
@@ -470,14 +481,14 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
       const TmaMatMaps* mm = maps + pr->mat;
       const int rep = pr->replica;
       const bool tr_p = SIDE == 1 || (SIDE == 2 && pr->tr);
-      const int colq = tr_p ? q * 32 + lane : q * 32 + 4 * (lane & 7) + (lane >> 3);  // strip element this lane's operands belong to
+      const int colq = tr_p || F32 ? q * 32 + lane : q * 32 + 4 * (lane & 7) + (lane >> 3);  // strip element this lane's operands belong to
       const long long col = (long long)n0 + colq;
       const float c = *pr->cptr;
       float cd[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        // right side: one strip element per thread (its own row); else the four columns of the thread's epilogue block
-        const long long ec = tr_p ? col : (long long)n0 + ecol0 + j;
+        // right side, fp32: one strip element per thread (its own row or column); else the four columns of the thread's epilogue block
+        const long long ec = tr_p || F32 ? col : (long long)n0 + ecol0 + j;
         const long long ecc = ec < n ? ec : (long long)n - 1;
         cd[j] = full ? (1.f - om) * c / (pr->dcol[ecc] + (pr->dcol2 ? pr->dcol2[ecc] : 0.f)) : 0.f;
       }
@@ -514,7 +525,40 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
         if (ok) ok = mbar_wait<32>(&acc_full[b], (jt >> 1) & 1u, status);
         if (!ok) break;
         tc_fence_after_sync();
-        if (tr_p) {
+        if constexpr (F32) {
+          // this thread: column 32 q + lane of the strip, rows 8 grp .. +7 of the step; a warp reads 128 bytes of a row
+          float a1[8], a2[8];
+          const uint32_t taddr = tmem + lane_base + 256 + b * 128 + (uint32_t)(grp * 8);
+          tmem_ld8x2(taddr, taddr + 64, a1, a2);
+          tc_fence_before_sync();
+          mbar_arrive(&acc_empty[b]);
+          float* at = reinterpret_cast<float*>(base) + grp * 8 * kStrip + q * 32 + lane;
+          float *ae = at + EOFF / 4, *aw = at + WOFF / 4;
+          float g[8], w[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) { g[i] = at[i * kStrip]; w[i] = aw[i * kStrip]; }
+          if (ef) {
+            float e[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) e[i] = ae[i * kStrip];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ae[i * kStrip] = (c * g[i] + e[i]) - a1[i];
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) aw[i * kStrip] = w[i] - lr * (cd[0] * g[i] + a2w * a2[i]);
+          fence_async_smem();
+          asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+          if ((ew & 3) == 0 && lane == 0) {  // a row group's 8 rows
+            const int row = t * ROWS + grp * 8;
+            if (row < pr->m) {
+              if (ef) tma_store_3d(mm->e_st, n0, row, rep, base + EOFF + grp * 4096);
+              tma_store_3d(mm->w_st, n0, row, rep, base + WOFF + grp * 4096);
+            }
+            tma_store_commit();
+            tma_store_wait_read();
+            mbar_arrive(&in_free[is]);
+          }
+        } else if (tr_p) {
           // this thread: stored row 32q + lane of the strip, stored columns 16 grp .. +15 of the step
           const int row = q * 32 + lane;
           const uint32_t o0 = swz_chunk(row, 2 * grp), o1 = swz_chunk(row, 2 * grp + 1);
@@ -556,8 +600,8 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
           asm volatile("bar.sync %0, 128;" ::"r"(6 + q) : "memory");
           if (grp == 0 && lane == 0) {
             if (n0 + q * 32 < n) {
-              if (DO_E && ef) tma_store_3d(mm->e_st32, t * kARows, n0 + q * 32, rep, base + EOFF + q * 4096);
-              if (DO_W) tma_store_3d(mm->w_st32, t * kARows, n0 + q * 32, rep, base + WOFF + q * 4096);
+              if (DO_E && ef) tma_store_3d(mm->e_st32, t * ROWS, n0 + q * 32, rep, base + EOFF + q * 4096);
+              if (DO_W) tma_store_3d(mm->w_st32, t * ROWS, n0 + q * 32, rep, base + WOFF + q * 4096);
             }
             tma_store_commit();
             tma_store_wait_read();
@@ -612,7 +656,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
           asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
           if ((ew & 3) == 0 && lane == 0) {
             unsigned char* sb = base + grp * 2048;
-            const int row = t * kARows + grp * 16;
+            const int row = t * ROWS + grp * 16;
             for (int hh = 0; hh < 2; ++hh) {
               if (n0 + hh * 64 >= n) break;
               if (DO_E && ef) tma_store_3d(mm->e_st, n0 + hh * 64, row, rep, sb + EOFF + hh * 8192);
@@ -657,12 +701,16 @@ cudaError_t tma_configure() {
   e = max_resident_pairs(project_tma_kernel, kPThreads, kPStages * kPStageBytes + 1024, &g_project_pairs);
   if (e != cudaSuccess) return e;
   const int smem = (int)(kAPStages * 65536 + kAInStages * 32768 + 1024);  // the largest of the three modes
-  const void* kernels[9] = {(const void*)apply_tma_kernel<0, 0>, (const void*)apply_tma_kernel<1, 0>, (const void*)apply_tma_kernel<2, 0>,
-                            (const void*)apply_tma_kernel<0, 1>, (const void*)apply_tma_kernel<1, 1>, (const void*)apply_tma_kernel<2, 1>,
-                            (const void*)apply_tma_kernel<0, 2>, (const void*)apply_tma_kernel<1, 2>, (const void*)apply_tma_kernel<2, 2>};
+  const void* kernels[9] = {(const void*)apply_tma_kernel<0, 0, false>, (const void*)apply_tma_kernel<1, 0, false>, (const void*)apply_tma_kernel<2, 0, false>,
+                            (const void*)apply_tma_kernel<0, 1, false>, (const void*)apply_tma_kernel<1, 1, false>, (const void*)apply_tma_kernel<2, 1, false>,
+                            (const void*)apply_tma_kernel<0, 2, false>, (const void*)apply_tma_kernel<1, 2, false>, (const void*)apply_tma_kernel<2, 2, false>};
   for (const void* k : kernels)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return e;
+}
+
+cudaError_t tma_configure_f32() {
+  return cudaFuncSetAttribute(apply_tma_kernel<0, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kAPStages * kAPStageBytes / 2 + kAInStages32 * kAInStageBytes + 1024));
 }
 
 int project_pairs(int sm_count) { return g_project_pairs > 0 ? std::min(sm_count / 2, g_project_pairs) : sm_count / 2; }
@@ -673,15 +721,18 @@ void launch_project_tma(const TcProblem* probs, const TcSeg* segs, const int* st
   launch_dep(project_tma_kernel, dim3(2u * (unsigned)pairs), kPThreads, kPStages * kPStageBytes + 1024, st, probs, segs, start, maps, gmaps, sc, status);
 }
 void launch_apply_tma(const TcProblem* probs, const TcSeg* segs, const int* start, int ctas, const TmaMatMaps* maps, const TmaGradMaps* gmaps,
-                      const StepScalars& sc, int mode, int side, unsigned* status, cudaStream_t st) {
+                      const StepScalars& sc, int f32, int mode, int side, unsigned* status, cudaStream_t st) {
   if (ctas <= 0) return;
   const size_t small = kAPStages * kAPStageBytes + kAInStages * kAInStageBytes + 1024, large = kAPStages * 65536 + kAInStages * 32768 + 1024;
-#define LORDO_APPLY(M, T, SM) launch_dep(apply_tma_kernel<M, T>, dim3((unsigned)ctas), kAThreads, SM, st, probs, segs, start, maps, gmaps, sc, status)
+#define LORDO_APPLY(M, T, SM) launch_dep(apply_tma_kernel<M, T, false>, dim3((unsigned)ctas), kAThreads, SM, st, probs, segs, start, maps, gmaps, sc, status)
 #define LORDO_APPLY_SIDE(T)                    \
   if (mode == 0) LORDO_APPLY(0, T, small);      \
   else if (mode == 1) LORDO_APPLY(1, T, large); \
   else LORDO_APPLY(2, T, large)
-  if (side == 0) { LORDO_APPLY_SIDE(0); }
+  if (f32)
+    launch_dep(apply_tma_kernel<0, 0, true>, dim3((unsigned)ctas), kAThreads, kAPStages * kAPStageBytes / 2 + kAInStages32 * kAInStageBytes + 1024, st, probs, segs,
+               start, maps, gmaps, sc, status);
+  else if (side == 0) { LORDO_APPLY_SIDE(0); }
   else if (side == 1) { LORDO_APPLY_SIDE(1); }
   else { LORDO_APPLY_SIDE(2); }
 #undef LORDO_APPLY_SIDE

@@ -73,8 +73,8 @@ def test_clip_coefficients_in_one_launch(dt, mats, K, scope):
 @pytest.mark.parametrize("m,n,r", [(2048, 136, 16), (1096, 264, 240), (528, 1032, 144), (1032, 264, 256), (600, 72, 40), (72, 64, 8)])
 @pytest.mark.parametrize("form", [1, 2])
 def test_fp32_storage_strips_dealt_out(m, n, r, form):
-    """Register-staged kernels (fp32 storage) with a strip's rows over one, two and four CTAs, ranks that do not
-    divide evenly among them, more CTAs than chunks of 16 ranks, and the update's rows in pieces."""
+    """fp32 storage: the projection with a strip's rows over one, two and four CTAs, ranks that do not divide evenly
+    among them, more CTAs than chunks of 16 ranks; the update's strips whole and in pieces."""
     wl = synth.Workload("t", ((m, n, r),), K=2, H=3, rounds=1, grad="gauss", clip_rho=30.0)
     spec = RunSpec(wl, variant=0, form=form, lr=0.01, omega=0.9, check_mode=0, eps=0.05, refresh=False)
     opt, orc = hz.run_gpu(spec), hz.run_oracle(spec)
@@ -82,4 +82,20 @@ def test_fp32_storage_strips_dealt_out(m, n, r, form):
     assert opt.poll_status() == 0
     tol = 8 * 2.0 ** -9  # bf16 operands, as for the other fast-mode tests
     assert st["u"] < tol and st["v"] < 2 * tol and st["E"] < tol and st["W"] < tol * 3 * 0.01 / 0.02, st
+    opt.close()
+
+
+@pytest.mark.parametrize("mats", [((9, 8, 8),), ((33, 136, 8), (1001, 264, 40)), ((265, 392, 256), (40, 2056, 24)), ((2053, 520, 72),) * 5])
+@pytest.mark.parametrize("ef", [True, False])
+def test_fp32_storage_update_tiles(mats, ef):
+    """The update's tiles of 32 rows x 128 columns in fp32: fewer rows than a tile or than the eight that are stored at a
+    time, a last row alone, fewer columns than a strip, strips of different lengths in one list, more strips than SMs."""
+    wl = synth.Workload("t", mats, K=2 if len(mats) < 5 else 8, H=2, rounds=1, grad="gauss", clip_rho=30.0)
+    spec = RunSpec(wl, variant=1, form=2, lr=0.01, omega=0.9, check_mode=0, eps=0.05, refresh=False, error_feedback=ef)
+    opt, orc = hz.run_gpu(spec), hz.run_oracle(spec)
+    st = hz.compare_states(opt, orc)
+    assert opt.poll_status() == 0
+    tol = 8 * 2.0 ** -9  # bf16 operands, as for the other fast-mode tests
+    assert st["u"] < tol and st["v"] < 2 * tol and st["W"] < tol * 2 * 0.01 / 0.02, st
+    assert not ef or st["E"] < tol, st
     opt.close()
