@@ -1232,6 +1232,9 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
     INIT_CUDA(gemm_configure());
     INIT_CUDA(chol_configure());
   }
+  std::vector<TmaMatMaps> hm;
+  std::vector<TcSeg> seg_list[2];
+  std::vector<int> seg_start[2];
   if (c->tc) {
     if (!c->tma) INIT_CUDA(tc_configure(c->tc_rn_max));  // register-staged kernels (fp32 storage)
     INIT_CUDA(cudaMemsetAsync(c->d_tc_bf16, 0, c->tc_bf16_bytes, st));
@@ -1240,7 +1243,7 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
     INIT_CUDA(cudaMemcpyAsync(c->d_prep_start, c->h_prep_start.data(), 8 * c->h_prep_start.size(), cudaMemcpyHostToDevice, st));
     {
       if (c->tma && c->sm_count < 2) return bail(LORDO_ERR_UNSUPPORTED);  // the projection and the refresh products run as CTA pairs
-      std::vector<TmaMatMaps> hm(nm);
+      hm.resize(nm);
       bool good = tmap_encoder() != nullptr;
       const bool loc = c->cfg.variant == LORDO_LOCAL;
       for (int i = 0; i < nm && good; ++i) {
@@ -1301,8 +1304,6 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
         int right = 0;
         for (const lordo_mat& a : c->mats) right += a.side;
         c->tma_side = right == 0 ? 0 : right == nm ? 1 : 2;
-        std::vector<TcSeg> seg_list[2];
-        std::vector<int> seg_start[2];
         for (int l = c->tma ? 0 : 1; l < 2; ++l) {
           std::vector<WorkItem> items;
           for (int x = 0; x < (int)c->h_tc.size(); ++x) {
@@ -1330,7 +1331,6 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
           INIT_CUDA(cudaMemcpyAsync(c->d_segs[l], list.data(), sizeof(TcSeg) * list.size(), cudaMemcpyHostToDevice, st));
           INIT_CUDA(cudaMemcpyAsync(c->d_seg_start[l], start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, st));
         }
-        INIT_CUDA(cudaStreamSynchronize(st));  // the tables above leave the host's stack
       } else {
         return bail(LORDO_ERR_CUDA);  // tensor maps could not be encoded (driver without cuTensorMapEncodeTiled?)
       }

@@ -1,7 +1,7 @@
 // Grouped fp32 FFMA GEMM with fused operand formation and epilogues: the fp32-accurate ("check
 // mode") realisation of every contraction of the path -- P^T(cG+E), P g, P U~, the sketch and
 // subspace-iteration products, Gram matrices, R^-1 application, Rot = P'^T P and the rotation of
-// the moments. 64 x 64 output tile (64 x 32 with two products), 16-deep k-slices, 256 threads, 16 outputs per thread.
+// the moments. 64 x 64 output tile (64 x 32 with two products), 16-deep k-slices, 256 threads of 4 rows or 128 of 8.
 // Products are formed and summed in fp32 inside a k-slice; the slice sums are carried across slices
 // in fp64, so a result is accurate to fp32 rounding whatever the contraction length.
 #include "lordo_kernels.h"
@@ -25,29 +25,31 @@ __device__ __forceinline__ Source resolve(const Operand& op) {
   return s;
 }
 
-// Four consecutive stored elements (row, col..col+3) of an operand as loaded, zero outside (rows, cols); their
-// value is formed when they are put into shared memory, so that nothing waits for a load before that.
+// Four consecutive stored elements of an operand as loaded; their value is formed when they are put into shared memory, so that
+// nothing waits for a load before that.
 struct Raw {
   float4 a, b;
 };
-__device__ __forceinline__ Raw source_load(const Source& op, long long row, long long col, long long rows, long long cols) {
-  Raw o;
+// What one thread fetches of an operand, slice after slice: once or twice four elements, where they are next, how far the ones after them, and
+// their k (of the row, or of the first of the four where k runs along the contiguous side). The contiguous side of every operand is
+// a multiple of four, so four elements are inside or outside together.
+struct Feed {
+  long long at, step, second;
+  int k, second_k, end, second_end;  // end: the contraction's length, or 0 where the other side's index is outside
+};
+__device__ __forceinline__ void feed_one(const Source& op, long long at, bool in, Raw& o) {
   o.a = o.b = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (row >= rows || col >= cols) return o;
-  const long long idx = row * op.ld + col;
-  if (col + 3 < cols) {
-    o.a = load4(op.p0, op.dt0, idx);
-    if (op.p1) o.b = load4(op.p1, op.dt1, idx);
-  } else {
-    float t[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int e = 0; e < 4 && col + e < cols; ++e) {
-      t[e] = load1(op.p0, op.dt0, idx + e);
-      if (op.p1) u[e] = load1(op.p1, op.dt1, idx + e);
-    }
-    o.a = make_float4(t[0], t[1], t[2], t[3]);
-    o.b = make_float4(u[0], u[1], u[2], u[3]);
+  if (in) {
+    o.a = load4(op.p0, op.dt0, at);
+    if (op.p1) o.b = load4(op.p1, op.dt1, at);
   }
-  return o;
+}
+template <int NL>
+__device__ __forceinline__ void feed_next(const Source& op, const Source& op2, Feed& f, Raw (&o)[NL]) {
+  feed_one(op, f.at, f.k < f.end, o[0]);
+  if constexpr (NL > 1) feed_one(op2, f.at + f.second, f.k + f.second_k < f.second_end, o[1]);
+  f.at += f.step;
+  f.k += BK;
 }
 __device__ __forceinline__ float4 source_value(const Source& op, const Raw& x, const GemmScalars& sc) {
   if (op.kind == OP_PLAIN) return make_float4(op.s0 * x.a.x + x.b.x, op.s0 * x.a.y + x.b.y, op.s0 * x.a.z + x.b.z, op.s0 * x.a.w + x.b.w);
@@ -146,8 +148,14 @@ __device__ __forceinline__ void partials_of(const double* p, unsigned rank, doub
 // accumulation, half the registers (the fp32 work of the fast mode: QR and moment rotation).
 // With two products a tile is half as wide (gemm_columns): a thread then holds two columns of each, two CTAs fit an SM and the
 // loads of one's epilogue (G, E, W) run under the other's products. Three ragged matrices with three workers, r up to 136: update
-// 175 us with 256 threads of 4 x 4 outputs, 146 with 512 threads of 4 x 2, now 120.
-constexpr int kGemmThreads = 256;
+// 175 us with 256 threads of 4 x 4 outputs, 146 with 512 threads of 4 x 2, 120 with 256 of 4 x 2 of each.
+// RN: rows per thread. A slice is latency as long as few warps run (fragments out of shared memory, conversions for the carry, a barrier):
+// 3400 clocks of two CTAs an SM where the multiply-adds take 1000. Eight rows make twice as many independent ones per fragment, three
+// CTAs fit an SM, and the sums' registers leave room for one slice on its way instead of two. Where CTAs are few, four rows in
+// twice as many warps end sooner (256 x 256, r = 16 step 21.6 and 23.5 us; see launch_gemm). With the sums of fast mode in 32 bits there are
+// registers for four rows to do as well (refresh of 768 x 1536, r = 128, K = 4 with eight 944 us, with four 752). Steps of three ragged
+// matrices with three workers, r up to 136: 186 -> 170 us; of 600 x 3000, r = 200, K = 2 252 -> 216; of 2048 x 2048, r = 128, K = 4 659 -> 584.
+// Loads by a pointer that moves on from slice to slice instead of an index formed anew gave 3 % of a step (192 -> 186, 262 -> 252).
 
 __device__ __forceinline__ void load_columns(float (&x)[4], const float* p) {
   const float4 v = *reinterpret_cast<const float4*>(p);
@@ -179,9 +187,9 @@ __device__ __forceinline__ f32x2 square2(f32x2 a) {
   return d;
 }
 
-template <int ATRANS, int DUAL, int CARRY>
-__global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
-  constexpr int NT = kGemmThreads, BN = gemm_columns(DUAL), CN = BN * BM / 4 / NT;  // threads, output columns per thread (rows: four)
+template <int ATRANS, int DUAL, int CARRY, int RN>
+__global__ void __launch_bounds__(1024 / RN, RN == 8 ? 3 : 2) gemm_ffma_kernel(const GemmProblem* __restrict__ probs, int nprobs, GemmScalars sc) {
+  constexpr int NT = 1024 / RN, NL = 256 / NT, BN = gemm_columns(DUAL), CN = BN * BM / RN / NT;  // output columns per thread
   __shared__ __align__(16) float sA[2][BK][BM + PADS];
   __shared__ __align__(16) float sB[2][BK][BN + PADS];
   __shared__ __align__(16) float sB2[2][DUAL ? BK : 1][BN + PADS];
@@ -211,19 +219,18 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
 
   const int t = threadIdx.x;
   const int tx = t % (BN / CN), ty = t / (BN / CN);
-  // loaders, a float4 of a slice each: every thread A; one product: every thread B, two: half of them B and the others B2.
-  const bool second = DUAL && t >= NT / 2;
-  const int lt = DUAL ? t & (NT / 2 - 1) : t;
-  // B: row kk, columns four at a time
-  const int bk = lt / (BN / 4), bc = lt % (BN / 4) * 4;
+  // loaders, NL float4 of each operand a slice; with two products B and B2 share them, one each or one by each half of the threads
+  const bool second = DUAL && NL == 1 && t >= NT / 2;
+  const int lt = DUAL && NL == 1 ? t & (NT / 2 - 1) : t;
+  const int bk = lt / (BN / 4), bc = lt % (BN / 4) * 4;  // row, columns four at a time; the second float4 NT / (BN / 4) rows on, or in B2
   const Source Bm = second ? B2 : B;
-  // A. ATRANS: as B (stored [Kd][M]). Otherwise stored [M][Kd]: row lt/4, k (lt%4)*4.
+  // A. ATRANS: as B (stored [Kd][M]), the second 8 rows of k on. Otherwise stored [M][Kd]: row t/4, k (t%4)*4, the second 32 rows on.
   const int ar = ATRANS ? (t >> 4) : (t >> 2), ac = ATRANS ? (t & 15) * 4 : (t & 3) * 4;
 
-  f32x2 acc[2][CN], acc2[DUAL ? 2 : 1][CN];  // rows in pairs
-  double tot[CARRY ? 4 : 1][CN], tot2[(CARRY && DUAL) ? 4 : 1][CN];
+  f32x2 acc[RN / 2][CN], acc2[DUAL ? RN / 2 : 1][CN];  // rows in pairs
+  double tot[CARRY ? RN : 1][CN], tot2[(CARRY && DUAL) ? RN : 1][CN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < RN; ++i)
 #pragma unroll
     for (int j = 0; j < CN; ++j) {
       acc[i / 2][j] = 0ull;
@@ -234,60 +241,74 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
       }
     }
 
-  // Two slices of k are on their way in registers while a third, in one of two buffers, is multiplied.
+  // One or two slices of k are on their way in registers while another, in one of two buffers, is multiplied.
+  constexpr int kSecond = DUAL ? 0 : NT / (BN / 4);
   struct Slice {
-    Raw x, y;
+    Raw a[NL], b[NL];
   };
-  auto fetch = [&](Slice& s, int k0) {
-    s.x = ATRANS ? source_load(A, k0 + ar, m0 + ac, Kd, M) : source_load(A, m0 + ar, k0 + ac, M, Kd);
-    s.y = source_load(Bm, k0 + bk, n0 + bc, Kd, N);
-  };
-  auto stash = [&](const Slice& s, int buf) {
-    const float4 v = source_value(A, s.x, sc);
-    if (ATRANS) {
-      *reinterpret_cast<float4*>(&sA[buf][ar][ac]) = v;
-    } else {
-      sA[buf][ac + 0][ar] = v.x; sA[buf][ac + 1][ar] = v.y; sA[buf][ac + 2][ar] = v.z; sA[buf][ac + 3][ar] = v.w;
-    }
-    *reinterpret_cast<float4*>(second ? &sB2[buf][DUAL ? bk : 0][bc] : &sB[buf][bk][bc]) = source_value(Bm, s.y, sc);
-  };
-
   // this CTA's range of k
   const int per = ((Kd + BK - 1) / BK + (int)csize - 1) / (int)csize * BK;
   const int kbeg = min((int)rank * per, Kd), kend = min(kbeg + per, Kd);
+  Feed fa, fb;
+  if (ATRANS) fa = {(long long)(kbeg + ar) * A.ld + m0 + ac, (long long)BK * A.ld, 8 * A.ld, kbeg + ar, 8, m0 + ac < M ? Kd : 0, m0 + ac < M ? Kd : 0};
+  else fa = {(m0 + ar) * A.ld + kbeg + ac, BK, 32 * A.ld, kbeg + ac, 0, m0 + ar < M ? Kd : 0, m0 + ar + 32 < M ? Kd : 0};
+  fb = {(long long)(kbeg + bk) * Bm.ld + n0 + bc, (long long)BK * Bm.ld, kSecond * Bm.ld, kbeg + bk, kSecond, n0 + bc < N ? Kd : 0, n0 + bc < N ? Kd : 0};
+  auto fetch = [&](Slice& s) {
+    feed_next<NL>(A, A, fa, s.a);
+    feed_next<NL>(Bm, DUAL ? B2 : B, fb, s.b);
+  };
+  auto stash = [&](const Slice& s, int buf) {
+#pragma unroll
+    for (int h = 0; h < NL; ++h) {
+      const float4 v = source_value(A, s.a[h], sc);
+      if (ATRANS) {
+        *reinterpret_cast<float4*>(&sA[buf][ar + 8 * h][ac]) = v;
+      } else {
+        sA[buf][ac + 0][ar + 32 * h] = v.x; sA[buf][ac + 1][ar + 32 * h] = v.y; sA[buf][ac + 2][ar + 32 * h] = v.z; sA[buf][ac + 3][ar + 32 * h] = v.w;
+      }
+      const bool to2 = DUAL && (NL == 1 ? second : h == 1);
+      *reinterpret_cast<float4*>(to2 ? &sB2[buf][DUAL ? bk : 0][bc] : &sB[buf][bk + kSecond * h][bc]) = source_value(DUAL && h ? B2 : Bm, s.b[h], sc);
+    }
+  };
   Slice x0, x1;
-  if (kbeg < kend) fetch(x0, kbeg);
-  if (kbeg + BK < kend) fetch(x1, kbeg + BK);
+  if (kbeg < kend) fetch(x0);
+  if (RN == 4 && kbeg + BK < kend) fetch(x1);
   if (kbeg < kend) stash(x0, 0);
   __syncthreads();
   int buf = 0;
   auto multiply = [&]() {
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][kk][ty * 4]);
-      const f32x2 a[2] = {pair_of(a4.x, a4.y), pair_of(a4.z, a4.w)};
+      f32x2 a[RN / 2];
+#pragma unroll
+      for (int h = 0; h < RN / 4; ++h) {
+        const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][kk][ty * RN + 4 * h]);
+        a[2 * h] = pair_of(a4.x, a4.y); a[2 * h + 1] = pair_of(a4.z, a4.w);
+      }
       float b[CN], c[CN];
       load_columns(b, &sB[buf][kk][tx * CN]);
 #pragma unroll
       for (int j = 0; j < CN; ++j) {
         const f32x2 bb = pair_of(b[j], b[j]);
-        acc[0][j] = fma2(a[0], bb, acc[0][j]);
-        acc[1][j] = fma2(a[1], bb, acc[1][j]);
+#pragma unroll
+        for (int p = 0; p < RN / 2; ++p) acc[p][j] = fma2(a[p], bb, acc[p][j]);
       }
       if constexpr (DUAL) {
         load_columns(c, &sB2[buf][kk][tx * CN]);
-        const f32x2 a2[2] = {sc.a_square ? square2(a[0]) : a[0], sc.a_square ? square2(a[1]) : a[1]};
+        f32x2 a2[RN / 2];
+#pragma unroll
+        for (int p = 0; p < RN / 2; ++p) a2[p] = sc.a_square ? square2(a[p]) : a[p];
 #pragma unroll
         for (int j = 0; j < CN; ++j) {
           const f32x2 cc = pair_of(c[j], c[j]);
-          acc2[0][j] = fma2(a2[0], cc, acc2[0][j]);
-          acc2[1][j] = fma2(a2[1], cc, acc2[1][j]);
+#pragma unroll
+          for (int p = 0; p < RN / 2; ++p) acc2[p][j] = fma2(a2[p], cc, acc2[p][j]);
         }
       }
     }
     if constexpr (CARRY) {
 #pragma unroll
-      for (int p = 0; p < 2; ++p)
+      for (int p = 0; p < RN / 2; ++p)
 #pragma unroll
         for (int j = 0; j < CN; ++j) {
           float lo, hi;
@@ -302,9 +323,9 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
         }
     }
   };
-  // on entry to a turn `far` is free, `near` holds the slice after the one in `buf`
+  // on entry to a turn `far` is free, `near` holds the slice after the one in `buf` (RN = 8: they are one)
   auto turn = [&](int k0, Slice& far, const Slice& near) {
-    if (k0 + 2 * BK < kend) fetch(far, k0 + 2 * BK);
+    if (k0 + (RN == 4 ? 2 : 1) * BK < kend) fetch(far);
     multiply();
     if (k0 + BK < kend) {
       stash(near, buf ^ 1);
@@ -312,14 +333,18 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
     }
     buf ^= 1;
   };
-  for (int k0 = kbeg; k0 < kend; k0 += 2 * BK) {
-    turn(k0, x0, x1);
-    if (k0 + BK < kend) turn(k0 + BK, x1, x0);
+  if constexpr (RN == 4) {
+    for (int k0 = kbeg; k0 < kend; k0 += 2 * BK) {
+      turn(k0, x0, x1);
+      if (k0 + BK < kend) turn(k0 + BK, x1, x0);
+    }
+  } else {
+    for (int k0 = kbeg; k0 < kend; k0 += BK) turn(k0, x0, x0);
   }
-  float out[4][CN], out2[DUAL ? 4 : 1][CN];  // without the carry: the sums
+  float out[RN][CN], out2[DUAL ? RN : 1][CN];  // without the carry: the sums
   if constexpr (!CARRY) {
 #pragma unroll
-    for (int p = 0; p < 2; ++p)
+    for (int p = 0; p < RN / 2; ++p)
 #pragma unroll
       for (int j = 0; j < CN; ++j) {
         unpair(acc[p][j], out[2 * p][j], out[2 * p + 1][j]);
@@ -329,10 +354,10 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
   const Epilogue& ep = pr.epi;
   if (DUAL || csize > 1) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RN; ++i)
 #pragma unroll
       for (int j = 0; j < CN; j += 2) {
-        double* o = part + (ty * 4 + i) * BN + tx * CN + j;
+        double* o = part + (ty * RN + i) * BN + tx * CN + j;
         if constexpr (CARRY) *reinterpret_cast<double2*>(o) = make_double2(tot[i][j], tot[i][j + 1]);
         else *reinterpret_cast<double2*>(o) = make_double2((double)out[i][j], (double)out[i][j + 1]);
         if constexpr (CARRY && DUAL) *reinterpret_cast<double2*>(o + BM * BN) = make_double2(tot2[i][j], tot2[i][j + 1]);
@@ -365,12 +390,12 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
     return;
   }
   if constexpr (!DUAL) {
-    // each thread owns rows m0+ty*4.., columns n0+tx*4..+3
+    // each thread owns rows m0+ty*RN.., columns n0+tx*4..+3
     const long long col = n0 + tx * 4;
     if (col >= N) return;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long long row = m0 + ty * 4 + i;
+    for (int i = 0; i < RN; ++i) {
+      const long long row = m0 + ty * RN + i;
       if (row >= M) break;
       if constexpr (CARRY) {
 #pragma unroll
@@ -384,39 +409,42 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_ffma_kernel(const GemmPr
 // CTAs per output tile, up to the portable cluster size: the count whose turns of CTAs on the device (two fit an SM) times
 // the slices of k of each, with about three more for its start and end, are least; each is left two slices. A product
 // with few tiles is a chain of slices, each about a trip to memory long: 256 x 256, r = 16, two replicas, P^T (c G + E) in
-// 8 CTAs 44 us, in 64 10.5; Gram matrices of 1000 rows and r up to 136 in 14 CTAs 105 us, in 112 17; 198 tiles of up to 63 slices
-// in 198 CTAs 78 us, in 792 74.
+// 8 CTAs 44 us, in 64 10.5; Gram matrices of 1000 rows and r up to 136 in 14 CTAs 105 us, in 112 17.
+// With eight rows a thread three fit an SM, a turn takes about a quarter longer, and the meeting of a cluster six slices: eight rows
+// where their turns are less than four fifths (without the quarter 1000 x 1000, r = 120 85 us against 71; with three slices for the meeting
+// too, 2048 x 2048, r = 128, K = 4 628 against 584 and three matrices of 400 54 against 51).
 void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
                  const GemmScalars& sc, cudaStream_t st) {
-  const long long room = (long long)sm_count * 2;  // by registers
   const int slices = (kd_max + BK - 1) / BK;
-  int c = 1;
-  long long best = -1;
-  for (int x = 1; x <= 8 && (x == 1 || slices >= 2 * x); x *= 2) {
-    const long long cost = ((total_tiles * x + room - 1) / room) * ((slices + x - 1) / x + 3);
-    if (best < 0 || cost < best) { best = cost; c = x; }
-  }
+  int c = 1, c8 = 1;
+  auto split = [&](long long room, int meet, int& count) {  // room: CTAs that fit, by registers
+    long long best = -1;
+    for (int x = 1; x <= 8 && (x == 1 || slices >= 2 * x); x *= 2) {
+      const long long cost = ((total_tiles * x + room - 1) / room) * ((slices + x - 1) / x + (x == 1 ? 3 : meet));
+      if (best < 0 || cost < best) { best = cost; count = x; }
+    }
+    return best;
+  };
+  const long long cost = split((long long)sm_count * 2, 3, c), cost8 = split((long long)sm_count * 3, 6, c8);
+  const bool eight = carry && 5 * cost8 < 4 * cost;
+  if (eight) c = c8;
   cudaLaunchConfig_t lc = {};
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)c; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_dep
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(kGemmThreads, 1, 1); lc.stream = st;
+  lc.gridDim = dim3((unsigned)(total_tiles * c), 1, 1); lc.blockDim = dim3(eight ? 128 : 256, 1, 1); lc.stream = st;
   lc.dynamicSmemBytes = c > 1 || dual ? sizeof(double) * BM * gemm_columns(dual) * (dual ? 2 : 1) : 0;
   lc.attrs = at; lc.numAttrs = 2;
-#define LORDO_GEMM(A, B, C) cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, C>, probs, nprobs, sc)
-  if (carry) {
-    if (atrans && !dual) LORDO_GEMM(1, 0, 1);
-    else if (!atrans && !dual) LORDO_GEMM(0, 0, 1);
-    else if (!atrans && dual) LORDO_GEMM(0, 1, 1);
-    else LORDO_GEMM(1, 1, 1);
-  } else {
-    if (atrans && !dual) LORDO_GEMM(1, 0, 0);
-    else if (!atrans && !dual) LORDO_GEMM(0, 0, 0);
-    else if (!atrans && dual) LORDO_GEMM(0, 1, 0);
-    else LORDO_GEMM(1, 1, 0);
-  }
+#define LORDO_GEMM(A, B)                                                                     \
+  if (eight) cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, 1, 8>, probs, nprobs, sc);        \
+  else if (carry) cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, 1, 4>, probs, nprobs, sc);   \
+  else cudaLaunchKernelEx(&lc, gemm_ffma_kernel<A, B, 0, 4>, probs, nprobs, sc)
+  if (atrans && !dual) LORDO_GEMM(1, 0);
+  else if (!atrans && !dual) LORDO_GEMM(0, 0);
+  else if (!atrans && dual) LORDO_GEMM(0, 1);
+  else LORDO_GEMM(1, 1);
 #undef LORDO_GEMM
 }
 
@@ -427,10 +455,10 @@ cudaError_t gemm_configure() {
   auto set = [&](const void* kernel, int smem) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   };
-  set((const void*)gemm_ffma_kernel<0, 0, 0>, one); set((const void*)gemm_ffma_kernel<0, 0, 1>, one);
-  set((const void*)gemm_ffma_kernel<1, 0, 0>, one); set((const void*)gemm_ffma_kernel<1, 0, 1>, one);
-  set((const void*)gemm_ffma_kernel<0, 1, 0>, two); set((const void*)gemm_ffma_kernel<0, 1, 1>, two);
-  set((const void*)gemm_ffma_kernel<1, 1, 0>, two); set((const void*)gemm_ffma_kernel<1, 1, 1>, two);
+  set((const void*)gemm_ffma_kernel<0, 0, 0, 4>, one); set((const void*)gemm_ffma_kernel<0, 0, 1, 4>, one); set((const void*)gemm_ffma_kernel<0, 0, 1, 8>, one);
+  set((const void*)gemm_ffma_kernel<1, 0, 0, 4>, one); set((const void*)gemm_ffma_kernel<1, 0, 1, 4>, one); set((const void*)gemm_ffma_kernel<1, 0, 1, 8>, one);
+  set((const void*)gemm_ffma_kernel<0, 1, 0, 4>, two); set((const void*)gemm_ffma_kernel<0, 1, 1, 4>, two); set((const void*)gemm_ffma_kernel<0, 1, 1, 8>, two);
+  set((const void*)gemm_ffma_kernel<1, 1, 0, 4>, two); set((const void*)gemm_ffma_kernel<1, 1, 1, 4>, two); set((const void*)gemm_ffma_kernel<1, 1, 1, 8>, two);
   return e;
 }
 

@@ -27,6 +27,22 @@ def test_fp32_products_in_ranges_of_k(shape, side):
     opt.close()
 
 
+@pytest.mark.parametrize("side", [0, 1])
+def test_fp32_products_of_many_tiles(side):
+    """More tiles than the device holds at once, worked on by threads of eight rows: ragged in every direction, a tile with 8 of 64 rows, a
+    contraction that ends within a slice, with one product and with two. Bound as above."""
+    mats = ((1001, 1336, 72), (527, 392, 136), (200, 136, 24))
+    if side:
+        mats = tuple((n, (m + 7) // 8 * 8, r) for m, n, r in mats)
+    wl = synth.Workload("t", mats, K=3, H=2, rounds=1, grad="gauss", clip_rho=30.0, sides=(side,) * 3)
+    spec = RunSpec(wl, variant=1, form=2, lr=0.01, omega=0.9, eps=0.05, refresh=False)
+    opt, orc = hz.run_gpu(spec), hz.run_oracle(spec)
+    st = hz.compare_states(opt, orc)
+    assert opt.poll_status() == 0
+    assert max(st["W"], st["E"], st["u"], st["v"]) < 2e-5, st
+    opt.close()
+
+
 @pytest.mark.parametrize("mats", [((72, 64, 8),), ((2056, 136, 24), (136, 2088, 64)), ((4104, 136, 24),), ((1544, 264, 72), (520, 1032, 264))])
 @pytest.mark.parametrize("side", [0, 1])
 def test_strips_in_pieces(mats, side):
