@@ -10,18 +10,17 @@ namespace lordo {
 // finish adds that pair's partial sums, the last pair of a worker the matrices' sums, both in a fixed order
 // whichever block it is. Bound by HBM (7 TB/s on 14 layers of 2048); with the two sums as kernels of their own a small
 // step spent 8 us more on launches, and 256 x 256 with chunks of 32768 had four blocks (step 40.0 -> 34.6 us).
+// The sums of a block meet by shuffles and one barrier (as a tree of nine barriers: 256 x 256 step 20.8 us, now 20.5).
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ double block_sum_256(double x, double* red) {  // all threads return the sum
-  const int t = threadIdx.x;
-  red[t] = x;
+// All threads return the sum of x, always in the same order; `red` is not used again before a barrier.
+__device__ __forceinline__ double block_sum_256(double x, double* red) {
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
   __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (t < s) red[t] += red[t + s];
-    __syncthreads();
-  }
-  const double r = red[0];
-  __syncthreads();
-  return r;
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s += red[w];
+  return s;
 }
 
 template <bool BF16>
@@ -29,7 +28,7 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
                                                    const long long* __restrict__ chunk_start, int n_mats, int K, long long chunk, double* partial,
                                                    float rho, int scope, float* __restrict__ coef, double* sumsq, unsigned* __restrict__ tickets,
                                                    unsigned* __restrict__ status) {
-  __shared__ double red[256];
+  __shared__ double red[3][8];
   __shared__ bool last_s;
   const int t = threadIdx.x;
   const long long blk = blockIdx.x;
@@ -70,13 +69,8 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
         }
       }
   }
-  double d = ((double)sum[0] + (double)sum[1]) + ((double)sum[2] + (double)sum[3]);
-  for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-  if ((t & 31) == 0) red[t >> 5] = d;
-  __syncthreads();
+  const double s = block_sum_256(((double)sum[0] + (double)sum[1]) + ((double)sum[2] + (double)sum[3]), red[0]);
   if (t == 0) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[w];
     partial[blk] = s;
     __threadfence();
     last_s = atomicInc(tickets + (long long)i * K + k, chunks - 1) == chunks - 1;  // back to zero with the last block
@@ -87,7 +81,7 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
   const double* p = partial + chunk_start[i] + (long long)k * chunks;
   double a = 0.0;
   for (unsigned c = t; c < chunks; c += 256) a += __ldcg(p + c);  // written by other SMs meanwhile: not from this one's L1
-  const double s_i = block_sum_256(a, red);
+  const double s_i = block_sum_256(a, red[1]);
   if (t == 0) {
     sumsq[(long long)i * K + k] = s_i;
     if (scope == 1) coef[(long long)i * K + k] = fminf(1.f, rho / ((float)sqrt(s_i) + 1e-6f));
@@ -99,7 +93,7 @@ __global__ void __launch_bounds__(256) clip_kernel(const MatDev* __restrict__ ma
   __threadfence();
   a = 0.0;
   for (int m = t; m < n_mats; m += 256) a += __ldcg(sumsq + (long long)m * K + k);
-  const double total = block_sum_256(a, red);
+  const double total = block_sum_256(a, red[2]);
   if (t == 0 && !isfinite(total)) atomicOr(status, LORDO_FLAG_NONFINITE_GRAD);
   const float c = fminf(1.f, rho / ((float)sqrt(total) + 1e-6f));
   if (scope == 0)
