@@ -25,7 +25,8 @@ enum Phase { PH_SUBSPACE = 0, PH_ROTATE = 1, PH_COMMIT = 2 };
 struct PlanStep {
   int type = ST_GEMM, phase = PH_SUBSPACE;
   int atrans = 0, dual = 0, a_square = 0;  // gemm
-  int r_max = 0;                           // chol, eig: largest size; gemm: longest contraction
+  ProductSplit split;                      // gemm, set by lordo_init
+  int r_max = 0;                           // chol, eig, rotate: largest size
   int with_e = 0;                          // sketch: the problems' A is c G + E
   int p0 = 0;                              // random: 1 = initial projection (draw index 0), 0 = sketch (index = refresh count)
   long long first = 0, tiles = 0;          // tiles: gemm tiles or 256-thread blocks
@@ -483,9 +484,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       PlanStep st = sl.st;
       if (st.type == ST_GEMM) {
         st.first = (long long)P.size(); st.count = (int)sl.g.size(); st.tiles = 0;
-        st.r_max = 0;
         for (GemmProblem& g : sl.g) {
-          if (g.Kd > st.r_max) st.r_max = g.Kd;
           g.tile_start = st.tiles;
           st.tiles += (long long)((g.M + 63) / 64) * g.tiles_n;
           P.push_back(g);
@@ -1025,12 +1024,28 @@ GemmScalars base_scalars(const lordo_ctx* c) {
   return s;
 }
 
+// How the fp32 products of a list of launches are split on this device.
+void split_products(const lordo_ctx* c, std::vector<PlanStep>& steps) {
+  for (PlanStep& s : steps) {
+    if (s.type != ST_GEMM) continue;
+    std::vector<ProductRun> runs;
+    for (int i = 0; i < s.count; ++i) {
+      const GemmProblem& g = c->h_probs[s.first + i];
+      const int slices = (g.Kd + 15) / 16;
+      const long long tiles = (long long)((g.M + 63) / 64) * g.tiles_n;
+      if (!runs.empty() && runs.back().slices == slices) runs.back().tiles += tiles;
+      else runs.push_back({slices, tiles});
+    }
+    s.split = c->cfg.check_mode ? split_by_time(std::move(runs), c->sm_count) : split_by_turns(runs, c->sm_count);
+  }
+}
+
 int run_plan_step(lordo_ctx* c, const PlanStep& s, GemmScalars sc, cudaStream_t st) {
   if (s.count == 0) return LORDO_OK;
   switch (s.type) {
     case ST_GEMM:
       sc.a_square = s.a_square;
-      launch_gemm(c->d_probs + s.first, s.count, s.tiles, s.r_max, s.atrans, s.dual, c->cfg.check_mode != 0, c->sm_count, sc, st);
+      launch_gemm(c->d_probs + s.first, s.count, s.tiles, s.split, s.atrans, s.dual, c->cfg.check_mode != 0, sc, st);
       c->launches += 1;
       return check_launch(c, "gemm");
     case ST_CHOL:
@@ -1229,6 +1244,7 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
     int dev = 0;
     INIT_CUDA(cudaGetDevice(&dev));
     INIT_CUDA(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev));
+    for (std::vector<PlanStep>* steps : {&c->inner_proj, &c->inner_apply, &c->refresh_steps, &c->init_steps, &c->tb_steps}) split_products(c, *steps);
     INIT_CUDA(gemm_configure());
     INIT_CUDA(chol_configure());
   }

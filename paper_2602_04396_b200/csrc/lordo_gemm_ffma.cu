@@ -143,7 +143,7 @@ __device__ __forceinline__ void partials_of(const double* p, unsigned rank, doub
 }
 
 // A cluster of CTAs works on one output tile, each on a range of k; the partial sums meet in fp64 through
-// distributed shared memory, every CTA finishing its share of the tile's rows (see launch_gemm for the size).
+// distributed shared memory, every CTA finishing its share of the tile's rows (see lordo_plan.h for the size).
 // CARRY = 1: slice sums carried across k-slices in fp64 (parity mode). CARRY = 0: plain fp32
 // accumulation, half the registers (the fp32 work of the fast mode: QR and moment rotation).
 // With two products a tile is half as wide (gemm_columns): a thread then holds two columns of each, two CTAs fit an SM and the
@@ -152,7 +152,7 @@ __device__ __forceinline__ void partials_of(const double* p, unsigned rank, doub
 // RN: rows per thread. A slice is latency as long as few warps run (fragments out of shared memory, conversions for the carry, a barrier):
 // 3400 clocks of two CTAs an SM where the multiply-adds take 1000. Eight rows make twice as many independent ones per fragment, three
 // CTAs fit an SM, and the sums' registers leave room for one slice on its way instead of two. Where CTAs are few, four rows in
-// twice as many warps end sooner (256 x 256, r = 16 step 21.6 and 23.5 us; see launch_gemm). With the sums of fast mode in 32 bits there are
+// twice as many warps end sooner (256 x 256, r = 16 step 21.6 and 23.5 us; see split_by_time). With the sums of fast mode in 32 bits there are
 // registers for four rows to do as well (refresh of 768 x 1536, r = 128, K = 4 with eight 944 us, with four 752). Steps of three ragged
 // matrices with three workers, r up to 136: 186 -> 170 us; of 600 x 3000, r = 200, K = 2 252 -> 216; of 2048 x 2048, r = 128, K = 4 659 -> 584.
 // Loads by a pointer that moves on from slice to slice instead of an index formed anew gave 3 % of a step (192 -> 186, 262 -> 252).
@@ -406,28 +406,11 @@ __global__ void __launch_bounds__(1024 / RN, RN == 8 ? 3 : 2) gemm_ffma_kernel(c
   }
 }
 
-// CTAs per output tile, up to the portable cluster size: the count whose turns of CTAs on the device (two fit an SM) times
-// the slices of k of each, with about three more for its start and end, are least; each is left two slices. A product
-// with few tiles is a chain of slices, each about a trip to memory long: 256 x 256, r = 16, two replicas, P^T (c G + E) in
-// 8 CTAs 44 us, in 64 10.5; Gram matrices of 1000 rows and r up to 136 in 14 CTAs 105 us, in 112 17.
-// With eight rows a thread three fit an SM, a turn takes about a quarter longer, and the meeting of a cluster six slices: eight rows
-// where their turns are less than four fifths (without the quarter 1000 x 1000, r = 120 85 us against 71; with three slices for the meeting
-// too, 2048 x 2048, r = 128, K = 4 628 against 584 and three matrices of 400 54 against 51).
-void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
+// Rows per thread and CTAs per output tile: see lordo_plan.h.
+void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, ProductSplit split, int atrans, int dual, int carry,
                  const GemmScalars& sc, cudaStream_t st) {
-  const int slices = (kd_max + BK - 1) / BK;
-  int c = 1, c8 = 1;
-  auto split = [&](long long room, int meet, int& count) {  // room: CTAs that fit, by registers
-    long long best = -1;
-    for (int x = 1; x <= 8 && (x == 1 || slices >= 2 * x); x *= 2) {
-      const long long cost = ((total_tiles * x + room - 1) / room) * ((slices + x - 1) / x + (x == 1 ? 3 : meet));
-      if (best < 0 || cost < best) { best = cost; count = x; }
-    }
-    return best;
-  };
-  const long long cost = split((long long)sm_count * 2, 3, c), cost8 = split((long long)sm_count * 3, 6, c8);
-  const bool eight = carry && 5 * cost8 < 4 * cost;
-  if (eight) c = c8;
+  const int c = split.ctas;
+  const bool eight = split.rows == 8;
   cudaLaunchConfig_t lc = {};
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;

@@ -89,7 +89,7 @@ struct GemmScalars {
   int form, ef, w_dt, e_dt, g_dt, a_square;
 };
 
-void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, int kd_max, int atrans, int dual, int carry, int sm_count,
+void launch_gemm(const GemmProblem* probs, int nprobs, long long total_tiles, ProductSplit split, int atrans, int dual, int carry,
                  const GemmScalars& sc, cudaStream_t st);
 cudaError_t gemm_configure();
 

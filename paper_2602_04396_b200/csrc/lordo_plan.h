@@ -1,6 +1,8 @@
 // Rules by which work is dealt out, on the host and free of CUDA: tests compile this file on its own.
 #pragma once
 #include <algorithm>
+#include <functional>
+#include <queue>
 #include <utility>
 #include <vector>
 
@@ -128,6 +130,91 @@ inline void deal_out(std::vector<WorkItem> items, int workers, bool split, int h
     start.push_back((int)list.size());
   }
   while (start.size() > 1 && start[start.size() - 2] == (int)list.size()) start.pop_back();
+}
+
+// ---- fp32 products: rows per thread and CTAs per output tile ------------------------------------
+// Consecutive tiles of a launch whose contraction takes `slices` slices of 16 k.
+struct ProductRun {
+  int slices;
+  long long tiles;
+};
+struct ProductSplit {
+  int rows = 4, ctas = 1;  // rows per thread (4 or 8); CTAs per tile, a cluster that shares the slices
+};
+inline int longest_run(const std::vector<ProductRun>& runs) {
+  int longest = 1;
+  for (const ProductRun& r : runs) longest = std::max(longest, r.slices);
+  return longest;
+}
+
+// How long a launch takes, in slices of a CTA of four rows that has an SM to itself. CTAs take their places in the order of the tiles; what
+// a slice takes depends on how many share an SM: four rows 1 and, two on an SM, 1.2, eight rows 1.375, 1.4 and, three, 1.475
+// (a slice of one CTA is latency: 0.85 us). A CTA takes some four slices more for its start and end, and the meeting of a cluster one
+// and 0.45 for each of its CTAs.
+inline double product_time(const std::vector<ProductRun>& runs, int rows, int ctas, int sms) {
+  typedef std::pair<double, long long> Group;  // when they end, at the pace of one to an SM, and how many
+  std::priority_queue<Group, std::vector<Group>, std::greater<Group>> running;
+  const long long room = (long long)sms * (rows == 4 ? 2 : 3);  // by registers
+  const double extra = (rows == 4 ? 4.5 : 4.0) + (ctas > 1 ? 1.0 + 0.45 * ctas : 0.0);
+  const auto pace = [&](double per_sm) {
+    if (rows == 4) return 1.0 + 0.2 * std::max(0.0, per_sm - 1.0);
+    return per_sm <= 2.0 ? 1.375 + 0.025 * std::max(0.0, per_sm - 1.0) : 1.4 + 0.075 * (per_sm - 2.0);
+  };
+  double at = 0.0, time = 0.0;
+  long long resident = 0;
+  size_t next = 0;
+  long long left = runs.empty() ? 0 : runs[0].tiles * ctas;
+  for (;;) {
+    while (next < runs.size() && resident < room) {
+      const long long n = std::min(left, room - resident);
+      if (n > 0) running.push(Group(at + (runs[next].slices + ctas - 1) / ctas + extra, n));
+      resident += n;
+      left -= n;
+      if (left == 0 && ++next < runs.size()) left = runs[next].tiles * ctas;
+    }
+    if (running.empty()) return time;
+    const double end = running.top().first;
+    time += (end - at) * pace((double)resident / sms);
+    at = end;
+    while (!running.empty() && running.top().first <= at) { resident -= running.top().second; running.pop(); }
+  }
+}
+
+// Sums carried in fp32 (fast mode): four rows, and the count of CTAs whose turns on the device times the slices of k of each, with about three
+// more for its start and end, are least; each is left two slices. A product with few tiles is a chain of slices, each about a
+// trip to memory long: 256 x 256, r = 16, two replicas, P^T (c G + E) in 8 CTAs 44 us, in 64 10.5; Gram matrices of 1000 rows and
+// r up to 136 in 14 CTAs 105 us, in 112 17.
+inline ProductSplit split_by_turns(const std::vector<ProductRun>& runs, int sms) {
+  const int slices = longest_run(runs);
+  long long tiles = 0, best = -1;
+  for (const ProductRun& r : runs) tiles += r.tiles;
+  ProductSplit s;
+  for (int x = 1; x <= 8 && (x == 1 || slices >= 2 * x); x *= 2) {
+    const long long cost = ((tiles * x + 2 * sms - 1) / (2 * sms)) * ((slices + x - 1) / x + 3);
+    if (best < 0 || cost < best) { best = cost; s.ctas = x; }
+  }
+  return s;
+}
+
+// Sums carried in fp64 (check mode): the rows and CTAs whose launch is over first by product_time. Turns of CTAs as long as the longest contraction
+// told eight rows from four only where the contractions are alike: matrices of 5472 rows, r = 120 and of 64 to 3704 rows, r <= 40
+// took 209 us in pairs of eight rows by that rule, 87 in fours of four rows, and take 71 now. Over 482 launches of parity runs of random
+// shapes the choice takes at most 1.015 of the best split's time for nine of ten, and 1.25 for the worst (by turns 1.2 and 3.2).
+// A launch of more than 2048 tiles is timed as one of that many: the same choice, and a bounded time to make it in.
+inline ProductSplit split_by_time(std::vector<ProductRun> runs, int sms) {
+  const int slices = longest_run(runs);
+  long long tiles = 0;
+  for (const ProductRun& r : runs) tiles += r.tiles;
+  if (tiles > 2048)
+    for (ProductRun& r : runs) r.tiles = (r.tiles * 2048 + tiles - 1) / tiles;
+  ProductSplit best;
+  double least = -1.0;
+  for (int rows = 4; rows <= 8; rows += 4)
+    for (int x = 1; x <= 8 && (x == 1 || slices >= 2 * x); x *= 2) {
+      const double t = product_time(runs, rows, x, sms);
+      if (least < 0.0 || t < least) { least = t; best.rows = rows; best.ctas = x; }
+    }
+  return best;
 }
 
 }  // namespace lordo

@@ -27,14 +27,15 @@ def test_fp32_products_in_ranges_of_k(shape, side):
     opt.close()
 
 
+@pytest.mark.parametrize("mats,K", [(((1001, 1336, 72), (527, 392, 136), (200, 136, 24)), 3), (((2200, 264, 72), (72, 4040, 24), (96, 1536, 8)), 1)])
 @pytest.mark.parametrize("side", [0, 1])
-def test_fp32_products_of_many_tiles(side):
+def test_fp32_products_of_many_tiles(side, mats, K):
     """More tiles than the device holds at once, worked on by threads of eight rows: ragged in every direction, a tile with 8 of 64 rows, a
-    contraction that ends within a slice, with one product and with two. Bound as above."""
-    mats = ((1001, 1336, 72), (527, 392, 136), (200, 136, 24))
+    contraction that ends within a slice, with one product and with two. Then a few tiles of a long contraction among many of a
+    short one, in clusters of eight CTAs of which most have no slice of the short ones. Bound as above."""
     if side:
         mats = tuple((n, (m + 7) // 8 * 8, r) for m, n, r in mats)
-    wl = synth.Workload("t", mats, K=3, H=2, rounds=1, grad="gauss", clip_rho=30.0, sides=(side,) * 3)
+    wl = synth.Workload("t", mats, K=K, H=2, rounds=1, grad="gauss", clip_rho=30.0, sides=(side,) * 3)
     spec = RunSpec(wl, variant=1, form=2, lr=0.01, omega=0.9, eps=0.05, refresh=False)
     opt, orc = hz.run_gpu(spec), hz.run_oracle(spec)
     st = hz.compare_states(opt, orc)

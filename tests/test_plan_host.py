@@ -22,6 +22,12 @@ extern "C" int deal(int n, const int* len, int workers, int split, int busy, int
   *starts = (int)st.size();
   return (int)list.size();
 }
+extern "C" int split(int n, const int* slices, const int* tiles, int carry, int sms) {
+  std::vector<lordo::ProductRun> runs;
+  for (int i = 0; i < n; ++i) runs.push_back({slices[i], tiles[i]});
+  const lordo::ProductSplit s = carry ? lordo::split_by_time(runs, sms) : lordo::split_by_turns(runs, sms);
+  return 10 * s.rows + s.ctas;
+}
 extern "C" int ranges(long long tiles, long long steps, long long most, long long pairs) { return lordo::k_ranges(tiles, steps, most, pairs); }
 """
 
@@ -105,3 +111,32 @@ def test_workspace_of_the_kept_signal():
     assert size([big], 16, 2) <= 4.88e9 and size([big] * 8, 16, 2) <= 39.04e9
     for m, n, r, K in ((2048, 2048, 64, 8), (7504, 3888, 168, 2), (200, 1112, 8, 1), (2048, 2048, 256, 8)):
         assert size([(m, n, r)], K, 1) - size([(m, n, r)], K, 1, ef=False) <= 2 * K * m * n
+
+
+# launches of the fp32 products, (slices of k, tiles) in the order of the tiles, and what each split of them took, us: contractions of one
+# length with few and with many tiles, and long ones among short ones
+@pytest.mark.parametrize("runs,took", [
+    ([(16, 8)], {41: 16.9, 42: 13.1, 44: 9.0, 48: 8.9, 81: 21.2, 82: 16.9, 84: 10.9, 88: 9.0}),
+    ([(250, 64)], {41: 205.6, 42: 107.4, 44: 78.7, 48: 86.8, 81: 283.3, 82: 148.2, 84: 94.0, 88: 105.2}),
+    ([(71, 264)], {41: 92.0, 42: 97.6, 44: 111.4, 48: 147.7, 81: 106.4, 82: 109.8, 84: 106.2, 88: 132.5}),
+    ([(9, 3168)], {41: 196.3, 42: 273.7, 44: 527.8, 48: 1166.9, 81: 173.0, 82: 236.8, 84: 421.8, 88: 929.8}),
+    ([(22, 9), (342, 18), (232, 2), (4, 62), (6, 95), (68, 3)], {41: 295.8, 42: 153.2, 44: 87.1, 48: 77.0, 81: 406.2, 82: 209.6, 84: 112.4, 88: 71.1}),
+    ([(216, 1), (29, 177), (36, 12), (15, 2)], {41: 193.5, 42: 102.1, 44: 61.9, 48: 82.2, 81: 258.8, 82: 138.0, 84: 78.6, 88: 69.0}),
+    ([(52, 57), (69, 184), (58, 156), (4, 1), (368, 3)], {41: 381.2, 42: 252.2, 44: 213.8, 48: 244.5, 81: 453.9, 82: 290.0, 84: 216.2, 88: 230.6}),
+])
+def test_fp32_products_split_by_time(plan, runs, took):
+    """The split that the rule chooses took at most a tenth longer than the best."""
+    n = len(runs)
+    chosen = plan.split(n, (C.c_int * n)(*[s for s, _ in runs]), (C.c_int * n)(*[t for _, t in runs]), 1, 148)
+    assert took[chosen] <= 1.1 * min(took.values()), chosen
+
+
+@pytest.mark.parametrize("carry", [0, 1])
+@pytest.mark.parametrize("sms", [148, 20])
+def test_fp32_products_split_of_any_launch(plan, carry, sms):
+    """A count that the longest contraction has two slices for, also at one slice, one tile and more tiles than are timed."""
+    for runs in ([(1, 1)], [(1, 100000)], [(3, 7)], [(4, 1), (1, 1)], [(2, 50000), (400, 1), (3, 50000)], [(8, 3), (9, 3000000)]):
+        n = len(runs)
+        got = plan.split(n, (C.c_int * n)(*[s for s, _ in runs]), (C.c_int * n)(*[t for _, t in runs]), carry, sms)
+        rows, ctas = got // 10, got % 10
+        assert rows in ((4, 8) if carry else (4,)) and ctas in (1, 2, 4, 8) and (ctas == 1 or max(s for s, _ in runs) >= 2 * ctas)
