@@ -1338,10 +1338,11 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
           for (const WorkItem& it : items) steps += it.len;
           // SMs whose update keeps the memory busy; two sweeps (r > 256) are bound by what an SM pulls out of L2
           const int busy = c->tc_rn_max > 256 ? c->sm_count : c->sm_count * 7 / 9;
+          const int shortest = c->tma ? kMinPiece : kMinPiece32;
           // no more workers than there are pieces
           const int most = l == 0 ? std::min(project_pairs(c->sm_count), (int)items.size())
-                                  : (int)std::min<long long>(c->sm_count, std::max<long long>((long long)items.size(), steps / kMinPiece));
-          deal_out(std::move(items), std::min(most, kMaxWorkers), l > 0, l > 0 ? kPieceHead : 0, busy, list, start);
+                                  : (int)std::min<long long>(c->sm_count, std::max<long long>((long long)items.size(), steps / shortest));
+          deal_out(std::move(items), std::min(most, kMaxWorkers), l > 0, l > 0 ? kPieceHead : 0, shortest, busy, list, start);
           c->seg_workers[l] = (int)start.size() - 1;
           if (list.size() > (size_t)(l == 0 ? c->tc_pairs : c->tc_strips + kMaxWorkers)) return bail(LORDO_ERR_NOMEM);
           INIT_CUDA(cudaMemcpyAsync(c->d_segs[l], list.data(), sizeof(TcSeg) * list.size(), cudaMemcpyHostToDevice, st));

@@ -26,8 +26,8 @@ inline int k_ranges(long long tiles, long long steps, long long most, long long 
   return (int)best;
 }
 
-// A piece of work of one CTA (update) or CTA pair (projection) of the TMA-fed kernels: steps [t0, t1) of 64 rows of one
-// strip, or one pair of strips. Workers walk their own part of a list, [start[w], start[w + 1]), dealt out by lordo_init so
+// A piece of work of one CTA (update) or CTA pair (projection) of the TMA-fed kernels: steps [t0, t1) of one strip, of 64 rows
+// each with bf16 storage and of 32 with fp32 (as many bytes), or one pair of strips. Workers walk their own part of a list, [start[w], start[w + 1]), dealt out by lordo_init so
 // that all of them end together.
 struct TcSeg {
   int prob, strip, t0, t1;
@@ -36,18 +36,22 @@ struct WorkItem {  // a strip (or a pair of strips) of `len` steps that costs `c
   int prob, strip, len;
   double cost;
 };
-constexpr int kMinPiece = 8;   // steps of a piece of a cut strip
+// Steps of a piece of a cut strip. With fp32 storage short ones pay: the products of a step are half as long, and with pieces of eight 1064 x 72,
+// r = 8 went to 5 CTAs (a round of four steps 170 us, with pieces of four 154, of two 146; the kernel before this one 161),
+// 456 x 592, r = 32 and two workers to 10 (38.9, 30.7, 28.7; 36.4). 190 steps and rounds of random shapes: 1.04 times as fast on average with pieces
+// of two as of eight, at worst 0.97. A smaller kPieceHead cost up to 4 % of some, a larger one changed nothing, nor did other shares of busy SMs.
+constexpr int kMinPiece = 8, kMinPiece32 = 2;
 constexpr int kPieceHead = 4;  // steps that a piece costs on top of its own: its operands are fetched anew
 
 // Deals items out, longest first, each to the worker with the least so far. Returns the longest worker's.
 //   WHOLE  strips are not cut
 //   EVEN   a strip that would take its worker past `share` is cut there and the rest dealt on; what finds no room is dealt on
-//          top, in the shortest pieces, and a remainder that would be too short stays with the piece before it
+//          top, in the shortest pieces (of `least` steps), and a remainder that would be too short stays with the piece before it
 //   WITHIN no worker gets more than `share`: a remainder that would be too short is made long enough at the cost of the piece
 //          before it. Returns -1 where something has no place. A worker is cut at most once, being left with less room
 //          than a piece needs, so there are at most items + workers pieces.
 enum Dealing { WHOLE, EVEN, WITHIN };
-inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, double share, std::vector<std::vector<TcSeg>>& lists) {
+inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, int least, double share, std::vector<std::vector<TcSeg>>& lists) {
   typedef std::pair<double, int> Load;  // what a worker has, the worker
   std::vector<Load> heap;
   for (int w = 0; w < (int)lists.size(); ++w) { lists[w].clear(); heap.push_back(Load(0.0, w)); }
@@ -60,11 +64,11 @@ inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, doubl
       const int rest = it.len - t0, room = (int)(share - ld.first - head + 0.5);
       int n = rest;
       if (how == EVEN && n > room) {
-        n = std::min(n, std::max(room, kMinPiece));
-        if (rest - n < kMinPiece) n = rest;
+        n = std::min(n, std::max(room, least));
+        if (rest - n < least) n = rest;
       } else if (how == WITHIN && n > room) {
-        n = std::min(room, rest - kMinPiece);
-        if (n < kMinPiece) return -1;
+        n = std::min(room, rest - least);
+        if (n < least) return -1;
       }
       lists[ld.second].push_back({it.prob, it.strip, t0, t0 + n});
       ld.first += how == WHOLE ? it.cost + head : n + head;
@@ -102,21 +106,21 @@ inline double time_of(const std::vector<std::vector<TcSeg>>& lists, int head, in
 // most SMs have a whole strip the memory is busy anyway and WHOLE is, since every piece fetches its operands. Either is taken where
 // it ends sooner than EVEN by a tenth by time_of, which is about how well that tells: update of 4096 rows, r = 256, EVEN, WHOLE and WITHIN:
 // 40 strips 50, 83, 43 us; 120 strips 122, 107, 121 us; 256 strips 241, 241, 245 us; mixes that it called 4 to 8 % better were 2 to 5 % slower.
-inline void deal_out(std::vector<WorkItem> items, int workers, bool split, int head, int busy, std::vector<TcSeg>& list, std::vector<int>& start) {
+inline void deal_out(std::vector<WorkItem> items, int workers, bool split, int head, int shortest, int busy, std::vector<TcSeg>& list, std::vector<int>& start) {
   std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.cost > b.cost; });
   std::vector<std::vector<TcSeg>> lists(workers);
-  const int longest = deal(items, WHOLE, head, 0.0, lists);
+  const int longest = deal(items, WHOLE, head, shortest, 0.0, lists);
   if (split) {
     double total = 0.0;
     for (const WorkItem& it : items) total += it.cost + head;
     std::vector<std::vector<TcSeg>> even(workers), cut(workers), within;
-    deal(items, EVEN, head, std::max(total / workers + head / 2.0, (double)(kMinPiece + head)), even);
+    deal(items, EVEN, head, shortest, std::max(total / workers + head / 2.0, (double)(shortest + head)), even);
     size_t pieces = 0;
     for (const std::vector<TcSeg>& l : even) pieces += l.size();
-    int least = std::max((int)(total / workers), kMinPiece + head) - 1, share = longest;  // nothing below, everything at WHOLE's longest
+    int least = std::max((int)(total / workers), shortest + head) - 1, share = longest;  // nothing below, everything at WHOLE's longest
     while (share - least > 1) {
       const int mid = least + (share - least) / 2;
-      if (deal(items, WITHIN, head, mid, cut) < 0) least = mid;
+      if (deal(items, WITHIN, head, shortest, mid, cut) < 0) least = mid;
       else { share = mid; within.swap(cut); cut.resize(workers); }
     }
     if (!within.empty() && time_of(within, head, busy) < time_of(lists, head, busy)) lists.swap(within);

@@ -10,12 +10,12 @@ from paper_2602_04396_b200 import lordo
 
 WRAPPER = """
 #include "lordo_plan.h"
-extern "C" int deal(int n, const int* len, int workers, int split, int busy, int* seg, int* start, int* starts) {
+extern "C" int deal(int n, const int* len, int workers, int split, int f32, int busy, int* seg, int* start, int* starts) {
   std::vector<lordo::WorkItem> items;
   for (int i = 0; i < n; ++i) items.push_back({i, i, len[i], (double)len[i]});
   std::vector<lordo::TcSeg> list;
   std::vector<int> st;
-  lordo::deal_out(items, workers, split != 0, split ? lordo::kPieceHead : 0, busy, list, st);
+  lordo::deal_out(items, workers, split != 0, split ? lordo::kPieceHead : 0, f32 ? lordo::kMinPiece32 : lordo::kMinPiece, busy, list, st);
   if ((int)list.size() > n + workers || (int)st.size() > workers + 1) return -1;
   for (size_t i = 0; i < list.size(); ++i) { seg[3 * i] = list[i].prob; seg[3 * i + 1] = list[i].t0; seg[3 * i + 2] = list[i].t1; }
   for (size_t i = 0; i < st.size(); ++i) start[i] = st[i];
@@ -41,7 +41,7 @@ def plan(tmp_path_factory):
     subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", lbuild.CSRC, "-o", so, src], check=True)
     lib = C.CDLL(so)
     lib.ranges.argtypes = [C.c_longlong] * 4
-    lib.deal.argtypes = [C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
+    lib.deal.argtypes = [C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]
     return lib
 
 
@@ -63,7 +63,7 @@ def test_strips_dealt_out(plan, strips, cut, most, sms, split):
     lens = [ln for count, ln in strips for _ in range(count)]
     workers = min(sms, max(len(lens), sum(lens) // MIN_PIECE))
     seg, start, starts = (C.c_int * (3 * (len(lens) + workers)))(), (C.c_int * (workers + 1))(), C.c_int()
-    pieces = plan.deal(len(lens), (C.c_int * len(lens))(*lens), workers, split, sms * 7 // 9, seg, start, C.byref(starts))
+    pieces = plan.deal(len(lens), (C.c_int * len(lens))(*lens), workers, split, 0, sms * 7 // 9, seg, start, C.byref(starts))
     assert 0 < pieces <= len(lens) + workers
     got = [(seg[3 * i], seg[3 * i + 1], seg[3 * i + 2]) for i in range(pieces)]
     at = [0] * len(lens)
@@ -76,6 +76,26 @@ def test_strips_dealt_out(plan, strips, cut, most, sms, split):
     if split and sms == 148:
         loads = [sum(t1 - t0 + HEAD for _, t0, t1 in got[a:b]) for a, b in zip(starts, starts[1:])]
         assert max(loads) <= most * sum(loads) / workers and (pieces > len(lens)) == cut
+
+
+# fp32 storage: strips (count, 32-row steps), and the workers and the longest worker's steps at most on 148 SMs
+@pytest.mark.parametrize("strips,workers,longest", [([(1, 34)], 17, 3), ([(10, 15)], 75, 3), ([(4, 44)], 88, 3), ([(1, 3)], 1, 3), ([(28, 4)], 56, 2),
+                                                    ([(64, 64)], 148, 32), ([(149, 3)], 148, 6)])
+def test_strips_of_fp32_storage_dealt_out(plan, strips, workers, longest):
+    """Every step of every strip once, in pieces of two steps or more: few short strips reach as many SMs as their rows allow."""
+    lens = [ln for count, ln in strips for _ in range(count)]
+    most = min(148, max(len(lens), sum(lens) // 2))
+    seg, start, starts = (C.c_int * (3 * (len(lens) + most)))(), (C.c_int * (most + 1))(), C.c_int()
+    pieces = plan.deal(len(lens), (C.c_int * len(lens))(*lens), most, 1, 1, 148 * 7 // 9, seg, start, C.byref(starts))
+    got = [(seg[3 * i], seg[3 * i + 1], seg[3 * i + 2]) for i in range(pieces)]
+    at = [0] * len(lens)
+    for prob, t0, t1 in sorted(got):
+        assert t0 == at[prob] and t1 - t0 >= 2
+        at[prob] = t1
+    assert at == lens
+    starts = list(start)[:starts.value]
+    loads = [sum(t1 - t0 for _, t0, t1 in got[a:b]) for a, b in zip(starts, starts[1:])]
+    assert len(loads) >= 0.8 * workers and max(loads) <= longest, loads
 
 
 @pytest.mark.parametrize("rows", [8, 64, 520, 4096, 65536, 65600, 70000, 87424, 128256, 151936, 1 << 20])
