@@ -125,8 +125,7 @@ struct lordo_ctx {
   bool tma = false;              // bf16 storage: projection and refresh too; with fp32 storage the update alone is fed by TMA
   int sm_count = 0;
   TmaMatMaps* d_maps = nullptr;
-  TmaGradMaps* d_gmaps = nullptr;
-  TmaGradMaps* h_gmaps = nullptr;  // pinned, two slots of n_mats entries
+  TmaGradMaps* d_gmaps = nullptr;  // behind d_Gtab, at maps_at
   std::vector<TcProblem> h_tc;
   std::vector<TcPrep> h_prep;
   std::vector<long long> h_prep_start;
@@ -156,8 +155,9 @@ struct lordo_ctx {
   std::vector<PlanStep> tb_steps;  // Delta rebuilt from the time buffers (lordo_outer_step with time_buffer)
 
   // pinned host staging
-  const void** h_Gtab = nullptr;  // pinned, two slots of n_mats entries
-  unsigned* h_status = nullptr;   // pinned (this and h_gmaps: in h_Gtab's block)
+  char* h_grads = nullptr;       // pinned: two slots of what d_Gtab and d_gmaps hold, copied as one, and the flag word
+  size_t maps_at = 0, slot_bytes = 0;
+  unsigned* h_status = nullptr;  // in h_grads' block
   std::vector<const void*> last_G;
   cudaEvent_t g_slot_ev[2] = {nullptr, nullptr};  // behind the last copy out of each staging slot
   bool g_slot_used[2] = {false, false};
@@ -303,6 +303,9 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   c->d_wblk_start = cv.take<long long>(n_mats + 1);
   c->d_sblk_start = cv.take<long long>(n_mats + 1);
   c->d_Gtab = cv.take<const void*>(n_mats);
+  c->maps_at = (sizeof(void*) * n_mats + 255) & ~size_t(255);
+  c->slot_bytes = c->maps_at + (c->tc ? sizeof(TmaGradMaps) * n_mats : 0);
+  if (c->tc) c->d_gmaps = cv.take<TmaGradMaps>(n_mats);
   c->d_status = cv.take<unsigned>(64);
   c->d_sumsq = cv.take<double>((size_t)n_mats * K);
   c->d_coef = cv.take<float>((size_t)n_mats * K);
@@ -452,7 +455,6 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
     c->d_tc_prep = cv.take<TcPrep>(c->h_prep.size());
     c->d_prep_start = cv.take<long long>(c->h_prep_start.size());
     c->d_maps = cv.take<TmaMatMaps>(n_mats);
-    c->d_gmaps = cv.take<TmaGradMaps>(n_mats);
     if (c->tma && !local)
       for (int i = 0; i < n_mats; ++i) c->h_mats[i].Delta16 = cv.take<__nv_bfloat16>((size_t)c->h_mats[i].m * c->h_mats[i].n);
   }
@@ -1111,8 +1113,9 @@ int set_gradients(lordo_ctx* c, const void* const* G, cudaStream_t st) {
   if (same) return LORDO_OK;
   const int slot = c->g_slot ^ 1;
   if (c->g_slot_used[slot]) CUDA_OK(c, cudaEventSynchronize(c->g_slot_ev[slot]));
-  const void** tab = c->h_Gtab + (size_t)slot * c->n_mats;
-  TmaGradMaps* gm = c->tc ? c->h_gmaps + (size_t)slot * c->n_mats : nullptr;
+  char* h = c->h_grads + (size_t)slot * c->slot_bytes;
+  const void** tab = reinterpret_cast<const void**>(h);
+  TmaGradMaps* gm = reinterpret_cast<TmaGradMaps*>(h + c->maps_at);
   if (c->tc) {
     for (int i = 0; i < c->n_mats; ++i) {
       const lordo_mat& a = c->mats[i];
@@ -1123,8 +1126,8 @@ int set_gradients(lordo_ctx* c, const void* const* G, cudaStream_t st) {
     }
   }
   for (int i = 0; i < c->n_mats; ++i) tab[i] = G[i];
-  cudaError_t e = cudaMemcpyAsync(c->d_Gtab, tab, sizeof(void*) * c->n_mats, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && c->tc) e = cudaMemcpyAsync(c->d_gmaps, gm, sizeof(TmaGradMaps) * c->n_mats, cudaMemcpyHostToDevice, st);
+  // one copy: a second took 1.5 us of the host (64 x 64 with fp32 storage, other pointers in every step, 29.6 us)
+  cudaError_t e = cudaMemcpyAsync(c->d_Gtab, h, c->slot_bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaEventRecord(c->g_slot_ev[slot], st);
   if (e != cudaSuccess) {
     // the device tables may be half written: force the next call to write them again
@@ -1209,10 +1212,8 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
 
   auto bail = [&](int code) { lordo_destroy(c); return code; };
   {  // one pinned block: an allocation takes some 80 us
-    const size_t status_at = (2 * sizeof(void*) * c->n_mats + 255) & ~size_t(255), maps_at = status_at + 256;
-    if (cudaHostAlloc((void**)&c->h_Gtab, maps_at + (c->tc ? 2 * sizeof(TmaGradMaps) * c->n_mats : 0), cudaHostAllocDefault) != cudaSuccess) return bail(LORDO_ERR_NOMEM);
-    c->h_status = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(c->h_Gtab) + status_at);
-    if (c->tc) c->h_gmaps = reinterpret_cast<TmaGradMaps*>(reinterpret_cast<char*>(c->h_Gtab) + maps_at);
+    if (cudaHostAlloc((void**)&c->h_grads, 2 * c->slot_bytes + 256, cudaHostAllocDefault) != cudaSuccess) return bail(LORDO_ERR_NOMEM);
+    c->h_status = reinterpret_cast<unsigned*>(c->h_grads + 2 * c->slot_bytes);
   }
   for (int sl = 0; sl < 2; ++sl)
     if (cudaEventCreateWithFlags(&c->g_slot_ev[sl], cudaEventDisableTiming) != cudaSuccess) return bail(LORDO_ERR_CUDA);
@@ -1690,7 +1691,7 @@ const char* lordo_last_error(const lordo_ctx* c) { return c ? c->err.c_str() : "
 
 int lordo_destroy(lordo_ctx* c) {
   if (!c) return LORDO_ERR_INVALID_ARG;
-  if (c->h_Gtab) cudaFreeHost(c->h_Gtab);
+  if (c->h_grads) cudaFreeHost(c->h_grads);
   for (int sl = 0; sl < 2; ++sl)
     if (c->g_slot_ev[sl]) cudaEventDestroy(c->g_slot_ev[sl]);
   for (const lordo_ctx::Span& sp : c->spans) { cudaEventDestroy(sp.a); cudaEventDestroy(sp.b); }

@@ -116,3 +116,26 @@ def test_fp32_storage_update_tiles(mats, ef):
     assert st["u"] < tol and st["v"] < 2 * tol and st["W"] < tol * 2 * 0.01 / 0.02, st
     assert not ef or st["E"] < tol, st
     opt.close()
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("count", [1, 33])
+def test_gradients_in_other_buffers_every_step(dt, count):
+    """The table of pointers and the tensor maps behind it, copied as one into either slot in turn: the same bits as
+    with every step's gradients copied into the buffers of the first."""
+    mats = [(72, 136, 16)] * count
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    G = [[torch.randn(2, m, n, device="cuda", generator=gen).to(dt) for m, n, _ in mats] for _ in range(4)]
+    kw = dict(check_mode=0, clip_rho=1.0, seed=1, g_dtype=dt, e_dtype=dt)
+    a, b = (lordo.Lordo(mats, 2, 8, [torch.zeros(m, n, dtype=dt) for m, n, _ in mats], **kw) for _ in range(2))
+    fixed = [g.clone() for g in G[0]]
+    for g in G:
+        a.inner_step(g, 0.01, 0.9, 0.9, 1)
+        for x, y in zip(fixed, g):
+            x.copy_(y)
+        b.inner_step(fixed, 0.01, 0.9, 0.9, 1)
+    assert a.poll_status() == 0 and b.poll_status() == 0
+    for x, y in zip(a.W + a.E + a.u + a.v, b.W + b.E + b.u + b.v):
+        assert torch.equal(x, y)
+    a.close()
+    b.close()
