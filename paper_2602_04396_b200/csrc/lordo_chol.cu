@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
   double* floors = piv + kB;                         // [2][kB] least pivots of this panel and the next
   double* Li = floors + 2 * kB;                      // [kB][kLd] inverse of the diagonal block of L
   __shared__ float wmax[kCholWarps];
-  __shared__ Plan plans[3], late;                    // of this panel, the next and the one after it; of blocks that find no unit at first
+  __shared__ Plan plans[3], late[2];                 // of this panel, the next and the one after it; of blocks that find no unit at first, in turn
   __shared__ float ga[2 * kB * kB];                  // the Gram matrix' diagonal blocks of this panel and the next, for warp 0
 
   // handed round, so that the compiler sees that the lanes of a warp agree on what depends on them
@@ -220,30 +220,34 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
   auto tile_block = [&](int k, int t) { return (int)rank + (int)csize * ((has(k) && t >= k / (int)csize) ? t + 1 : t); };
   // The panels behind the blocks' sums, dealt out to the units (a block above the diagonal has panels from itself on): every block has
   // a unit, those left over go, one after the other, to the block with the most panels a unit. With as many units for each
-  // block one was idle with three blocks, and a block of two panels had as many as one of fourteen. Laid down by one thread two panels
-  // ahead.
+  // block one was idle with three blocks, and a block of two panels had as many as one of fourteen. Laid down by a warp, two panels ahead or
+  // while it has nothing else to do: by one thread, between two barriers that all wait at, it took a tenth where a matrix has one CTA
+  // (r = 192 and 148 matrices 140 us, now 128; r = 256 and 300 543, now 494).
   auto lay_out = [&](Plan& pl, int k, int t0, int cnt) {
-    int n[kUnits], of[kUnits];
+    int block[kUnits], n[kUnits], of[kUnits];
+#pragma unroll
     for (int t = 0; t < kUnits; ++t) {
-      const int b = t < cnt ? tile_block(k, t0 + t) : 0;
-      pl.block[t] = b;
-      n[t] = b > k ? k : k - b;
+      block[t] = t < cnt ? tile_block(k, t0 + t) : 0;
+      n[t] = block[t] > k ? k : k - block[t];
       of[t] = t < cnt ? 1 : 0;
     }
-    for (int left = cnt > 0 ? kUnits - cnt : 0; left > 0; --left) {
-      int best = 0;
-      for (int t = 1; t < cnt; ++t)
-        if (n[t] * of[best] > n[best] * of[t]) best = t;
-      ++of[best];
+#pragma unroll
+    for (int left = 1; left < kUnits; ++left) {
+      if (cnt == 0 || left > kUnits - cnt) continue;
+      int best = 0, bn = n[0], bof = of[0];
+#pragma unroll
+      for (int t = 1; t < kUnits; ++t)
+        if (t < cnt && n[t] * bof > bn * of[t]) { best = t; bn = n[t]; bof = of[t]; }
+#pragma unroll
+      for (int t = 0; t < kUnits; ++t) of[t] += t == best ? 1 : 0;
     }
-    for (int t = 0, at = 0; t < kUnits; ++t) {
-      pl.first[t] = at;
-      pl.of[t] = of[t];
-      for (int x = 0; x < of[t]; ++x) { pl.tile[at + x] = t; pl.slice[at + x] = x; }
-      at += of[t];
+    int first = 0, mine = 0, count = 0, tile = -1, slice = 0;
+#pragma unroll
+    for (int t = 0, at = 0; t < kUnits; at += of[t], ++t) {
+      if (lane == t) { first = at; mine = block[t]; count = of[t]; }
+      if (lane >= at && lane < at + of[t]) { tile = t; slice = lane - at; }
     }
-    if (cnt == 0)
-      for (int x = 0; x < kUnits; ++x) pl.tile[x] = -1;
+    if (lane < kUnits) { pl.block[lane] = mine; pl.first[lane] = first; pl.of[lane] = count; pl.tile[lane] = tile; pl.slice[lane] = slice; }
   };
   auto a_diag = [&](int k, int j) {  // element (lane, j) of the Gram matrix' diagonal block; A is symmetric
     const int k0 = k * kB, kw = r - k0 < kB ? r - k0 : kB;
@@ -263,7 +267,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
     }
   };
   if (warp == 0) stage_diag(0);
-  if (warp > 1 && warp < 4 && lane == 0 && warp - 2 < nb) lay_out(plans[warp - 2], warp - 2, 0, min(tiles(warp - 2), kUnits));
+  if (warp > 1 && warp < 4 && warp - 2 < nb) lay_out(plans[warp - 2], warp - 2, 0, min(tiles(warp - 2), kUnits));
   __syncthreads();
 
 #pragma unroll 1
@@ -356,7 +360,7 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
       clear(c);  // not held in registers meanwhile
     } else if (warp < 3) {
       if (warp == 2 && k + 1 < nb) stage_diag(k + 1);
-      if (warp == 1 && lane == 0 && k + 2 < nb) lay_out(plans[(k + 2) % 3], k + 2, 0, min(tiles(k + 2), kUnits));
+      if (warp == 1 && k + 2 < nb) lay_out(plans[(k + 2) % 3], k + 2, 0, min(tiles(k + 2), kUnits));
       __syncwarp();
       if (k + 1 < nb) block_sum<true>(c, L, k0 + kB, L, k0 + kB, r, warp - 1, k, 2);
     } else if (warp == 7) {
@@ -386,6 +390,8 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
         const int b = pl.block[t];
         block_sum<false>(c, b > k + 1 ? L : Z, b * kB, L, k0 + kB, r, (b > k + 1 ? 0 : b) + pl.slice[u], k, pl.of[t]);
       }
+    } else if (!ahead && u == 0 && ntiles > kUnits) {
+      lay_out(late[0], k, kUnits, min(ntiles - kUnits, kUnits));
     }
 
     // ---- Z_k = M Lkk^-T, eight rows of a block per warp and turn; the panel's own rows of rinv are Lkk^-T itself
@@ -453,22 +459,23 @@ __global__ void __launch_bounds__(kCholWarps * 32, 1) chol_inverse_kernel(const 
         if (row < kw && col < kw) put(k, k0 + row, col, (float)Li[col * kLd + row], (float)Li[(col + 1) * kLd + row]);
       }
     }
-    for (int base = kUnits; base < ntiles; base += kUnits) {
-      const int cnt = ntiles - base < kUnits ? ntiles - base : kUnits;
+    for (int base = kUnits, i = 0; base < ntiles; base += kUnits, i ^= 1) {
+      const Plan& pl = late[i];
+      const int cnt = min(ntiles - base, kUnits), more = min(ntiles - base - kUnits, kUnits);
       __syncthreads();  // the blocks before are done with their sums
-      if (tid == 0) lay_out(late, k, base, cnt);
-      __syncthreads();
       if (u < kUnits) {
-        const int t = late.tile[u], b = late.block[t];
-        block_sum<false>(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + late.slice[u], k, late.of[t]);
+        const int t = pl.tile[u], b = pl.block[t];
+        block_sum<false>(c, b > k ? L : Z, b * kB, L, k0, r, (b > k ? 0 : b) + pl.slice[u], k, pl.of[t]);
         store_part(part + u * kPartDoubles, c);
         clear(c);
+      } else if (warp == 7 && more > 0) {
+        lay_out(late[i ^ 1], k, base + kUnits, more);
       }
       __syncthreads();
       for (int q = warp; q < cnt * 4; q += kCholWarps) {
-        const int b = late.block[q >> 2];
+        const int b = pl.block[q >> 2];
         gram_init(b, b * kB + (q & 3) * 8 + lr, g[0]);
-        finish(late, q >> 2, (q & 3) * 8, g[0]);
+        finish(pl, q >> 2, (q & 3) * 8, g[0]);
       }
     }
     // the panel is in memory for every CTA of the cluster

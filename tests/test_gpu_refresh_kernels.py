@@ -43,7 +43,7 @@ def test_gram_of_a_vocabulary_sized_matrix(shape, q):
     assert w["P_angle_bf16rhs"] < ANGLE_TOL, w
 
 
-@pytest.mark.parametrize("r,count", [(8, 1), (32, 1), (40, 3), (256, 2), (264, 40), (504, 1), (296, 80), (512, 75), (136, 3), (512, 16)])
+@pytest.mark.parametrize("r,count", [(8, 1), (32, 1), (40, 3), (256, 2), (264, 40), (504, 1), (296, 80), (512, 75), (136, 3), (512, 16), (192, 148), (256, 60)])
 def test_cholesky_panels_and_clusters(r, count):
     """The factorisation behind P_0 = Q of a 2r x r integer matrix, against a QR in fp64: one panel, whole and
     ragged panels, clusters of eight CTAs (few matrices) down to one (many), more blocks per CTA than it sums at
