@@ -302,10 +302,10 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
   c->d_mom_start = cv.take<long long>(n_mats + 1);
   c->d_wblk_start = cv.take<long long>(n_mats + 1);
   c->d_sblk_start = cv.take<long long>(n_mats + 1);
-  c->d_Gtab = cv.take<const void*>(n_mats);
-  c->maps_at = (sizeof(void*) * n_mats + 255) & ~size_t(255);
-  c->slot_bytes = c->maps_at + (c->tc ? sizeof(TmaGradMaps) * n_mats : 0);
-  if (c->tc) c->d_gmaps = cv.take<TmaGradMaps>(n_mats);
+  c->maps_at = (sizeof(void*) * n_mats + 127) & ~size_t(127);
+  c->slot_bytes = c->maps_at + (c->tc ? (c->tma ? 2 : 1) * 128 * (size_t)n_mats : 0);
+  c->d_Gtab = reinterpret_cast<const void**>(cv.take<char>(c->slot_bytes));
+  c->d_gmaps = reinterpret_cast<TmaGradMaps*>(reinterpret_cast<char*>(c->d_Gtab) + c->maps_at);
   c->d_status = cv.take<unsigned>(64);
   c->d_sumsq = cv.take<double>((size_t)n_mats * K);
   c->d_coef = cv.take<float>((size_t)n_mats * K);
@@ -1115,19 +1115,24 @@ int set_gradients(lordo_ctx* c, const void* const* G, cudaStream_t st) {
   if (c->g_slot_used[slot]) CUDA_OK(c, cudaEventSynchronize(c->g_slot_ev[slot]));
   char* h = c->h_grads + (size_t)slot * c->slot_bytes;
   const void** tab = reinterpret_cast<const void**>(h);
-  TmaGradMaps* gm = reinterpret_cast<TmaGradMaps*>(h + c->maps_at);
   if (c->tc) {
+    unsigned char* gm = reinterpret_cast<unsigned char*>(h + c->maps_at);
     for (int i = 0; i < c->n_mats; ++i) {
       const lordo_mat& a = c->mats[i];
-      const bool good = !c->tma ? encode_map3(gm[i].g_kb, G[i], a.n, a.m, c->K, 128, 32, false, true)
-                                : encode_map3(gm[i].g_sw, G[i], a.n, a.m, c->K, 64, 64, true) && encode_map3(gm[i].g_kb, G[i], a.n, a.m, c->K, 64, 128, true);
+      const bool good = !c->tma ? encode_map3(gm + 128 * i, G[i], a.n, a.m, c->K, 128, 32, false, true)
+                                : encode_map3(gm + 256 * i, G[i], a.n, a.m, c->K, 64, 64, true) && encode_map3(gm + 256 * i + 128, G[i], a.n, a.m, c->K, 64, 128, true);
       if (!good)
         return fail(c, LORDO_ERR_CUDA, "tensor map encoding failed for a gradient");
     }
   }
   for (int i = 0; i < c->n_mats; ++i) tab[i] = G[i];
-  // one copy: a second took 1.5 us of the host (64 x 64 with fp32 storage, other pointers in every step, 29.6 us)
-  cudaError_t e = cudaMemcpyAsync(c->d_Gtab, h, c->slot_bytes, cudaMemcpyHostToDevice, st);
+  // One copy where it can be: up to 1024 bytes it holds the stream up for 4 us, above that for 9. Two where either is that short and both
+  // together are not (four matrices with bf16 storage). Steps on other buffers each time, us, with two copies always and now: 256 x 256,
+  // K = 1, in fp32 38 and 30, seven of them 47 and 32, in bf16 31 and 27, seven 38 and 35.
+  const size_t maps = c->slot_bytes - c->maps_at;
+  const bool apart = c->slot_bytes > 1024 && maps > 0 && maps <= 1024;
+  cudaError_t e = cudaMemcpyAsync(c->d_Gtab, h, apart ? c->maps_at : c->slot_bytes, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && apart) e = cudaMemcpyAsync(c->d_gmaps, h + c->maps_at, maps, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaEventRecord(c->g_slot_ev[slot], st);
   if (e != cudaSuccess) {
     // the device tables may be half written: force the next call to write them again

@@ -149,6 +149,8 @@ struct alignas(128) TmaMatMaps {
 struct alignas(128) TmaGradMaps {  // re-encoded whenever the caller's gradient pointer changes
   unsigned char g_sw[128], g_kb[128];
 };
+// ... with fp32 storage one map per matrix, of boxes of 32 rows x 128 columns as they are stored
+__device__ __forceinline__ const unsigned char* grad_map_f32(const TmaGradMaps* maps, int mat) { return maps->g_sw + 128ll * mat; }
 
 struct TcPrep {
   const float* P;              // [m][r]

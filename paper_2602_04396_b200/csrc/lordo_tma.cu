@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(kAThreads, 1) apply_tma_kernel(const TcProblem
           const bool ld_e = DO_E && ef;
           mbar_expect_tx(&in_full[is], 16384u + (ld_e ? 16384u : 0u) + (DO_W ? 16384u : 0u), one);
           if (F32) {  // one box of 32 rows x 128 columns per tile
-            tma_load_3d(base, gm->g_kb, n0, t * ROWS, rep, &in_full[is], one);
+            tma_load_3d(base, grad_map_f32(gmaps, pr->mat), n0, t * ROWS, rep, &in_full[is], one);
             if (ld_e) tma_load_3d(base + EOFF, mm->e_kb, n0, t * ROWS, rep, &in_full[is], one);
             tma_load_3d(base + WOFF, mm->w_kb, n0, t * ROWS, rep, &in_full[is], one);
           } else if (SIDE == 1 || (SIDE == 2 && pr->tr)) {  // one box of 128 stored rows x 64 stored columns per tile
