@@ -152,6 +152,7 @@ struct lordo_ctx {
   std::vector<SketchBufs> h_skbufs;  // per matrix: bf16 right-hand sides of the sketch products (refresh scratch)
   std::vector<PlanStep> inner_proj, inner_apply;  // one launch per side present
   std::vector<PlanStep> refresh_steps, init_steps;
+  bool products_ok = true;         // every fp32 product is one that its kernel takes
   std::vector<PlanStep> tb_steps;  // Delta rebuilt from the time buffers (lordo_outer_step with time_buffer)
 
   // pinned host staging
@@ -258,6 +259,12 @@ Operand plain(const void* p0, long long ld, int dt0 = LORDO_F32) {
   std::memset(&o, 0, sizeof(o));
   o.p0 = p0; o.ld = ld; o.dt0 = dt0; o.dt1 = LORDO_F32; o.kind = OP_PLAIN;
   return o;
+}
+
+// What the fp32 products take for granted: four elements along the contiguous side of an operand are inside or outside together and
+// 16 bytes in step (8 in bf16), and the second product's operand lies as the first's.
+bool product_fits(const GemmProblem& g, int atrans, int dual) {
+  return (atrans ? g.M : g.Kd) % 4 == 0 && g.N % 4 == 0 && g.A.ld % 4 == 0 && g.B.ld % 4 == 0 && (!dual || g.B2.ld == g.B.ld);
 }
 
 long long clip_chunk(const lordo_config& cfg) {
@@ -487,6 +494,7 @@ size_t build(lordo_ctx* c, const lordo_buffers* buf, void* ws) {
       if (st.type == ST_GEMM) {
         st.first = (long long)P.size(); st.count = (int)sl.g.size(); st.tiles = 0;
         for (GemmProblem& g : sl.g) {
+          c->products_ok = c->products_ok && product_fits(g, st.atrans, st.dual);
           g.tile_start = st.tiles;
           st.tiles += (long long)((g.M + 63) / 64) * g.tiles_n;
           P.push_back(g);
@@ -1184,7 +1192,7 @@ int lordo_query_workspace(const lordo_config* cfg, size_t* bytes) {
   tmp.cfg = *cfg;
   tmp.n_mats = cfg->n_mats; tmp.K = cfg->K;
   *bytes = build(&tmp, nullptr, nullptr);
-  return LORDO_OK;
+  return tmp.products_ok ? LORDO_OK : LORDO_ERR_ALIGN;
 }
 
 int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspace, size_t workspace_bytes, void* stream,
@@ -1214,6 +1222,7 @@ int lordo_init(const lordo_config* cfg, const lordo_buffers* buf, void* workspac
   c->n_mats = cfg->n_mats; c->K = cfg->K;
   const size_t need = build(c, buf, workspace);
   if (need > workspace_bytes) { delete c; return LORDO_ERR_NOMEM; }
+  if (!c->products_ok) { delete c; return LORDO_ERR_ALIGN; }
 
   auto bail = [&](int code) { lordo_destroy(c); return code; };
   {  // one pinned block: an allocation takes some 80 us

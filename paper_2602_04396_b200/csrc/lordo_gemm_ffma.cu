@@ -32,7 +32,8 @@ struct Raw {
 };
 // What one thread fetches of an operand, slice after slice: once or twice four elements, where they are next, how far the ones after them, and
 // their k (of the row, or of the first of the four where k runs along the contiguous side). The contiguous side of every operand is
-// a multiple of four, so four elements are inside or outside together.
+// a multiple of four, so four elements are inside or outside together; with two products and eight rows a thread the second
+// four come from B2 at B's index, so both have one ld (the plans are checked for either).
 struct Feed {
   long long at, step, second;
   int k, second_k, end, second_end;  // end: the contraction's length, or 0 where the other side's index is outside

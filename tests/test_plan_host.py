@@ -110,6 +110,17 @@ def test_a_range_of_k_has_at_most_64_steps(plan, rows, pairs_of_planes, most, ti
     assert ns <= max(most, (steps + 63) // 64)
 
 
+@pytest.mark.parametrize("kw", [dict(), dict(variant=lordo.LOCAL, power_iters=1), dict(sides=(1, 0)), dict(oversample=8, power_iters=1), dict(time_buffer=1),
+                                dict(check_mode=0), dict(w_dtype=lordo.BF16, g_dtype=lordo.BF16, e_dtype=lordo.BF16, check_mode=0)])
+def test_every_product_is_one_that_its_kernel_takes(kw):
+    """The plans of every kind of run at the least multiples of n, r (and m, projected from the right) that are accepted: extents and
+    strides of the fp32 products' operands are multiples of four, the second product's operand lies as the first's. A plan
+    that breaks this is refused."""
+    m = 1000 if "sides" in kw else 1001
+    cfg, _keep = lordo.make_config([(m, 72, 8), (129, 1336, 24)], 3, 2, **kw)
+    assert lordo.query_workspace(cfg) > 0
+
+
 def test_workspace_holds_the_ranges_of_tall_matrices():
     """The partial Gram matrices are sized by the same rule: more rows never need fewer of them."""
     def size(m, **kw):
