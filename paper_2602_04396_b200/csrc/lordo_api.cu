@@ -1457,8 +1457,7 @@ int lordo_inner_step(lordo_ctx* c, const void* const* G, float lr, float beta1, 
     } else {
     {
       ProfScope ps(c, st, PC_PROJECT);  // includes the moment update (fused epilogue)
-      launch_project_tc(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips, c->tc_rn_max, c->tc_steps_min, c->sm_count, ss, c->cfg.w_dtype == LORDO_BF16,
-                        c->d_status, st);
+      launch_project_tc(c->d_tc_probs, (int)c->h_tc.size(), c->tc_strips, c->tc_rn_max, c->tc_steps_min, c->sm_count, ss, c->d_status, st);
     }
     {
       ProfScope ps(c, st, PC_APPLY);

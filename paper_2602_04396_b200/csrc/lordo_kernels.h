@@ -162,10 +162,10 @@ struct TcPrep {
 
 cudaError_t tc_configure(int r_n_max);
 void launch_prep_projection(const TcPrep* items, const long long* blk_start, int nitems, long long total_blocks, cudaStream_t st);
-// bf16 != 0: G, E, W are all bf16; else all fp32 (mixed storage runs on the fp32 path).
+// G and E in fp32, ranks up to 256 (mixed storage and larger ranks run on the fp32 path).
 void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, int steps, int sm_count, const StepScalars& sc,
-                       int bf16, unsigned* status, cudaStream_t st);
-// TMA-fed persistent kernels for bf16 storage (lordo_tma.cu).
+                       unsigned* status, cudaStream_t st);
+// TMA-fed persistent kernels (lordo_tma.cu): all of bf16 storage, the update of fp32 storage.
 cudaError_t tma_configure();      // bf16 storage
 cudaError_t tma_configure_f32();  // fp32 storage
 int project_pairs(int sm_count);  // CTA pairs of the projection that the device holds at once

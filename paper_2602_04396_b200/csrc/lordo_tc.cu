@@ -35,28 +35,16 @@ __device__ __forceinline__ int find_problem(const TcProblem* __restrict__ probs,
   return lo;
 }
 
-// Storage type of G, E and W inside the tensor-core kernels: all bf16 or all fp32. Loads are kept
-// as raw values in registers (no use before the whole batch has been issued), converted afterwards.
+// Storage type of G and E: fp32 alone (bf16 storage takes the TMA-fed projection), although the kernel is written for either and for ranks up
+// to 512: as a plain function its loop compiles into one that is up to 2 % slower, and without the branches for ranks above 256, which
+// nothing reaches, up to 5 % (2832 x 752, r = 256, K = 1 104.9 and 109.5 us).
 template <bool BF16>
 struct Elem;
-template <>
-struct Elem<true> {
-  using one = unsigned short;
-  using pair = uint32_t;
-  static __device__ __forceinline__ float cvt(one x) { return __uint_as_float(((uint32_t)x) << 16); }
-  static __device__ __forceinline__ float2 cvt2(pair x) { return make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u)); }
-  static __device__ __forceinline__ one pack(float v) {
-    const __nv_bfloat16 h = __float2bfloat16_rn(v);
-    return *reinterpret_cast<const unsigned short*>(&h);
-  }
-};
 template <>
 struct Elem<false> {
   using one = float;
   using pair = float2;
-  static __device__ __forceinline__ float cvt(one x) { return x; }
   static __device__ __forceinline__ float2 cvt2(pair x) { return x; }
-  static __device__ __forceinline__ one pack(float v) { return v; }
 };
 
 }  // namespace
@@ -202,7 +190,7 @@ __global__ void __launch_bounds__(kProjThreads, 2) project_tc_kernel(const TcPro
         const int idx = tid + t * 256;
         if (idx < pt_chunks) *reinterpret_cast<uint4*>(sB + swz_chunk(idx >> 3, idx & 7)) = pt[t];
       }
-      if (r_n > 256) {  // rows 256.. of the P^T tile (r up to 512)
+      if (r_n > 256) {  // rows 256.. of the P^T tile: not reached, see Elem
         for (int idx = 2048 + tid; idx < pt_chunks; idx += 256) {
           const uint4 v = *reinterpret_cast<const uint4*>(PT + (long long)(idx >> 3) * m_k + kb * 64 + (idx & 7) * 8);
           *reinterpret_cast<uint4*>(sB + swz_chunk(idx >> 3, idx & 7)) = v;
@@ -353,8 +341,6 @@ size_t project_tc_smem(int r_n_max) {
   return std::max(2 * stage, (nch - nch / 4) * 16 * kStrip * sizeof(float)) + 1024;
 }
 cudaError_t tc_configure(int r_n_max) {
-  const cudaError_t e = cudaFuncSetAttribute(project_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
-  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(project_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)project_tc_smem(r_n_max));
 }
 
@@ -363,7 +349,7 @@ void launch_prep_projection(const TcPrep* items, const long long* blk_start, int
 }
 // `steps`: 64-row steps of the problem with the fewest
 void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strips, int r_n_max, int steps, int sm_count, const StepScalars& sc,
-                       int bf16, unsigned* status, cudaStream_t st) {
+                       unsigned* status, cudaStream_t st) {
   // two CTAs fit an SM; each is left four steps at least
   int c = 1;
   while (c < 4 && total_strips * 2 * c <= 2 * (long long)sm_count && steps >= 8 * c) c *= 2;
@@ -375,7 +361,6 @@ void launch_project_tc(const TcProblem* probs, int nprobs, long long total_strip
   at.val.clusterDim.x = (unsigned)c; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
   lc.gridDim = dim3((unsigned)(total_strips * c), 1, 1); lc.blockDim = dim3(kProjThreads, 1, 1); lc.dynamicSmemBytes = project_tc_smem(r_n_max);
   lc.stream = st; lc.attrs = &at; lc.numAttrs = c > 1 ? 1 : 0;
-  if (bf16) cudaLaunchKernelEx(&lc, project_tc_kernel<true>, probs, nprobs, sc, status);
-  else cudaLaunchKernelEx(&lc, project_tc_kernel<false>, probs, nprobs, sc, status);
+  cudaLaunchKernelEx(&lc, project_tc_kernel<false>, probs, nprobs, sc, status);
 }
 }  // namespace lordo
