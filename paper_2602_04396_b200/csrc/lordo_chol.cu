@@ -41,7 +41,7 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
 // Sums of products of rows: lane l of a warp holds rows l/4 + 8i of both 32-row blocks (rows from r on read as
 // zeros). The columns may be dealt to the lanes in any order as long as it is the same on both sides.
 // DIAG: both blocks are the same one, so its rows are fetched once and only the 8 x 8 tiles on and above the diagonal are
-// multiplied (every CTA of a cluster sums the diagonal block for itself: r = 512, 16 matrices
+// multiplied (every CTA of a cluster sums the diagonal block for itself: in the kernel whose factor took roots, r = 512, 16 matrices
 // 359 -> 345 us, r = 256, 7 matrices 90 -> 88 us).
 // c += X_cols L_cols^T over 8 columns from `col` on.
 template <bool DIAG>
@@ -497,13 +497,8 @@ static cudaLaunchConfig_t chol_launch(cudaLaunchAttribute* at, int nprobs, int c
   return lc;
 }
 
-// CTAs per problem: as many, up to the portable cluster size, as leave every problem a place on the device at
-// once (fifteen clusters of seven or eight fit, 22 of six: r = 512, 16 problems 375 us with four CTAs each, 325 with
-// six) and every CTA about two row blocks.
 void launch_chol_inverse(const CholProblem* probs, int nprobs, int r_max, unsigned* status, cudaStream_t st) {
-  const int panels = (r_max + kB - 1) / kB;
-  int c = 8;
-  while (c > 1 && (2 * c > panels + 1 || nprobs > g_clusters[c])) --c;
+  const int c = factor_ctas((r_max + kB - 1) / kB, nprobs, g_clusters);
   cudaLaunchAttribute at[2];
   const cudaLaunchConfig_t lc = chol_launch(at, nprobs, c, st);
   cudaLaunchKernelEx(&lc, chol_inverse_kernel, probs, status);

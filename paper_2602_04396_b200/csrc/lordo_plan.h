@@ -26,6 +26,16 @@ inline int k_ranges(long long tiles, long long steps, long long most, long long 
   return (int)best;
 }
 
+// CTAs per matrix of the factorisation: as many, up to the portable cluster size, as leave every matrix a place on the device at once (`fits`:
+// clusters of that many CTAs that the device holds) and every CTA about two row blocks. r = 512, 16 matrices, us: one CTA each 906, two 524,
+// four 321, six 288; seven or eight, of which fifteen clusters fit, 519 and 396. r = 256, 7 matrices: 162, 96, with four 76. Above 75 matrices
+// one CTA each: 300 of r = 256 would take a tenth less in two, but 148 of r = 192 a tenth more.
+inline int factor_ctas(int panels, int matrices, const int* fits) {
+  int c = 8;
+  while (c > 1 && (2 * c > panels + 1 || matrices > fits[c])) --c;
+  return c;
+}
+
 // A piece of work of one CTA (update) or CTA pair (projection) of the TMA-fed kernels: steps [t0, t1) of one strip, of 64 rows
 // each with bf16 storage and of 32 with fp32 (as many bytes), or one pair of strips. Workers walk their own part of a list, [start[w], start[w + 1]), dealt out by lordo_init so
 // that all of them end together.

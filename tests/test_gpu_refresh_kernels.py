@@ -47,8 +47,8 @@ def test_gram_of_a_vocabulary_sized_matrix(shape, q):
 def test_cholesky_panels_and_clusters(r, count):
     """The factorisation behind P_0 = Q of a 2r x r integer matrix, against a QR in fp64: one panel, whole and
     ragged panels, clusters of eight CTAs (few matrices) down to one (many), more blocks per CTA than it sums at
-    once (r = 296, 512 in one CTA), one to four blocks for four units (r = 136 in two CTAs, 512 in six). The condition of such a matrix is about 6 (the ratio of the edges of its
-    singular values): CholeskyQR2 in fp32 is off by a small multiple of 6^2 2^-24 = 2e-6."""
+    once (r = 192, 296, 512 in one CTA), one to four blocks for four units (test_plan_host.py holds the counts). The condition of such a matrix
+    is about 6 (the ratio of the edges of its singular values): CholeskyQR2 in fp32 is off by a small multiple of 6^2 2^-24 = 2e-6."""
     mats = [(2 * r, r, r)] * count
     opt = lordo.Lordo(mats, 1, 1, [torch.zeros(2 * r, r)] * count, check_mode=0, seed=5)
     assert opt.poll_status() == 0

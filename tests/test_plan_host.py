@@ -28,6 +28,7 @@ extern "C" int split(int n, const int* slices, const int* tiles, int carry, int 
   const lordo::ProductSplit s = carry ? lordo::split_by_time(runs, sms) : lordo::split_by_turns(runs, sms);
   return 10 * s.rows + s.ctas;
 }
+extern "C" int factor(int panels, int matrices, const int* fits) { return lordo::factor_ctas(panels, matrices, fits); }
 extern "C" int ranges(long long tiles, long long steps, long long most, long long pairs) { return lordo::k_ranges(tiles, steps, most, pairs); }
 """
 
@@ -171,3 +172,13 @@ def test_fp32_products_split_of_any_launch(plan, carry, sms):
         got = plan.split(n, (C.c_int * n)(*[s for s, _ in runs]), (C.c_int * n)(*[t for _, t in runs]), carry, sms)
         rows, ctas = got // 10, got % 10
         assert rows in ((4, 8) if carry else (4,)) and ctas in (1, 2, 4, 8) and (ctas == 1 or max(s for s, _ in runs) >= 2 * ctas)
+
+
+# the cases of the factorisation's GPU test: CTAs per matrix on a B200 and row blocks of a CTA at most (up to four have a unit each, of which
+# those left over help; with more, some blocks wait for a second batch, or with more than eight beside the diagonal's a third)
+@pytest.mark.parametrize("r,count,ctas,blocks", [(8, 1, 1, 1), (32, 1, 1, 1), (40, 3, 1, 2), (256, 2, 4, 2), (264, 40, 3, 3), (504, 1, 8, 2), (296, 80, 1, 10),
+                                                 (512, 75, 1, 16), (136, 3, 3, 2), (512, 16, 6, 3), (192, 148, 1, 6), (256, 60, 2, 4)])
+def test_ctas_of_the_factorisation(plan, r, count, ctas, blocks):
+    fits = (C.c_int * 9)(0, 148, 74, 45, 33, 26, 22, 15, 15)  # clusters of 0 to 8 CTAs that a B200 holds
+    panels = (r + 31) // 32
+    assert plan.factor(panels, count, fits) == ctas and (panels + ctas - 1) // ctas == blocks
