@@ -27,9 +27,9 @@ inline int k_ranges(long long tiles, long long steps, long long most, long long 
 }
 
 // CTAs per matrix of the factorisation: as many, up to the portable cluster size, as leave every matrix a place on the device at once (`fits`:
-// clusters of that many CTAs that the device holds) and every CTA about two row blocks. r = 512, 16 matrices, us: one CTA each 906, two 524,
-// four 321, six 288; seven or eight, of which fifteen clusters fit, 519 and 396. r = 256, 7 matrices: 162, 96, with four 76. Above 75 matrices
-// one CTA each: 300 of r = 256 would take a tenth less in two, but 148 of r = 192 a tenth more.
+// clusters of that many CTAs that the device holds) and every CTA about two row blocks. r = 512, 16 matrices, us: one CTA each 828, two 499,
+// four 301, six 275; seven or eight, of which fifteen clusters fit, 504 and 392. r = 256, 7 matrices: 150, 97, with four 76. Above 74 matrices
+// one CTA each: 148 of r = 192 take 128 us that way, 152 in two, 300 of r = 256 488 and 480.
 inline int factor_ctas(int panels, int matrices, const int* fits) {
   int c = 8;
   while (c > 1 && (2 * c > panels + 1 || matrices > fits[c])) --c;
@@ -212,8 +212,8 @@ inline ProductSplit split_by_turns(const std::vector<ProductRun>& runs, int sms)
 
 // Sums carried in fp64 (check mode): the rows and CTAs whose launch is over first by product_time. Turns of CTAs as long as the longest contraction
 // told eight rows from four only where the contractions are alike: matrices of 5472 rows, r = 120 and of 64 to 3704 rows, r <= 40
-// took 209 us in pairs of eight rows by that rule, 87 in fours of four rows, and take 71 now. Over 482 launches of parity runs of random
-// shapes the choice takes at most 1.015 of the best split's time for nine of ten, and 1.25 for the worst (by turns 1.2 and 3.2).
+// took 209 us in pairs of eight rows by that rule, 87 in fours of four rows, and take 71 now. Over 790 launches of parity runs of random
+// shapes the choice takes at most 1.02 of the best split's time for nine of ten, and 1.3 for the worst (by turns 1.2 and 3.2).
 // A launch of more than 2048 tiles is timed as one of that many: the same choice, and a bounded time to make it in.
 inline ProductSplit split_by_time(std::vector<ProductRun> runs, int sms) {
   const int slices = longest_run(runs);
