@@ -142,6 +142,9 @@ typedef struct {
 LORDO_API int lordo_query_workspace(const lordo_config* cfg, size_t* bytes);
 
 /*
+ * Needs an sm_100a device; with check_mode = 0 and one storage type throughout (bf16 with r <= 512, fp32 with
+ * r <= 256 and side 0) also a driver that offers cuTensorMapEncodeTiled (CUDA 12.0 or later), else LORDO_ERR_CUDA.
+ *
  * Algorithm 1 / 2 "Require": copies W[0] to every replica and to X0, zeroes E, u, v, B, Delta,
  * writes P_0 (Global: orthonormalised random matrix from `seed`; Local: first r columns of the
  * identity for every worker). Synchronises `stream` before returning. `*out` owns host memory

@@ -37,8 +37,8 @@ inline int factor_ctas(int panels, int matrices, const int* fits) {
 }
 
 // A piece of work of one CTA (update) or CTA pair (projection) of the TMA-fed kernels: steps [t0, t1) of one strip, of 64 rows
-// each with bf16 storage and of 32 with fp32 (as many bytes), or one pair of strips. Workers walk their own part of a list, [start[w], start[w + 1]), dealt out by lordo_init so
-// that all of them end together.
+// each with bf16 storage and of 32 with fp32 (as many bytes), or one pair of strips. Workers walk their own part of a list,
+// [start[w], start[w + 1]), dealt out by lordo_init so that all of them end together.
 struct TcSeg {
   int prob, strip, t0, t1;
 };
