@@ -61,16 +61,21 @@ constexpr int kPieceHead = 4;  // steps that a piece costs on top of its own: it
 //          before it. Returns -1 where something has no place. A worker is cut at most once, being left with less room
 //          than a piece needs, so there are at most items + workers pieces.
 enum Dealing { WHOLE, EVEN, WITHIN };
-inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, int least, double share, std::vector<std::vector<TcSeg>>& lists) {
+struct Dealt {
   typedef std::pair<double, int> Load;  // what a worker has, the worker
-  std::vector<Load> heap;
-  for (int w = 0; w < (int)lists.size(); ++w) { lists[w].clear(); heap.push_back(Load(0.0, w)); }
-  const auto later = [](const Load& a, const Load& b) { return a > b; };
+  std::vector<TcSeg> piece;
+  std::vector<int> worker;    // of a piece
+  std::vector<Load> least;    // a heap, the worker with the least first
+};
+inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, int least, double share, int workers, Dealt& d) {
+  d.piece.clear();
+  d.worker.clear();
+  d.least.clear();
+  for (int w = 0; w < workers; ++w) d.least.push_back(Dealt::Load(0.0, w));
   double longest = 0.0;
   for (const WorkItem& it : items) {
     for (int t0 = 0; t0 < it.len;) {
-      std::pop_heap(heap.begin(), heap.end(), later);
-      Load& ld = heap.back();
+      Dealt::Load ld = d.least.front();
       const int rest = it.len - t0, room = (int)(share - ld.first - head + 0.5);
       int n = rest;
       if (how == EVEN && n > room) {
@@ -80,11 +85,19 @@ inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, int l
         n = std::min(room, rest - least);
         if (n < least) return -1;
       }
-      lists[ld.second].push_back({it.prob, it.strip, t0, t0 + n});
+      d.piece.push_back({it.prob, it.strip, t0, t0 + n});
+      d.worker.push_back(ld.second);
       ld.first += how == WHOLE ? it.cost + head : n + head;
       longest = std::max(longest, ld.first);
       t0 += n;
-      std::push_heap(heap.begin(), heap.end(), later);
+      int at = 0;
+      for (int c = 1; c < workers; c = 2 * at + 1) {
+        if (c + 1 < workers && d.least[c + 1] < d.least[c]) ++c;
+        if (ld < d.least[c]) break;
+        d.least[at] = d.least[c];
+        at = c;
+      }
+      d.least[at] = ld;
     }
   }
   return (int)(longest + 0.5);
@@ -92,13 +105,10 @@ inline int deal(const std::vector<WorkItem>& items, Dealing how, int head, int l
 
 // How long the workers of a cut or uncut list take, in steps of a worker that has the memory to itself: up to `busy` of them run at that
 // pace, more share what the memory gives.
-inline double time_of(const std::vector<std::vector<TcSeg>>& lists, int head, int busy) {
+inline double time_of(const Dealt& d, int busy) {
   std::vector<double> load;
-  for (const std::vector<TcSeg>& l : lists) {
-    double x = 0.0;
-    for (const TcSeg& s : l) x += s.t1 - s.t0 + head;
-    if (x > 0.0) load.push_back(x);
-  }
+  for (const Dealt::Load& l : d.least)
+    if (l.first > 0.0) load.push_back(l.first);
   std::sort(load.begin(), load.end());
   double t = 0.0, before = 0.0;
   for (size_t i = 0; i < load.size(); ++i) {
@@ -118,31 +128,29 @@ inline double time_of(const std::vector<std::vector<TcSeg>>& lists, int head, in
 // 40 strips 50, 83, 43 us; 120 strips 122, 107, 121 us; 256 strips 241, 241, 245 us; mixes that it called 4 to 8 % better were 2 to 5 % slower.
 inline void deal_out(std::vector<WorkItem> items, int workers, bool split, int head, int shortest, int busy, std::vector<TcSeg>& list, std::vector<int>& start) {
   std::stable_sort(items.begin(), items.end(), [](const WorkItem& a, const WorkItem& b) { return a.cost > b.cost; });
-  std::vector<std::vector<TcSeg>> lists(workers);
-  const int longest = deal(items, WHOLE, head, shortest, 0.0, lists);
+  Dealt dealt;
+  const int longest = deal(items, WHOLE, head, shortest, 0.0, workers, dealt);
   if (split) {
     double total = 0.0;
     for (const WorkItem& it : items) total += it.cost + head;
-    std::vector<std::vector<TcSeg>> even(workers), cut(workers), within;
-    deal(items, EVEN, head, shortest, std::max(total / workers + head / 2.0, (double)(shortest + head)), even);
-    size_t pieces = 0;
-    for (const std::vector<TcSeg>& l : even) pieces += l.size();
+    Dealt even, cut, within;
+    deal(items, EVEN, head, shortest, std::max(total / workers + head / 2.0, (double)(shortest + head)), workers, even);
     int least = std::max((int)(total / workers), shortest + head) - 1, share = longest;  // nothing below, everything at WHOLE's longest
     while (share - least > 1) {
       const int mid = least + (share - least) / 2;
-      if (deal(items, WITHIN, head, shortest, mid, cut) < 0) least = mid;
-      else { share = mid; within.swap(cut); cut.resize(workers); }
+      if (deal(items, WITHIN, head, shortest, mid, workers, cut) < 0) least = mid;
+      else { share = mid; std::swap(within, cut); }
     }
-    if (!within.empty() && time_of(within, head, busy) < time_of(lists, head, busy)) lists.swap(within);
-    const bool fits = pieces <= items.size() + workers;  // the room that the table has; either of the others does
-    if (fits && time_of(lists, head, busy) > 0.9 * time_of(even, head, busy)) lists.swap(even);
+    if (!within.piece.empty() && time_of(within, busy) < time_of(dealt, busy)) std::swap(dealt, within);
+    const bool fits = even.piece.size() <= items.size() + workers;  // the room that the table has; either of the others does
+    if (fits && time_of(dealt, busy) > 0.9 * time_of(even, busy)) std::swap(dealt, even);
   }
-  list.clear();
-  start.assign(1, 0);
-  for (const std::vector<TcSeg>& l : lists) {
-    list.insert(list.end(), l.begin(), l.end());
-    start.push_back((int)list.size());
-  }
+  start.assign(workers + 1, 0);
+  for (int w : dealt.worker) ++start[w + 1];
+  for (int w = 0; w < workers; ++w) start[w + 1] += start[w];
+  list.resize(dealt.piece.size());
+  std::vector<int> next(start.begin(), start.end() - 1);
+  for (size_t i = 0; i < dealt.piece.size(); ++i) list[next[dealt.worker[i]]++] = dealt.piece[i];
   while (start.size() > 1 && start[start.size() - 2] == (int)list.size()) start.pop_back();
 }
 
